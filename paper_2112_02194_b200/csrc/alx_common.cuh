@@ -188,21 +188,27 @@ struct CgOptions {
 // alx_umma.cu: tensor-core path, d = 128 and bf16 tables only
 int64_t gramian_umma_partials();
 cudaError_t launch_gramian_umma(const void *X, int64_t n, float *partials, cudaStream_t s, int64_t *launches);
-// ---- evaluation (alx_eval.cu, alx_topk_umma.cu)
-// slabs of items per query tile (each slab's best k are listed separately and merged)
-int topk_slabs(int64_t n_items, int64_t m);
-// exact Top-K of <q, h_i>: H [n_items x d] (storage type), Q [m x d] fp32; lists: [slabs][m][k] scratch;
-// ids_out [m x k] (-1 where fewer than k items qualify), scores_out [m x k] or nullptr; ex_*: per-query ids to leave out
-cudaError_t launch_topk(const void *H, bool bf16, int64_t n_items, int d, const float *Q, int64_t m, int k,
-                        const int64_t *ex_ptr, const int32_t *ex_idx, int slabs, float *list_s, int32_t *list_id,
-                        int32_t *list_cnt, int32_t *ids_out, float *scores_out, bool tensor_cores, void *scratch_q,
+// ---- evaluation (alx_topk.cu, alx_topk_umma.cu, alx_eval.cu)
+// exact Top-K of <q, h_i>: H [n_items x d] (storage type), Q [m x d] fp32; ids_out [m x k] (-1 where fewer than k items
+// qualify), scores_out [m x k] or nullptr; ex_*: per-query ids to leave out
+struct TopkPlan {
+    static constexpr int kMostPhases = 8;
+    struct Phase {
+        int64_t begin, end, slab;  // items of the phase; items per slab
+        int slabs;
+    };
+    bool tensor_cores;
+    int cap, qt, tile_items;       // elements of a candidate list; queries per block; items per step of a block
+    int phases;
+    Phase phase[kMostPhases];
+    int64_t m_batch;               // queries per batch
+    int64_t list_bytes, cnt_bytes, tau_bytes, carry_bytes, query_bytes;
+    int64_t workspace_bytes() const { return list_bytes + cnt_bytes + tau_bytes + carry_bytes + query_bytes; }
+};
+TopkPlan topk_plan(int64_t n_items, int64_t m, int k, bool tensor_cores);
+cudaError_t launch_topk(const TopkPlan &p, const void *H, bool bf16, int64_t n_items, int d, const float *Q, int64_t m, int k,
+                        const int64_t *ex_ptr, const int32_t *ex_idx, void *workspace, int32_t *ids_out, float *scores_out,
                         DevStatus *st, cudaStream_t s, int64_t *launches);
-// the tensor-core scoring kernel (d = 128, bfloat16 table); scratch_q: topk_query_scratch_bytes(m) bytes for the queries'
-// bfloat16 parts
-int64_t topk_query_scratch_bytes(int64_t m);
-cudaError_t launch_topk_umma(const void *H, int64_t n_items, const float *Q, int64_t m, int k, const int64_t *ex_ptr,
-                             const int32_t *ex_idx, int slabs, int64_t slab, float *list_s, int32_t *list_id,
-                             int32_t *list_cnt, void *scratch_q, DevStatus *st, cudaStream_t s, int64_t *launches);
 cudaError_t launch_recall(const int32_t *ids, int64_t m, int k_stride, int k, const int64_t *tptr, const int32_t *tidx,
                           double *per_query, double *out2, cudaStream_t s, int64_t *launches);
 cudaError_t launch_rows_fold(const SideView &sv, const int64_t *class_offs_host, int64_t n_chunks, int64_t n_split_rows,
