@@ -370,10 +370,11 @@ alx_status half_epoch_impl(alx_ctx *c, int side, const int32_t *cap_slot, float 
                                             c->stream));
         }
     } else {
-        ALX_CUDA(c, launch_rows_simple(side_view(c, side), c->class_offs[side], c->n_chunks[side],
-                                       c->n_split_rows[side], c->table[fixed], c->bf16, c->opt.d, c->Bmat,
-                                       c->split_partials, out, c->status, c->stream, &c->launches));
-        c->stats.kernel_path[side] = 0;
+        const bool warp_rows = c->opt.kernels != 1 && c->opt.d <= 64;
+        ALX_CUDA(c, (warp_rows ? launch_rows_warp : launch_rows_simple)(side_view(c, side), c->class_offs[side], c->n_chunks[side],
+                                                                       c->n_split_rows[side], c->table[fixed], c->bf16, c->opt.d, c->Bmat,
+                                                                       c->split_partials, out, c->status, c->stream, &c->launches));
+        c->stats.kernel_path[side] = warp_rows ? 1 : 0;
         c->dual_candidates = 0;
     }
     ALX_CUDA(c, cudaEventRecord(c->ev[2], c->stream));

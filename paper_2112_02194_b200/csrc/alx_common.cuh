@@ -140,6 +140,11 @@ cudaError_t launch_rows_simple(const SideView &sv, const int64_t *class_offs_hos
                                float *split_partials, RowOut out, DevStatus *st, cudaStream_t s,
                                int64_t *launches);
 
+// alx_rows_warp.cu: d = 16, 32, 64, a warp per row (kernels != 1)
+cudaError_t launch_rows_warp(const SideView &sv, const int64_t *class_offs_host, int64_t n_chunks, int64_t n_split_rows, const void *X,
+                             int bf16, int d, const float *Bmat, float *split_partials, RowOut out, DevStatus *st, cudaStream_t s,
+                             int64_t *launches);
+
 // Tensor-core path: the first degree class whose rows (with all longer whole rows) get their sums from the chunks
 // kernel instead of the rows kernel.  Classes 8 .. 10 (1025 .. 8192 observations at the default split) qualify, from
 // the top, as long as they hold at most kLongRowBudget rows together (one d x d + d sum of workspace each).
