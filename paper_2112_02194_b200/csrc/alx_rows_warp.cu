@@ -41,22 +41,16 @@ template <int D, typename T> struct WGeo {
     static constexpr int STAGE = kEntries * RAW;
     static constexpr int TILE = kF32 ? 3 * kEntries * ROW : 0;      // bfloat16 parts of a stage
     static constexpr int ROWS = D == 16 ? 2 : 1;            // matrices a warp solves at a time
-    // columns of L, four at a time from the diagonal block down; the stride of a group's columns is 4 mod 8 floats
-    static constexpr int group_stride(int g) { return D - 4 * g + ((D / 4 - g) % 2 == 0 ? 4 : 0); }
-    __host__ __device__ static constexpr int group_base(int g)
-    {
-        // sum of 4 * group_stride over the groups before g (D / 4 is even: the even ones are padded)
-        return 4 * (D * g - 2 * g * (g - 1) + 4 * ((g + 1) / 2));
-    }
-    static constexpr int L_FLOATS = group_base(D / 4);
-    static constexpr int T_FLOATS = (D < 32 ? D : 32) * ((D < 32 ? D : 32) + 4);      // transposition buffer of one matrix
-    static constexpr int SOLVE = 4 * (ROWS * (L_FLOATS > T_FLOATS ? L_FLOATS : T_FLOATS) + ROWS * D);
-    static constexpr int B_AT = ROWS * (L_FLOATS > T_FLOATS ? L_FLOATS : T_FLOATS);      // right-hand sides, behind the factor
-    static constexpr int WORK = SOLVE;                      // the parts share the factor's place
-    static_assert(TILE <= 4 * B_AT, "the parts leave the right-hand sides alone");
+    // panel k of L: rows 16 k .. D - 1, 16 columns, 64 bytes a row.  The bfloat16 parts of a panel lie where later panels
+    // will: 3 x (rows below the diagonal block) x 32 bytes, which only the last but one panel has too little room for
+    __host__ __device__ static constexpr int panel_at(int k) { return 16 * (16 * MB * k - 8 * k * (k - 1)); }      // floats
+    static constexpr int L_FLOATS = panel_at(MB) + (MB > 1 ? 128 : 0);
+    static constexpr int B_AT = 4 * ROWS * L_FLOATS > TILE ? ROWS * L_FLOATS : TILE / 4;      // right-hand sides, reciprocal pivots
+    static constexpr int SOLVE = 4 * (B_AT + 2 * ROWS * D);
+    static constexpr int WORK = SOLVE;                      // the parts of a gathered stage share the factor's place
     static constexpr int WARP = 2 * STAGE + (WORK + 15) / 16 * 16;
     static constexpr int BASE = NB * 32 * 16;               // the base matrix in fragment order, per block
-    static constexpr int REGS_WARPS = D == 64 ? 12 : 20;      // warps per SM
+    static constexpr int REGS_WARPS = D == 64 ? (kF32 ? 11 : 12) : 20;      // warps per SM
 };
 
 __device__ __forceinline__ void cp_async16_zfill(uint32_t dst, const void *src, bool valid)
@@ -66,6 +60,13 @@ __device__ __forceinline__ void cp_async16_zfill(uint32_t dst, const void *src, 
 __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t addr, uint32_t (&r)[4])
 {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr)
+                 : "memory");
+}
+__device__ __forceinline__ void ldmatrix_x4(uint32_t addr, uint32_t (&r)[4])
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                  : "r"(addr)
                  : "memory");
@@ -221,104 +222,199 @@ __device__ __forceinline__ float rsqrt_full(float p)
     return inv * fmaf(-0.5f * p * inv, inv, 1.5f);      // one Newton step: full fp32 accuracy
 }
 
-// Cholesky, forward and back substitution of the warp's matrix (two for d = 16, one per half-warp).  Lane: row r = lane % 32
-// (% 16) in a0, row r + 32 in a1 for d = 64; b likewise.  L: the warp's columns in shared memory.  The solution replaces b.
-// Returns whether every pivot was positive.
+// address (floats) of 16-byte chunk c of row r of a panel, swizzled so that eight lanes reading rows in a row meet every bank once
+__device__ __forceinline__ int panel_chunk(int r, int c) { return r * 16 + 4 * (c ^ ((r >> 1) & 3)); }
+
+// Cholesky, forward and back substitution of the warp's matrix: the sums in acc (lower triangle, base matrix added), the
+// right-hand side in b_s; the solution replaces b_s.  Blocked, 16 columns per panel: the panel goes through shared memory to
+// lane = row (rows l and l + 32 below the diagonal block's first), is factored there two columns per step, stays in shared
+// memory as part of L and, in three bfloat16 parts, is both operands of the trailing update: the blocks of the matrix never
+// leave the mma fragments.  (With the whole matrix in lane = row, every column of L had to be read by every lane: 2200
+// shared-memory wavefronts per 64 x 64 matrix, 85 % of that pipe.)  d = 16: two matrices, one per half-warp, `acc2` the second.
 template <int D, typename T>
-__device__ __forceinline__ bool factor_solve(float (&a0)[D < 32 ? D : 32], float (&a1)[D == 64 ? 64 : 1], float &b0, float &b1, float *L,
-                                             int lane)
+__device__ __forceinline__ bool factor_solve(Sums<D, T> &acc, Sums<D, T> &acc2, float *L, float *b_s, int lane)
 {
     using G = WGeo<D, T>;
-    constexpr int H = D < 32 ? D : 32;
-    const int r = lane & (H - 1);
-    const int half = lane & ~(H - 1);      // first lane of this matrix
+    constexpr int MB = G::MB;
+    float *dinv_s = b_s + G::ROWS * D;
+    const int half = D == 16 ? lane & 16 : 0;      // first lane of this lane's matrix
+    const int rl = D == 16 ? lane & 15 : lane;
+    float *b_m = b_s + half;                       // d = 16: 16 floats a matrix
+    float *dinv_m = dinv_s + half;
     bool ok = true;
-    float d0 = 0.f, d1 = 0.f;              // reciprocal pivots of the lane's rows
+    auto put_block = [&](float *P, const float(&c)[4], int i, int n) {      // block (16 i .., 8 n ..) of the panel
+        const int r = 16 * i + lane / 4, q = 2 * n + (lane % 4) / 2, o = 2 * (lane & 1);
+        *reinterpret_cast<float2 *>(P + panel_chunk(r, q) + o) = make_float2(c[0], c[1]);
+        *reinterpret_cast<float2 *>(P + panel_chunk(r + 8, q) + o) = make_float2(c[2], c[3]);
+    };
+#pragma unroll 1
+    for (int k = 0; k < MB; ++k) {
+        float *P = L + G::panel_at(k);
+        const int rows = D - 16 * k;
+        // the panel's blocks to shared memory
 #pragma unroll
-    for (int j = 0; j < D; j += 2) {
-        const int src = half + (j & (H - 1));
-        float p, q, s, z0, z1;
-        if (j < 32) {
-            p = __shfl_sync(0xFFFFFFFFu, a0[j & (H - 1)], src);
-            q = __shfl_sync(0xFFFFFFFFu, a0[j & (H - 1)], src + 1);
-            s = __shfl_sync(0xFFFFFFFFu, a0[(j + 1) & (H - 1)], src + 1);
-            z0 = __shfl_sync(0xFFFFFFFFu, b0, src);
-            z1 = __shfl_sync(0xFFFFFFFFu, b0, src + 1);
-        } else {
-            p = __shfl_sync(0xFFFFFFFFu, a1[D == 64 ? j : 0], src);
-            q = __shfl_sync(0xFFFFFFFFu, a1[D == 64 ? j : 0], src + 1);
-            s = __shfl_sync(0xFFFFFFFFu, a1[D == 64 ? j + 1 : 0], src + 1);
-            z0 = __shfl_sync(0xFFFFFFFFu, b1, src);
-            z1 = __shfl_sync(0xFFFFFFFFu, b1, src + 1);
-        }
-        const float i0 = rsqrt_full(p), l10 = q * i0, dd = fmaf(-l10, l10, s), i1 = rsqrt_full(dd);
-        ok = ok && p > 0.f && dd > 0.f;
-        z0 *= i0;
-        z1 = fmaf(-z0, l10, z1) * i1;
-        float *c0 = L + G::group_base(j / 4) + (j % 4) * G::group_stride(j / 4) - 4 * (j / 4);
-        float *c1 = c0 + G::group_stride(j / 4);
-        float x00 = 0.f, x01 = 0.f, x10 = 0.f, x11 = 0.f;
-        if (j < 32) {
-            x00 = a0[j & (H - 1)] * i0;
-            x01 = fmaf(-x00, l10, a0[(j + 1) & (H - 1)]) * i1;
-            if (r >= 4 * (j / 4)) { c0[r] = x00; c1[r] = x01; }
-            const float nb = fmaf(-x01, z1, fmaf(-x00, z0, b0));
-            b0 = r > j + 1 ? nb : r == j ? z0 : r == j + 1 ? z1 : b0;
-            d0 = r == j ? i0 : r == j + 1 ? i1 : d0;
-        }
-        if constexpr (D == 64) {
-            x10 = a1[j] * i0;
-            x11 = fmaf(-x10, l10, a1[j + 1]) * i1;
-            if (j < 32 || r + 32 >= 4 * (j / 4)) { c0[r + 32] = x10; c1[r + 32] = x11; }
-            const float nb = fmaf(-x11, z1, fmaf(-x10, z0, b1));
-            b1 = r + 32 > j + 1 ? nb : r + 32 == j ? z0 : r + 32 == j + 1 ? z1 : b1;
-            d1 = r + 32 == j ? i0 : r + 32 == j + 1 ? i1 : d1;
+        for (int kk = 0; kk < MB; ++kk)
+            if (kk == k) {
+#pragma unroll
+                for (int i = kk; i < MB; ++i)
+#pragma unroll
+                    for (int n = 0; n < 2; ++n) put_block(P, acc.c[i * (i + 1) + 2 * kk + n], i - kk, n);
+            }
+        if (D == 16) {
+            put_block(L + G::L_FLOATS, acc2.c[0], 0, 0);
+            put_block(L + G::L_FLOATS, acc2.c[1], 0, 1);
         }
         __syncwarp();
+        float *Pm = D == 16 ? L + (half ? G::L_FLOATS : 0) : P;
+        const bool two = D == 64 && lane + 32 < rows;
+        float a0[16], a1[16];
 #pragma unroll
-        for (int c = (j + 2) & ~3; c < D; c += 4) {
-            const float4 u = *reinterpret_cast<const float4 *>(c0 + c), v = *reinterpret_cast<const float4 *>(c1 + c);
-            const float2 m00 = make_float2(-x00, -x00), m01 = make_float2(-x01, -x01);
-            const float2 m10 = make_float2(-x10, -x10), m11 = make_float2(-x11, -x11);
+        for (int c = 0; c < 4; ++c) {
+            const float4 v = *reinterpret_cast<const float4 *>(Pm + panel_chunk(rl < rows ? rl : 0, c));
+            a0[4 * c] = v.x; a0[4 * c + 1] = v.y; a0[4 * c + 2] = v.z; a0[4 * c + 3] = v.w;
+            if (D == 64) {
+                const float4 w = *reinterpret_cast<const float4 *>(Pm + panel_chunk(two ? rl + 32 : 0, c));
+                a1[4 * c] = w.x; a1[4 * c + 1] = w.y; a1[4 * c + 2] = w.z; a1[4 * c + 3] = w.w;
+            }
+        }
+        float b0 = rl < rows ? b_m[16 * k + rl] : 0.f, b1 = two ? b_m[16 * k + 32 + rl] : 0.f, d = 0.f;
+        __syncwarp();
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int cc = c + 2 * h;
-                if (cc < j + 2) continue;
-                const float2 uu = h ? make_float2(u.z, u.w) : make_float2(u.x, u.y), vv = h ? make_float2(v.z, v.w) : make_float2(v.x, v.y);
-                if (cc < 32) {
-                    float2 t = make_float2(a0[cc & (H - 1)], a0[(cc + 1) & (H - 1)]);
-                    t = __ffma2_rn(m01, vv, __ffma2_rn(m00, uu, t));
-                    a0[cc & (H - 1)] = t.x;
-                    a0[(cc + 1) & (H - 1)] = t.y;
-                }
-                if constexpr (D == 64) {
-                    float2 t = make_float2(a1[cc], a1[cc + 1]);
-                    t = __ffma2_rn(m11, vv, __ffma2_rn(m10, uu, t));
-                    a1[cc] = t.x;
-                    a1[cc + 1] = t.y;
+        for (int j = 0; j < 16; j += 2) {
+            const float p = __shfl_sync(0xFFFFFFFFu, a0[j], half + j), q = __shfl_sync(0xFFFFFFFFu, a0[j], half + j + 1);
+            const float s = __shfl_sync(0xFFFFFFFFu, a0[j + 1], half + j + 1);
+            float z0 = __shfl_sync(0xFFFFFFFFu, b0, half + j), z1 = __shfl_sync(0xFFFFFFFFu, b0, half + j + 1);
+            const float i0 = rsqrt_full(p), l10 = q * i0, dd = fmaf(-l10, l10, s), i1 = rsqrt_full(dd);
+            ok = ok && p > 0.f && dd > 0.f;
+            z0 *= i0;
+            z1 = fmaf(-z0, l10, z1) * i1;
+            const float x0 = a0[j] * i0, x1 = fmaf(-x0, l10, a0[j + 1]) * i1;
+            a0[j] = x0;
+            a0[j + 1] = x1;
+            const float nb = fmaf(-x1, z1, fmaf(-x0, z0, b0));
+            b0 = rl > j + 1 ? nb : rl == j ? z0 : rl == j + 1 ? z1 : b0;
+            d = rl == j ? i0 : rl == j + 1 ? i1 : d;
+            float y0 = 0.f, y1 = 0.f;
+            if (D == 64) {
+                y0 = a1[j] * i0;
+                y1 = fmaf(-y0, l10, a1[j + 1]) * i1;
+                a1[j] = y0;
+                a1[j + 1] = y1;
+                b1 = fmaf(-y1, z1, fmaf(-y0, z0, b1));
+            }
+            if (j < 14) {
+                // the two columns of the diagonal block's rows to everybody: the place of the panel's first two rows serves
+                // as the exchange (its rows are in registers)
+                float *ex = Pm + 32 * ((j / 2) & 1);
+                if (rl < 16) { ex[rl] = x0; ex[16 + rl] = x1; }
+                __syncwarp();
+#pragma unroll
+                for (int c = (j + 2) & ~3; c < 16; c += 4) {
+                    const float4 u = *reinterpret_cast<const float4 *>(ex + c), v = *reinterpret_cast<const float4 *>(ex + 16 + c);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int cc = c + 2 * h;
+                        if (cc < j + 2) continue;
+                        const float2 uu = h ? make_float2(u.z, u.w) : make_float2(u.x, u.y), vv = h ? make_float2(v.z, v.w) : make_float2(v.x, v.y);
+                        float2 t = make_float2(a0[cc], a0[cc + 1]);
+                        t = __ffma2_rn(make_float2(-x1, -x1), vv, __ffma2_rn(make_float2(-x0, -x0), uu, t));
+                        a0[cc] = t.x;
+                        a0[cc + 1] = t.y;
+                        if (D == 64) {
+                            float2 w = make_float2(a1[cc], a1[cc + 1]);
+                            w = __ffma2_rn(make_float2(-y1, -y1), vv, __ffma2_rn(make_float2(-y0, -y0), uu, w));
+                            a1[cc] = w.x;
+                            a1[cc + 1] = w.y;
+                        }
+                    }
                 }
             }
         }
-    }
-    // back substitution, from the last column: x_j to everybody, then row i < j takes L[j][i] x_j off
-    const int g0 = r / 4;
-    const float *l0 = L + G::group_base(g0) + (r % 4) * (D - 4 * g0 + ((D / 4 - g0) % 2 == 0 ? 4 : 0)) - 4 * g0;
-    if constexpr (D == 64) {
-        const int g1 = (r + 32) / 4;
-        const float *l1 = L + G::group_base(g1) + (r % 4) * (D - 4 * g1 + ((D / 4 - g1) % 2 == 0 ? 4 : 0)) - 4 * g1;
-#pragma unroll 8
-        for (int j = 63; j >= 32; --j) {
-            const float x = __shfl_sync(0xFFFFFFFFu, b1 * d1, j - 32);
-            const float m0 = l0[j], m1 = l1[j];
-            b0 = fmaf(-m0, x, b0);
-            b1 = r + 32 < j ? fmaf(-m1, x, b1) : r + 32 == j ? x : b1;
+        __syncwarp();
+        // L's rows back, the right-hand side, the reciprocal pivots
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            if (rl < rows) *reinterpret_cast<float4 *>(Pm + panel_chunk(rl, c)) = make_float4(a0[4 * c], a0[4 * c + 1], a0[4 * c + 2], a0[4 * c + 3]);
+            if (two) *reinterpret_cast<float4 *>(Pm + panel_chunk(rl + 32, c)) = make_float4(a1[4 * c], a1[4 * c + 1], a1[4 * c + 2], a1[4 * c + 3]);
         }
+        if (rl < rows) b_m[16 * k + rl] = b0;
+        if (two) b_m[16 * k + 32 + rl] = b1;
+        if (rl < 16) dinv_m[16 * k + rl] = d;
+        if (D > 16 && k + 1 < MB) {
+            // the rows below the diagonal block as bfloat16 parts, [part][row][16 columns]: 32-byte rows, the two 16-byte
+            // chunks exchanged in every other group of four rows (ldmatrix without conflicts)
+            unsigned char *tile = reinterpret_cast<unsigned char *>(L + G::panel_at(k + 1));
+            const int below = rows - 16;
+            auto put_parts = [&](const float(&x)[16], int r) {      // r: row below the diagonal block
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    uint32_t p[3][4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const float u = x[8 * c + 2 * e], v = x[8 * c + 2 * e + 1];
+                        p[0][e] = pack_bf16(u, v);
+                        const float u1 = u - bf16_lo(p[0][e]), v1 = v - bf16_hi(p[0][e]);
+                        p[1][e] = pack_bf16(u1, v1);
+                        p[2][e] = pack_bf16(u1 - bf16_lo(p[1][e]), v1 - bf16_hi(p[1][e]));
+                    }
+#pragma unroll
+                    for (int part = 0; part < 3; ++part)
+                        *reinterpret_cast<uint4 *>(tile + (part * below + r) * 32 + 16 * (c ^ ((r >> 2) & 1))) =
+                            make_uint4(p[part][0], p[part][1], p[part][2], p[part][3]);
+                }
+            };
+            if (rl >= 16 && rl < rows) put_parts(a0, rl - 16);
+            if (two) put_parts(a1, rl + 16);
+            __syncwarp();
+            // trailing update of the blocks (i, n), i > k, n >= 2 (k + 1)
+            const int lr = (lane & 7) + 8 * ((lane >> 3) & 1);
+            const uint32_t src = ptx::smem_u32(tile) + lr * 32 + 16 * ((lane >> 4) ^ ((lr >> 2) & 1));
+#pragma unroll
+            for (int kk = 0; kk + 1 < MB; ++kk)
+                if (kk == k) {
+                    constexpr int pa[6] = {2, 0, 1, 1, 0, 0}, pb[6] = {0, 2, 1, 0, 1, 0};
+                    uint32_t f[3][MB][4];
+#pragma unroll
+                    for (int part = 0; part < 3; ++part)
+#pragma unroll
+                        for (int i = kk + 1; i < MB; ++i) ldmatrix_x4(src + (part * (D - 16 * (kk + 1)) + 16 * (i - kk - 1)) * 32, f[part][i]);
+#pragma unroll
+                    for (int i = kk + 1; i < MB; ++i)
+#pragma unroll
+                        for (int q = 0; q < 6; ++q) {
+                            uint32_t neg[4];
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) neg[e] = f[pa[q]][i][e] ^ 0x80008000u;
+#pragma unroll
+                            for (int n = 2 * (kk + 1); n < 2 * (i + 1); ++n)
+                                mma_bf16(acc.c[i * (i + 1) + n], neg, f[pb[q]][n / 2][n % 2], f[pb[q]][n / 2][2 + n % 2]);
+                        }
+                }
+        }
+        __syncwarp();
     }
-#pragma unroll 8
-    for (int j = H - 1; j >= 0; --j) {
-        const float x = __shfl_sync(0xFFFFFFFFu, b0 * d0, half + j);
-        const float m0 = l0[j];
-        b0 = r < j ? fmaf(-m0, x, b0) : r == j ? x : b0;
+    // back substitution, panel by panel from the last: what the solved rows below take off (lanes: column c, rows of one
+    // parity), then the 16 x 16 triangle
+    const int c = lane & 15;
+#pragma unroll 1
+    for (int k = MB - 1; k >= 0; --k) {
+        const float *Pm = D == 16 ? L + (half ? G::L_FLOATS : 0) : L + G::panel_at(k);
+        float s = 0.f;
+        if (D > 16) {
+#pragma unroll 4
+            for (int r = 16 + (lane >> 4); r < D - 16 * k; r += 2) s = fmaf(Pm[panel_chunk(r, c >> 2) + (c & 3)], b_s[16 * k + r], s);
+            s += __shfl_xor_sync(0xFFFFFFFFu, s, 16);
+        }
+        float x = b_m[16 * k + c] - s;
+        const float d = dinv_m[16 * k + c];
+#pragma unroll
+        for (int j = 15; j >= 0; --j) {
+            const float xj = __shfl_sync(0xFFFFFFFFu, x * d, half + j);
+            x = c < j ? fmaf(-Pm[panel_chunk(j, c >> 2) + (c & 3)], xj, x) : c == j ? xj : x;
+        }
+        __syncwarp();
+        if (D == 16 || lane < 16) b_m[16 * k + c] = x;
+        __syncwarp();
     }
     const unsigned bad = __ballot_sync(0xFFFFFFFFu, !ok);
     return D == 16 ? (bad >> half & 0xFFFFu) == 0 : bad == 0;
@@ -330,54 +426,22 @@ template <int D, typename T> __device__ __forceinline__ void put_b(const Sums<D,
     __syncwarp();
 }
 
-// adds the base matrix to the sums and hands the rows to their lanes through shared memory; matrix `which` of a d = 16 pair
-template <int D, typename T>
-__device__ __forceinline__ void place_rows(const Sums<D, T> &acc, const float4 *base, float *work, float (&a0)[D < 32 ? D : 32],
-                                           float (&a1)[D == 64 ? 64 : 1], int which, int lane)
+template <int D, typename T> __device__ __forceinline__ void add_base(Sums<D, T> &acc, const float4 *base, int lane)
 {
-    using G = WGeo<D, T>;
-    constexpr int H = D < 32 ? D : 32, S = H + 4;
-    float *t = work + which * G::T_FLOATS;
-    // passes of H rows x H columns: (rows 0..31), and for d = 64 (rows 32..63) x two halves of the columns
 #pragma unroll
-    for (int pass = 0; pass < (D == 64 ? 3 : 1); ++pass) {
-        const int i0 = pass == 0 ? 0 : 2, n0 = pass == 2 ? 4 : 0;
-#pragma unroll
-        for (int i = i0; i < (D == 16 ? 1 : i0 + 2); ++i)
-#pragma unroll
-            for (int n = n0; n < n0 + H / 8; ++n)
-                if (n < 2 * (i + 1)) {
-                    const int blk = i * (i + 1) + n;
-                    const float4 v = base[blk * 32 + lane];
-                    float *dst = t + (16 * (i - i0) + lane / 4) * S + 8 * (n - n0) + 2 * (lane % 4);
-                    *reinterpret_cast<float2 *>(dst) = make_float2(acc.c[blk][0] + v.x, acc.c[blk][1] + v.y);
-                    *reinterpret_cast<float2 *>(dst + 8 * S) = make_float2(acc.c[blk][2] + v.z, acc.c[blk][3] + v.w);
-                }
-        __syncwarp();
-        if (D != 16 || (lane >> 4) == which) {
-            const float *row = t + (lane & (H - 1)) * S;
-#pragma unroll
-            for (int c = 0; c < H; c += 4) {
-                const float4 v = *reinterpret_cast<const float4 *>(row + c);
-                if (pass == 0) {
-                    a0[c] = v.x; a0[c + 1] = v.y; a0[c + 2] = v.z; a0[c + 3] = v.w;
-                } else if constexpr (D == 64) {
-                    const int o = 32 * (pass - 1) + c;
-                    a1[o] = v.x; a1[o + 1] = v.y; a1[o + 2] = v.z; a1[o + 3] = v.w;
-                }
-            }
-        }
-        __syncwarp();
+    for (int n = 0; n < WGeo<D, T>::NB; ++n) {
+        const float4 v = base[n * 32 + lane];
+        acc.c[n][0] += v.x; acc.c[n][1] += v.y; acc.c[n][2] += v.z; acc.c[n][3] += v.w;
     }
 }
 
 template <int D, typename T>
-__device__ __forceinline__ void store_row(float b0, float b1, bool ok, int64_t u, const RowOut &out, DevStatus *st, int lane)
+__device__ __forceinline__ void store_row(const float *x, bool ok, int64_t u, const RowOut &out, DevStatus *st, int lane)
 {
     constexpr int H = D < 32 ? D : 32;
     const int r = lane & (H - 1);
     T *row = reinterpret_cast<T *>(out.table) + u * D;
-    const float v0 = ok ? b0 : 0.f, v1 = ok ? b1 : 0.f;
+    const float v0 = ok ? x[r] : 0.f, v1 = D == 64 && ok ? x[D == 64 ? r + 32 : 0] : 0.f;
     store_elem(row + r, v0);
     if (D == 64) store_elem(row + 32 + r, v1);
     if (out.cap_slot) {
@@ -433,44 +497,35 @@ k_rows_warp(SideView sv, int64_t last, int64_t count, const T *__restrict__ X, c
     feed.start(beg, end, lane);
     float *b_s = reinterpret_cast<float *>(work) + G::B_AT;
     while (true) {
-        float a0[D < 32 ? D : 32], a1[D == 64 ? 64 : 1], b0 = 0.f, b1 = 0.f;
         int64_t u_pair = -1;
         const int64_t next = item + warps * G::ROWS;
-        int64_t un = next < count ? sv.order[last - next] : -1, bn = 0, en = 0;
-        {
-            Sums<D, T> acc;
-            acc.zero();
-            sum_entries<D, T>(feed, end - beg, mine, work, acc, lane);
-            if constexpr (D == 16) {
-                put_b<D, T>(acc, b_s, lane);
-                place_rows<D, T>(acc, base, reinterpret_cast<float *>(work), a0, a1, 0, lane);
-                if (item + 1 < count) {
-                    u_pair = sv.order[last - item - 1];
-                    const int64_t b2 = sv.ptr[u_pair], e2 = sv.ptr[u_pair + 1];
-                    feed.start(b2, e2, lane);
-                    acc.zero();
-                    sum_entries<D, T>(feed, e2 - b2, mine, work, acc, lane);
-                }      // (a lone last row: the second matrix is the first one again, and is not stored)
-                put_b<D, T>(acc, b_s + D, lane);
-                place_rows<D, T>(acc, base, reinterpret_cast<float *>(work), a0, a1, 1, lane);
-                b0 = b_s[lane];
-            } else {
-                put_b<D, T>(acc, b_s, lane);
-                place_rows<D, T>(acc, base, reinterpret_cast<float *>(work), a0, a1, 0, lane);
-                b0 = b_s[lane];
-                if (D == 64) b1 = b_s[lane + 32];
+        const int64_t un = next < count ? sv.order[last - next] : -1;
+        int64_t bn = 0, en = 0;
+        Sums<D, T> acc, acc2;
+        acc.zero();
+        sum_entries<D, T>(feed, end - beg, mine, work, acc, lane);
+        put_b<D, T>(acc, b_s, lane);
+        if constexpr (D == 16) {      // a second matrix; a lone last row goes without
+            acc2.zero();
+            if (item + 1 < count) {
+                u_pair = sv.order[last - item - 1];
+                const int64_t b2 = sv.ptr[u_pair], e2 = sv.ptr[u_pair + 1];
+                feed.start(b2, e2, lane);
+                sum_entries<D, T>(feed, e2 - b2, mine, work, acc2, lane);
             }
+            put_b<D, T>(acc2, b_s + D, lane);
+            add_base<D, T>(acc2, base, lane);
         }
-        __syncwarp();
+        add_base<D, T>(acc, base, lane);
         // the next row's first entries travel while this one is solved
         if (un >= 0) {
             bn = sv.ptr[un];
             en = sv.ptr[un + 1];
             feed.start(bn, en, lane);
         }
-        const bool ok = factor_solve<D, T>(a0, a1, b0, b1, reinterpret_cast<float *>(work) + (D == 16 ? (lane >> 4) * G::L_FLOATS : 0), lane);
-        if (D != 16 || lane < 16) store_row<D, T>(b0, b1, ok, u, out, st, lane);
-        else if (u_pair >= 0) store_row<D, T>(b0, b1, ok, u_pair, out, st, lane);
+        const bool ok = factor_solve<D, T>(acc, acc2, reinterpret_cast<float *>(work), b_s, lane);
+        if (D != 16 || lane < 16) store_row<D, T>(b_s, ok, u, out, st, lane);
+        else if (u_pair >= 0) store_row<D, T>(b_s + D, ok, u_pair, out, st, lane);
         if (un < 0) return;
         __syncwarp();
         item = next;
@@ -495,18 +550,19 @@ template <int D, typename T>
 __device__ __forceinline__ void solve_sums(const float *sums, const float4 *base, float *work, int64_t u, const RowOut &out, DevStatus *st, int lane)
 {
     using G = WGeo<D, T>;
-    Sums<D, T> acc;
+    Sums<D, T> acc, acc2;
 #pragma unroll
     for (int n = 0; n < G::NB; ++n) {
         const float4 v = *reinterpret_cast<const float4 *>(sums + (n * 32 + lane) * 4);
         acc.c[n][0] = v.x; acc.c[n][1] = v.y; acc.c[n][2] = v.z; acc.c[n][3] = v.w;
     }
-    float a0[D < 32 ? D : 32], a1[D == 64 ? 64 : 1], b0, b1 = 0.f;
-    for (int w = 0; w < G::ROWS; ++w) place_rows<D, T>(acc, base, work, a0, a1, w, lane);
-    b0 = sums[G::NB * 128 + (lane & (D < 32 ? D - 1 : 31))];
-    if (D == 64) b1 = sums[G::NB * 128 + 32 + lane];
-    const bool ok = factor_solve<D, T>(a0, a1, b0, b1, work + (D == 16 ? (lane >> 4) * G::L_FLOATS : 0), lane);
-    if (D != 16 || lane < 16) store_row<D, T>(b0, b1, ok, u, out, st, lane);
+    float *b_s = work + G::B_AT;
+    for (int e = lane; e < G::ROWS * D; e += 32) b_s[e] = sums[G::NB * 128 + (e & (D - 1))];
+    add_base<D, T>(acc, base, lane);
+    if constexpr (D == 16) acc2 = acc;
+    __syncwarp();
+    const bool ok = factor_solve<D, T>(acc, acc2, work, b_s, lane);
+    if (D != 16 || lane < 16) store_row<D, T>(b_s, ok, u, out, st, lane);
 }
 
 template <int D, typename T, bool CHUNK>
