@@ -295,20 +295,21 @@ CgOptions cg_options(const alx_ctx *c, int solved_side)
     return o;
 }
 
-alx_status gramian_of(alx_ctx *c, int table_side)
+// the Gramian and the base matrix of a table; `solve`: also what the rows' dual form needs of the base matrix
+alx_status gramian_of(alx_ctx *c, int table_side, bool solve)
 {
     if (tensor_path(c)) {
         ALX_CUDA(c, launch_gramian_umma(c->table[table_side], c->n[table_side], c->gram_partials, c->stream, &c->launches));
         ALX_CUDA(c, launch_gramian_reduce(c->gram_partials, gramian_umma_partials(), c->opt.d, c->G64[table_side], c->Bmat,
                                           c->opt.alpha0, c->opt.lambda, c->stream, &c->launches));
-        if (dual_form(c)) ALX_CUDA(c, launch_dual_prepare(c->Bmat, c->dual_ws, dual_cond_limit(c), c->opt.solver == ALX_SOLVER_AUTO, c->stream,
+        if (solve && dual_form(c)) ALX_CUDA(c, launch_dual_prepare(c->Bmat, c->dual_ws, dual_cond_limit(c), c->opt.solver == ALX_SOLVER_AUTO, c->stream,
                                                          &c->launches));
         c->have_gram[table_side] = true;
         return ALX_OK;
     }
     ALX_CUDA(c, launch_gramian(c->table[table_side], c->bf16, c->n[table_side], c->opt.d, c->gram_partials,
                                c->G64[table_side], c->Bmat, c->opt.alpha0, c->opt.lambda, c->stream, &c->launches));
-    if (fold_path(c) && c->dual_ws)
+    if (solve && fold_path(c) && c->dual_ws)
         ALX_CUDA(c, launch_dual64_prepare(c->Bmat, c->dual_ws, dual_cond_limit(c), c->stream, &c->launches));
     c->have_gram[table_side] = true;
     return ALX_OK;
@@ -324,7 +325,7 @@ alx_status half_epoch_impl(alx_ctx *c, int side, const int32_t *cap_slot, float 
     alx_status st;
     {
         NvtxRange r("alx Gramian + base matrix");
-        st = gramian_of(c, fixed);
+        st = gramian_of(c, fixed, true);
     }
     if (st != ALX_OK) return st;
     ALX_CUDA(c, cudaEventRecord(c->ev[1], c->stream));
@@ -463,6 +464,7 @@ alx_status create_impl(const alx_options *opt, const alx_ctx *parent, alx_ctx **
         if (gramian_umma_partials() > n_part) n_part = gramian_umma_partials();
         ALX_ALLOC(c, c->gram_partials, n_part * d * d);
         ALX_ALLOC(c, c->loss_result, 4);
+        ALX_CUDA(c, cudaMemsetAsync(c->loss_result, 0, 4 * sizeof(double), c->stream));
         ALX_ALLOC(c, c->status, 1);
         ALX_CUDA(c, cudaMemsetAsync(c->status, 0, sizeof(DevStatus), c->stream));
         ALX_ALLOC(c, c->cg_counters, 5);
@@ -855,7 +857,7 @@ alx_status alx_gramian(alx_ctx *c, alx_side table, double *dst)
     if (!dst || (table != ALX_ROWS && table != ALX_COLS)) return fail(c, ALX_ERR_INVALID_ARG, "bad argument");
     if (!c->have_table[table]) return fail(c, ALX_ERR_BAD_STATE, "table has not been set");
     DeviceGuard guard(c->device);
-    alx_status st = gramian_of(c, table);
+    alx_status st = gramian_of(c, table, false);
     if (st != ALX_OK) return st;
     return alx_get_gramian(c, table, dst);
 }
@@ -880,14 +882,12 @@ alx_status alx_loss(alx_ctx *c, double *total, double *components)
     DeviceGuard guard(c->device);
     for (int s = 0; s < 2; ++s)
         if (!c->have_gram[s]) {
-            alx_status st = gramian_of(c, s);
+            alx_status st = gramian_of(c, s, false);
             if (st != ALX_OK) return st;
         }
-    ALX_CUDA(c, launch_loss_obs(c->ptr[0], c->idx[0], c->val[0], c->n[0], c->nnz, c->table[0], c->table[1], c->bf16,
-                                c->opt.d, c->loss_partials_buf, c->loss_result, c->stream, &c->launches));
-    ALX_CUDA(c, launch_loss_finish(c->loss_partials_buf, c->nnz > 0 ? loss_partials(c->nnz) : 0, c->G64[0], c->G64[1],
-                                   c->opt.d, (double)c->opt.alpha0, (double)c->opt.lambda, c->loss_result, c->stream,
-                                   &c->launches));
+    ALX_CUDA(c, launch_loss(c->ptr[0], c->idx[0], c->val[0], c->n[0], c->nnz, c->table[0], c->table[1], c->bf16, c->opt.d, c->G64[0],
+                            c->G64[1], (double)c->opt.alpha0, (double)c->opt.lambda, c->loss_partials_buf, c->loss_result, c->stream,
+                            &c->launches));
     double h[3];
     ALX_CUDA(c, cudaMemcpyAsync(h, c->loss_result, sizeof h, cudaMemcpyDeviceToHost, c->stream));
     alx_status st = check_device_status(c);

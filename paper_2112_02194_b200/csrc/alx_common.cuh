@@ -125,7 +125,6 @@ cudaError_t launch_convert(const void *src, int src_bf16, void *dst, int dst_bf1
                            int64_t *launches);
 
 // alx_gramian.cu
-constexpr int kGramRowsPerPartial = 4096;
 int64_t gramian_partials(int64_t n);
 cudaError_t launch_gramian(const void *X, int bf16, int64_t n, int d, float *partials, double *G64, float *Bmat,
                            float alpha0, float lambda, cudaStream_t s, int64_t *launches);
@@ -248,10 +247,9 @@ cudaError_t launch_rows_dual(const SideView &sv, int64_t first16, int64_t count1
 
 // alx_loss.cu
 int64_t loss_partials(int64_t nnz);
-cudaError_t launch_loss_obs(const int64_t *rowptr, const int32_t *colidx, const float *values, int64_t n_rows,
-                            int64_t nnz, const void *W, const void *H, int bf16, int d, double *partials,
-                            double *result, cudaStream_t s, int64_t *launches);
-cudaError_t launch_loss_finish(const double *partials, int64_t n_partials, const double *GW, const double *GH, int d,
-                               double alpha0, double lambda, double *result, cudaStream_t s, int64_t *launches);
+// result: [0] observed, [1] all-pairs, [2] regulariser, and [3] a counter that is zero between calls
+cudaError_t launch_loss(const int64_t *rowptr, const int32_t *colidx, const float *values, int64_t n_rows,
+                            int64_t nnz, const void *W, const void *H, int bf16, int d, const double *GW, const double *GH,
+                            double alpha0, double lambda, double *partials, double *result, cudaStream_t s, int64_t *launches);
 
 }  // namespace alx

@@ -18,6 +18,7 @@
 // 128-byte-swizzled operand layout), 1 MMA warp, 3 solver groups of 128 threads (thread = tensor-memory lane =
 // one padded observation).  Every wait is bounded; a block that gives up sets a status flag and returns.
 #include "alx_common.cuh"
+#include "alx_inverse.cuh"
 #include "alx_ptx.cuh"
 
 namespace alx {
@@ -53,65 +54,15 @@ __host__ __device__ constexpr uint32_t idesc_bf16_k_major(int M, int N)
 }
 
 // ---------------------------------------------------------------------------------------------------------
-// B^-1 in fp64 by Cholesky (one block of 128 threads, thread i = row i), written as three bfloat16 parts in the
-// operand layout of the dual kernel; flag = 1 if B is positive definite and ||B||_F ||B^-1||_F <= cond_limit,
-// 2 if it is positive definite but beyond the limit and the caller can use the dual solutions as start vectors, else 0
-// (the product is 128 for a multiple of the identity).
-__global__ void __launch_bounds__(128, 1) k_binv_prepare(const float *__restrict__ Bmat, unsigned char *__restrict__ tiles,
-                                                         int *__restrict__ flag, double cond_limit, int allow_start)
+// B^-1 in fp64 (alx_inverse.cuh), written as three bfloat16 parts in the operand layout of the dual kernel; flag = 1 if B is
+// positive definite and ||B||_F ||B^-1||_F <= cond_limit, 2 if it is positive definite but beyond the limit and the caller
+// can use the dual solutions as start vectors, else 0 (the product is 128 for a multiple of the identity).
+__global__ void __launch_bounds__(SweepGeo<D>::THREADS, 1) k_binv_prepare(const float *__restrict__ Bmat, unsigned char *__restrict__ tiles,
+                                                                         int *__restrict__ flag, double cond_limit, int allow_start)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    double *A = reinterpret_cast<double *>(smem_raw);          // [128][129]: lower = L, strict upper = (L^-1)^T
-    double *dinv = A + D * (D + 1);                            // [128]: 1 / L[i][i]
-    double *red = dinv + D;                                    // [128]
-    __shared__ int s_ok;
-    constexpr int LD = D + 1;
-    const int i = threadIdx.x;
-    if (i == 0) s_ok = 1;
-    double fro = 0.0;
-    for (int c = 0; c < D; ++c) {
-        const double v = (double)Bmat[i * D + c];
-        A[i * LD + c] = v;
-        fro += v * v;
-    }
-    red[i] = fro;
-    __syncthreads();
-    // right-looking Cholesky, lower triangle
-    for (int j = 0; j < D; ++j) {
-        if (i == j) {
-            const double p = A[j * LD + j];
-            if (!(p > 0.0)) s_ok = 0;
-            const double l = sqrt(p > 0.0 ? p : 1.0);
-            A[j * LD + j] = l;
-            dinv[j] = 1.0 / l;
-        }
-        __syncthreads();
-        if (i > j) A[i * LD + j] *= dinv[j];
-        __syncthreads();
-        if (i > j) {
-            const double lij = A[i * LD + j];
-            for (int c = j + 1; c <= i; ++c) A[i * LD + c] -= lij * A[c * LD + j];
-        }
-        __syncthreads();
-    }
-    // column i of L^-1 (stored transposed in the strict upper triangle: A[i][r] = Linv[r][i], r > i)
-    for (int r = i + 1; r < D; ++r) {
-        double s = A[r * LD + i] * dinv[i];
-        for (int k = i + 1; k < r; ++k) s += A[r * LD + k] * A[i * LD + k];
-        A[i * LD + r] = -s * dinv[r];
-    }
-    __syncthreads();
-    // row i of B^-1 = (L^-1)^T L^-1
-    double fro_inv = 0.0;
-    for (int c = 0; c < D; ++c) {
-        const int m = i > c ? i : c;
-        double s = 0.0;
-        for (int k = m; k < D; ++k) {
-            const double a = (k == i) ? dinv[i] : A[i * LD + k];
-            const double b = (k == c) ? dinv[c] : A[c * LD + k];
-            s += a * b;
-        }
-        fro_inv += s * s;
+    __shared__ SweepSmem<D> sm;
+    double cond;
+    const bool ok = sweep_inverse<D>(Bmat, sm, &cond, [&](int i, int c, double s) {
         const float v = (float)s;
         // three bfloat16 parts: the first rounds to nearest, the others keep the leading 8 bits of what is left
         const __nv_bfloat16 p1 = __float2bfloat16_rn(v);
@@ -123,15 +74,8 @@ __global__ void __launch_bounds__(128, 1) k_binv_prepare(const float *__restrict
         *reinterpret_cast<__nv_bfloat16 *>(tiles + off) = p1;
         *reinterpret_cast<unsigned short *>(tiles + kTileBytes + off) = (unsigned short)(m2 >> 16);
         *reinterpret_cast<unsigned short *>(tiles + 2 * kTileBytes + off) = (unsigned short)(m3 >> 16);
-    }
-    __syncthreads();
-    dinv[i] = fro_inv;       // dinv is no longer needed
-    __syncthreads();
-    if (i == 0) {
-        double a = 0.0, b = 0.0;
-        for (int k = 0; k < D; ++k) { a += red[k]; b += dinv[k]; }
-        *flag = !s_ok ? 0 : (sqrt(a) * sqrt(b) <= cond_limit) ? 1 : (allow_start ? 2 : 0);
-    }
+    });
+    if (threadIdx.x == 0) *flag = !ok ? 0 : cond <= cond_limit ? 1 : allow_start ? 2 : 0;
 }
 
 // ---------------------------------------------------------------------------------------------------------
@@ -703,11 +647,8 @@ size_t dual_workspace_bytes() { return (size_t)kBinvBytes + 256; }
 cudaError_t launch_dual_prepare(const float *Bmat, void *ws, float cond_limit, bool allow_start, cudaStream_t s,
                                 int64_t *launches)
 {
-    const size_t smem = sizeof(double) * (D * (D + 1) + 2 * D);
-    cudaError_t e = cudaFuncSetAttribute(k_binv_prepare, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
     unsigned char *w = static_cast<unsigned char *>(ws);
-    k_binv_prepare<<<1, 128, smem, s>>>(Bmat, w, reinterpret_cast<int *>(w + kBinvBytes), (double)cond_limit, allow_start ? 1 : 0);
+    k_binv_prepare<<<1, SweepGeo<D>::THREADS, 0, s>>>(Bmat, w, reinterpret_cast<int *>(w + kBinvBytes), (double)cond_limit, allow_start ? 1 : 0);
     ++*launches;
     return cudaGetLastError();
 }

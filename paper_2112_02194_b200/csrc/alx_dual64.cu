@@ -10,6 +10,7 @@
 // B^-1 in fp64 once per half-epoch and sets a flag from ||B||_F ||B^-1||_F; with the flag clear this kernel does
 // nothing and the whole-rows kernel takes these rows as well.
 #include "alx_common.cuh"
+#include "alx_inverse.cuh"
 
 namespace alx {
 
@@ -18,70 +19,14 @@ namespace {
 constexpr int D = 64;
 constexpr int kWarps = 8;
 
-// B^-1 in fp64 by Cholesky (one block of 64 threads, thread i = row i), written in fp32
-__global__ void __launch_bounds__(D, 1) k_binv64_prepare(const float *__restrict__ Bmat, float *__restrict__ Binv,
-                                                         int *__restrict__ flag, double cond_limit)
+// B^-1 in fp64 (alx_inverse.cuh), written in fp32
+__global__ void __launch_bounds__(SweepGeo<D>::THREADS, 1) k_binv64_prepare(const float *__restrict__ Bmat, float *__restrict__ Binv,
+                                                                           int *__restrict__ flag, double cond_limit)
 {
-    constexpr int LD = D + 1;
-    __shared__ double A[D * LD];       // lower = L, strict upper = (L^-1)^T
-    __shared__ double dinv[D], red[D];
-    __shared__ int s_ok;
-    const int i = threadIdx.x;
-    if (i == 0) s_ok = 1;
-    double fro = 0.0;
-    for (int c = 0; c < D; ++c) {
-        const double v = (double)Bmat[i * D + c];
-        A[i * LD + c] = v;
-        fro += v * v;
-    }
-    red[i] = fro;
-    __syncthreads();
-    for (int j = 0; j < D; ++j) {
-        if (i == j) {
-            const double p = A[j * LD + j];
-            if (!(p > 0.0)) s_ok = 0;
-            const double l = sqrt(p > 0.0 ? p : 1.0);
-            A[j * LD + j] = l;
-            dinv[j] = 1.0 / l;
-        }
-        __syncthreads();
-        if (i > j) A[i * LD + j] *= dinv[j];
-        __syncthreads();
-        if (i > j) {
-            const double lij = A[i * LD + j];
-            for (int c = j + 1; c <= i; ++c) A[i * LD + c] -= lij * A[c * LD + j];
-        }
-        __syncthreads();
-    }
-    // column i of L^-1, stored transposed in the strict upper triangle: A[i][r] = Linv[r][i], r > i
-    for (int r = i + 1; r < D; ++r) {
-        double s = A[r * LD + i] * dinv[i];
-        for (int k = i + 1; k < r; ++k) s += A[r * LD + k] * A[i * LD + k];
-        A[i * LD + r] = -s * dinv[r];
-    }
-    __syncthreads();
-    // row i of B^-1 = (L^-1)^T L^-1
-    double fro_inv = 0.0;
-    for (int c = 0; c < D; ++c) {
-        const int m = i > c ? i : c;
-        double s = 0.0;
-        for (int k = m; k < D; ++k) {
-            const double a = (k == i) ? dinv[i] : A[i * LD + k];
-            const double b = (k == c) ? dinv[c] : A[c * LD + k];
-            s += a * b;
-        }
-        fro_inv += s * s;
-        Binv[i * D + c] = (float)s;
-    }
-    __syncthreads();
-    dinv[i] = fro_inv;      // (dinv is not needed any more)
-    __syncthreads();
-    if (i == 0) {
-        double f = 0.0, g = 0.0;
-        for (int k = 0; k < D; ++k) { f += red[k]; g += dinv[k]; }
-        const double cond = sqrt(f) * sqrt(g);
-        *flag = (s_ok && cond <= cond_limit) ? 1 : 0;
-    }
+    __shared__ SweepSmem<D> sm;
+    double cond;
+    const bool ok = sweep_inverse<D>(Bmat, sm, &cond, [&](int i, int c, double v) { Binv[i * D + c] = (float)v; });
+    if (threadIdx.x == 0) *flag = (ok && cond <= cond_limit) ? 1 : 0;
 }
 
 // sum over the 32 lanes of each of N values (N a power of two <= 16): afterwards the sum of v[c] is in v[0] of the lanes
@@ -250,7 +195,7 @@ int *dual64_flag_ptr(void *ws) { return reinterpret_cast<int *>(static_cast<unsi
 
 cudaError_t launch_dual64_prepare(const float *Bmat, void *ws, float cond_limit, cudaStream_t s, int64_t *launches)
 {
-    k_binv64_prepare<<<1, D, 0, s>>>(Bmat, static_cast<float *>(ws), dual64_flag_ptr(ws), (double)cond_limit);
+    k_binv64_prepare<<<1, SweepGeo<D>::THREADS, 0, s>>>(Bmat, static_cast<float *>(ws), dual64_flag_ptr(ws), (double)cond_limit);
     ++*launches;
     return cudaGetLastError();
 }
