@@ -31,23 +31,39 @@ __device__ __forceinline__ int64_t warp_row_of(const int64_t *__restrict__ ptr, 
     return lo;
 }
 
-__device__ __forceinline__ float dot16(const uint4 &a, const uint4 &b, float)
+// 16 bytes of a table row as floats
+__device__ __forceinline__ void unpack16(const uint4 &a, float (&v)[4])
 {
-    float s = __uint_as_float(a.x) * __uint_as_float(b.x);
-    s = fmaf(__uint_as_float(a.y), __uint_as_float(b.y), s);
-    s = fmaf(__uint_as_float(a.z), __uint_as_float(b.z), s);
-    return fmaf(__uint_as_float(a.w), __uint_as_float(b.w), s);
+    v[0] = __uint_as_float(a.x); v[1] = __uint_as_float(a.y); v[2] = __uint_as_float(a.z); v[3] = __uint_as_float(a.w);
 }
-__device__ __forceinline__ float dot16(const uint4 &a, const uint4 &b, __nv_bfloat16)
+__device__ __forceinline__ void unpack16(const uint4 &a, float (&v)[8])
 {
-    const uint32_t x[4] = {a.x, a.y, a.z, a.w}, y[4] = {b.x, b.y, b.z, b.w};
-    float s = 0.f;
+    const uint32_t x[4] = {a.x, a.y, a.z, a.w};
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        s = fmaf(__uint_as_float(x[k] << 16), __uint_as_float(y[k] << 16), s);
-        s = fmaf(__uint_as_float(x[k] & 0xFFFF0000u), __uint_as_float(y[k] & 0xFFFF0000u), s);
+        v[2 * k] = __uint_as_float(x[k] << 16);
+        v[2 * k + 1] = __uint_as_float(x[k] & 0xFFFF0000u);
     }
-    return s;
+}
+
+// sums over the LANES lanes of a group of each of U values (U = 4, or 2 for LANES = 2): lane `part` of a group with
+// t0 <= part < t0 + U receives the sum of v[part - t0].  The values are halved with the lanes: U - 1 shuffles, then one value's
+// butterfly, then one shuffle to the lane that wants it.
+template <int LANES, int U> __device__ __forceinline__ float group_sums(float (&v)[U], int t0, int lane)
+{
+    int o = LANES / 2;
+#pragma unroll
+    for (int n = U / 2; n > 0; n /= 2, o /= 2) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int k = 0; k < n; ++k) {
+            const float send = up ? v[k] : v[k + n], keep = up ? v[k + n] : v[k];
+            v[k] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, o);
+        }
+    }
+#pragma unroll
+    for (; o > 0; o /= 2) v[0] += __shfl_xor_sync(0xFFFFFFFFu, v[0], o);
+    return __shfl_sync(0xFFFFFFFFu, v[0], (lane & ~(LANES - 1)) + (((lane & (LANES - 1)) - t0) & (U - 1)) * (LANES / U));
 }
 
 __device__ __forceinline__ double block_sum(double v, double *buf)
@@ -62,9 +78,10 @@ __device__ __forceinline__ double block_sum(double v, double *buf)
     return r;
 }
 
-// A warp takes spans of entries, 32 at a time: every lane looks up its entry's column, label and row (a window of
-// the row offsets, searched by shuffles), then LANES lanes share an entry, 16 bytes of both rows each, 32 / LANES entries
-// side by side and four such rounds of loads in flight.  Bound: the gather of the H rows (L2 where they are local).  The last
+// A warp takes spans of entries, 32 at a time: every lane looks up its entry's column, label and row (a window of the row offsets,
+// searched by shuffles).  A group of LANES lanes then works through LANES of the entries in turn, 16 bytes of a row a lane, so
+// that the W row stays in registers while the row goes on; four entries' loads are in flight and their sums share a
+// butterfly.  Bound: the gather of the H rows, and the 16 instructions an entry of 128 bfloat16 features takes.  The last
 // block to finish adds the blocks' sums in order and the two Gramian terms.
 template <int D, typename T>
 __global__ void __launch_bounds__(kWarps * 32) k_loss(const int64_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
@@ -73,19 +90,20 @@ __global__ void __launch_bounds__(kWarps * 32) k_loss(const int64_t *__restrict_
                                                       const double *__restrict__ GH, double alpha0, double lambda, double *partials,
                                                       double *result)
 {
-    constexpr int EL = 16 / (int)sizeof(T), LANES = D / EL, SIDE = 32 / LANES;      // lanes per entry, entries side by side
-    constexpr int UNROLL = 32 / SIDE < 4 ? 32 / SIDE : 4;
+    constexpr int EL = 16 / (int)sizeof(T), LANES = D / EL, U = LANES < 4 ? LANES : 4;
     __shared__ double buf[kWarps];
     __shared__ int last_s;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int part = lane % LANES, sub = lane / LANES;
+    const int part = lane % LANES, first = lane - part;      // first lane of the group
     double acc = 0.0;
     for (int64_t e0 = ((int64_t)blockIdx.x * kWarps + warp) * kSpan; e0 < nnz; e0 += (int64_t)gridDim.x * kWarps * kSpan) {
         const int64_t e1 = e0 + kSpan < nnz ? e0 + kSpan : nnz;
         int64_t u = warp_row_of(rowptr, n_rows, e0, lane);
+        int w_row = -1;
+        float w[EL];
         for (int64_t base = e0; base < e1; base += 32) {
             const int64_t e = base + lane;
-            const int64_t lastE = e1 - 1 < base + 31 ? e1 - 1 : base + 31;
+            const int64_t last = e1 - 1 < base + 31 ? e1 - 1 : base + 31;
             const int32_t c = e < e1 ? colidx[e] : 0;
             const float y = values && e < e1 ? values[e] : 1.f;
             // row of this lane's entry: count the offsets ptr[u + 1 ..] that are <= e
@@ -101,31 +119,39 @@ __global__ void __launch_bounds__(kWarps * 32) k_loss(const int64_t *__restrict_
                 const int64_t q = __shfl_sync(0xFFFFFFFFu, p, 31);
                 if (lo == 31 && q <= e) lo = 32;
                 row += lo;
-                if (q > lastE) break;      // (warp-uniform: the 32nd offset lies beyond the batch)
+                if (q > last) break;      // (warp-uniform: the 32nd offset lies beyond the batch)
                 at += 32;
             }
-            u = __shfl_sync(0xFFFFFFFFu, row, (int)(lastE - base));
+            u = __shfl_sync(0xFFFFFFFFu, row, (int)(last - base));
+            float dot = 0.f;
 #pragma unroll 1
-            for (int t0 = 0; t0 < 32 / SIDE; t0 += UNROLL) {
-                if (base + t0 * SIDE > lastE) break;
-                uint4 h[UNROLL], w[UNROLL];
+            for (int t0 = 0; t0 < LANES; t0 += U) {
+                uint4 h[U];
+                int wr[U];
 #pragma unroll
-                for (int k = 0; k < UNROLL; ++k) {
-                    const int src = (t0 + k) * SIDE + sub;
-                    const int64_t hc = __shfl_sync(0xFFFFFFFFu, c, src), wr = __shfl_sync(0xFFFFFFFFu, row, src);
+                for (int k = 0; k < U; ++k) {
+                    const int64_t hc = __shfl_sync(0xFFFFFFFFu, c, first + t0 + k);
+                    wr[k] = __shfl_sync(0xFFFFFFFFu, (int)row, first + t0 + k);
                     h[k] = __ldg(reinterpret_cast<const uint4 *>(H + hc * D) + part);
-                    w[k] = __ldg(reinterpret_cast<const uint4 *>(W + wr * D) + part);
                 }
+                float s[U];
 #pragma unroll
-                for (int k = 0; k < UNROLL; ++k) {
-                    const int src = (t0 + k) * SIDE + sub;
-                    float dot = dot16(w[k], h[k], T());
+                for (int k = 0; k < U; ++k) {
+                    if (wr[k] != w_row) {
+                        w_row = wr[k];
+                        unpack16(__ldg(reinterpret_cast<const uint4 *>(W + (int64_t)w_row * D) + part), w);
+                    }
+                    float hv[EL];
+                    unpack16(h[k], hv);
+                    s[k] = w[0] * hv[0];
 #pragma unroll
-                    for (int o = LANES / 2; o > 0; o >>= 1) dot += __shfl_xor_sync(0xFFFFFFFFu, dot, o);
-                    const double r = (double)__shfl_sync(0xFFFFFFFFu, y, src) - (double)dot;
-                    if (part == 0 && base + src <= lastE) acc = fma(r, r, acc);
+                    for (int j = 1; j < EL; ++j) s[k] = fmaf(w[j], hv[j], s[k]);
                 }
+                const float d = group_sums<LANES, U>(s, t0, lane);
+                if (part - t0 >= 0 && part - t0 < U) dot = d;
             }
+            const double r = (double)y - (double)dot;
+            if (e < e1) acc = fma(r, r, acc);
         }
     }
     const double mine = block_sum(acc, buf);
