@@ -9,7 +9,8 @@ namespace alx {
 namespace {
 
 constexpr int kWarps = 8;
-constexpr int64_t kMostBlocks = 148 * 8;
+constexpr int kBlocksPerSm = 3;
+constexpr int64_t kMostBlocks = 148 * kBlocksPerSm;
 // Entries a warp takes at a time; the warps then go on together to the next stretch of the matrix, so that at any time they
 // read neighbouring rows of W, and of H where the matrix is local (one long range per warp spread them over the whole table:
 // 70 ms instead of 35 ms for 1e9 entries within 1 % of the diagonal)
@@ -81,10 +82,10 @@ __device__ __forceinline__ double block_sum(double v, double *buf)
 // A warp takes spans of entries, 32 at a time: every lane looks up its entry's column, label and row (a window of the row offsets,
 // searched by shuffles).  A group of LANES lanes then works through LANES of the entries in turn, 16 bytes of a row a lane, so
 // that the W row stays in registers while the row goes on; four entries' loads are in flight and their sums share a
-// butterfly.  Bound: the gather of the H rows, and the 16 instructions an entry of 128 bfloat16 features takes.  The last
+// butterfly.  Bound: the latency of the H rows' gather (two rounds in flight, 24 warps per SM), and the 16 instructions an entry of 128 bfloat16 features takes.  The last
 // block to finish adds the blocks' sums in order and the two Gramian terms.
 template <int D, typename T>
-__global__ void __launch_bounds__(kWarps * 32) k_loss(const int64_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
+__global__ void __launch_bounds__(kWarps * 32, kBlocksPerSm) k_loss(const int64_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
                                                       const float *__restrict__ values, int64_t n_rows, int64_t nnz,
                                                       const T *__restrict__ W, const T *__restrict__ H, const double *__restrict__ GW,
                                                       const double *__restrict__ GH, double alpha0, double lambda, double *partials,
@@ -124,25 +125,28 @@ __global__ void __launch_bounds__(kWarps * 32) k_loss(const int64_t *__restrict_
             }
             u = __shfl_sync(0xFFFFFFFFu, row, (int)(last - base));
             float dot = 0.f;
-#pragma unroll 1
-            for (int t0 = 0; t0 < LANES; t0 += U) {
-                uint4 h[U];
-                int wr[U];
+            uint4 h[2][U];
+            auto load = [&](int t0, uint4(&to)[U]) {
 #pragma unroll
                 for (int k = 0; k < U; ++k) {
                     const int64_t hc = __shfl_sync(0xFFFFFFFFu, c, first + t0 + k);
-                    wr[k] = __shfl_sync(0xFFFFFFFFu, (int)row, first + t0 + k);
-                    h[k] = __ldg(reinterpret_cast<const uint4 *>(H + hc * D) + part);
+                    to[k] = __ldg(reinterpret_cast<const uint4 *>(H + hc * D) + part);
                 }
+            };
+            load(0, h[0]);
+#pragma unroll
+            for (int t0 = 0; t0 < LANES; t0 += U) {
+                if (t0 + U < LANES) load(t0 + U, h[(t0 / U + 1) & 1]);      // one round ahead
                 float s[U];
 #pragma unroll
                 for (int k = 0; k < U; ++k) {
-                    if (wr[k] != w_row) {
-                        w_row = wr[k];
+                    const int wr = __shfl_sync(0xFFFFFFFFu, (int)row, first + t0 + k);
+                    if (wr != w_row) {
+                        w_row = wr;
                         unpack16(__ldg(reinterpret_cast<const uint4 *>(W + (int64_t)w_row * D) + part), w);
                     }
                     float hv[EL];
-                    unpack16(h[k], hv);
+                    unpack16(h[(t0 / U) & 1][k], hv);
                     s[k] = w[0] * hv[0];
 #pragma unroll
                     for (int j = 1; j < EL; ++j) s[k] = fmaf(w[j], hv[j], s[k]);
