@@ -21,30 +21,27 @@ struct alx_ctx {
     cudaStream_t stream = nullptr;
     int bf16 = 0;
     size_t elem = 4;
-    int64_t n[4] = {0, 0, 0, 0};   // n[ALX_ROWS] = n_rows, n[ALX_COLS] = n_cols (and again for the doubled lists, see below)
+    int64_t n[2] = {0, 0};         // n[ALX_ROWS] = n_rows, n[ALX_COLS] = n_cols
     int64_t nnz = -1;
     int64_t split = ALX_DEFAULT_SPLIT;
     bool has_values = false;
     bool have_table[2] = {false, false};
     bool have_gram[2] = {false, false};
 
-    // per orientation: [ALX_ROWS] = CSR (rows of the matrix), [ALX_COLS] = CSC.  Slots 2 and 3 (fp32 tables of 64 features
-    // on the tensor cores only): the same two orientations with every row's entry list doubled over the table of
-    // bfloat16 parts, which is what that path's kernels walk; with degree classes and chunks of their own.
-    int64_t *ptr[4] = {nullptr, nullptr, nullptr, nullptr};
-    int32_t *idx[4] = {nullptr, nullptr, nullptr, nullptr};
-    float *val[4] = {nullptr, nullptr, nullptr, nullptr};
-    int32_t *order[4] = {nullptr, nullptr, nullptr, nullptr};
-    int64_t *class_offs_dev[4] = {nullptr, nullptr, nullptr, nullptr};
-    int64_t class_offs[4][ALX_N_CLASSES + 1] = {};
-    int64_t *chunk_desc[4] = {nullptr, nullptr, nullptr, nullptr};
-    int64_t *split_first[4] = {nullptr, nullptr, nullptr, nullptr};
-    int64_t n_chunks[4] = {0, 0, 0, 0};
-    int64_t n_split_rows[4] = {0, 0, 0, 0};
+    // per orientation: [ALX_ROWS] = CSR (rows of the matrix), [ALX_COLS] = CSC
+    int64_t *ptr[2] = {nullptr, nullptr};
+    int32_t *idx[2] = {nullptr, nullptr};
+    float *val[2] = {nullptr, nullptr};
+    int32_t *order[2] = {nullptr, nullptr};
+    int64_t *class_offs_dev[2] = {nullptr, nullptr};
+    int64_t class_offs[2][ALX_N_CLASSES + 1] = {};
+    int64_t *chunk_desc[2] = {nullptr, nullptr};
+    int64_t *split_first[2] = {nullptr, nullptr};
+    int64_t n_chunks[2] = {0, 0};
+    int64_t n_split_rows[2] = {0, 0};
     // tensor path with the dual form: the rows of 1 .. 16 entries once more per orientation, those with at most 8 entries first
     int32_t *order16[2] = {nullptr, nullptr};
     int64_t n4[2] = {0, 0}, n8[2] = {0, 0};      // ... and those with at most 4 before them
-    void *fold_table = nullptr;   // that path's fixed table: [2 N x 128] bfloat16 parts of the fp32 table, rebuilt every half-epoch
 
     void *table[2] = {nullptr, nullptr};
     double *G64[2] = {nullptr, nullptr};   // Gramian of table [side]
@@ -249,16 +246,14 @@ alx_status build_buckets(alx_ctx *c, int side, int64_t *scratch_a, int64_t *scra
                                       c->chunk_desc[side], c->stream, &c->launches));
         ALX_CUDA(c, cudaStreamSynchronize(c->stream));
     }
-    if (side < 2) {
-        for (int k = 0; k < ALX_N_CLASSES; ++k) c->stats.rows_in_class[side][k] = offs[k + 1] - offs[k];
-        c->stats.n_chunks[side] = c->n_chunks[side];
-    }
+    for (int k = 0; k < ALX_N_CLASSES; ++k) c->stats.rows_in_class[side][k] = offs[k + 1] - offs[k];
+    c->stats.n_chunks[side] = c->n_chunks[side];
     return ALX_OK;
 }
 
 void release_matrix(alx_ctx *c)
 {
-    for (int s = 0; s < 4; ++s) {
+    for (int s = 0; s < 2; ++s) {
         dev_free(c, c->ptr[s]); c->ptr[s] = nullptr;
         dev_free(c, c->idx[s]); c->idx[s] = nullptr;
         dev_free(c, c->val[s]); c->val[s] = nullptr;
@@ -273,11 +268,14 @@ void release_matrix(alx_ctx *c)
 }
 
 bool tensor_path(const alx_ctx *c) { return c->bf16 && c->opt.d == 128 && c->opt.kernels != 1; }
-// fp32 tables of 64 features: tensor cores through bfloat16 parts and doubled entry lists (ids up to 2 N must fit int32)
-bool fold_path(const alx_ctx *c)
-{
-    return !c->bf16 && c->opt.d == 64 && c->opt.kernels != 1 && c->n[0] < (1ll << 30) && c->n[1] < (1ll << 30);
-}
+// d <= 64: a warp per row (alx_rows_warp.cu)
+bool warp_path(const alx_ctx *c) { return c->opt.d <= 64 && c->opt.kernels != 1; }
+// of those, fp32 tables of 64 features: conjugate gradients, and the dual form for rows of at most 16 observations
+bool cg64(const alx_ctx *c) { return warp_path(c) && !c->bf16 && c->opt.d == 64; }
+bool dual64(const alx_ctx *c) { return cg64(c) && c->opt.kernels == 0; }
+// Fewer rows than this are not worth the inverse of the base matrix that the dual form starts with (25 us and more, against
+// a few ns per row): they take the d x d solve with the others
+constexpr int64_t kDualLeastRows = 256;
 bool dual_form(const alx_ctx *c) { return tensor_path(c) && c->opt.kernels == 0; }
 float dual_cond_limit(const alx_ctx *c) { return c->opt.dual_cond_limit > 0.f ? c->opt.dual_cond_limit : ALX_DEFAULT_DUAL_COND_LIMIT; }
 CgOptions cg_options(const alx_ctx *c, int solved_side)
@@ -295,6 +293,14 @@ CgOptions cg_options(const alx_ctx *c, int solved_side)
     return o;
 }
 
+// rows of a side that the dual form is offered (class 1, and class 2 for d = 128); 0: none, or too few
+int64_t dual_rows_of(const alx_ctx *c, int side)
+{
+    const int64_t *offs = c->class_offs[side];
+    const int64_t n = dual_form(c) ? offs[3] - offs[1] : dual64(c) ? offs[2] - offs[1] : 0;
+    return n >= kDualLeastRows ? n : 0;
+}
+
 // the Gramian and the base matrix of a table; `solve`: also what the rows' dual form needs of the base matrix
 alx_status gramian_of(alx_ctx *c, int table_side, bool solve)
 {
@@ -309,7 +315,7 @@ alx_status gramian_of(alx_ctx *c, int table_side, bool solve)
     }
     ALX_CUDA(c, launch_gramian(c->table[table_side], c->bf16, c->n[table_side], c->opt.d, c->gram_partials,
                                c->G64[table_side], c->Bmat, c->opt.alpha0, c->opt.lambda, c->stream, &c->launches));
-    if (solve && fold_path(c) && c->dual_ws)
+    if (solve && dual64(c))
         ALX_CUDA(c, launch_dual64_prepare(c->Bmat, c->dual_ws, dual_cond_limit(c), c->stream, &c->launches));
     c->have_gram[table_side] = true;
     return ALX_OK;
@@ -325,45 +331,44 @@ alx_status half_epoch_impl(alx_ctx *c, int side, const int32_t *cap_slot, float 
     alx_status st;
     {
         NvtxRange r("alx Gramian + base matrix");
-        st = gramian_of(c, fixed, true);
+        st = gramian_of(c, fixed, dual_rows_of(c, side) > 0);
     }
     if (st != ALX_OK) return st;
     ALX_CUDA(c, cudaEventRecord(c->ev[1], c->stream));
     NvtxRange rows_range("alx rows: gather, sums, solve, store");
     RowOut out{c->table[side], cap_slot, cap_out};
-    if (fold_path(c)) {
-        ALX_CUDA(c, cudaMemsetAsync(c->cg_counters, 0, 5 * sizeof(unsigned long long), c->stream));
-        ALX_CUDA(c, launch_split_table(static_cast<const float *>(c->table[fixed]), c->n[fixed], c->fold_table, c->stream,
-                                       &c->launches));
-        // rows of 1 .. 16 observations (class 1 of the entry lists as given = classes 1 and 2 of the doubled ones): dual form
-        const int64_t n_dual = c->dual_ws ? c->class_offs[side][2] - c->class_offs[side][1] : 0;
+    c->dual_candidates = c->dual_candidates32 = 0;
+    c->dual_flag_latched = 0;
+    c->policy_latched = CgPolicy{};
+    if (warp_path(c)) {
+        if (cg64(c)) ALX_CUDA(c, cudaMemsetAsync(c->cg_counters, 0, 5 * sizeof(unsigned long long), c->stream));
+        const int64_t n_dual = dual_rows_of(c, side);
         if (n_dual > 0)
             ALX_CUDA(c, launch_rows_dual64(side_view(c, side), c->class_offs[side][1], n_dual, c->table[fixed], c->dual_ws, out,
                                            c->stream, &c->launches));
-        ALX_CUDA(c, launch_rows_fold(side_view(c, 2 + side), c->class_offs[2 + side], c->n_chunks[2 + side],
-                                     c->n_split_rows[2 + side], c->fold_table, 2 * c->n[fixed], c->Bmat, c->split_partials,
-                                     out, c->status, c->stream, &c->launches, c->ev[3], c->ev[4], cg_options(c, side),
-                                     n_dual > 0 ? dual64_flag_ptr(c->dual_ws) : nullptr));
+        ALX_CUDA(c, cudaEventRecord(c->ev[3], c->stream));
+        ALX_CUDA(c, launch_rows_warp(side_view(c, side), c->class_offs[side], c->n_chunks[side], c->n_split_rows[side], c->table[fixed],
+                                     c->bf16, c->opt.d, c->Bmat, c->split_partials, out, c->status, cg_options(c, side),
+                                     n_dual > 0 ? dual64_flag_ptr(c->dual_ws) : nullptr, c->stream, &c->launches));
+        ALX_CUDA(c, cudaEventRecord(c->ev[4], c->stream));
         c->stats.kernel_path[side] = 1;
         c->main_timed = true;
         c->dual_candidates = n_dual;
-        c->dual_flag_latched = 0;
         if (n_dual > 0)
             ALX_CUDA(c, cudaMemcpyAsync(&c->dual_flag_latched, dual64_flag_ptr(c->dual_ws), sizeof(int), cudaMemcpyDeviceToHost,
                                         c->stream));
     } else if (tensor_path(c)) {
+        const int64_t n_dual = dual_rows_of(c, side);
         ALX_CUDA(c, cudaMemsetAsync(c->cg_counters, 0, 5 * sizeof(unsigned long long), c->stream));
         ALX_CUDA(c, launch_rows_umma(side_view(c, side), c->class_offs[side], c->n_chunks[side], c->n_split_rows[side],
                                      c->table[fixed], c->Bmat, c->split_partials, out, c->status, c->stream,
-                                     &c->launches, c->ev[3], c->ev[4], dual_form(c) ? c->dual_ws : nullptr, c->n[fixed],
+                                     &c->launches, c->ev[3], c->ev[4], n_dual > 0 ? c->dual_ws : nullptr, c->n[fixed],
                                      cg_options(c, side), c->order16[side], c->n4[side], c->n8[side]));
         c->stats.kernel_path[side] = 1;
         c->main_timed = true;
-        c->dual_candidates = dual_form(c) ? c->class_offs[side][3] - c->class_offs[side][1] : 0;
-        c->dual_candidates32 = dual_form(c) ? c->class_offs[side][3] - c->class_offs[side][2] : 0;
-        c->dual_flag_latched = 0;
-        c->policy_latched = CgPolicy{};
-        if (c->dual_candidates > 0) {
+        c->dual_candidates = n_dual;
+        c->dual_candidates32 = n_dual > 0 ? c->class_offs[side][3] - c->class_offs[side][2] : 0;
+        if (n_dual > 0) {
             ALX_CUDA(c, cudaMemcpyAsync(&c->dual_flag_latched, dual_flag_ptr(c->dual_ws), sizeof(int), cudaMemcpyDeviceToHost,
                                         c->stream));
             if (c->cg_policy && c->opt.solver == ALX_SOLVER_AUTO)
@@ -371,12 +376,9 @@ alx_status half_epoch_impl(alx_ctx *c, int side, const int32_t *cap_slot, float 
                                             c->stream));
         }
     } else {
-        const bool warp_rows = c->opt.kernels != 1 && c->opt.d <= 64;
-        ALX_CUDA(c, (warp_rows ? launch_rows_warp : launch_rows_simple)(side_view(c, side), c->class_offs[side], c->n_chunks[side],
-                                                                       c->n_split_rows[side], c->table[fixed], c->bf16, c->opt.d, c->Bmat,
-                                                                       c->split_partials, out, c->status, c->stream, &c->launches));
-        c->stats.kernel_path[side] = warp_rows ? 1 : 0;
-        c->dual_candidates = 0;
+        ALX_CUDA(c, launch_rows_simple(side_view(c, side), c->class_offs[side], c->n_chunks[side], c->n_split_rows[side], c->table[fixed],
+                                       c->bf16, c->opt.d, c->Bmat, c->split_partials, out, c->status, c->stream, &c->launches));
+        c->stats.kernel_path[side] = 0;
     }
     ALX_CUDA(c, cudaEventRecord(c->ev[2], c->stream));
     c->have_table[side] = true;
@@ -436,8 +438,8 @@ alx_status create_impl(const alx_options *opt, const alx_ctx *parent, alx_ctx **
     c->stream = static_cast<cudaStream_t>(opt->stream);
     c->bf16 = opt->storage == ALX_BF16;
     c->elem = c->bf16 ? 2 : 4;
-    c->n[ALX_ROWS] = c->n[2 + ALX_ROWS] = opt->n_rows;
-    c->n[ALX_COLS] = c->n[2 + ALX_COLS] = opt->n_cols;
+    c->n[ALX_ROWS] = opt->n_rows;
+    c->n[ALX_COLS] = opt->n_cols;
     c->split = opt->split ? opt->split : ALX_DEFAULT_SPLIT;
     DeviceGuard guard(dev);
     auto body = [&]() -> alx_status {
@@ -448,18 +450,13 @@ alx_status create_impl(const alx_options *opt, const alx_ctx *parent, alx_ctx **
             c->table[s] = t;
             ALX_ALLOC(c, c->G64[s], d * d);
             ALX_ALLOC(c, c->class_offs_dev[s], ALX_N_CLASSES + 1);
-            if (fold_path(c)) ALX_ALLOC(c, c->class_offs_dev[2 + s], ALX_N_CLASSES + 1);
         }
         ALX_ALLOC(c, c->Bmat, d * d);
-        if (dual_form(c) || (fold_path(c) && c->opt.kernels == 0)) {
+        if (dual_form(c) || dual64(c)) {
             c->dual_ws = dev_alloc(c, dual_form(c) ? dual_workspace_bytes() : dual64_workspace_bytes());
             if (!c->dual_ws) return fail(c, ALX_ERR_OOM, "device allocation of the dual-form workspace failed");
         }
         const int64_t nmax = c->n[0] > c->n[1] ? c->n[0] : c->n[1];
-        if (fold_path(c)) {
-            c->fold_table = dev_alloc(c, (size_t)2 * nmax * 128 * 2);
-            if (!c->fold_table) return fail(c, ALX_ERR_OOM, "device allocation of the table of bfloat16 parts failed");
-        }
         int64_t n_part = gramian_partials(nmax);
         if (gramian_umma_partials() > n_part) n_part = gramian_umma_partials();
         ALX_ALLOC(c, c->gram_partials, n_part * d * d);
@@ -468,8 +465,8 @@ alx_status create_impl(const alx_options *opt, const alx_ctx *parent, alx_ctx **
         ALX_ALLOC(c, c->status, 1);
         ALX_CUDA(c, cudaMemsetAsync(c->status, 0, sizeof(DevStatus), c->stream));
         ALX_ALLOC(c, c->cg_counters, 5);
+        if ((tensor_path(c) || cg64(c)) && c->opt.solver == ALX_SOLVER_AUTO) ALX_ALLOC(c, c->cg_fallback_list, nmax);
         if (tensor_path(c) && c->opt.solver == ALX_SOLVER_AUTO) {
-            ALX_ALLOC(c, c->cg_fallback_list, nmax);
             ALX_ALLOC(c, c->cg_policy, 2);
             ALX_CUDA(c, cudaMemsetAsync(c->cg_policy, 0, 2 * sizeof(CgPolicy), c->stream));
         }
@@ -570,19 +567,6 @@ alx_status alx_set_csr(alx_ctx *c, const int64_t *rowptr, const int32_t *colidx,
     }
     st = build_buckets(c, ALX_ROWS, blk_counts, blk_offs, scan_scratch, scan_elems);
     if (st != ALX_OK) return st;
-    if (fold_path(c)) {
-        // the doubled entry lists of both orientations, with degree classes and chunks of their own
-        for (int s = 0; s < 2; ++s) {
-            ALX_ALLOC(c, c->ptr[2 + s], c->n[s] + 1);
-            ALX_ALLOC(c, c->idx[2 + s], 2 * nz);
-            if (values) ALX_ALLOC(c, c->val[2 + s], 2 * nz);
-            ALX_ALLOC(c, c->order[2 + s], c->n[s]);
-            ALX_CUDA(c, launch_double_entries(c->ptr[s], c->idx[s], c->val[s], c->n[s], c->n[1 - s], c->ptr[2 + s],
-                                              c->idx[2 + s], c->val[2 + s], c->stream, &c->launches));
-            st = build_buckets(c, 2 + s, blk_counts, blk_offs, scan_scratch, scan_elems);
-            if (st != ALX_OK) return st;
-        }
-    }
     if (dual_form(c)) {
         // the rows of 1 .. 16 entries, ordered by length class (at most 4, 5 .. 8, 9 .. 16): kernel instances with four and
         // eight observations per row take the first two parts at a quarter and half of the cost per row
@@ -629,28 +613,25 @@ alx_status alx_set_csr(alx_ctx *c, const int64_t *rowptr, const int32_t *colidx,
     tmp.release(class_entries);
 
     const int d = c->opt.d;
-    const int kb = fold_path(c) ? 2 : 0;      // the lists the row kernels walk
-    const int dk = fold_path(c) ? 128 : d;    // the width of the sums they form
-    int64_t sums[2] = {c->n_chunks[kb], c->n_chunks[kb + 1]};
+    int64_t sums[2] = {c->n_chunks[0], c->n_chunks[1]};
     for (int s = 0; s < 2; ++s) c->stats.long_rows[s] = c->stats.long_entries[s] = 0;
-    if (tensor_path(c) || fold_path(c)) {    // one more sum per long whole row
+    if (tensor_path(c) || warp_path(c)) {    // d = 128: one more sum per long whole row
         int64_t *total = nullptr;
         ALX_TMP(c, tmp, total, 2);
         for (int s = 0; s < 2; ++s) {
-            const int64_t *offs = c->class_offs[kb + s];
-            const int64_t first = offs[long_class_begin(offs)];
+            const int64_t *offs = c->class_offs[s];
+            const int64_t first = offs[tensor_path(c) ? long_class_begin(offs) : kWarpLongClass];
             const int64_t n_long = offs[kNClasses - 1] - first;
-            sums[s] += n_long;
+            if (tensor_path(c)) sums[s] += n_long;
             c->stats.long_rows[s] = n_long;
-            ALX_CUDA(c, launch_sum_row_lengths(c->ptr[kb + s], c->order[kb + s] + first, n_long, total + s, c->stream, &c->launches));
+            ALX_CUDA(c, launch_sum_row_lengths(c->ptr[s], c->order[s] + first, n_long, total + s, c->stream, &c->launches));
         }
         ALX_CUDA(c, cudaMemcpyAsync(c->stats.long_entries, total, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost, c->stream));
         ALX_CUDA(c, cudaStreamSynchronize(c->stream));
-        if (fold_path(c)) for (int s = 0; s < 2; ++s) c->stats.long_entries[s] /= 2;      // (every entry is listed twice there)
         tmp.release(total);
     }
     const int64_t max_chunks = sums[0] > sums[1] ? sums[0] : sums[1];
-    if (max_chunks > 0) ALX_ALLOC(c, c->split_partials, max_chunks * (int64_t)(dk * dk + dk));
+    if (max_chunks > 0) ALX_ALLOC(c, c->split_partials, max_chunks * (int64_t)(d * d + d));
     ALX_ALLOC(c, c->loss_partials_buf, loss_partials(nnz));
     c->stats.nnz = nnz;
     return ALX_OK;

@@ -139,11 +139,6 @@ cudaError_t launch_rows_simple(const SideView &sv, const int64_t *class_offs_hos
                                float *split_partials, RowOut out, DevStatus *st, cudaStream_t s,
                                int64_t *launches);
 
-// alx_rows_warp.cu: d = 16, 32, 64, a warp per row (kernels != 1)
-cudaError_t launch_rows_warp(const SideView &sv, const int64_t *class_offs_host, int64_t n_chunks, int64_t n_split_rows, const void *X,
-                             int bf16, int d, const float *Bmat, float *split_partials, RowOut out, DevStatus *st, cudaStream_t s,
-                             int64_t *launches);
-
 // Tensor-core path: the first degree class whose rows (with all longer whole rows) get their sums from the chunks
 // kernel instead of the rows kernel.  Classes 8 .. 10 (1025 .. 8192 observations at the default split) qualify, from
 // the top, as long as they hold at most kLongRowBudget rows together (one d x d + d sum of workspace each).
@@ -188,6 +183,13 @@ struct CgOptions {
     CgPolicy *policy;              // device, this side's record
     float switch_products;         // mean products per row beyond which the side's next half-epochs take Cholesky
 };
+
+constexpr int kWarpLongClass = 6;      // degree classes from here on (more than 256 entries) get a block of eight warps per row
+// alx_rows_warp.cu: d = 16, 32, 64, a warp per row (kernels != 1); conjugate gradients for fp32 tables of 64 features where
+// cg.enabled.  dual_flag (may be null): device flag, set when the rows of class 1 have been solved in the dual form
+cudaError_t launch_rows_warp(const SideView &sv, const int64_t *class_offs_host, int64_t n_chunks, int64_t n_split_rows, const void *X,
+                             int bf16, int d, const float *Bmat, float *split_partials, RowOut out, DevStatus *st, const CgOptions &cg,
+                             const int *dual_flag, cudaStream_t s, int64_t *launches);
 
 // alx_umma.cu: tensor-core path, d = 128 and bf16 tables only
 int64_t gramian_umma_partials();

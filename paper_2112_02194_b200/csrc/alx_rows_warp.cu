@@ -28,7 +28,7 @@ namespace {
 
 constexpr int kEntries = 16;       // entries per stage = the K of one mma
 constexpr int kBlockWarps = 8;     // warps per row in the long-row kernels
-constexpr int kLongClass = 6;      // degree classes from here on (more than 256 entries) go to the long-row kernel
+constexpr int kLongClass = kWarpLongClass;
 
 template <int D, typename T> struct WGeo {
     static constexpr bool kF32 = sizeof(T) == 4;
@@ -435,6 +435,146 @@ template <int D, typename T> __device__ __forceinline__ void add_base(Sums<D, T>
     }
 }
 
+// ---- conjugate gradients (Sec. 4.5): fp32 tables of 64 features with ALX_SOLVER_AUTO
+struct WarpCg {
+    int max_iter, warm;                // step limit; start from the stored embedding
+    float tol2;
+    unsigned long long *counters;      // rows, products, rows left to the Cholesky kernel (nullptr: Cholesky for every row)
+    int32_t *fallback_list;
+};
+constexpr int kCgVerifyProducts = 24;
+
+// sums over the warp of two values, to every lane: six shuffles
+__device__ __forceinline__ void warp_sums(float &a, float &b, int lane)
+{
+    const bool up = (lane & 16) != 0;
+    float t = (up ? b : a) + __shfl_xor_sync(0xFFFFFFFFu, up ? a : b, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
+    const float other = __shfl_xor_sync(0xFFFFFFFFu, t, 16);
+    a = up ? other : t;
+    b = up ? t : other;
+}
+
+// the warp's 64 x 64 matrix (lower triangle in mma fragments) to lane = rows l and l + 32, whole rows, quadrant by quadrant
+// through shared memory (t: 32 x 36 floats)
+__device__ __forceinline__ void symmetric_rows(const Sums<64, float> &acc, float *t, float (&a0)[64], float (&a1)[64], int lane)
+{
+    constexpr int S = 36;
+    const int r = lane / 4, q = 2 * (lane % 4);
+#pragma unroll
+    for (int pass = 0; pass < 3; ++pass) {      // rows 0..31 x columns 0..31; rows 32..63 x columns 0..31; rows and columns 32..63
+        const int i0 = pass == 0 ? 0 : 2, n0 = pass == 2 ? 4 : 0;
+#pragma unroll
+        for (int i = i0; i < i0 + 2; ++i)
+#pragma unroll
+            for (int n = n0; n < n0 + 4; ++n)
+                if (n < 2 * (i + 1)) {
+                    const float(&c)[4] = acc.c[i * (i + 1) + n];
+                    const int row = 16 * (i - i0) + r, col = 8 * (n - n0) + q;
+                    *reinterpret_cast<float2 *>(t + row * S + col) = make_float2(c[0], c[1]);
+                    *reinterpret_cast<float2 *>(t + (row + 8) * S + col) = make_float2(c[2], c[3]);
+                    if (pass != 1 && i == i0 + 1 && n < n0 + 2) {      // the block above the diagonal is this one's transpose
+                        t[col * S + row] = c[0];
+                        t[(col + 1) * S + row] = c[1];
+                        t[col * S + row + 8] = c[2];
+                        t[(col + 1) * S + row + 8] = c[3];
+                    }
+                }
+        __syncwarp();
+#pragma unroll
+        for (int c = 0; c < 32; c += 4) {
+            const float4 v = *reinterpret_cast<const float4 *>(t + lane * S + c);
+            float *a = pass == 0 ? a0 + c : pass == 1 ? a1 + c : a1 + 32 + c;
+            a[0] = v.x; a[1] = v.y; a[2] = v.z; a[3] = v.w;
+        }
+        if (pass == 1) {
+#pragma unroll
+            for (int c = 0; c < 32; ++c) a0[32 + c] = t[c * S + lane];
+        }
+        __syncwarp();
+    }
+}
+
+// Single-reduction conjugate gradients (Chronopoulos-Gear): one product w = A r and one pair of sums (r.r, r.w) per step.
+// x: the lane's two components of the start vector, then of the solution.  vec: 64 floats of shared memory.  Returns whether
+// |r| <= tol |b| was reached; after many products the true residual is looked at once (the recurrence's can drift).
+__device__ __forceinline__ bool conjugate_gradients(const WarpCg &cg, const float (&a0)[64], const float (&a1)[64], float *vec, float b0, float b1,
+                                                    float &x0, float &x1, int &products, int lane)
+{
+    auto product = [&](float v0, float v1, float &w0, float &w1) {
+        __syncwarp();
+        vec[lane] = v0;
+        vec[lane + 32] = v1;
+        __syncwarp();
+        float2 s0 = make_float2(0.f, 0.f), s1 = s0, t0 = s0, t1 = s0;
+#pragma unroll
+        for (int c = 0; c < 64; c += 4) {
+            const float4 v = *reinterpret_cast<const float4 *>(vec + c);
+            const float2 lo = make_float2(v.x, v.y), hi = make_float2(v.z, v.w);
+            s0 = __ffma2_rn(make_float2(a0[c], a0[c + 1]), lo, s0);
+            s1 = __ffma2_rn(make_float2(a0[c + 2], a0[c + 3]), hi, s1);
+            t0 = __ffma2_rn(make_float2(a1[c], a1[c + 1]), lo, t0);
+            t1 = __ffma2_rn(make_float2(a1[c + 2], a1[c + 3]), hi, t1);
+        }
+        w0 = (s0.x + s0.y) + (s1.x + s1.y);
+        w1 = (t0.x + t0.y) + (t1.x + t1.y);
+        ++products;
+    };
+    bool warm = cg.warm != 0;
+    float w0, w1, r0 = b0, r1 = b1, p0 = 0.f, p1 = 0.f, s0 = 0.f, s1 = 0.f;
+    float bb = b0 * b0 + b1 * b1, unused = 0.f;
+    warp_sums(bb, unused, lane);
+    if (warm) {                 // r = b - A x0
+        product(x0, x1, w0, w1);
+        r0 = b0 - w0;
+        r1 = b1 - w1;
+    } else {
+        x0 = x1 = 0.f;
+    }
+    float rg_old = 0.f, inv_alpha_old = 0.f;
+    bool ok = false;
+    for (int it = 0;; ++it) {
+        product(r0, r1, w0, w1);
+        float g = r0 * r0 + r1 * r1, dl = r0 * w0 + r1 * w1;
+        warp_sums(g, dl, lane);
+        if (it == 0 && warm && !(g <= bb)) {
+            // the start vector is further from the solution than zero is: start again from zero
+            warm = false;
+            x0 = x1 = 0.f;
+            r0 = b0;
+            r1 = b1;
+            it = -1;
+            continue;
+        }
+        if (g <= cg.tol2 * bb) { ok = true; break; }        // (also b = 0: x = 0)
+        if (it >= cg.max_iter) break;
+        const float rg = __fdividef(1.f, g);
+        const float beta = g * rg_old;                           // 0 at the first step
+        const float inv_alpha = dl * rg - beta * inv_alpha_old;  // p.A p / |r|^2
+        if (!(inv_alpha > 0.f) || !(inv_alpha <= 3.0e38f)) break;
+        const float alpha = __fdividef(1.f, inv_alpha);
+        p0 = fmaf(beta, p0, r0);
+        p1 = fmaf(beta, p1, r1);
+        s0 = fmaf(beta, s0, w0);
+        s1 = fmaf(beta, s1, w1);
+        x0 = fmaf(alpha, p0, x0);
+        x1 = fmaf(alpha, p1, x1);
+        r0 = fmaf(-alpha, s0, r0);
+        r1 = fmaf(-alpha, s1, r1);
+        rg_old = rg;
+        inv_alpha_old = inv_alpha;
+    }
+    if (ok && products >= kCgVerifyProducts) {
+        product(x0, x1, w0, w1);
+        float t = (b0 - w0) * (b0 - w0) + (b1 - w1) * (b1 - w1);
+        unused = 0.f;
+        warp_sums(t, unused, lane);
+        ok = t <= 4.f * cg.tol2 * bb;
+    }
+    return ok;
+}
+
 template <int D, typename T>
 __device__ __forceinline__ void store_row(const float *x, bool ok, int64_t u, const RowOut &out, DevStatus *st, int lane)
 {
@@ -471,9 +611,12 @@ template <int D, typename T> __device__ __forceinline__ void load_base(const flo
 
 // ---- rows of at most 256 entries: a warp each, items dealt round-robin (they are sorted by length class, so a warp's items
 // are of all lengths); item 0 is the last of the order, i.e. of the longest class
-template <int D, typename T>
+// `primal_count`, where *dual_flag is set: the items before the rows that the dual form has solved.  `list`: the rows to solve
+// instead of the order's, *list_count of them (negative entries are skipped).
+template <int D, typename T, bool CG>
 __global__ void __launch_bounds__(WGeo<D, T>::REGS_WARPS * 32, 1)
-k_rows_warp(SideView sv, int64_t last, int64_t count, const T *__restrict__ X, const float *__restrict__ Bmat, RowOut out, DevStatus *st)
+k_rows_warp(SideView sv, int64_t last, int64_t count, const int *dual_flag, int64_t primal_count, const int32_t *list,
+            const unsigned long long *list_count, const T *__restrict__ X, const float *__restrict__ Bmat, RowOut out, WarpCg cg, DevStatus *st)
 {
     using G = WGeo<D, T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -481,9 +624,14 @@ k_rows_warp(SideView sv, int64_t last, int64_t count, const T *__restrict__ X, c
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     unsigned char *mine = smem_raw + G::BASE + warp * G::WARP;
     unsigned char *work = mine + 2 * G::STAGE;
+    if (dual_flag && *dual_flag) count = primal_count;
+    if (list_count) count = (int64_t)*list_count;
+    if ((int64_t)blockIdx.x * G::ROWS >= count) return;
     load_base<D, T>(Bmat, base);
     __syncthreads();
     const int64_t warps = (int64_t)gridDim.x * G::REGS_WARPS;
+    unsigned cg_rows = 0, cg_products = 0;
+    auto row_at = [&](int64_t k) -> int64_t { return list ? list[k] : sv.order[last - k]; };
     int64_t item = ((int64_t)warp * gridDim.x + blockIdx.x) * G::ROWS;
     if (item >= count) return;
     Feed<D, T> feed;
@@ -492,46 +640,74 @@ k_rows_warp(SideView sv, int64_t last, int64_t count, const T *__restrict__ X, c
     feed.val = sv.val;
     feed.ring = ptx::smem_u32(mine);
     feed.g = 0;
-    int64_t u = sv.order[last - item];
-    int64_t beg = sv.ptr[u], end = sv.ptr[u + 1];
+    int64_t u = row_at(item);
+    int64_t beg = u < 0 ? 0 : sv.ptr[u], end = u < 0 ? 0 : sv.ptr[u + 1];
     feed.start(beg, end, lane);
     float *b_s = reinterpret_cast<float *>(work) + G::B_AT;
     while (true) {
         int64_t u_pair = -1;
         const int64_t next = item + warps * G::ROWS;
-        const int64_t un = next < count ? sv.order[last - next] : -1;
+        const bool more = next < count;
+        const int64_t un = more ? row_at(next) : -1;
         int64_t bn = 0, en = 0;
         Sums<D, T> acc, acc2;
         acc.zero();
-        sum_entries<D, T>(feed, end - beg, mine, work, acc, lane);
+        sum_entries<D, T>(feed, u < 0 ? 1 : end - beg, mine, work, acc, lane);      // (a skipped row: one stage of zeros)
         put_b<D, T>(acc, b_s, lane);
         if constexpr (D == 16) {      // a second matrix; a lone last row goes without
             acc2.zero();
             if (item + 1 < count) {
-                u_pair = sv.order[last - item - 1];
-                const int64_t b2 = sv.ptr[u_pair], e2 = sv.ptr[u_pair + 1];
+                u_pair = row_at(item + 1);
+                const int64_t b2 = u_pair < 0 ? 0 : sv.ptr[u_pair], e2 = u_pair < 0 ? 0 : sv.ptr[u_pair + 1];
                 feed.start(b2, e2, lane);
-                sum_entries<D, T>(feed, e2 - b2, mine, work, acc2, lane);
+                sum_entries<D, T>(feed, u_pair < 0 ? 1 : e2 - b2, mine, work, acc2, lane);
             }
             put_b<D, T>(acc2, b_s + D, lane);
             add_base<D, T>(acc2, base, lane);
         }
         add_base<D, T>(acc, base, lane);
         // the next row's first entries travel while this one is solved
-        if (un >= 0) {
-            bn = sv.ptr[un];
-            en = sv.ptr[un + 1];
+        if (more) {
+            if (un >= 0) {
+                bn = sv.ptr[un];
+                en = sv.ptr[un + 1];
+            }
             feed.start(bn, en, lane);
         }
-        const bool ok = factor_solve<D, T>(acc, acc2, reinterpret_cast<float *>(work), b_s, lane);
-        if (D != 16 || lane < 16) store_row<D, T>(b_s, ok, u, out, st, lane);
-        else if (u_pair >= 0) store_row<D, T>(b_s + D, ok, u_pair, out, st, lane);
-        if (un < 0) return;
+        if constexpr (CG) {
+            const float b0 = b_s[lane], b1 = b_s[lane + 32];
+            const float *stored = reinterpret_cast<const float *>(out.table) + u * D;
+            float x0 = cg.warm ? stored[lane] : 0.f, x1 = cg.warm ? stored[lane + 32] : 0.f;
+            float a0[64], a1[64];
+            symmetric_rows(acc, reinterpret_cast<float *>(work), a0, a1, lane);
+            int products = 0;
+            const bool ok = conjugate_gradients(cg, a0, a1, b_s, b0, b1, x0, x1, products, lane);
+            ++cg_rows;
+            cg_products += products;
+            __syncwarp();
+            b_s[lane] = x0;
+            b_s[lane + 32] = x1;
+            __syncwarp();
+            if (ok) store_row<D, T>(b_s, true, u, out, st, lane);
+            else if (lane == 0) cg.fallback_list[atomicAdd(&cg.counters[2], 1ull)] = (int32_t)u;
+        } else {
+            const bool ok = factor_solve<D, T>(acc, acc2, reinterpret_cast<float *>(work), b_s, lane);
+            if (D != 16 || lane < 16) {
+                if (u >= 0) store_row<D, T>(b_s, ok, u, out, st, lane);
+            } else if (u_pair >= 0) {
+                store_row<D, T>(b_s + D, ok, u_pair, out, st, lane);
+            }
+        }
+        if (!more) break;
         __syncwarp();
         item = next;
         u = un;
         beg = bn;
         end = en;
+    }
+    if (CG && lane == 0) {
+        atomicAdd(&cg.counters[0], (unsigned long long)cg_rows);
+        atomicAdd(&cg.counters[1], (unsigned long long)cg_products);
     }
 }
 
@@ -546,17 +722,48 @@ template <int D, typename T> struct BGeo {
     static constexpr size_t SMEM = (size_t)G::BASE + G::WORK + SHARED + 16;
 };
 
-template <int D, typename T>
-__device__ __forceinline__ void solve_sums(const float *sums, const float4 *base, float *work, int64_t u, const RowOut &out, DevStatus *st, int lane)
+template <int D, typename T> __device__ __forceinline__ void load_sums(const float *sums, Sums<D, T> &acc, int lane)
 {
-    using G = WGeo<D, T>;
-    Sums<D, T> acc, acc2;
 #pragma unroll
-    for (int n = 0; n < G::NB; ++n) {
+    for (int n = 0; n < WGeo<D, T>::NB; ++n) {
         const float4 v = *reinterpret_cast<const float4 *>(sums + (n * 32 + lane) * 4);
         acc.c[n][0] = v.x; acc.c[n][1] = v.y; acc.c[n][2] = v.z; acc.c[n][3] = v.w;
     }
+}
+
+template <int D, typename T, bool CG>
+__device__ __forceinline__ void solve_sums(const float *sums, const float4 *base, float *work, int64_t u, const RowOut &out, const WarpCg &cg,
+                                           DevStatus *st, int lane)
+{
+    using G = WGeo<D, T>;
     float *b_s = work + G::B_AT;
+    if constexpr (CG) {
+        Sums<D, T> acc;
+        load_sums<D, T>(sums, acc, lane);
+        add_base<D, T>(acc, base, lane);
+        const float b0 = sums[G::NB * 128 + lane], b1 = sums[G::NB * 128 + 32 + lane];
+        const float *stored = reinterpret_cast<const float *>(out.table) + u * D;
+        float x0 = cg.warm ? stored[lane] : 0.f, x1 = cg.warm ? stored[lane + 32] : 0.f;
+        float a0[64], a1[64];
+        symmetric_rows(acc, work, a0, a1, lane);
+        int products = 0;
+        const bool ok = conjugate_gradients(cg, a0, a1, b_s, b0, b1, x0, x1, products, lane);
+        if (lane == 0) {
+            atomicAdd(&cg.counters[0], 1ull);
+            atomicAdd(&cg.counters[1], (unsigned long long)products);
+            if (!ok) cg.fallback_list[atomicAdd(&cg.counters[2], 1ull)] = -1;      // solved below: nothing for the list's kernel
+        }
+        if (ok) {
+            __syncwarp();
+            b_s[lane] = x0;
+            b_s[lane + 32] = x1;
+            __syncwarp();
+            store_row<D, T>(b_s, true, u, out, st, lane);
+            return;
+        }
+    }
+    Sums<D, T> acc, acc2;
+    load_sums<D, T>(sums, acc, lane);
     for (int e = lane; e < G::ROWS * D; e += 32) b_s[e] = sums[G::NB * 128 + (e & (D - 1))];
     add_base<D, T>(acc, base, lane);
     if constexpr (D == 16) acc2 = acc;
@@ -565,10 +772,10 @@ __device__ __forceinline__ void solve_sums(const float *sums, const float4 *base
     if (D != 16 || lane < 16) store_row<D, T>(b_s, ok, u, out, st, lane);
 }
 
-template <int D, typename T, bool CHUNK>
+template <int D, typename T, bool CHUNK, bool CG>
 __global__ void __launch_bounds__(kBlockWarps * 32, 1)
 k_rows_block(SideView sv, int64_t last, const T *__restrict__ X, const float *__restrict__ Bmat, float *__restrict__ partials, RowOut out,
-             DevStatus *st)
+             WarpCg cg, DevStatus *st)
 {
     using G = WGeo<D, T>;
     using B = BGeo<D, T>;
@@ -620,13 +827,13 @@ k_rows_block(SideView sv, int64_t last, const T *__restrict__ X, const float *__
     }
     if (CHUNK) return;
     __syncthreads();
-    if (warp == 0) solve_sums<D, T>(red, base, work, u, out, st, lane);
+    if (warp == 0) solve_sums<D, T, CG>(red, base, work, u, out, cg, st, lane);
 }
 
 // one warp per split row: its chunks' sums in ascending order, then the solve
-template <int D, typename T>
+template <int D, typename T, bool CG>
 __global__ void __launch_bounds__(32) k_split_solve_warp(SideView sv, int64_t split_begin, const float *__restrict__ partials,
-                                                         const float *__restrict__ Bmat, RowOut out, DevStatus *st)
+                                                         const float *__restrict__ Bmat, RowOut out, WarpCg cg, DevStatus *st)
 {
     using G = WGeo<D, T>;
     using B = BGeo<D, T>;
@@ -647,7 +854,7 @@ __global__ void __launch_bounds__(32) k_split_solve_warp(SideView sv, int64_t sp
         *reinterpret_cast<float4 *>(sums + e) = s;
     }
     __syncwarp();
-    solve_sums<D, T>(sums, base, work, u, out, st, lane);
+    solve_sums<D, T, CG>(sums, base, work, u, out, cg, st, lane);
 }
 
 // rows without observations: A^-1 0 = 0
@@ -665,43 +872,65 @@ __global__ void k_zero_rows_warp(const int32_t *__restrict__ rows, int64_t count
     }
 }
 
-template <int D, typename T>
-cudaError_t rows_warp_dt(const SideView &sv, const int64_t *offs, int64_t n_chunks, int64_t n_split_rows, const void *Xv, const float *Bmat,
-                         float *partials, RowOut out, DevStatus *st, cudaStream_t s, int64_t *launches)
+struct WarpRows {
+    SideView sv;
+    const int64_t *offs;
+    int64_t n_chunks, n_split_rows;
+    const void *X;
+    const float *Bmat;
+    float *partials;
+    RowOut out;
+    DevStatus *st;
+    WarpCg cg;
+    const int *dual_flag;      // set on the device when the rows of class 1 have been solved in the dual form
+    cudaStream_t s;
+    int64_t *launches;
+};
+
+template <int D, typename T, bool CG> cudaError_t rows_warp_dt(const WarpRows &a)
 {
     using G = WGeo<D, T>;
     using B = BGeo<D, T>;
     static_assert(B::SUMS <= D * D + D, "a chunk's sums fit its place in the workspace");
     static_assert(B::SMEM <= 232448 && (size_t)G::BASE + G::REGS_WARPS * G::WARP <= 232448, "shared memory");
-    const T *X = reinterpret_cast<const T *>(Xv);
+    const T *X = reinterpret_cast<const T *>(a.X);
+    const int64_t *offs = a.offs;
     const size_t smem_warp = (size_t)G::BASE + G::REGS_WARPS * G::WARP;
     const size_t smem_split = (size_t)G::BASE + G::WORK + 4 * B::SUMS;
     cudaError_t e;
     // longest work first
-    if (n_chunks > 0) {
-        if ((e = cudaFuncSetAttribute(k_rows_block<D, T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B::SMEM)) != cudaSuccess) return e;
-        k_rows_block<D, T, true><<<(unsigned)n_chunks, kBlockWarps * 32, B::SMEM, s>>>(sv, 0, X, Bmat, partials, out, st);
-        k_split_solve_warp<D, T><<<(unsigned)n_split_rows, 32, smem_split, s>>>(sv, offs[kNClasses - 1], partials, Bmat, out, st);
-        *launches += 2;
+    if (a.n_chunks > 0) {
+        if ((e = cudaFuncSetAttribute(k_rows_block<D, T, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B::SMEM)) != cudaSuccess) return e;
+        k_rows_block<D, T, true, false><<<(unsigned)a.n_chunks, kBlockWarps * 32, B::SMEM, a.s>>>(a.sv, 0, X, a.Bmat, a.partials, a.out, a.cg, a.st);
+        k_split_solve_warp<D, T, CG><<<(unsigned)a.n_split_rows, 32, smem_split, a.s>>>(a.sv, offs[kNClasses - 1], a.partials, a.Bmat, a.out, a.cg, a.st);
+        *a.launches += 2;
     }
     const int64_t n_long = offs[kNClasses - 1] - offs[kLongClass];
     if (n_long > 0) {
-        if ((e = cudaFuncSetAttribute(k_rows_block<D, T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B::SMEM)) != cudaSuccess) return e;
-        k_rows_block<D, T, false><<<(unsigned)n_long, kBlockWarps * 32, B::SMEM, s>>>(sv, offs[kNClasses - 1] - 1, X, Bmat, partials, out, st);
-        ++*launches;
+        if ((e = cudaFuncSetAttribute(k_rows_block<D, T, false, CG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B::SMEM)) != cudaSuccess) return e;
+        k_rows_block<D, T, false, CG><<<(unsigned)n_long, kBlockWarps * 32, B::SMEM, a.s>>>(a.sv, offs[kNClasses - 1] - 1, X, a.Bmat, a.partials, a.out,
+                                                                                          a.cg, a.st);
+        ++*a.launches;
     }
     const int64_t n_warp = offs[kLongClass] - offs[1];
     if (n_warp > 0) {
-        if ((e = cudaFuncSetAttribute(k_rows_warp<D, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_warp)) != cudaSuccess) return e;
-        const int64_t per_warp = G::ROWS, blocks = (n_warp + per_warp - 1) / per_warp;      // few rows: one per SM before two
-        k_rows_warp<D, T><<<(unsigned)(blocks < 148 ? blocks : 148), G::REGS_WARPS * 32, smem_warp, s>>>(sv, offs[kLongClass] - 1, n_warp, X,
-                                                                                                       Bmat, out, st);
-        ++*launches;
+        if ((e = cudaFuncSetAttribute(k_rows_warp<D, T, CG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_warp)) != cudaSuccess) return e;
+        const int64_t blocks = (n_warp + G::ROWS - 1) / G::ROWS;      // few rows: one per SM before two
+        k_rows_warp<D, T, CG><<<(unsigned)(blocks < 148 ? blocks : 148), G::REGS_WARPS * 32, smem_warp, a.s>>>(
+            a.sv, offs[kLongClass] - 1, n_warp, a.dual_flag, offs[kLongClass] - offs[2], nullptr, nullptr, X, a.Bmat, a.out, a.cg, a.st);
+        ++*a.launches;
+    }
+    if (CG && offs[kNClasses] > offs[1]) {
+        // the rows conjugate gradients did not finish (none, as a rule: its blocks then return at once)
+        if ((e = cudaFuncSetAttribute(k_rows_warp<D, T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_warp)) != cudaSuccess) return e;
+        k_rows_warp<D, T, false><<<148, G::REGS_WARPS * 32, smem_warp, a.s>>>(a.sv, 0, 0, nullptr, 0, a.cg.fallback_list, a.cg.counters + 2, X, a.Bmat,
+                                                                             a.out, a.cg, a.st);
+        ++*a.launches;
     }
     const int64_t n_zero = offs[1] - offs[0];
     if (n_zero > 0) {
-        k_zero_rows_warp<T><<<(unsigned)((n_zero * D + 255) / 256), 256, 0, s>>>(sv.order + offs[0], n_zero, D, out);
-        ++*launches;
+        k_zero_rows_warp<T><<<(unsigned)((n_zero * D + 255) / 256), 256, 0, a.s>>>(a.sv.order + offs[0], n_zero, D, a.out);
+        ++*a.launches;
     }
     return cudaGetLastError();
 }
@@ -709,16 +938,19 @@ cudaError_t rows_warp_dt(const SideView &sv, const int64_t *offs, int64_t n_chun
 }  // namespace
 
 cudaError_t launch_rows_warp(const SideView &sv, const int64_t *offs, int64_t n_chunks, int64_t n_split_rows, const void *X, int bf16, int d,
-                             const float *Bmat, float *partials, RowOut out, DevStatus *st, cudaStream_t s, int64_t *launches)
+                             const float *Bmat, float *partials, RowOut out, DevStatus *st, const CgOptions &cg, const int *dual_flag,
+                             cudaStream_t s, int64_t *launches)
 {
-#define ALX_CASE(DD)                                                                                                                      case DD:                                                                                                                                  return bf16 ? rows_warp_dt<DD, __nv_bfloat16>(sv, offs, n_chunks, n_split_rows, X, Bmat, partials, out, st, s, launches)                          : rows_warp_dt<DD, float>(sv, offs, n_chunks, n_split_rows, X, Bmat, partials, out, st, s, launches);
+    const bool use_cg = cg.enabled && d == 64 && !bf16;
+    const WarpRows a{sv, offs, n_chunks, n_split_rows, X, Bmat, partials, out, st,
+                     WarpCg{cg.max_iter, cg.warm_start ? 1 : 0, cg.tol * cg.tol, use_cg ? cg.counters : nullptr, cg.fallback_list},
+                     dual_flag, s, launches};
     switch (d) {
-        ALX_CASE(16)
-        ALX_CASE(32)
-        ALX_CASE(64)
+    case 16: return bf16 ? rows_warp_dt<16, __nv_bfloat16, false>(a) : rows_warp_dt<16, float, false>(a);
+    case 32: return bf16 ? rows_warp_dt<32, __nv_bfloat16, false>(a) : rows_warp_dt<32, float, false>(a);
+    case 64: return bf16 ? rows_warp_dt<64, __nv_bfloat16, false>(a) : use_cg ? rows_warp_dt<64, float, true>(a) : rows_warp_dt<64, float, false>(a);
     default: return cudaErrorInvalidValue;
     }
-#undef ALX_CASE
 }
 
 }  // namespace alx
