@@ -620,7 +620,7 @@ alx_status alx_set_csr(alx_ctx *c, const int64_t *rowptr, const int32_t *colidx,
         ALX_TMP(c, tmp, total, 2);
         for (int s = 0; s < 2; ++s) {
             const int64_t *offs = c->class_offs[s];
-            const int64_t first = offs[tensor_path(c) ? long_class_begin(offs) : kWarpLongClass];
+            const int64_t first = offs[tensor_path(c) ? long_class_begin(offs) : warp_long_class(offs)];
             const int64_t n_long = offs[kNClasses - 1] - first;
             if (tensor_path(c)) sums[s] += n_long;
             c->stats.long_rows[s] = n_long;

@@ -184,7 +184,10 @@ struct CgOptions {
     float switch_products;         // mean products per row beyond which the side's next half-epochs take Cholesky
 };
 
-constexpr int kWarpLongClass = 6;      // degree classes from here on (more than 256 entries) get a block of eight warps per row
+// The degree class from which on a row gets a block of warps instead of one: more than 1024 entries (a warp takes about 50 us
+// for as many) where there are so many rows that every warp has several anyway, else more than 256, so that a few longer
+// rows do not outlast the others.
+inline int warp_long_class(const int64_t *class_offs_host) { return class_offs_host[8] - class_offs_host[1] >= 148 * 20 * 8 ? 8 : 6; }
 // alx_rows_warp.cu: d = 16, 32, 64, a warp per row (kernels != 1); conjugate gradients for fp32 tables of 64 features where
 // cg.enabled.  dual_flag (may be null): device flag, set when the rows of class 1 have been solved in the dual form
 cudaError_t launch_rows_warp(const SideView &sv, const int64_t *class_offs_host, int64_t n_chunks, int64_t n_split_rows, const void *X,

@@ -15,8 +15,8 @@
 //   - Cholesky with lane = row (d = 64: rows l and l + 32; d = 16: two matrices per warp), two columns per step, the finished
 //     columns of L in shared memory: their broadcast reads drive the trailing update (packed FMAs), and the back
 //     substitution reads them across.
-// Rows of more than 256 entries, and the chunks of rows longer than `split`, are summed by a block of eight warps, each a
-// slice of the entries; the slices are added in a fixed order.
+// Long rows (warp_long_class), and the chunks of rows longer than `split`, are summed by a block of warps, each a slice of the
+// entries; the slices are added in a fixed order.
 //
 // Bound: issue slots of the solve (d = 64: about 3400 per row) and, for long rows, the mma rate.
 #include "alx_common.cuh"
@@ -27,8 +27,6 @@ namespace alx {
 namespace {
 
 constexpr int kEntries = 16;       // entries per stage = the K of one mma
-constexpr int kBlockWarps = 8;     // warps per row in the long-row kernels
-constexpr int kLongClass = kWarpLongClass;
 
 template <int D, typename T> struct WGeo {
     static constexpr bool kF32 = sizeof(T) == 4;
@@ -134,15 +132,29 @@ template <int D, typename T> struct Feed {
         }
         ptx::cp_async_commit();
     }
-    // first stage of a row's entries [beg, e): ids, then its copies, then the ids of the second stage
-    __device__ __forceinline__ void start(int64_t beg, int64_t e, int lane)
+    // a row's entries [beg, e): the loads of the ids of its first two stages ...
+    int id_first;
+    __device__ __forceinline__ void start_ids(int64_t beg, int64_t e, int lane)
     {
         at = beg;
         end = e;
         load_ids(lane);
         y = y_next;
-        issue(g & 1, lane);
+        id_first = id;
         load_ids(lane);
+    }
+    // ... and, later, the copies of the first stage
+    __device__ __forceinline__ void start_copies(int lane)
+    {
+        const int second = id;
+        id = id_first;
+        issue(g & 1, lane);
+        id = second;
+    }
+    __device__ __forceinline__ void start(int64_t beg, int64_t e, int lane)
+    {
+        start_ids(beg, e, lane);
+        start_copies(lane);
     }
 };
 
@@ -609,7 +621,7 @@ template <int D, typename T> __device__ __forceinline__ void load_base(const flo
     }
 }
 
-// ---- rows of at most 256 entries: a warp each, items dealt round-robin (they are sorted by length class, so a warp's items
+// ---- rows up to the long ones: a warp each, items dealt round-robin (they are sorted by length class, so a warp's items
 // are of all lengths); item 0 is the last of the order, i.e. of the longest class
 // `primal_count`, where *dual_flag is set: the items before the rows that the dual form has solved.  `list`: the rows to solve
 // instead of the order's, *list_count of them (negative entries are skipped).
@@ -644,12 +656,14 @@ k_rows_warp(SideView sv, int64_t last, int64_t count, const int *dual_flag, int6
     int64_t beg = u < 0 ? 0 : sv.ptr[u], end = u < 0 ? 0 : sv.ptr[u + 1];
     feed.start(beg, end, lane);
     float *b_s = reinterpret_cast<float *>(work) + G::B_AT;
+    // the row after this one is looked up while this one is summed: its id a row ahead, its range now
+    int64_t un = item + warps * G::ROWS < count ? row_at(item + warps * G::ROWS) : -1;
     while (true) {
         int64_t u_pair = -1;
-        const int64_t next = item + warps * G::ROWS;
+        const int64_t next = item + warps * G::ROWS, after = next + warps * G::ROWS;
         const bool more = next < count;
-        const int64_t un = more ? row_at(next) : -1;
-        int64_t bn = 0, en = 0;
+        const int64_t bn = un < 0 ? 0 : sv.ptr[un], en = un < 0 ? 0 : sv.ptr[un + 1];
+        const int64_t ua = after < count ? row_at(after) : -1;
         Sums<D, T> acc, acc2;
         acc.zero();
         sum_entries<D, T>(feed, u < 0 ? 1 : end - beg, mine, work, acc, lane);      // (a skipped row: one stage of zeros)
@@ -665,21 +679,16 @@ k_rows_warp(SideView sv, int64_t last, int64_t count, const int *dual_flag, int6
             put_b<D, T>(acc2, b_s + D, lane);
             add_base<D, T>(acc2, base, lane);
         }
-        add_base<D, T>(acc, base, lane);
         // the next row's first entries travel while this one is solved
-        if (more) {
-            if (un >= 0) {
-                bn = sv.ptr[un];
-                en = sv.ptr[un + 1];
-            }
-            feed.start(bn, en, lane);
-        }
+        if (more) feed.start_ids(bn, en, lane);
+        add_base<D, T>(acc, base, lane);
         if constexpr (CG) {
             const float b0 = b_s[lane], b1 = b_s[lane + 32];
             const float *stored = reinterpret_cast<const float *>(out.table) + u * D;
             float x0 = cg.warm ? stored[lane] : 0.f, x1 = cg.warm ? stored[lane + 32] : 0.f;
             float a0[64], a1[64];
             symmetric_rows(acc, reinterpret_cast<float *>(work), a0, a1, lane);
+            if (more) feed.start_copies(lane);
             int products = 0;
             const bool ok = conjugate_gradients(cg, a0, a1, b_s, b0, b1, x0, x1, products, lane);
             ++cg_rows;
@@ -691,6 +700,7 @@ k_rows_warp(SideView sv, int64_t last, int64_t count, const int *dual_flag, int6
             if (ok) store_row<D, T>(b_s, true, u, out, st, lane);
             else if (lane == 0) cg.fallback_list[atomicAdd(&cg.counters[2], 1ull)] = (int32_t)u;
         } else {
+            if (more) feed.start_copies(lane);
             const bool ok = factor_solve<D, T>(acc, acc2, reinterpret_cast<float *>(work), b_s, lane);
             if (D != 16 || lane < 16) {
                 if (u >= 0) store_row<D, T>(b_s, ok, u, out, st, lane);
@@ -702,6 +712,7 @@ k_rows_warp(SideView sv, int64_t last, int64_t count, const int *dual_flag, int6
         __syncwarp();
         item = next;
         u = un;
+        un = ua;
         beg = bn;
         end = en;
     }
@@ -711,10 +722,12 @@ k_rows_warp(SideView sv, int64_t last, int64_t count, const int *dual_flag, int6
     }
 }
 
-// ---- longer rows and chunks of split rows: a block of eight warps, each a slice of the entries; the slices' sums are added in
-// warp order.  A chunk's sums go to the workspace in fragment order ([NB x 128] and b); a row is solved by the first warp.
+// ---- long rows and chunks of split rows: a block of warps, each a slice of the entries; the slices' sums are added in warp
+// order.  A chunk's sums go to the workspace in fragment order ([NB x 128] and b); a row is solved by the first warp.
 template <int D, typename T> struct BGeo {
     using G = WGeo<D, T>;
+    static constexpr int kBlockWarps = D == 64 ? 12 : 8;                 // warps per row, and blocks per SM: the registers of the sums
+    static constexpr int kBlocks = D == 64 ? 1 : D == 32 ? 3 : 4;
     static constexpr int SUMS = G::NB * 128 + D;      // floats
     static constexpr int FEED = kBlockWarps * (2 * G::STAGE + G::TILE);
     static constexpr int RED = kBlockWarps * SUMS * 4;
@@ -773,12 +786,13 @@ __device__ __forceinline__ void solve_sums(const float *sums, const float4 *base
 }
 
 template <int D, typename T, bool CHUNK, bool CG>
-__global__ void __launch_bounds__(kBlockWarps * 32, 1)
+__global__ void __launch_bounds__(BGeo<D, T>::kBlockWarps * 32, BGeo<D, T>::kBlocks)
 k_rows_block(SideView sv, int64_t last, const T *__restrict__ X, const float *__restrict__ Bmat, float *__restrict__ partials, RowOut out,
              WarpCg cg, DevStatus *st)
 {
     using G = WGeo<D, T>;
     using B = BGeo<D, T>;
+    constexpr int kBlockWarps = B::kBlockWarps;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float4 *base = reinterpret_cast<float4 *>(smem_raw);
     float *work = reinterpret_cast<float *>(smem_raw + G::BASE);
@@ -895,20 +909,21 @@ template <int D, typename T, bool CG> cudaError_t rows_warp_dt(const WarpRows &a
     static_assert(B::SMEM <= 232448 && (size_t)G::BASE + G::REGS_WARPS * G::WARP <= 232448, "shared memory");
     const T *X = reinterpret_cast<const T *>(a.X);
     const int64_t *offs = a.offs;
+    const int kLongClass = warp_long_class(offs);
     const size_t smem_warp = (size_t)G::BASE + G::REGS_WARPS * G::WARP;
     const size_t smem_split = (size_t)G::BASE + G::WORK + 4 * B::SUMS;
     cudaError_t e;
     // longest work first
     if (a.n_chunks > 0) {
         if ((e = cudaFuncSetAttribute(k_rows_block<D, T, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B::SMEM)) != cudaSuccess) return e;
-        k_rows_block<D, T, true, false><<<(unsigned)a.n_chunks, kBlockWarps * 32, B::SMEM, a.s>>>(a.sv, 0, X, a.Bmat, a.partials, a.out, a.cg, a.st);
+        k_rows_block<D, T, true, false><<<(unsigned)a.n_chunks, B::kBlockWarps * 32, B::SMEM, a.s>>>(a.sv, 0, X, a.Bmat, a.partials, a.out, a.cg, a.st);
         k_split_solve_warp<D, T, CG><<<(unsigned)a.n_split_rows, 32, smem_split, a.s>>>(a.sv, offs[kNClasses - 1], a.partials, a.Bmat, a.out, a.cg, a.st);
         *a.launches += 2;
     }
     const int64_t n_long = offs[kNClasses - 1] - offs[kLongClass];
     if (n_long > 0) {
         if ((e = cudaFuncSetAttribute(k_rows_block<D, T, false, CG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B::SMEM)) != cudaSuccess) return e;
-        k_rows_block<D, T, false, CG><<<(unsigned)n_long, kBlockWarps * 32, B::SMEM, a.s>>>(a.sv, offs[kNClasses - 1] - 1, X, a.Bmat, a.partials, a.out,
+        k_rows_block<D, T, false, CG><<<(unsigned)n_long, B::kBlockWarps * 32, B::SMEM, a.s>>>(a.sv, offs[kNClasses - 1] - 1, X, a.Bmat, a.partials, a.out,
                                                                                           a.cg, a.st);
         ++*a.launches;
     }
