@@ -4,6 +4,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <string>
 #include <utility>
@@ -14,6 +15,13 @@
 #include <nvtx3/nvToolsExt.h>      // header-only: ranges show up in a profiler's timeline, and cost nothing without one
 
 using namespace alx;
+
+// Device memory that a context keeps from call to call (grown as needed, given back when it is large, freed with the context)
+enum Kept { kKeptRows, kKeptOrder, kKeptScratch, kKeptSums, kKeptTable, kKeptFallback, kKeptOut, kKeptUpload, kKeptWork, kKeptCount };
+constexpr size_t kKeepMost = 256ull << 20;
+// Page-locked staging of small transfers: the status word and small results come back together behind one wait, the arrays of
+// a small call go up in one copy
+constexpr size_t kBoxBytes = 64 << 10, kBoxSmall = 1 << 10;
 
 struct alx_ctx {
     alx_options opt{};
@@ -50,9 +58,8 @@ struct alx_ctx {
     float *split_partials = nullptr;
     void *dual_ws = nullptr;      // tensor path: B^-1 operand tiles and the flag of the dual form
     int64_t dual_candidates = 0;  // rows of classes 1 and 2 of the last half-epoch (solved in the dual form if the flag is set)
-    int dual_flag_latched = 0;
     int64_t dual_candidates32 = 0; // of them, the rows of 17 .. 32 observations (which the whole-rows kernel may have taken instead)
-    CgPolicy policy_latched{};    // the side's policy record as the last half-epoch's kernels saw it    // that flag as the last half-epoch's kernels saw it (the loss and the Gramian calls rewrite it)
+    int last_side = 0;             // side of the last half-epoch: its flag and policy record stay on the device until alx_get_stats asks
     double *loss_partials_buf = nullptr;
     double *loss_result = nullptr;
     DevStatus *status = nullptr;
@@ -64,6 +71,11 @@ struct alx_ctx {
     cudaStream_t copy_stream = nullptr;
     cudaEvent_t copy_ev = nullptr;
     const void *upload_after_csr[2] = {nullptr, nullptr};   // alx_load_host: tables to upload behind the upload of S
+
+    unsigned char *box = nullptr;                  // kBoxBytes, page-locked: DevStatus, then small results, payload from kBoxSmall on
+    struct { void *p; size_t bytes; } kept[kKeptCount] = {};
+    alx_ctx *fold = nullptr;                       // alx_fold_in's context for the new rows, made at the first call
+    std::mutex calls;                              // alx_fold_in, alx_topk and alx_recall_at_k, which use what is kept
 
     cudaEvent_t ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
     bool main_timed = false;
@@ -181,12 +193,106 @@ struct Scratch {
         (scratch).keep(dst);                                                                       \
     } while (0)
 
-// read and clear the device status word (after a stream synchronise)
+alx_status ensure_box(alx_ctx *c)
+{
+    if (!c->box) ALX_CUDA(c, cudaHostAlloc(reinterpret_cast<void **>(&c->box), kBoxBytes, cudaHostAllocDefault));
+    return ALX_OK;
+}
+
+// device memory of a slot, at least `bytes`; its old contents are gone when it had to grow.  The calls that use the slots wait
+// for the stream before they return, so nothing in flight uses an old one.
+alx_status keep(alx_ctx *c, Kept slot, size_t bytes, void **out)
+{
+    auto &k = c->kept[slot];
+    if (k.bytes < bytes) {
+        dev_free(c, k.p);
+        k.p = nullptr;
+        k.bytes = 0;
+        const size_t want = bytes > kKeepMost ? bytes : bytes + bytes / 4;
+        k.p = dev_alloc(c, want);
+        if (!k.p) return fail(c, ALX_ERR_OOM, "device allocation of %zu bytes failed", want);
+        k.bytes = want;
+    }
+    *out = k.p;
+    return ALX_OK;
+}
+void give_back_large(alx_ctx *c)
+{
+    for (auto &k : c->kept)
+        if (k.bytes > kKeepMost) { dev_free(c, k.p); k.p = nullptr; k.bytes = 0; }
+}
+constexpr size_t aligned(size_t bytes) { return (bytes + 255) / 256 * 256; }
+
+// A host call's arrays, laid out one behind the other in a slot of device memory; small ones go up in one copy through the box.
+struct Upload {
+    alx_ctx *c;
+    struct { const void *src; size_t bytes, at; } part[4];
+    int n = 0;
+    size_t total = 0;
+    explicit Upload(alx_ctx *ctx) : c(ctx) {}
+    int add(const void *src, size_t bytes)      // number of the part
+    {
+        part[n] = {src, bytes, total};
+        total += aligned(bytes > 0 ? bytes : 1);
+        return n++;
+    }
+    alx_status send(Kept slot, void *(&dev)[4])
+    {
+        void *base = nullptr;
+        alx_status st = keep(c, slot, total, &base);
+        if (st != ALX_OK) return st;
+        for (int k = 0; k < n; ++k) dev[k] = static_cast<unsigned char *>(base) + part[k].at;
+        if (total <= kBoxBytes - kBoxSmall) {
+            if ((st = ensure_box(c)) != ALX_OK) return st;
+            for (int k = 0; k < n; ++k)
+                if (part[k].bytes) memcpy(c->box + kBoxSmall + part[k].at, part[k].src, part[k].bytes);
+            ALX_CUDA(c, cudaMemcpyAsync(base, c->box + kBoxSmall, total, cudaMemcpyHostToDevice, c->stream));
+        } else {
+            for (int k = 0; k < n; ++k)
+                if (part[k].bytes) ALX_CUDA(c, cudaMemcpyAsync(dev[k], part[k].src, part[k].bytes, cudaMemcpyHostToDevice, c->stream));
+        }
+        return ALX_OK;
+    }
+};
+
+// Results on their way back to the host with the status word: small ones through the box (`take` hands them out after the wait).
+// The box's payload is free by then: the upload that used it has been read.
+struct Download {
+    alx_ctx *c;
+    struct { void *dst; size_t bytes, at; } part[4];
+    int n = 0;
+    size_t used = kBoxSmall;
+    explicit Download(alx_ctx *ctx) : c(ctx) {}
+    alx_status add(void *dst, const void *dev, size_t bytes)
+    {
+        alx_status st = ensure_box(c);
+        if (st != ALX_OK) return st;
+        if (used + aligned(bytes) <= kBoxBytes) {
+            part[n++] = {dst, bytes, used};
+            ALX_CUDA(c, cudaMemcpyAsync(c->box + used, dev, bytes, cudaMemcpyDeviceToHost, c->stream));
+            used += aligned(bytes);
+        } else {
+            ALX_CUDA(c, cudaMemcpyAsync(dst, dev, bytes, cudaMemcpyDeviceToHost, c->stream));
+        }
+        return ALX_OK;
+    }
+    void take()
+    {
+        for (int k = 0; k < n; ++k) memcpy(part[k].dst, c->box + part[k].at, part[k].bytes);
+    }
+};
+
+// wait for the stream, read and clear the device status word
 alx_status check_device_status(alx_ctx *c)
 {
     DevStatus h;
-    ALX_CUDA(c, cudaMemcpyAsync(&h, c->status, sizeof h, cudaMemcpyDeviceToHost, c->stream));
+    {
+        alx_status st = ensure_box(c);
+        if (st != ALX_OK) return st;
+    }
+    ALX_CUDA(c, cudaMemcpyAsync(c->box, c->status, sizeof h, cudaMemcpyDeviceToHost, c->stream));
     ALX_CUDA(c, cudaStreamSynchronize(c->stream));
+    memcpy(&h, c->box, sizeof h);
     c->stats.not_spd += (int64_t)h.not_spd;
     if (h.flags == 0) return ALX_OK;
     ALX_CUDA(c, cudaMemsetAsync(c->status, 0, sizeof(DevStatus), c->stream));
@@ -214,16 +320,9 @@ SideView side_view(const alx_ctx *c, int side)
     return v;
 }
 
-// degree classes, order and chunk descriptors of one orientation
-alx_status build_buckets(alx_ctx *c, int side, int64_t *scratch_a, int64_t *scratch_b, int64_t *scan_scratch,
-                         int64_t scan_elems)
+// chunk descriptors of the rows longer than `split` of one orientation, from its class offsets
+alx_status build_chunks(alx_ctx *c, int side, int64_t *scan_scratch, int64_t scan_elems)
 {
-    const int64_t n = c->n[side];
-    ALX_CUDA(c, launch_bucket(c->ptr[side], n, c->split, scratch_a, scratch_b, scan_scratch, scan_elems,
-                              c->order[side], c->class_offs_dev[side], c->stream, &c->launches));
-    ALX_CUDA(c, cudaMemcpyAsync(c->class_offs[side], c->class_offs_dev[side], sizeof(int64_t) * (ALX_N_CLASSES + 1),
-                                cudaMemcpyDeviceToHost, c->stream));
-    ALX_CUDA(c, cudaStreamSynchronize(c->stream));
     const int64_t *offs = c->class_offs[side];
     const int64_t n_split = offs[ALX_N_CLASSES] - offs[ALX_N_CLASSES - 1];
     c->n_split_rows[side] = n_split;
@@ -246,6 +345,22 @@ alx_status build_buckets(alx_ctx *c, int side, int64_t *scratch_a, int64_t *scra
                                       c->chunk_desc[side], c->stream, &c->launches));
         ALX_CUDA(c, cudaStreamSynchronize(c->stream));
     }
+    return ALX_OK;
+}
+
+// degree classes, order and chunk descriptors of one orientation
+alx_status build_buckets(alx_ctx *c, int side, int64_t *scratch_a, int64_t *scratch_b, int64_t *scan_scratch,
+                         int64_t scan_elems)
+{
+    const int64_t n = c->n[side];
+    ALX_CUDA(c, launch_bucket(c->ptr[side], n, c->split, scratch_a, scratch_b, scan_scratch, scan_elems,
+                              c->order[side], c->class_offs_dev[side], c->stream, &c->launches));
+    ALX_CUDA(c, cudaMemcpyAsync(c->class_offs[side], c->class_offs_dev[side], sizeof(int64_t) * (ALX_N_CLASSES + 1),
+                                cudaMemcpyDeviceToHost, c->stream));
+    ALX_CUDA(c, cudaStreamSynchronize(c->stream));
+    alx_status st = build_chunks(c, side, scan_scratch, scan_elems);
+    if (st != ALX_OK) return st;
+    const int64_t *offs = c->class_offs[side];
     for (int k = 0; k < ALX_N_CLASSES; ++k) c->stats.rows_in_class[side][k] = offs[k + 1] - offs[k];
     c->stats.n_chunks[side] = c->n_chunks[side];
     return ALX_OK;
@@ -338,8 +453,7 @@ alx_status half_epoch_impl(alx_ctx *c, int side, const int32_t *cap_slot, float 
     NvtxRange rows_range("alx rows: gather, sums, solve, store");
     RowOut out{c->table[side], cap_slot, cap_out};
     c->dual_candidates = c->dual_candidates32 = 0;
-    c->dual_flag_latched = 0;
-    c->policy_latched = CgPolicy{};
+    c->last_side = side;
     if (warp_path(c)) {
         if (cg64(c)) ALX_CUDA(c, cudaMemsetAsync(c->cg_counters, 0, 5 * sizeof(unsigned long long), c->stream));
         const int64_t n_dual = dual_rows_of(c, side);
@@ -354,9 +468,6 @@ alx_status half_epoch_impl(alx_ctx *c, int side, const int32_t *cap_slot, float 
         c->stats.kernel_path[side] = 1;
         c->main_timed = true;
         c->dual_candidates = n_dual;
-        if (n_dual > 0)
-            ALX_CUDA(c, cudaMemcpyAsync(&c->dual_flag_latched, dual64_flag_ptr(c->dual_ws), sizeof(int), cudaMemcpyDeviceToHost,
-                                        c->stream));
     } else if (tensor_path(c)) {
         const int64_t n_dual = dual_rows_of(c, side);
         ALX_CUDA(c, cudaMemsetAsync(c->cg_counters, 0, 5 * sizeof(unsigned long long), c->stream));
@@ -368,13 +479,6 @@ alx_status half_epoch_impl(alx_ctx *c, int side, const int32_t *cap_slot, float 
         c->main_timed = true;
         c->dual_candidates = n_dual;
         c->dual_candidates32 = n_dual > 0 ? c->class_offs[side][3] - c->class_offs[side][2] : 0;
-        if (n_dual > 0) {
-            ALX_CUDA(c, cudaMemcpyAsync(&c->dual_flag_latched, dual_flag_ptr(c->dual_ws), sizeof(int), cudaMemcpyDeviceToHost,
-                                        c->stream));
-            if (c->cg_policy && c->opt.solver == ALX_SOLVER_AUTO)
-                ALX_CUDA(c, cudaMemcpyAsync(&c->policy_latched, c->cg_policy + side, sizeof(CgPolicy), cudaMemcpyDeviceToHost,
-                                            c->stream));
-        }
     } else {
         ALX_CUDA(c, launch_rows_simple(side_view(c, side), c->class_offs[side], c->n_chunks[side], c->n_split_rows[side], c->table[fixed],
                                        c->bf16, c->opt.d, c->Bmat, c->split_partials, out, c->status, c->stream, &c->launches));
@@ -410,7 +514,7 @@ alx_status create_impl(const alx_options *opt, const alx_ctx *parent, alx_ctx **
 alx_status alx_create_ex(const alx_options *opt, alx_ctx **out) { return create_impl(opt, nullptr, out); }
 
 namespace {
-// parent: the new context borrows the parent's column table (alx_fold_in) instead of holding one of its own
+// parent: the new context borrows the parent's column table (alx_fold_in) and gets its rows' buffers call by call
 alx_status create_impl(const alx_options *opt, const alx_ctx *parent, alx_ctx **out)
 {
     if (!opt || !out) return ALX_ERR_INVALID_ARG;
@@ -445,8 +549,8 @@ alx_status create_impl(const alx_options *opt, const alx_ctx *parent, alx_ctx **
     auto body = [&]() -> alx_status {
         const int d = opt->d;
         for (int s = 0; s < 2; ++s) {
-            void *t = parent && s == ALX_COLS ? parent->table[s] : dev_alloc(c, (size_t)c->n[s] * d * c->elem);
-            if (!t) return fail(c, ALX_ERR_OOM, "device allocation of a %lld x %d table failed", (long long)c->n[s], d);
+            void *t = parent ? (s == ALX_COLS ? parent->table[s] : nullptr) : dev_alloc(c, (size_t)c->n[s] * d * c->elem);
+            if (!t && !(parent && s == ALX_ROWS)) return fail(c, ALX_ERR_OOM, "device allocation of a %lld x %d table failed", (long long)c->n[s], d);
             c->table[s] = t;
             ALX_ALLOC(c, c->G64[s], d * d);
             ALX_ALLOC(c, c->class_offs_dev[s], ALX_N_CLASSES + 1);
@@ -465,7 +569,7 @@ alx_status create_impl(const alx_options *opt, const alx_ctx *parent, alx_ctx **
         ALX_ALLOC(c, c->status, 1);
         ALX_CUDA(c, cudaMemsetAsync(c->status, 0, sizeof(DevStatus), c->stream));
         ALX_ALLOC(c, c->cg_counters, 5);
-        if ((tensor_path(c) || cg64(c)) && c->opt.solver == ALX_SOLVER_AUTO) ALX_ALLOC(c, c->cg_fallback_list, nmax);
+        if ((tensor_path(c) || cg64(c)) && c->opt.solver == ALX_SOLVER_AUTO && !parent) ALX_ALLOC(c, c->cg_fallback_list, nmax);
         if (tensor_path(c) && c->opt.solver == ALX_SOLVER_AUTO) {
             ALX_ALLOC(c, c->cg_policy, 2);
             ALX_CUDA(c, cudaMemsetAsync(c->cg_policy, 0, 2 * sizeof(CgPolicy), c->stream));
@@ -490,6 +594,8 @@ alx_status alx_destroy(alx_ctx *c)
     if (!c) return ALX_OK;
     DeviceGuard guard(c->device);
     cudaStreamSynchronize(c->stream);
+    if (c->fold) alx_destroy(c->fold);
+    if (c->box) cudaFreeHost(c->box);
     for (auto &e : c->ev) if (e) cudaEventDestroy(e);
     if (c->copy_stream) { cudaStreamSynchronize(c->copy_stream); cudaStreamDestroy(c->copy_stream); }
     if (c->copy_ev) cudaEventDestroy(c->copy_ev);
@@ -870,9 +976,11 @@ alx_status alx_loss(alx_ctx *c, double *total, double *components)
                             c->G64[1], (double)c->opt.alpha0, (double)c->opt.lambda, c->loss_partials_buf, c->loss_result, c->stream,
                             &c->launches));
     double h[3];
-    ALX_CUDA(c, cudaMemcpyAsync(h, c->loss_result, sizeof h, cudaMemcpyDeviceToHost, c->stream));
-    alx_status st = check_device_status(c);
+    Download down(c);
+    alx_status st = down.add(h, c->loss_result, sizeof h);
+    if (st == ALX_OK) st = check_device_status(c);
     if (st != ALX_OK) return st;
+    down.take();
     *total = h[0] + h[1] + h[2];
     if (components) { components[0] = h[0]; components[1] = h[1]; components[2] = h[2]; }
     return ALX_OK;
@@ -909,6 +1017,92 @@ alx_status alx_get_buckets(alx_ctx *c, alx_side side, int32_t *order, int64_t *c
     return ALX_OK;
 }
 
+namespace {
+// The rows half-step of Eq. 4 on new rows, in a context that borrows the column table.  What alx_set_csr does for the rows'
+// side and nothing of its columns' (the transpose and the degree classes of a million columns were most of the time of a
+// call with a few rows); buffers are kept from call to call, the solver's history is not.
+alx_status fold_in_impl(alx_ctx *k, const int64_t *rowptr, const int32_t *colidx, const float *values, int64_t n, int64_t nnz, int on_device,
+                        float *x_out)
+{
+    const int d = k->opt.d;
+    alx_status st = ensure_box(k);
+    if (st != ALX_OK) return st;
+    // what the last call left
+    dev_free(k, k->chunk_desc[0]); k->chunk_desc[0] = nullptr;
+    dev_free(k, k->split_first[0]); k->split_first[0] = nullptr;
+    k->nnz = -1;
+    k->n[ALX_ROWS] = n;
+    k->has_values = values != nullptr;
+    k->have_table[ALX_ROWS] = false;
+    // upload (or take the caller's device arrays as they are: they are only read, and not after the call)
+    if (on_device) {
+        k->ptr[0] = const_cast<int64_t *>(rowptr);
+        k->idx[0] = const_cast<int32_t *>(colidx);
+        k->val[0] = const_cast<float *>(values);
+    } else {
+        Upload up(k);
+        void *dev[4];
+        up.add(rowptr, sizeof(int64_t) * (n + 1));
+        up.add(colidx, sizeof(int32_t) * nnz);
+        if (values) up.add(values, sizeof(float) * nnz);
+        if ((st = up.send(kKeptRows, dev)) != ALX_OK) return st;
+        k->ptr[0] = static_cast<int64_t *>(dev[0]);
+        k->idx[0] = static_cast<int32_t *>(dev[1]);
+        k->val[0] = values ? static_cast<float *>(dev[2]) : nullptr;
+    }
+    void *order = nullptr, *scratch = nullptr, *table = nullptr, *list = nullptr, *sums = nullptr;
+    const int64_t nb = bucket_blocks(n);
+    const int64_t scan_elems = scan_scratch_elems(nb * kNClasses > n ? nb * kNClasses : n) + 16;
+    if ((st = keep(k, kKeptOrder, sizeof(int32_t) * n, &order)) != ALX_OK) return st;
+    if ((st = keep(k, kKeptScratch, sizeof(int64_t) * (2 * nb * kNClasses + 1 + scan_elems), &scratch)) != ALX_OK) return st;
+    if ((st = keep(k, kKeptTable, (size_t)n * d * k->elem, &table)) != ALX_OK) return st;
+    k->order[0] = static_cast<int32_t *>(order);
+    k->table[0] = table;
+    if (k->opt.solver == ALX_SOLVER_AUTO && (tensor_path(k) || cg64(k))) {
+        if ((st = keep(k, kKeptFallback, sizeof(int32_t) * n, &list)) != ALX_OK) return st;
+        k->cg_fallback_list = static_cast<int32_t *>(list);
+    }
+    if (k->cg_policy) ALX_CUDA(k, cudaMemsetAsync(k->cg_policy, 0, 2 * sizeof(CgPolicy), k->stream));
+    int64_t *blk_counts = static_cast<int64_t *>(scratch), *blk_offs = blk_counts + nb * kNClasses, *scan = blk_offs + nb * kNClasses + 1;
+    ALX_CUDA(k, launch_validate(k->ptr[0], k->idx[0], n, k->n[1], nnz, k->status, k->stream, &k->launches));
+    // (the degree classes only look at the offsets' differences: nothing is indexed with them before the check below)
+    ALX_CUDA(k, launch_bucket(k->ptr[0], n, k->split, blk_counts, blk_offs, scan, scan_elems, k->order[0], k->class_offs_dev[0], k->stream,
+                              &k->launches));
+    {
+        Download down(k);
+        if ((st = down.add(k->class_offs[0], k->class_offs_dev[0], sizeof(int64_t) * (ALX_N_CLASSES + 1))) != ALX_OK) return st;
+        if ((st = check_device_status(k)) != ALX_OK) return st;
+        down.take();
+    }
+    if ((st = build_chunks(k, 0, scan, scan_elems)) != ALX_OK) return st;
+    const int64_t *offs = k->class_offs[0];
+    const int64_t n_sums = k->n_chunks[0] + (tensor_path(k) ? offs[kNClasses - 1] - offs[long_class_begin(offs)] : 0);
+    if (n_sums > 0) {
+        if ((st = keep(k, kKeptSums, sizeof(float) * n_sums * (d * d + d), &sums)) != ALX_OK) return st;
+        k->split_partials = static_cast<float *>(sums);
+    }
+    k->nnz = nnz;
+    if ((st = half_epoch_impl(k, ALX_ROWS, nullptr, nullptr)) != ALX_OK) return st;
+    const size_t bytes = sizeof(float) * n * d;
+    if (on_device) {
+        ALX_CUDA(k, launch_convert(k->table[0], k->bf16, x_out, 0, n * d, k->stream, &k->launches));
+        return check_device_status(k);
+    }
+    const void *x = k->table[0];
+    if (k->bf16) {
+        void *wide = nullptr;
+        if ((st = keep(k, kKeptOut, bytes, &wide)) != ALX_OK) return st;
+        ALX_CUDA(k, launch_convert(k->table[0], 1, wide, 0, n * d, k->stream, &k->launches));
+        x = wide;
+    }
+    Download down(k);
+    if ((st = down.add(x_out, x, bytes)) != ALX_OK) return st;
+    st = check_device_status(k);
+    if (st == ALX_OK) down.take();
+    return st;
+}
+}  // namespace
+
 alx_status alx_fold_in(alx_ctx *c, const int64_t *rowptr, const int32_t *colidx, const float *values, int64_t n_new,
                        int64_t nnz, int on_device, float *x_out)
 {
@@ -918,22 +1112,25 @@ alx_status alx_fold_in(alx_ctx *c, const int64_t *rowptr, const int32_t *colidx,
     if (!c->have_table[ALX_COLS]) return fail(c, ALX_ERR_BAD_STATE, "the column table has not been set or solved yet");
     if (n_new == 0) return ALX_OK;
     DeviceGuard guard(c->device);
-    ALX_CUDA(c, cudaStreamSynchronize(c->stream));
-    // a context of its own for the new rows: same options, the column table borrowed, the rows half-step of Eq. 4
-    alx_options o = c->opt;
-    o.n_rows = n_new;
-    o.device = c->device;
-    alx_ctx *k = nullptr;
-    alx_status st = create_impl(&o, c, &k);
-    if (st != ALX_OK) return fail(c, st, "alx_fold_in: the context for the new rows could not be created");
-    k->have_table[ALX_COLS] = true;
-    st = alx_set_csr(k, rowptr, colidx, values, nnz, on_device);
-    if (st == ALX_OK) st = alx_half_epoch(k, ALX_ROWS);
-    if (st == ALX_OK) st = alx_get_embeddings(k, ALX_ROWS, x_out, ALX_F32, 0, n_new, on_device);
-    if (st == ALX_OK) st = alx_synchronize(k);
-    c->launches += k->launches;
-    if (st != ALX_OK) c->err = "alx_fold_in: " + k->err;
-    alx_destroy(k);
+    std::lock_guard<std::mutex> lock(c->calls);
+    if (!c->fold) {
+        // a context of its own for the new rows: same options, the column table borrowed
+        alx_options o = c->opt;
+        o.n_rows = 1;
+        o.device = c->device;
+        alx_status st = create_impl(&o, c, &c->fold);
+        if (st != ALX_OK) return fail(c, st, "alx_fold_in: the context for the new rows could not be created");
+        c->fold->have_table[ALX_COLS] = true;
+    }
+    alx_ctx *k = c->fold;
+    const int64_t before = k->launches;
+    alx_status st = fold_in_impl(k, rowptr, colidx, values, n_new, nnz, on_device, x_out);
+    c->launches += k->launches - before;
+    if (st != ALX_OK) {
+        cudaStreamSynchronize(k->stream);
+        c->err = "alx_fold_in: " + k->err;
+    }
+    give_back_large(k);
     return st;
 }
 
@@ -950,44 +1147,52 @@ alx_status alx_topk(alx_ctx *c, alx_side items, const float *queries, int64_t m,
     NvtxRange range("alx_topk");
     const int d = c->opt.d;
     const int64_t n_items = c->n[items];
-    Scratch tmp(c);
+    std::lock_guard<std::mutex> lock(c->calls);
     const float *Q = queries;
     const int64_t *ex_ptr = exclude_ptr;
     const int32_t *ex_idx = exclude_idx;
     int32_t *ids_dev = ids_out;
     float *scores_dev = scores_out;
-    int64_t n_ex = 0;
+    alx_status st;
     if (!on_device) {
-        float *q_dev = nullptr;
-        ALX_TMP(c, tmp, q_dev, m * d);
-        ALX_CUDA(c, cudaMemcpyAsync(q_dev, queries, sizeof(float) * m * d, cudaMemcpyHostToDevice, c->stream));
-        Q = q_dev;
+        Upload up(c);
+        void *dev[4];
+        up.add(queries, sizeof(float) * m * d);
         if (exclude_ptr) {
-            n_ex = exclude_ptr[m];
-            if (n_ex < 0) return fail(c, ALX_ERR_INVALID_ARG, "alx_topk: negative length of the exclusion lists");
-            int64_t *p_dev = nullptr;
-            int32_t *i_dev = nullptr;
-            ALX_TMP(c, tmp, p_dev, m + 1);
-            ALX_TMP(c, tmp, i_dev, n_ex > 0 ? n_ex : 1);
-            ALX_CUDA(c, cudaMemcpyAsync(p_dev, exclude_ptr, sizeof(int64_t) * (m + 1), cudaMemcpyHostToDevice, c->stream));
-            if (n_ex > 0) ALX_CUDA(c, cudaMemcpyAsync(i_dev, exclude_idx, sizeof(int32_t) * n_ex, cudaMemcpyHostToDevice, c->stream));
-            ex_ptr = p_dev;
-            ex_idx = i_dev;
+            if (exclude_ptr[m] < 0) return fail(c, ALX_ERR_INVALID_ARG, "alx_topk: negative length of the exclusion lists");
+            up.add(exclude_ptr, sizeof(int64_t) * (m + 1));
+            up.add(exclude_idx, sizeof(int32_t) * exclude_ptr[m]);
         }
-        ALX_TMP(c, tmp, ids_dev, m * k);
-        if (scores_out) ALX_TMP(c, tmp, scores_dev, m * k);
+        if ((st = up.send(kKeptUpload, dev)) != ALX_OK) return st;
+        Q = static_cast<const float *>(dev[0]);
+        if (exclude_ptr) {
+            ex_ptr = static_cast<const int64_t *>(dev[1]);
+            ex_idx = static_cast<const int32_t *>(dev[2]);
+        }
+        void *out = nullptr;
+        const size_t list = aligned(sizeof(int32_t) * m * k);
+        if ((st = keep(c, kKeptOut, 2 * list, &out)) != ALX_OK) return st;
+        ids_dev = static_cast<int32_t *>(out);
+        scores_dev = scores_out ? reinterpret_cast<float *>(static_cast<unsigned char *>(out) + list) : nullptr;
     }
     const TopkPlan plan = topk_plan(n_items, m, k, c->opt.kernels != 1 && c->bf16 && d == 128);
-    unsigned char *work = nullptr;
-    ALX_TMP(c, tmp, work, plan.workspace_bytes());
-    ALX_CUDA(c, launch_topk(plan, c->table[items], c->bf16 != 0, n_items, d, Q, m, k, ex_ptr, ex_idx, work, ids_dev, scores_dev,
-                            c->status, c->stream, &c->launches));
-    if (!on_device) {
-        ALX_CUDA(c, cudaMemcpyAsync(ids_out, ids_dev, sizeof(int32_t) * m * k, cudaMemcpyDeviceToHost, c->stream));
-        if (scores_out) ALX_CUDA(c, cudaMemcpyAsync(scores_out, scores_dev, sizeof(float) * m * k, cudaMemcpyDeviceToHost, c->stream));
+    void *work = nullptr;
+    if ((st = keep(c, kKeptWork, plan.workspace_bytes(), &work)) != ALX_OK) return st;
+    const cudaError_t e = launch_topk(plan, c->table[items], c->bf16 != 0, n_items, d, Q, m, k, ex_ptr, ex_idx, work, ids_dev, scores_dev,
+                                      c->status, c->stream, &c->launches);
+    if (e != cudaSuccess) {
+        cudaStreamSynchronize(c->stream);
+        return fail(c, ALX_ERR_CUDA, "alx_topk: %s", cudaGetErrorString(e));
     }
-    ALX_CUDA(c, cudaStreamSynchronize(c->stream));
-    return check_device_status(c);
+    Download down(c);
+    if (!on_device) {
+        if ((st = down.add(ids_out, ids_dev, sizeof(int32_t) * m * k)) != ALX_OK) return st;
+        if (scores_out && (st = down.add(scores_out, scores_dev, sizeof(float) * m * k)) != ALX_OK) return st;
+    }
+    st = check_device_status(c);
+    if (st == ALX_OK) down.take();
+    give_back_large(c);
+    return st;
 }
 
 alx_status alx_recall_at_k(alx_ctx *c, const int32_t *ids, int64_t m, int32_t k_stride, int32_t k, const int64_t *truth_ptr,
@@ -997,30 +1202,34 @@ alx_status alx_recall_at_k(alx_ctx *c, const int32_t *ids, int64_t m, int32_t k_
     if (m < 0 || k < 1 || k > k_stride || !recall || (m > 0 && (!ids || !truth_ptr)))
         return fail(c, ALX_ERR_INVALID_ARG, "bad argument to alx_recall_at_k");
     DeviceGuard guard(c->device);
-    Scratch tmp(c);
+    std::lock_guard<std::mutex> lock(c->calls);
     const int32_t *ids_dev = ids;
     const int64_t *tp = truth_ptr;
     const int32_t *ti = truth_idx;
+    alx_status st;
     if (!on_device && m > 0) {
         const int64_t nt = truth_ptr[m];
         if (nt < 0 || (nt > 0 && !truth_idx)) return fail(c, ALX_ERR_INVALID_ARG, "alx_recall_at_k: bad ground-truth lists");
-        int32_t *a = nullptr, *t = nullptr;
-        int64_t *p = nullptr;
-        ALX_TMP(c, tmp, a, m * k_stride);
-        ALX_TMP(c, tmp, p, m + 1);
-        ALX_TMP(c, tmp, t, nt > 0 ? nt : 1);
-        ALX_CUDA(c, cudaMemcpyAsync(a, ids, sizeof(int32_t) * m * k_stride, cudaMemcpyHostToDevice, c->stream));
-        ALX_CUDA(c, cudaMemcpyAsync(p, truth_ptr, sizeof(int64_t) * (m + 1), cudaMemcpyHostToDevice, c->stream));
-        if (nt > 0) ALX_CUDA(c, cudaMemcpyAsync(t, truth_idx, sizeof(int32_t) * nt, cudaMemcpyHostToDevice, c->stream));
-        ids_dev = a; tp = p; ti = t;
+        Upload up(c);
+        void *dev[4];
+        up.add(ids, sizeof(int32_t) * m * k_stride);
+        up.add(truth_ptr, sizeof(int64_t) * (m + 1));
+        up.add(truth_idx, sizeof(int32_t) * nt);
+        if ((st = up.send(kKeptUpload, dev)) != ALX_OK) return st;
+        ids_dev = static_cast<const int32_t *>(dev[0]);
+        tp = static_cast<const int64_t *>(dev[1]);
+        ti = static_cast<const int32_t *>(dev[2]);
     }
-    double *per_query = nullptr, *out2 = nullptr;
-    ALX_TMP(c, tmp, per_query, m > 0 ? m : 1);
-    ALX_TMP(c, tmp, out2, 2);
+    void *work = nullptr;
+    if ((st = keep(c, kKeptWork, sizeof(double) * (2 + (m > 0 ? m : 1)), &work)) != ALX_OK) return st;
+    double *out2 = static_cast<double *>(work), *per_query = out2 + 2;
     ALX_CUDA(c, launch_recall(ids_dev, m, k_stride, k, tp, ti, per_query, out2, c->stream, &c->launches));
     double h[2] = {0.0, 0.0};
-    ALX_CUDA(c, cudaMemcpyAsync(h, out2, sizeof h, cudaMemcpyDeviceToHost, c->stream));
+    Download down(c);
+    if ((st = down.add(h, out2, sizeof h)) != ALX_OK) return st;
     ALX_CUDA(c, cudaStreamSynchronize(c->stream));
+    down.take();
+    give_back_large(c);
     *recall = h[1] > 0.0 ? h[0] / h[1] : 0.0;
     if (n_counted) *n_counted = (int64_t)h[1];
     return ALX_OK;
@@ -1039,8 +1248,15 @@ alx_status alx_get_stats(alx_ctx *c, alx_stats *out)
     if (c->main_timed) {
         if (cudaEventElapsedTime(&ms, c->ev[3], c->ev[4]) == cudaSuccess) c->stats.ms_main_kernel = ms; else cudaGetLastError();
     }
-    c->stats.dual_rows = c->dual_candidates > 0 && c->dual_flag_latched
-                             ? c->dual_candidates - (c->policy_latched.short_rows_by_cg ? c->dual_candidates32 : 0) : 0;
+    // (the flag and the record are rewritten by half-epochs only)
+    c->stats.dual_rows = 0;
+    if (c->dual_candidates > 0) {
+        int flag = 0;
+        CgPolicy pol{};
+        ALX_CUDA(c, cudaMemcpy(&flag, tensor_path(c) ? dual_flag_ptr(c->dual_ws) : dual64_flag_ptr(c->dual_ws), sizeof flag, cudaMemcpyDeviceToHost));
+        if (c->cg_policy) ALX_CUDA(c, cudaMemcpy(&pol, c->cg_policy + c->last_side, sizeof pol, cudaMemcpyDeviceToHost));
+        if (flag) c->stats.dual_rows = c->dual_candidates - (pol.short_rows_by_cg ? c->dual_candidates32 : 0);
+    }
     {
         unsigned long long h[5] = {0, 0, 0, 0, 0};
         ALX_CUDA(c, cudaMemcpy(h, c->cg_counters, sizeof h, cudaMemcpyDeviceToHost));

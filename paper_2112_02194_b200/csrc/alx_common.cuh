@@ -90,10 +90,6 @@ int64_t scan_scratch_elems(int64_t n);
 cudaError_t launch_validate(const int64_t *rowptr, const int32_t *colidx, int64_t n_rows, int64_t n_cols,
                             int64_t nnz, DevStatus *st, cudaStream_t s, int64_t *launches);
 cudaError_t launch_degrees(const int64_t *ptr, int64_t n, int32_t *deg, cudaStream_t s, int64_t *launches);
-// Entry lists over a table of 2N rows (the bfloat16 parts of an fp32 table, see launch_rows_fold): row u of length L
-// becomes a row of 2L entries, its L ids followed by the same ids + N (labels repeated); vptr = 2 ptr.
-cudaError_t launch_double_entries(const int64_t *ptr, const int32_t *idx, const float *val, int64_t n, int64_t n_fixed,
-                                  int64_t *vptr, int32_t *vidx, float *vval, cudaStream_t s, int64_t *launches);
 // stable partition of a list of rows by length (see alx_setup.cu)
 cudaError_t launch_partition_by_length(const int64_t *ptr, const int32_t *rows, int64_t count, int limit, int32_t *out,
                                        int64_t *block_counts, int64_t *block_offsets, int64_t *n_short_dev,
@@ -220,12 +216,6 @@ cudaError_t launch_topk(const TopkPlan &p, const void *H, bool bf16, int64_t n_i
                         DevStatus *st, cudaStream_t s, int64_t *launches);
 cudaError_t launch_recall(const int32_t *ids, int64_t m, int k_stride, int k, const int64_t *tptr, const int32_t *tidx,
                           double *per_query, double *out2, cudaStream_t s, int64_t *launches);
-cudaError_t launch_rows_fold(const SideView &sv, const int64_t *class_offs_host, int64_t n_chunks, int64_t n_split_rows,
-                             const void *T, int64_t n_table, const float *Bmat, float *split_partials, RowOut out,
-                             DevStatus *st, cudaStream_t s, int64_t *launches, cudaEvent_t main_begin, cudaEvent_t main_end,
-                             const CgOptions &cg, const int *dual_flag);
-// fp32 table [n x 64] -> bfloat16 parts [2n x 128]
-cudaError_t launch_split_table(const float *X, int64_t n, void *T, cudaStream_t s, int64_t *launches);
 cudaError_t launch_rows_umma(const SideView &sv, const int64_t *class_offs_host, int64_t n_chunks,
                              int64_t n_split_rows, const void *X, const float *Bmat, float *split_partials,
                              RowOut out, DevStatus *st, cudaStream_t s, int64_t *launches, cudaEvent_t main_begin,
