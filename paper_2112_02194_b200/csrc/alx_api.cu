@@ -385,7 +385,9 @@ void release_matrix(alx_ctx *c)
 bool tensor_path(const alx_ctx *c) { return c->bf16 && c->opt.d == 128 && c->opt.kernels != 1; }
 // d <= 64: a warp per row (alx_rows_warp.cu)
 bool warp_path(const alx_ctx *c) { return c->opt.d <= 64 && c->opt.kernels != 1; }
-// of those, fp32 tables of 64 features: conjugate gradients, and the dual form for rows of at most 16 observations
+// fp32 tables of 128 features: four warps per row (alx_rows_team.cu)
+bool team_path(const alx_ctx *c) { return c->opt.d == 128 && !c->bf16 && c->opt.kernels != 1; }
+// of the warp path, fp32 tables of 64 features: conjugate gradients, and the dual form for rows of at most 16 observations
 bool cg64(const alx_ctx *c) { return warp_path(c) && !c->bf16 && c->opt.d == 64; }
 bool dual64(const alx_ctx *c) { return cg64(c) && c->opt.kernels == 0; }
 // Fewer rows than this are not worth the inverse of the base matrix that the dual form starts with (25 us and more, against
@@ -406,6 +408,15 @@ CgOptions cg_options(const alx_ctx *c, int solved_side)
     o.policy = c->cg_policy ? c->cg_policy + solved_side : nullptr;
     o.switch_products = c->opt.cg_switch_products > 0.f ? c->opt.cg_switch_products : ALX_DEFAULT_CG_SWITCH_PRODUCTS;
     return o;
+}
+
+// floats of workspace that the sums of a side's chunks and long rows need
+int64_t sums_floats(const alx_ctx *c, int side)
+{
+    const int64_t *offs = c->class_offs[side];
+    const int64_t d = c->opt.d;
+    if (team_path(c)) return team_sums_floats(offs, c->n_chunks[side]);
+    return (c->n_chunks[side] + (tensor_path(c) ? offs[kNClasses - 1] - offs[long_class_begin(offs)] : 0)) * (d * d + d);
 }
 
 // rows of a side that the dual form is offered (class 1, and class 2 for d = 128); 0: none, or too few
@@ -479,6 +490,11 @@ alx_status half_epoch_impl(alx_ctx *c, int side, const int32_t *cap_slot, float 
         c->main_timed = true;
         c->dual_candidates = n_dual;
         c->dual_candidates32 = n_dual > 0 ? c->class_offs[side][3] - c->class_offs[side][2] : 0;
+    } else if (team_path(c)) {
+        ALX_CUDA(c, launch_rows_team(side_view(c, side), c->class_offs[side], c->n_chunks[side], c->n_split_rows[side],
+                                     static_cast<const float *>(c->table[fixed]), c->Bmat, c->split_partials, out, c->status, c->stream,
+                                     &c->launches));
+        c->stats.kernel_path[side] = 1;
     } else {
         ALX_CUDA(c, launch_rows_simple(side_view(c, side), c->class_offs[side], c->n_chunks[side], c->n_split_rows[side], c->table[fixed],
                                        c->bf16, c->opt.d, c->Bmat, c->split_partials, out, c->status, c->stream, &c->launches));
@@ -718,17 +734,14 @@ alx_status alx_set_csr(alx_ctx *c, const int64_t *rowptr, const int32_t *colidx,
     tmp.release(scan_scratch);
     tmp.release(class_entries);
 
-    const int d = c->opt.d;
-    int64_t sums[2] = {c->n_chunks[0], c->n_chunks[1]};
     for (int s = 0; s < 2; ++s) c->stats.long_rows[s] = c->stats.long_entries[s] = 0;
-    if (tensor_path(c) || warp_path(c)) {    // d = 128: one more sum per long whole row
+    if (tensor_path(c) || warp_path(c)) {
         int64_t *total = nullptr;
         ALX_TMP(c, tmp, total, 2);
         for (int s = 0; s < 2; ++s) {
             const int64_t *offs = c->class_offs[s];
             const int64_t first = offs[tensor_path(c) ? long_class_begin(offs) : warp_long_class(offs)];
             const int64_t n_long = offs[kNClasses - 1] - first;
-            if (tensor_path(c)) sums[s] += n_long;
             c->stats.long_rows[s] = n_long;
             ALX_CUDA(c, launch_sum_row_lengths(c->ptr[s], c->order[s] + first, n_long, total + s, c->stream, &c->launches));
         }
@@ -736,8 +749,8 @@ alx_status alx_set_csr(alx_ctx *c, const int64_t *rowptr, const int32_t *colidx,
         ALX_CUDA(c, cudaStreamSynchronize(c->stream));
         tmp.release(total);
     }
-    const int64_t max_chunks = sums[0] > sums[1] ? sums[0] : sums[1];
-    if (max_chunks > 0) ALX_ALLOC(c, c->split_partials, max_chunks * (int64_t)(d * d + d));
+    const int64_t sums = sums_floats(c, 0) > sums_floats(c, 1) ? sums_floats(c, 0) : sums_floats(c, 1);
+    if (sums > 0) ALX_ALLOC(c, c->split_partials, sums);
     ALX_ALLOC(c, c->loss_partials_buf, loss_partials(nnz));
     c->stats.nnz = nnz;
     return ALX_OK;
@@ -1075,10 +1088,8 @@ alx_status fold_in_impl(alx_ctx *k, const int64_t *rowptr, const int32_t *colidx
         down.take();
     }
     if ((st = build_chunks(k, 0, scan, scan_elems)) != ALX_OK) return st;
-    const int64_t *offs = k->class_offs[0];
-    const int64_t n_sums = k->n_chunks[0] + (tensor_path(k) ? offs[kNClasses - 1] - offs[long_class_begin(offs)] : 0);
-    if (n_sums > 0) {
-        if ((st = keep(k, kKeptSums, sizeof(float) * n_sums * (d * d + d), &sums)) != ALX_OK) return st;
+    if (sums_floats(k, 0) > 0) {
+        if ((st = keep(k, kKeptSums, sizeof(float) * sums_floats(k, 0), &sums)) != ALX_OK) return st;
         k->split_partials = static_cast<float *>(sums);
     }
     k->nnz = nnz;

@@ -190,6 +190,11 @@ cudaError_t launch_rows_warp(const SideView &sv, const int64_t *class_offs_host,
                              int bf16, int d, const float *Bmat, float *split_partials, RowOut out, DevStatus *st, const CgOptions &cg,
                              const int *dual_flag, cudaStream_t s, int64_t *launches);
 
+// alx_rows_team.cu: fp32 tables of 128 features, four warps per row (kernels != 1); `sums`: team_sums_floats() floats
+int64_t team_sums_floats(const int64_t *class_offs_host, int64_t n_chunks);
+cudaError_t launch_rows_team(const SideView &sv, const int64_t *class_offs_host, int64_t n_chunks, int64_t n_split_rows, const float *X,
+                             const float *Bmat, float *sums, RowOut out, DevStatus *st, cudaStream_t s, int64_t *launches);
+
 // alx_umma.cu: tensor-core path, d = 128 and bf16 tables only
 int64_t gramian_umma_partials();
 cudaError_t launch_gramian_umma(const void *X, int64_t n, float *partials, cudaStream_t s, int64_t *launches);
