@@ -387,13 +387,19 @@ bool tensor_path(const alx_ctx *c) { return c->bf16 && c->opt.d == 128 && c->opt
 bool warp_path(const alx_ctx *c) { return c->opt.d <= 64 && c->opt.kernels != 1; }
 // fp32 tables of 128 features: four warps per row (alx_rows_team.cu)
 bool team_path(const alx_ctx *c) { return c->opt.d == 128 && !c->bf16 && c->opt.kernels != 1; }
-// of the warp path, fp32 tables of 64 features: conjugate gradients, and the dual form for rows of at most 16 observations
+// of the warp path, fp32 tables of 64 features: conjugate gradients
 bool cg64(const alx_ctx *c) { return warp_path(c) && !c->bf16 && c->opt.d == 64; }
+// rows of at most 16 observations in the dual form, by a warp each: on the FP32 ALUs (alx_dual64.cu) or by mma (alx_dual_warp.cu)
 bool dual64(const alx_ctx *c) { return cg64(c) && c->opt.kernels == 0; }
+bool dual_warp(const alx_ctx *c) { return c->opt.kernels == 0 && (team_path(c) || (warp_path(c) && c->bf16 && c->opt.d == 64)); }
 // Fewer rows than this are not worth the inverse of the base matrix that the dual form starts with (25 us and more, against
 // a few ns per row): they take the d x d solve with the others
 constexpr int64_t kDualLeastRows = 256;
 bool dual_form(const alx_ctx *c) { return tensor_path(c) && c->opt.kernels == 0; }
+const int *dual_flag_of(const alx_ctx *c)
+{
+    return dual_form(c) ? dual_flag_ptr(c->dual_ws) : dual64(c) ? dual64_flag_ptr(c->dual_ws) : dual_warp_flag_ptr(c->dual_ws, c->opt.d);
+}
 float dual_cond_limit(const alx_ctx *c) { return c->opt.dual_cond_limit > 0.f ? c->opt.dual_cond_limit : ALX_DEFAULT_DUAL_COND_LIMIT; }
 CgOptions cg_options(const alx_ctx *c, int solved_side)
 {
@@ -423,7 +429,7 @@ int64_t sums_floats(const alx_ctx *c, int side)
 int64_t dual_rows_of(const alx_ctx *c, int side)
 {
     const int64_t *offs = c->class_offs[side];
-    const int64_t n = dual_form(c) ? offs[3] - offs[1] : dual64(c) ? offs[2] - offs[1] : 0;
+    const int64_t n = dual_form(c) ? offs[3] - offs[1] : dual_warp(c) || dual64(c) ? offs[2] - offs[1] : 0;
     return n >= kDualLeastRows ? n : 0;
 }
 
@@ -441,8 +447,12 @@ alx_status gramian_of(alx_ctx *c, int table_side, bool solve)
     }
     ALX_CUDA(c, launch_gramian(c->table[table_side], c->bf16, c->n[table_side], c->opt.d, c->gram_partials,
                                c->G64[table_side], c->Bmat, c->opt.alpha0, c->opt.lambda, c->stream, &c->launches));
-    if (solve && dual64(c))
-        ALX_CUDA(c, launch_dual64_prepare(c->Bmat, c->dual_ws, dual_cond_limit(c), c->stream, &c->launches));
+    if (solve && dual64(c)) ALX_CUDA(c, launch_dual64_prepare(c->Bmat, c->dual_ws, dual_cond_limit(c), c->stream, &c->launches));
+    if (solve && dual_warp(c)) {
+        const float most = c->bf16 ? kDualWarpLimitBf16 : kDualWarpLimitF32;
+        ALX_CUDA(c, launch_dual_warp_prepare(c->Bmat, c->dual_ws, c->opt.d, dual_cond_limit(c) < most ? dual_cond_limit(c) : most, c->stream,
+                                             &c->launches));
+    }
     c->have_gram[table_side] = true;
     return ALX_OK;
 }
@@ -469,12 +479,14 @@ alx_status half_epoch_impl(alx_ctx *c, int side, const int32_t *cap_slot, float 
         if (cg64(c)) ALX_CUDA(c, cudaMemsetAsync(c->cg_counters, 0, 5 * sizeof(unsigned long long), c->stream));
         const int64_t n_dual = dual_rows_of(c, side);
         if (n_dual > 0)
-            ALX_CUDA(c, launch_rows_dual64(side_view(c, side), c->class_offs[side][1], n_dual, c->table[fixed], c->dual_ws, out,
-                                           c->stream, &c->launches));
+            ALX_CUDA(c, dual64(c) ? launch_rows_dual64(side_view(c, side), c->class_offs[side][1], n_dual, c->table[fixed], c->dual_ws, out,
+                                                       c->stream, &c->launches)
+                                  : launch_rows_dual_warp(side_view(c, side), c->class_offs[side][1], n_dual, c->table[fixed], c->bf16,
+                                                          c->opt.d, c->dual_ws, out, c->status, c->stream, &c->launches));
         ALX_CUDA(c, cudaEventRecord(c->ev[3], c->stream));
         ALX_CUDA(c, launch_rows_warp(side_view(c, side), c->class_offs[side], c->n_chunks[side], c->n_split_rows[side], c->table[fixed],
                                      c->bf16, c->opt.d, c->Bmat, c->split_partials, out, c->status, cg_options(c, side),
-                                     n_dual > 0 ? dual64_flag_ptr(c->dual_ws) : nullptr, c->stream, &c->launches));
+                                     n_dual > 0 ? dual_flag_of(c) : nullptr, c->stream, &c->launches));
         ALX_CUDA(c, cudaEventRecord(c->ev[4], c->stream));
         c->stats.kernel_path[side] = 1;
         c->main_timed = true;
@@ -491,10 +503,15 @@ alx_status half_epoch_impl(alx_ctx *c, int side, const int32_t *cap_slot, float 
         c->dual_candidates = n_dual;
         c->dual_candidates32 = n_dual > 0 ? c->class_offs[side][3] - c->class_offs[side][2] : 0;
     } else if (team_path(c)) {
+        const int64_t n_dual = dual_rows_of(c, side);
+        if (n_dual > 0)
+            ALX_CUDA(c, launch_rows_dual_warp(side_view(c, side), c->class_offs[side][1], n_dual, c->table[fixed], 0, c->opt.d, c->dual_ws, out,
+                                              c->status, c->stream, &c->launches));
         ALX_CUDA(c, launch_rows_team(side_view(c, side), c->class_offs[side], c->n_chunks[side], c->n_split_rows[side],
-                                     static_cast<const float *>(c->table[fixed]), c->Bmat, c->split_partials, out, c->status, c->stream,
-                                     &c->launches));
+                                     static_cast<const float *>(c->table[fixed]), c->Bmat, c->split_partials, out, c->status,
+                                     n_dual > 0 ? dual_flag_of(c) : nullptr, c->stream, &c->launches));
         c->stats.kernel_path[side] = 1;
+        c->dual_candidates = n_dual;
     } else {
         ALX_CUDA(c, launch_rows_simple(side_view(c, side), c->class_offs[side], c->n_chunks[side], c->n_split_rows[side], c->table[fixed],
                                        c->bf16, c->opt.d, c->Bmat, c->split_partials, out, c->status, c->stream, &c->launches));
@@ -572,8 +589,8 @@ alx_status create_impl(const alx_options *opt, const alx_ctx *parent, alx_ctx **
             ALX_ALLOC(c, c->class_offs_dev[s], ALX_N_CLASSES + 1);
         }
         ALX_ALLOC(c, c->Bmat, d * d);
-        if (dual_form(c) || dual64(c)) {
-            c->dual_ws = dev_alloc(c, dual_form(c) ? dual_workspace_bytes() : dual64_workspace_bytes());
+        if (dual_form(c) || dual_warp(c) || dual64(c)) {
+            c->dual_ws = dev_alloc(c, dual_form(c) ? dual_workspace_bytes() : dual64(c) ? dual64_workspace_bytes() : dual_warp_workspace_bytes(opt->d));
             if (!c->dual_ws) return fail(c, ALX_ERR_OOM, "device allocation of the dual-form workspace failed");
         }
         const int64_t nmax = c->n[0] > c->n[1] ? c->n[0] : c->n[1];
@@ -1264,7 +1281,7 @@ alx_status alx_get_stats(alx_ctx *c, alx_stats *out)
     if (c->dual_candidates > 0) {
         int flag = 0;
         CgPolicy pol{};
-        ALX_CUDA(c, cudaMemcpy(&flag, tensor_path(c) ? dual_flag_ptr(c->dual_ws) : dual64_flag_ptr(c->dual_ws), sizeof flag, cudaMemcpyDeviceToHost));
+        ALX_CUDA(c, cudaMemcpy(&flag, dual_flag_of(c), sizeof flag, cudaMemcpyDeviceToHost));
         if (c->cg_policy) ALX_CUDA(c, cudaMemcpy(&pol, c->cg_policy + c->last_side, sizeof pol, cudaMemcpyDeviceToHost));
         if (flag) c->stats.dual_rows = c->dual_candidates - (pol.short_rows_by_cg ? c->dual_candidates32 : 0);
     }

@@ -193,7 +193,8 @@ cudaError_t launch_rows_warp(const SideView &sv, const int64_t *class_offs_host,
 // alx_rows_team.cu: fp32 tables of 128 features, four warps per row (kernels != 1); `sums`: team_sums_floats() floats
 int64_t team_sums_floats(const int64_t *class_offs_host, int64_t n_chunks);
 cudaError_t launch_rows_team(const SideView &sv, const int64_t *class_offs_host, int64_t n_chunks, int64_t n_split_rows, const float *X,
-                             const float *Bmat, float *sums, RowOut out, DevStatus *st, cudaStream_t s, int64_t *launches);
+                             const float *Bmat, float *sums, RowOut out, DevStatus *st, const int *dual_flag, cudaStream_t s,
+                             int64_t *launches);
 
 // alx_umma.cu: tensor-core path, d = 128 and bf16 tables only
 int64_t gramian_umma_partials();
@@ -236,6 +237,16 @@ int *dual64_flag_ptr(void *ws);
 cudaError_t launch_dual64_prepare(const float *Bmat, void *ws, float cond_limit, cudaStream_t s, int64_t *launches);
 cudaError_t launch_rows_dual64(const SideView &sv, int64_t first, int64_t count, const void *X, void *ws, RowOut out,
                                cudaStream_t s, int64_t *launches);
+// alx_dual_warp.cu (bfloat16 tables of 64 features, fp32 tables of 128): B^-1 as mma fragments + flag; rows of 1 .. 16
+// observations in the dual form.  Its sums truncate like every tensor-core sum, so it takes part only where B is better
+// conditioned than the other dual kernels ask for: the worst residual was 8e-5 at a product of norms of 8100 and is in proportion
+// below, so 512 (fp32 tables) keeps it at the 5e-6 of the direct solves, and 1024 at 1e-5 for results rounded to 2^-9
+constexpr float kDualWarpLimitF32 = 512.f, kDualWarpLimitBf16 = 1024.f;
+size_t dual_warp_workspace_bytes(int d);
+const int *dual_warp_flag_ptr(const void *ws, int d);
+cudaError_t launch_dual_warp_prepare(const float *Bmat, void *ws, int d, float cond_limit, cudaStream_t s, int64_t *launches);
+cudaError_t launch_rows_dual_warp(const SideView &sv, int64_t first, int64_t count, const void *X, int bf16, int d, const void *ws, RowOut out,
+                                  DevStatus *st, cudaStream_t s, int64_t *launches);
 const int *dual_flag_ptr(const void *ws);
 // route: set where conjugate gradients run; the kernel of the rows of 17 .. 32 observations returns at once when it says so.
 // order16 (may be null): the count16 rows of 1 .. 16 observations again, ordered by length class: the n4 rows of at most 4

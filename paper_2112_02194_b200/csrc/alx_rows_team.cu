@@ -8,7 +8,7 @@
 // the column steps need shuffles only; the block meets at a barrier before and after a panel.
 //
 // The FP32-ALU kernels (alx_rows.cu) gave such a row 256 threads that met at a barrier three times per 16 columns and did the
-// trailing update with FMAs from shared memory: 60k x 25k, 2e6 entries, one epoch 17.4 ms; here 4.3 ms.
+// trailing update with FMAs from shared memory: 60k x 25k, 2e6 entries, one epoch 17.4 ms; here 8.7 ms.
 // Bound: the chain of 64 double column steps and the 128 steps of the back substitution (three teams per SM hide what they can).
 #include "alx_common.cuh"
 #include "alx_mma.cuh"
@@ -40,7 +40,7 @@ struct __align__(16) TeamSmem {
         float L[kLFloats];
         unsigned char tile[kTile];
     };
-    float b[D], dinv[D];
+    float b[D], z[D], dinv[D];      // right-hand side, then the solution; L^-1 b; reciprocal pivots
     float exchange[kWarps][64];
     float part[kWarps][16];
     float y[2][kEntries];
@@ -181,7 +181,6 @@ __device__ __forceinline__ bool factor_solve(Acc &acc, TeamSmem &sm, const float
 #pragma unroll
     for (int n = 0; n < kHi; ++n)
         if (n < 2 * (ihi + 1)) add_base(acc.hi[n], Bmat, ihi, n, lane);
-    bool ok = true;
     auto put_block = [&](float *P, const float(&c)[4], int i, int n) {      // block (16 i .., 8 n ..) of the panel
         const int r = 16 * i + lane / 4, q = 2 * n + (lane % 4) / 2, o = 2 * (lane & 1);
         *reinterpret_cast<float2 *>(P + panel_chunk(r, q) + o) = make_float2(c[0], c[1]);
@@ -212,30 +211,32 @@ __device__ __forceinline__ bool factor_solve(Acc &acc, TeamSmem &sm, const float
             const float4 w = *reinterpret_cast<const float4 *>(P + panel_chunk(mine ? own : 0, c));
             a1[4 * c] = w.x; a1[4 * c + 1] = w.y; a1[4 * c + 2] = w.z; a1[4 * c + 3] = w.w;
         }
-        float b0 = sm.b[16 * k + dl], b1 = mine ? sm.b[16 * k + own] : 0.f, d = 0.f;
+        float b0 = sm.b[16 * k + dl], b1 = mine ? sm.b[16 * k + own] : 0.f;
         // (the first write to the diagonal block's rows and to b comes after the barrier below)
 #pragma unroll
         for (int j = 0; j < 16; j += 2) {
             const float p = __shfl_sync(0xFFFFFFFFu, a0[j], j), q = __shfl_sync(0xFFFFFFFFu, a0[j], j + 1);
             const float s = __shfl_sync(0xFFFFFFFFu, a0[j + 1], j + 1);
             float z0 = __shfl_sync(0xFFFFFFFFu, b0, j), z1 = __shfl_sync(0xFFFFFFFFu, b0, j + 1);
+            // (a pivot that is not positive makes its reciprocal root a NaN, and is reported for that at the end)
             const float i0 = rsqrt_full(p), l10 = q * i0, dd = fmaf(-l10, l10, s), i1 = rsqrt_full(dd);
-            ok = ok && p > 0.f && dd > 0.f;
             z0 *= i0;
             z1 = fmaf(-z0, l10, z1) * i1;
+            if (tid == 0) {
+                *reinterpret_cast<float2 *>(sm.z + 16 * k + j) = make_float2(z0, z1);
+                *reinterpret_cast<float2 *>(sm.dinv + 16 * k + j) = make_float2(i0, i1);
+            }
             const float x0 = a0[j] * i0, x1 = fmaf(-x0, l10, a0[j + 1]) * i1;
             const float y0 = a1[j] * i0, y1 = fmaf(-y0, l10, a1[j + 1]) * i1;
             a0[j] = x0;
             a0[j + 1] = x1;
             a1[j] = y0;
             a1[j + 1] = y1;
-            const float nb = fmaf(-x1, z1, fmaf(-x0, z0, b0));
-            b0 = dl > j + 1 ? nb : dl == j ? z0 : dl == j + 1 ? z1 : b0;
+            b0 = fmaf(-x1, z1, fmaf(-x0, z0, b0));      // (what it becomes in the rows up to j + 1 is not used)
             b1 = fmaf(-y1, z1, fmaf(-y0, z0, b1));
-            d = dl == j ? i0 : dl == j + 1 ? i1 : d;
             if (j < 14) {
                 float *ex = sm.exchange[warp] + 32 * ((j / 2) & 1);
-                if (lane < 16) { ex[lane] = x0; ex[16 + lane] = x1; }
+                if (lane < 16) { ex[lane] = -x0; ex[16 + lane] = -x1; }
                 __syncwarp();
 #pragma unroll
                 for (int c = (j + 2) & ~3; c < 16; c += 4) {
@@ -246,8 +247,8 @@ __device__ __forceinline__ bool factor_solve(Acc &acc, TeamSmem &sm, const float
                         if (cc < j + 2) continue;
                         const float2 uu = h ? make_float2(u.z, u.w) : make_float2(u.x, u.y), vv = h ? make_float2(v.z, v.w) : make_float2(v.x, v.y);
                         float2 t = make_float2(a0[cc], a0[cc + 1]), w = make_float2(a1[cc], a1[cc + 1]);
-                        t = __ffma2_rn(make_float2(-x1, -x1), vv, __ffma2_rn(make_float2(-x0, -x0), uu, t));
-                        w = __ffma2_rn(make_float2(-y1, -y1), vv, __ffma2_rn(make_float2(-y0, -y0), uu, w));
+                        t = __ffma2_rn(make_float2(x1, x1), vv, __ffma2_rn(make_float2(x0, x0), uu, t));
+                        w = __ffma2_rn(make_float2(y1, y1), vv, __ffma2_rn(make_float2(y0, y0), uu, w));
                         a0[cc] = t.x;
                         a0[cc + 1] = t.y;
                         a1[cc] = w.x;
@@ -261,8 +262,6 @@ __device__ __forceinline__ bool factor_solve(Acc &acc, TeamSmem &sm, const float
 #pragma unroll
             for (int c = 0; c < 4; ++c)
                 *reinterpret_cast<float4 *>(P + panel_chunk(lane, c)) = make_float4(a0[4 * c], a0[4 * c + 1], a0[4 * c + 2], a0[4 * c + 3]);
-            sm.b[16 * k + lane] = b0;
-            sm.dinv[16 * k + lane] = d;
         }
         if (mine) {
 #pragma unroll
@@ -325,28 +324,32 @@ __device__ __forceinline__ bool factor_solve(Acc &acc, TeamSmem &sm, const float
     // back substitution, panel by panel from the last: what the solved rows below take off (column c = tid % 16, every eighth
     // row a thread), then the 16 x 16 triangle by the first warp
     const int c = lane & 15;
+    int at[4];      // column c of a row r of a panel: r * 16 + at[(r / 2) % 4]
+#pragma unroll
+    for (int v = 0; v < 4; ++v) at[v] = 4 * ((c >> 2) ^ v) + (c & 3);
+    const int at_mine = 4 * ((c >> 2) ^ warp) + (c & 3);      // ... of this thread's rows 16 + 2 warp + lane / 16 (+ 8, ...)
 #pragma unroll 1
     for (int k = kBlocks - 1; k >= 0; --k) {
         const float *P = sm.L + panel_at(k);
         float s = 0.f;
 #pragma unroll 4
-        for (int r = 16 + (tid >> 4); r < D - 16 * k; r += 8) s = fmaf(P[panel_chunk(r, c >> 2) + (c & 3)], sm.b[16 * k + r], s);
+        for (int r = 16 + (tid >> 4); r < D - 16 * k; r += 8) s = fmaf(P[r * 16 + at_mine], sm.b[16 * k + r], s);
         s += __shfl_xor_sync(0xFFFFFFFFu, s, 16);
         if (lane < 16) sm.part[warp][lane] = s;
         __syncthreads();
         if (warp == 0) {
-            float x = sm.b[16 * k + c] - ((sm.part[0][c] + sm.part[1][c]) + (sm.part[2][c] + sm.part[3][c]));
+            float x = sm.z[16 * k + c] - ((sm.part[0][c] + sm.part[1][c]) + (sm.part[2][c] + sm.part[3][c]));
             const float d = sm.dinv[16 * k + c];
 #pragma unroll
             for (int j = 15; j >= 0; --j) {
                 const float xj = __shfl_sync(0xFFFFFFFFu, x * d, j);
-                x = c < j ? fmaf(-P[panel_chunk(j, c >> 2) + (c & 3)], xj, x) : c == j ? xj : x;
+                if (lane == 0) sm.b[16 * k + j] = xj;
+                x = fmaf(-P[j * 16 + at[(j >> 1) & 3]], xj, x);      // (columns from j on are done with)
             }
-            if (lane < 16) sm.b[16 * k + c] = x;
         }
         __syncthreads();
     }
-    return ok;      // (every warp has seen every pivot)
+    return !__syncthreads_or(!(sm.dinv[tid] == sm.dinv[tid]));
 }
 
 __device__ __forceinline__ void store_row(const TeamSmem &sm, bool ok, int64_t u, const RowOut &out, DevStatus *st, int tid)
@@ -364,12 +367,14 @@ __device__ __forceinline__ void store_row(const TeamSmem &sm, bool ok, int64_t u
 }
 
 // ---- whole rows: a team each, items dealt round-robin, item 0 the last of the order (the longest class)
-__global__ void __launch_bounds__(kTeam, kTeamsPerSm) k_rows_team(SideView sv, int64_t last, int64_t count, const float *__restrict__ X,
+__global__ void __launch_bounds__(kTeam, kTeamsPerSm) k_rows_team(SideView sv, int64_t last, int64_t count, const int *dual_flag,
+                                                                  int64_t primal_count, const float *__restrict__ X,
                                                                   const float *__restrict__ Bmat, RowOut out, DevStatus *st)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     TeamSmem &sm = *reinterpret_cast<TeamSmem *>(smem_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (dual_flag && *dual_flag) count = primal_count;      // the rows behind them have been solved in the dual form
     int64_t item = blockIdx.x;
     if (item >= count) return;
     Feed feed;
@@ -513,7 +518,7 @@ int64_t team_sums_floats(const int64_t *offs, int64_t n_chunks)
 }
 
 cudaError_t launch_rows_team(const SideView &sv, const int64_t *offs, int64_t n_chunks, int64_t n_split_rows, const float *X, const float *Bmat,
-                             float *sums, RowOut out, DevStatus *st, cudaStream_t s, int64_t *launches)
+                             float *sums, RowOut out, DevStatus *st, const int *dual_flag, cudaStream_t s, int64_t *launches)
 {
     const size_t smem = sizeof(TeamSmem);
     cudaError_t e;
@@ -537,7 +542,8 @@ cudaError_t launch_rows_team(const SideView &sv, const int64_t *offs, int64_t n_
     }
     const int64_t n = end - offs[1];
     if (n > 0) {
-        k_rows_team<<<(unsigned)(n < 148 * kTeamsPerSm ? n : 148 * kTeamsPerSm), kTeam, smem, s>>>(sv, end - 1, n, X, Bmat, out, st);
+        k_rows_team<<<(unsigned)(n < 148 * kTeamsPerSm ? n : 148 * kTeamsPerSm), kTeam, smem, s>>>(sv, end - 1, n, dual_flag, end - offs[2], X,
+                                                                                                           Bmat, out, st);
         ++*launches;
     }
     const int64_t n_zero = offs[1] - offs[0];

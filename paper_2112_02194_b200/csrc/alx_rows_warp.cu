@@ -212,7 +212,7 @@ __device__ __forceinline__ bool factor_solve(Sums<D, T> &acc, Sums<D, T> &acc2, 
     const int rl = D == 16 ? lane & 15 : lane;
     float *b_m = b_s + half;                       // d = 16: 16 floats a matrix
     float *dinv_m = dinv_s + half;
-    bool ok = true;
+    const bool first = rl == 0;                    // the lane that writes down what all lanes of the matrix know
     auto put_block = [&](float *P, const float(&c)[4], int i, int n) {      // block (16 i .., 8 n ..) of the panel
         const int r = 16 * i + lane / 4, q = 2 * n + (lane % 4) / 2, o = 2 * (lane & 1);
         *reinterpret_cast<float2 *>(P + panel_chunk(r, q) + o) = make_float2(c[0], c[1]);
@@ -248,23 +248,25 @@ __device__ __forceinline__ bool factor_solve(Sums<D, T> &acc, Sums<D, T> &acc2, 
                 a1[4 * c] = w.x; a1[4 * c + 1] = w.y; a1[4 * c + 2] = w.z; a1[4 * c + 3] = w.w;
             }
         }
-        float b0 = rl < rows ? b_m[16 * k + rl] : 0.f, b1 = two ? b_m[16 * k + 32 + rl] : 0.f, d = 0.f;
+        float b0 = rl < rows ? b_m[16 * k + rl] : 0.f, b1 = two ? b_m[16 * k + 32 + rl] : 0.f;
         __syncwarp();
 #pragma unroll
         for (int j = 0; j < 16; j += 2) {
             const float p = __shfl_sync(0xFFFFFFFFu, a0[j], half + j), q = __shfl_sync(0xFFFFFFFFu, a0[j], half + j + 1);
             const float s = __shfl_sync(0xFFFFFFFFu, a0[j + 1], half + j + 1);
             float z0 = __shfl_sync(0xFFFFFFFFu, b0, half + j), z1 = __shfl_sync(0xFFFFFFFFu, b0, half + j + 1);
+            // (a pivot that is not positive makes its reciprocal root a NaN, and is reported for that at the end)
             const float i0 = rsqrt_full(p), l10 = q * i0, dd = fmaf(-l10, l10, s), i1 = rsqrt_full(dd);
-            ok = ok && p > 0.f && dd > 0.f;
             z0 *= i0;
             z1 = fmaf(-z0, l10, z1) * i1;
+            if (first) {
+                *reinterpret_cast<float2 *>(b_m + 16 * k + j) = make_float2(z0, z1);
+                *reinterpret_cast<float2 *>(dinv_m + 16 * k + j) = make_float2(i0, i1);
+            }
             const float x0 = a0[j] * i0, x1 = fmaf(-x0, l10, a0[j + 1]) * i1;
             a0[j] = x0;
             a0[j + 1] = x1;
-            const float nb = fmaf(-x1, z1, fmaf(-x0, z0, b0));
-            b0 = rl > j + 1 ? nb : rl == j ? z0 : rl == j + 1 ? z1 : b0;
-            d = rl == j ? i0 : rl == j + 1 ? i1 : d;
+            b0 = fmaf(-x1, z1, fmaf(-x0, z0, b0));      // (what it becomes in the rows up to j + 1 is not used)
             float y0 = 0.f, y1 = 0.f;
             if (D == 64) {
                 y0 = a1[j] * i0;
@@ -277,7 +279,7 @@ __device__ __forceinline__ bool factor_solve(Sums<D, T> &acc, Sums<D, T> &acc2, 
                 // the two columns of the diagonal block's rows to everybody: the place of the panel's first two rows serves
                 // as the exchange (its rows are in registers)
                 float *ex = Pm + 32 * ((j / 2) & 1);
-                if (rl < 16) { ex[rl] = x0; ex[16 + rl] = x1; }
+                if (rl < 16) { ex[rl] = -x0; ex[16 + rl] = -x1; }
                 __syncwarp();
 #pragma unroll
                 for (int c = (j + 2) & ~3; c < 16; c += 4) {
@@ -288,12 +290,12 @@ __device__ __forceinline__ bool factor_solve(Sums<D, T> &acc, Sums<D, T> &acc2, 
                         if (cc < j + 2) continue;
                         const float2 uu = h ? make_float2(u.z, u.w) : make_float2(u.x, u.y), vv = h ? make_float2(v.z, v.w) : make_float2(v.x, v.y);
                         float2 t = make_float2(a0[cc], a0[cc + 1]);
-                        t = __ffma2_rn(make_float2(-x1, -x1), vv, __ffma2_rn(make_float2(-x0, -x0), uu, t));
+                        t = __ffma2_rn(make_float2(x1, x1), vv, __ffma2_rn(make_float2(x0, x0), uu, t));
                         a0[cc] = t.x;
                         a0[cc + 1] = t.y;
                         if (D == 64) {
                             float2 w = make_float2(a1[cc], a1[cc + 1]);
-                            w = __ffma2_rn(make_float2(-y1, -y1), vv, __ffma2_rn(make_float2(-y0, -y0), uu, w));
+                            w = __ffma2_rn(make_float2(y1, y1), vv, __ffma2_rn(make_float2(y0, y0), uu, w));
                             a1[cc] = w.x;
                             a1[cc + 1] = w.y;
                         }
@@ -302,15 +304,14 @@ __device__ __forceinline__ bool factor_solve(Sums<D, T> &acc, Sums<D, T> &acc2, 
             }
         }
         __syncwarp();
-        // L's rows back, the right-hand side, the reciprocal pivots
+        // L's rows back, and the right-hand side of the rows below the diagonal block
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
             if (rl < rows) *reinterpret_cast<float4 *>(Pm + panel_chunk(rl, c)) = make_float4(a0[4 * c], a0[4 * c + 1], a0[4 * c + 2], a0[4 * c + 3]);
             if (two) *reinterpret_cast<float4 *>(Pm + panel_chunk(rl + 32, c)) = make_float4(a1[4 * c], a1[4 * c + 1], a1[4 * c + 2], a1[4 * c + 3]);
         }
-        if (rl < rows) b_m[16 * k + rl] = b0;
+        if (rl >= 16 && rl < rows) b_m[16 * k + rl] = b0;
         if (two) b_m[16 * k + 32 + rl] = b1;
-        if (rl < 16) dinv_m[16 * k + rl] = d;
         if (D > 16 && k + 1 < MB) {
             // the rows below the diagonal block as bfloat16 parts, [part][row][16 columns]: 32-byte rows, the two 16-byte
             // chunks exchanged in every other group of four rows (ldmatrix without conflicts)
@@ -367,28 +368,36 @@ __device__ __forceinline__ bool factor_solve(Sums<D, T> &acc, Sums<D, T> &acc2, 
     // back substitution, panel by panel from the last: what the solved rows below take off (lanes: column c, rows of one
     // parity), then the 16 x 16 triangle
     const int c = lane & 15;
+    int at[4];      // column c of a row r of a panel: r * 16 + at[(r / 2) % 4]
+#pragma unroll
+    for (int v = 0; v < 4; ++v) at[v] = 4 * ((c >> 2) ^ v) + (c & 3);
+    bool bad = false;
 #pragma unroll 1
     for (int k = MB - 1; k >= 0; --k) {
         const float *Pm = D == 16 ? L + (half ? G::L_FLOATS : 0) : L + G::panel_at(k);
         float s = 0.f;
         if (D > 16) {
-#pragma unroll 4
-            for (int r = 16 + (lane >> 4); r < D - 16 * k; r += 2) s = fmaf(Pm[panel_chunk(r, c >> 2) + (c & 3)], b_s[16 * k + r], s);
+            const float *row = Pm + (16 + (lane >> 4)) * 16, *xs = b_s + 16 * k + 16 + (lane >> 4);
+#pragma unroll 1
+            for (int r = 16; r < D - 16 * k; r += 8, row += 128, xs += 8)
+#pragma unroll
+                for (int v = 0; v < 4; ++v) s = fmaf(row[32 * v + at[v]], xs[2 * v], s);
             s += __shfl_xor_sync(0xFFFFFFFFu, s, 16);
         }
         float x = b_m[16 * k + c] - s;
         const float d = dinv_m[16 * k + c];
+        bad |= !(d == d);
+        __syncwarp();
 #pragma unroll
         for (int j = 15; j >= 0; --j) {
             const float xj = __shfl_sync(0xFFFFFFFFu, x * d, half + j);
-            x = c < j ? fmaf(-Pm[panel_chunk(j, c >> 2) + (c & 3)], xj, x) : c == j ? xj : x;
+            if (first) b_m[16 * k + j] = xj;
+            x = fmaf(-Pm[j * 16 + at[(j >> 1) & 3]], xj, x);      // (columns from j on are done with)
         }
         __syncwarp();
-        if (D == 16 || lane < 16) b_m[16 * k + c] = x;
-        __syncwarp();
     }
-    const unsigned bad = __ballot_sync(0xFFFFFFFFu, !ok);
-    return D == 16 ? (bad >> half & 0xFFFFu) == 0 : bad == 0;
+    const unsigned who = __ballot_sync(0xFFFFFFFFu, bad);
+    return D == 16 ? (who >> half & 0xFFFFu) == 0 : who == 0;
 }
 
 template <int D, typename T> __device__ __forceinline__ void put_b(const Sums<D, T> &acc, float *b_s, int lane)
