@@ -52,6 +52,7 @@ struct alx_ctx {
     int64_t n4[2] = {0, 0}, n8[2] = {0, 0};      // ... and those with at most 4 before them
 
     void *table[2] = {nullptr, nullptr};
+    void *parts = nullptr;        // fp32 tables of 64 features: bfloat16 parts of the fixed table, [larger side][3][64], rewritten every half-epoch
     double *G64[2] = {nullptr, nullptr};   // Gramian of table [side]
     float *Bmat = nullptr;
     float *gram_partials = nullptr;
@@ -422,7 +423,9 @@ int64_t sums_floats(const alx_ctx *c, int side)
     const int64_t *offs = c->class_offs[side];
     const int64_t d = c->opt.d;
     if (team_path(c)) return team_sums_floats(offs, c->n_chunks[side]);
-    return (c->n_chunks[side] + (tensor_path(c) ? offs[kNClasses - 1] - offs[long_class_begin(offs)] : 0)) * (d * d + d);
+    const int64_t n_long = tensor_path(c) ? offs[kNClasses - 1] - offs[long_class_begin(offs)]
+                           : cg64(c)      ? offs[kNClasses - 1] - offs[parts64_long_class(offs)] : 0;
+    return (c->n_chunks[side] + n_long) * (d * d + d);
 }
 
 // rows of a side that the dual form is offered (class 1, and class 2 for d = 128); 0: none, or too few
@@ -485,7 +488,7 @@ alx_status half_epoch_impl(alx_ctx *c, int side, const int32_t *cap_slot, float 
                                                           c->opt.d, c->dual_ws, out, c->status, c->stream, &c->launches));
         ALX_CUDA(c, cudaEventRecord(c->ev[3], c->stream));
         ALX_CUDA(c, launch_rows_warp(side_view(c, side), c->class_offs[side], c->n_chunks[side], c->n_split_rows[side], c->table[fixed],
-                                     c->bf16, c->opt.d, c->Bmat, c->split_partials, out, c->status, cg_options(c, side),
+                                     c->n[fixed], c->parts, c->bf16, c->opt.d, c->Bmat, c->split_partials, out, c->status, cg_options(c, side),
                                      n_dual > 0 ? dual_flag_of(c) : nullptr, c->stream, &c->launches));
         ALX_CUDA(c, cudaEventRecord(c->ev[4], c->stream));
         c->stats.kernel_path[side] = 1;
@@ -594,6 +597,10 @@ alx_status create_impl(const alx_options *opt, const alx_ctx *parent, alx_ctx **
             if (!c->dual_ws) return fail(c, ALX_ERR_OOM, "device allocation of the dual-form workspace failed");
         }
         const int64_t nmax = c->n[0] > c->n[1] ? c->n[0] : c->n[1];
+        if (cg64(c)) {
+            c->parts = parent ? parent->parts : dev_alloc(c, (size_t)nmax * 384);
+            if (!c->parts) return fail(c, ALX_ERR_OOM, "device allocation of the table of bfloat16 parts failed");
+        }
         int64_t n_part = gramian_partials(nmax);
         if (gramian_umma_partials() > n_part) n_part = gramian_umma_partials();
         ALX_ALLOC(c, c->gram_partials, n_part * d * d);
@@ -757,7 +764,7 @@ alx_status alx_set_csr(alx_ctx *c, const int64_t *rowptr, const int32_t *colidx,
         ALX_TMP(c, tmp, total, 2);
         for (int s = 0; s < 2; ++s) {
             const int64_t *offs = c->class_offs[s];
-            const int64_t first = offs[tensor_path(c) ? long_class_begin(offs) : warp_long_class(offs)];
+            const int64_t first = offs[tensor_path(c) ? long_class_begin(offs) : cg64(c) ? parts64_long_class(offs) : warp_long_class(offs)];
             const int64_t n_long = offs[kNClasses - 1] - first;
             c->stats.long_rows[s] = n_long;
             ALX_CUDA(c, launch_sum_row_lengths(c->ptr[s], c->order[s] + first, n_long, total + s, c->stream, &c->launches));

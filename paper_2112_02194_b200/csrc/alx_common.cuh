@@ -184,11 +184,20 @@ struct CgOptions {
 // for as many) where there are so many rows that every warp has several anyway, else more than 256, so that a few longer
 // rows do not outlast the others.
 inline int warp_long_class(const int64_t *class_offs_host) { return class_offs_host[8] - class_offs_host[1] >= 148 * 20 * 8 ? 8 : 6; }
+// ... and for fp32 tables of 64 features, where a long row's sums take a place in the workspace: more than 512 entries (256 where rows
+// are few), as long as those rows are at most kLongRowBudget
+inline int parts64_long_class(const int64_t *class_offs_host)
+{
+    int c = class_offs_host[7] - class_offs_host[1] >= 148 * 12 * 8 ? 7 : 6;
+    while (c < kNClasses - 1 && class_offs_host[kNClasses - 1] - class_offs_host[c] > kLongRowBudget) ++c;
+    return c;
+}
 // alx_rows_warp.cu: d = 16, 32, 64, a warp per row (kernels != 1); conjugate gradients for fp32 tables of 64 features where
-// cg.enabled.  dual_flag (may be null): device flag, set when the rows of class 1 have been solved in the dual form
+// cg.enabled, over the table's bfloat16 parts (n_table rows of 384 bytes, rewritten by the call).  dual_flag (may be null): device
+// flag, set when the rows of class 1 have been solved in the dual form
 cudaError_t launch_rows_warp(const SideView &sv, const int64_t *class_offs_host, int64_t n_chunks, int64_t n_split_rows, const void *X,
-                             int bf16, int d, const float *Bmat, float *split_partials, RowOut out, DevStatus *st, const CgOptions &cg,
-                             const int *dual_flag, cudaStream_t s, int64_t *launches);
+                             int64_t n_table, void *parts, int bf16, int d, const float *Bmat, float *split_partials, RowOut out, DevStatus *st,
+                             const CgOptions &cg, const int *dual_flag, cudaStream_t s, int64_t *launches);
 
 // alx_rows_team.cu: fp32 tables of 128 features, four warps per row (kernels != 1); `sums`: team_sums_floats() floats
 int64_t team_sums_floats(const int64_t *class_offs_host, int64_t n_chunks);

@@ -106,6 +106,24 @@ struct Feed {
     __device__ __forceinline__ void start_copies(TeamSmem &sm, int warp, int lane) { issue(sm, g, id_first, y_first, warp, lane); }
 };
 
+// c0, c1 (two blocks of 8 columns) += or -= A B^T, the six products of the parts from the smallest up
+template <bool SUB>
+__device__ __forceinline__ void add_products(float (&c0)[4], float (&c1)[4], const uint32_t (&a)[3][4], const uint32_t (&b)[3][4])
+{
+    constexpr int pa[6] = {2, 0, 1, 1, 0, 0}, pb[6] = {0, 2, 1, 0, 1, 0};
+    float t0[4] = {0.f, 0.f, 0.f, 0.f}, t1[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+        mma_bf16(t0, a[pa[q]], b[pb[q]][0], b[pb[q]][2]);
+        mma_bf16(t1, a[pa[q]], b[pb[q]][1], b[pb[q]][3]);
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        c0[e] += SUB ? -t0[e] : t0[e];
+        c1[e] += SUB ? -t1[e] : t1[e];
+    }
+}
+
 // sums over `len` entries of the row that the feed was started on; b: this thread's feature of the right-hand side
 __device__ __forceinline__ void sum_entries(Feed &feed, int64_t len, TeamSmem &sm, Acc &acc, float &b, int warp, int lane)
 {
@@ -145,20 +163,15 @@ __device__ __forceinline__ void sum_entries(Feed &feed, int64_t len, TeamSmem &s
             ldmatrix_x4_trans(src + q * kEntries * kRow + 32 * ilo, al[q]);
             ldmatrix_x4_trans(src + q * kEntries * kRow + 32 * ihi, ah[q]);
         }
-        constexpr int pa[6] = {2, 0, 1, 1, 0, 0}, pb[6] = {0, 2, 1, 0, 1, 0};      // the parts' products from the smallest up
 #pragma unroll
         for (int j = 0; j < kBlocks; ++j) {
             if (j > ihi) break;
             uint32_t bf[3][4];
 #pragma unroll
             for (int q = 0; q < 3; ++q) ldmatrix_x4_trans(src + q * kEntries * kRow + 32 * j, bf[q]);
-#pragma unroll
-            for (int q = 0; q < 6; ++q)
-#pragma unroll
-                for (int n = 0; n < 2; ++n) {
-                    mma_bf16(acc.hi[2 * j + n], ah[pa[q]], bf[pb[q]][n], bf[pb[q]][2 + n]);
-                    if (j < kLo / 2 && j <= ilo) mma_bf16(acc.lo[2 * (j < kLo / 2 ? j : 0) + n], al[pa[q]], bf[pb[q]][n], bf[pb[q]][2 + n]);
-                }
+            // (from zero in every stage, the sums by FADD: the accumulator of an mma truncates)
+            add_products<false>(acc.hi[2 * j], acc.hi[2 * j + 1], ah, bf);
+            if (j < kLo / 2 && j <= ilo) add_products<false>(acc.lo[2 * (j < kLo / 2 ? j : 0)], acc.lo[2 * (j < kLo / 2 ? j : 0) + 1], al, bf);
         }
     }
 }
@@ -289,18 +302,12 @@ __device__ __forceinline__ bool factor_solve(Acc &acc, TeamSmem &sm, const float
             // trailing update of the warp's blocks (i, n), i > k, n >= 2 (k + 1)
             const int lr = (lane & 7) + 8 * ((lane >> 3) & 1);
             const uint32_t src = ptx::smem_u32(tile) + lr * 32 + 16 * ((lane >> 4) ^ ((lr >> 2) & 1));
-            constexpr int pa[6] = {2, 0, 1, 1, 0, 0}, pb[6] = {0, 2, 1, 0, 1, 0};
             if (ihi > k) {
                 uint32_t al[3][4], ah[3][4];
 #pragma unroll
                 for (int q = 0; q < 3; ++q) {
                     ldmatrix_x4(src + (q * below + 16 * (ihi - k - 1)) * 32, ah[q]);
                     if (ilo > k) ldmatrix_x4(src + (q * below + 16 * (ilo - k - 1)) * 32, al[q]);
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        ah[q][e] ^= 0x80008000u;
-                        al[q][e] ^= 0x80008000u;
-                    }
                 }
 #pragma unroll
                 for (int j = 1; j < kBlocks; ++j) {
@@ -308,13 +315,8 @@ __device__ __forceinline__ bool factor_solve(Acc &acc, TeamSmem &sm, const float
                     uint32_t bf[3][4];
 #pragma unroll
                     for (int q = 0; q < 3; ++q) ldmatrix_x4(src + (q * below + 16 * (j - k - 1)) * 32, bf[q]);
-#pragma unroll
-                    for (int q = 0; q < 6; ++q)
-#pragma unroll
-                        for (int n = 0; n < 2; ++n) {
-                            mma_bf16(acc.hi[2 * j + n], ah[pa[q]], bf[pb[q]][n], bf[pb[q]][2 + n]);
-                            if (j < kLo / 2 && j <= ilo) mma_bf16(acc.lo[2 * (j < kLo / 2 ? j : 0) + n], al[pa[q]], bf[pb[q]][n], bf[pb[q]][2 + n]);
-                        }
+                    add_products<true>(acc.hi[2 * j], acc.hi[2 * j + 1], ah, bf);
+                    if (j < kLo / 2 && j <= ilo) add_products<true>(acc.lo[2 * (j < kLo / 2 ? j : 0)], acc.lo[2 * (j < kLo / 2 ? j : 0) + 1], al, bf);
                 }
             }
             __syncthreads();      // the parts have been read: the next panel takes their place

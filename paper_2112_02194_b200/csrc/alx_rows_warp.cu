@@ -174,18 +174,26 @@ __device__ __forceinline__ void sum_entries(Feed<D, T> &feed, int64_t len, unsig
         for (int p = 0; p < G::PARTS; ++p)
 #pragma unroll
             for (int i = 0; i < G::MB; ++i) ldmatrix_x4_trans(src + p * kEntries * G::ROW + 32 * i, a[p][i]);
-        // the parts' products from the smallest up
+        // the parts' products from the smallest up, each stage's from zero: the accumulator of an mma truncates, and adding up a
+        // whole row in it biases long rows by 1e-5 (the final sums are ordinary FADDs)
         constexpr int kPairs = G::kF32 ? 6 : 1;
         constexpr int pa[6] = {G::kF32 ? 2 : 0, 0, 1, 1, 0, 0}, pb[6] = {0, G::kF32 ? 2 : 0, 1, 0, 1, 0};
 #pragma unroll
-        for (int q = 0; q < kPairs; ++q)
+        for (int i = 0; i < G::MB; ++i)
 #pragma unroll
-            for (int i = 0; i < G::MB; ++i)
+            for (int j = 0; j <= i; ++j) {
+                float t[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
 #pragma unroll
-                for (int n = 0; n < 2 * (i + 1); ++n) {
-                    const uint32_t(&bf)[4] = a[G::kF32 ? pb[q] : 0][n / 2];
-                    mma_bf16(acc.c[i * (i + 1) + n], a[G::kF32 ? pa[q] : 0][i], bf[n % 2], bf[2 + n % 2]);
+                for (int q = 0; q < kPairs; ++q) {
+                    const uint32_t(&bf)[4] = a[G::kF32 ? pb[q] : 0][j];
+                    mma_bf16(t[0], a[G::kF32 ? pa[q] : 0][i], bf[0], bf[2]);
+                    mma_bf16(t[1], a[G::kF32 ? pa[q] : 0][i], bf[1], bf[3]);
                 }
+#pragma unroll
+                for (int n = 0; n < 2; ++n)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) acc.c[i * (i + 1) + 2 * j + n][e] += t[n][e];
+            }
         __syncwarp();      // the slot and the parts may be overwritten
         ++feed.g;
     }
@@ -353,13 +361,17 @@ __device__ __forceinline__ bool factor_solve(Sums<D, T> &acc, Sums<D, T> &acc2, 
 #pragma unroll
                     for (int i = kk + 1; i < MB; ++i)
 #pragma unroll
-                        for (int q = 0; q < 6; ++q) {
-                            uint32_t neg[4];
+                        for (int j = kk + 1; j <= i; ++j) {
+                            float t[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) neg[e] = f[pa[q]][i][e] ^ 0x80008000u;
+                            for (int q = 0; q < 6; ++q) {
+                                mma_bf16(t[0], f[pa[q]][i], f[pb[q]][j][0], f[pb[q]][j][2]);
+                                mma_bf16(t[1], f[pa[q]][i], f[pb[q]][j][1], f[pb[q]][j][3]);
+                            }
 #pragma unroll
-                            for (int n = 2 * (kk + 1); n < 2 * (i + 1); ++n)
-                                mma_bf16(acc.c[i * (i + 1) + n], neg, f[pb[q]][n / 2][n % 2], f[pb[q]][n / 2][2 + n % 2]);
+                            for (int n = 0; n < 2; ++n)
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) acc.c[i * (i + 1) + 2 * j + n][e] -= t[n][e];
                         }
                 }
         }
@@ -593,10 +605,10 @@ template <int D, typename T> __device__ __forceinline__ void load_base(const flo
 // are of all lengths); item 0 is the last of the order, i.e. of the longest class
 // `primal_count`, where *dual_flag is set: the items before the rows that the dual form has solved.  `list`: the rows to solve
 // instead of the order's, *list_count of them (negative entries are skipped).
-template <int D, typename T, bool CG>
+template <int D, typename T>
 __global__ void __launch_bounds__(WGeo<D, T>::REGS_WARPS * 32, 1)
 k_rows_warp(SideView sv, int64_t last, int64_t count, const int *dual_flag, int64_t primal_count, const int32_t *list,
-            const unsigned long long *list_count, const T *__restrict__ X, const float *__restrict__ Bmat, RowOut out, WarpCg cg, DevStatus *st)
+            const unsigned long long *list_count, const T *__restrict__ X, const float *__restrict__ Bmat, RowOut out, DevStatus *st)
 {
     using G = WGeo<D, T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -610,7 +622,6 @@ k_rows_warp(SideView sv, int64_t last, int64_t count, const int *dual_flag, int6
     load_base<D, T>(Bmat, base);
     __syncthreads();
     const int64_t warps = (int64_t)gridDim.x * G::REGS_WARPS;
-    unsigned cg_rows = 0, cg_products = 0;
     auto row_at = [&](int64_t k) -> int64_t { return list ? list[k] : sv.order[last - k]; };
     int64_t item = ((int64_t)warp * gridDim.x + blockIdx.x) * G::ROWS;
     if (item >= count) return;
@@ -650,31 +661,12 @@ k_rows_warp(SideView sv, int64_t last, int64_t count, const int *dual_flag, int6
         // the next row's first entries travel while this one is solved
         if (more) feed.start_ids(bn, en, lane);
         add_base<D, T>(acc, base, lane);
-        if constexpr (CG) {
-            const float b0 = b_s[lane], b1 = b_s[lane + 32];
-            const float *stored = reinterpret_cast<const float *>(out.table) + u * D;
-            float x0 = cg.warm ? stored[lane] : 0.f, x1 = cg.warm ? stored[lane + 32] : 0.f;
-            float a0[64], a1[64];
-            symmetric_rows(acc, reinterpret_cast<float *>(work), a0, a1, lane);
-            if (more) feed.start_copies(lane);
-            int products = 0;
-            const bool ok = conjugate_gradients(cg, a0, a1, b_s, b0, b1, x0, x1, products, lane);
-            ++cg_rows;
-            cg_products += products;
-            __syncwarp();
-            b_s[lane] = x0;
-            b_s[lane + 32] = x1;
-            __syncwarp();
-            if (ok) store_row<D, T>(b_s, true, u, out, st, lane);
-            else if (lane == 0) cg.fallback_list[atomicAdd(&cg.counters[2], 1ull)] = (int32_t)u;
-        } else {
-            if (more) feed.start_copies(lane);
-            const bool ok = factor_solve<D, T>(acc, acc2, reinterpret_cast<float *>(work), b_s, lane);
-            if (D != 16 || lane < 16) {
-                if (u >= 0) store_row<D, T>(b_s, ok, u, out, st, lane);
-            } else if (u_pair >= 0) {
-                store_row<D, T>(b_s + D, ok, u_pair, out, st, lane);
-            }
+        if (more) feed.start_copies(lane);
+        const bool ok = factor_solve<D, T>(acc, acc2, reinterpret_cast<float *>(work), b_s, lane);
+        if (D != 16 || lane < 16) {
+            if (u >= 0) store_row<D, T>(b_s, ok, u, out, st, lane);
+        } else if (u_pair >= 0) {
+            store_row<D, T>(b_s + D, ok, u_pair, out, st, lane);
         }
         if (!more) break;
         __syncwarp();
@@ -683,10 +675,6 @@ k_rows_warp(SideView sv, int64_t last, int64_t count, const int *dual_flag, int6
         un = ua;
         beg = bn;
         end = en;
-    }
-    if (CG && lane == 0) {
-        atomicAdd(&cg.counters[0], (unsigned long long)cg_rows);
-        atomicAdd(&cg.counters[1], (unsigned long long)cg_products);
     }
 }
 
@@ -753,10 +741,10 @@ __device__ __forceinline__ void solve_sums(const float *sums, const float4 *base
     if (D != 16 || lane < 16) store_row<D, T>(b_s, ok, u, out, st, lane);
 }
 
-template <int D, typename T, bool CHUNK, bool CG>
+template <int D, typename T, bool CHUNK>
 __global__ void __launch_bounds__(BGeo<D, T>::kBlockWarps * 32, BGeo<D, T>::kBlocks)
 k_rows_block(SideView sv, int64_t last, const T *__restrict__ X, const float *__restrict__ Bmat, float *__restrict__ partials, RowOut out,
-             WarpCg cg, DevStatus *st)
+             DevStatus *st)
 {
     using G = WGeo<D, T>;
     using B = BGeo<D, T>;
@@ -809,13 +797,15 @@ k_rows_block(SideView sv, int64_t last, const T *__restrict__ X, const float *__
     }
     if (CHUNK) return;
     __syncthreads();
-    if (warp == 0) solve_sums<D, T, CG>(red, base, work, u, out, cg, st, lane);
+    if (warp == 0) solve_sums<D, T, false>(red, base, work, u, out, WarpCg{}, st, lane);
 }
 
-// one warp per split row: its chunks' sums in ascending order, then the solve
+// one warp per row whose sums are in the workspace: split rows first (their chunks' sums are added in ascending order), then
+// n_long whole rows of one sum each, behind the n_chunks of the others
 template <int D, typename T, bool CG>
-__global__ void __launch_bounds__(32) k_split_solve_warp(SideView sv, int64_t split_begin, const float *__restrict__ partials,
-                                                         const float *__restrict__ Bmat, RowOut out, WarpCg cg, DevStatus *st)
+__global__ void __launch_bounds__(32) k_solve_sums_warp(SideView sv, int64_t split_begin, int64_t n_split, int64_t n_chunks,
+                                                        const float *__restrict__ partials, const float *__restrict__ Bmat, RowOut out,
+                                                        WarpCg cg, DevStatus *st)
 {
     using G = WGeo<D, T>;
     using B = BGeo<D, T>;
@@ -825,8 +815,9 @@ __global__ void __launch_bounds__(32) k_split_solve_warp(SideView sv, int64_t sp
     float *sums = reinterpret_cast<float *>(smem_raw + G::BASE + G::WORK);
     const int lane = threadIdx.x;
     load_base<D, T>(Bmat, base);
-    const int64_t u = sv.order[split_begin + blockIdx.x];
-    const int64_t c0 = sv.split_first[blockIdx.x], c1 = sv.split_first[blockIdx.x + 1];
+    const int64_t k = blockIdx.x, whole = k - n_split;      // whole rows: from the end of their classes, as k_sums64 takes them
+    const int64_t u = sv.order[whole < 0 ? split_begin + k : split_begin - 1 - whole];
+    const int64_t c0 = whole < 0 ? sv.split_first[k] : n_chunks + whole, c1 = whole < 0 ? sv.split_first[k + 1] : c0 + 1;
     for (int e = 4 * lane; e < B::SUMS; e += 128) {
         float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
         for (int64_t c = c0; c < c1; ++c) {
@@ -837,6 +828,384 @@ __global__ void __launch_bounds__(32) k_split_solve_warp(SideView sv, int64_t sp
     }
     __syncwarp();
     solve_sums<D, T, CG>(sums, base, work, u, out, cg, st, lane);
+}
+
+// ---- fp32 tables of 64 features over a table of their bfloat16 parts: [row][x1 | x2 | x3][64], x = x1 + x2 + x3 to 2^-24, written once
+// per half-epoch, so that a gathered row is an mma operand as it lands (converting every gathered entry was a third of the
+// instructions of the sums).  The right-hand side is a product too, with the labels' three parts as columns.
+__global__ void __launch_bounds__(256) k_parts64(const float *__restrict__ X, int64_t n, uint32_t *__restrict__ P)
+{
+    const int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x;      // four features of a row
+    if (e >= n * 16) return;
+    const float4 x = reinterpret_cast<const float4 *>(X)[e];
+    uint32_t p[3][2];
+    split_bf16(x.x, x.y, p[0][0], p[1][0], p[2][0]);
+    split_bf16(x.z, x.w, p[0][1], p[1][1], p[2][1]);
+    uint32_t *row = P + (e / 16) * 96 + 2 * (e % 16);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) *reinterpret_cast<uint2 *>(row + 32 * q) = make_uint2(p[q][0], p[q][1]);
+}
+
+struct PGeo {
+    using G = WGeo<64, float>;
+    static constexpr int ROW = 144;                       // bytes between the rows of a staged part
+    static constexpr int PART = kEntries * ROW, STAGE = 3 * PART;
+    static constexpr int PIECES = 24;                     // 16-byte pieces of a table row
+    static constexpr int WARPS = 12;                      // per SM: registers
+    static constexpr int WARP = 2 * STAGE + 512;          // ring, vector, right-hand side
+    static constexpr int SUMS = G::NB * 128 + 64;
+    static constexpr int RING = 4;                        // stages of the long-row kernel
+};
+static_assert(PGeo::G::BASE + PGeo::WARPS * PGeo::WARP <= 232448 && 32 * 36 * 4 <= PGeo::STAGE, "shared memory");
+
+// labels of a stage as an mma B operand: column 0, 1, 2 = their bfloat16 parts; y0 .. y3 = labels of entries 2 q, 2 q + 1, 2 q + 8,
+// 2 q + 9, q = lane % 4
+__device__ __forceinline__ void label_operand(float y0, float y1, float y2, float y3, uint32_t &b0, uint32_t &b1, int lane)
+{
+    uint32_t p[2][3];
+    split_bf16(y0, y1, p[0][0], p[0][1], p[0][2]);
+    split_bf16(y2, y3, p[1][0], p[1][1], p[1][2]);
+    const int n = lane >> 2;
+    b0 = n == 0 ? p[0][0] : n == 1 ? p[0][1] : n == 2 ? p[0][2] : 0u;
+    b1 = n == 0 ? p[1][0] : n == 1 ? p[1][1] : n == 2 ? p[1][2] : 0u;
+}
+
+// Whole rows by a warp each: conjugate gradients, the matrix in registers.
+struct PartsFeed {
+    const uint4 *P;
+    const int32_t *idx;
+    const float *val;
+    uint32_t ring;
+    int g;                          // next stage to be consumed; stage g lives in slot g % 2
+    int64_t at, end;
+    int id, id_first;               // (lane < 16) ids of the stage after the one in flight; of a row's first stage
+    float y, y_next;                // labels of the stage in flight, of the one after it
+
+    __device__ __forceinline__ void load_ids(int lane)
+    {
+        id = -1;
+        y_next = 0.f;
+        if (lane < kEntries && at + lane < end) {
+            id = __ldg(idx + at + lane);
+            y_next = val ? __ldg(val + at + lane) : 1.f;
+        }
+        at += kEntries;
+    }
+    __device__ __forceinline__ void issue(int slot, int ids, int lane)
+    {
+        const uint32_t dst = ring + (uint32_t)slot * PGeo::STAGE;
+#pragma unroll
+        for (int k = 0; k < kEntries * PGeo::PIECES / 32; ++k) {
+            const int p = lane + 32 * k, r = p / PGeo::PIECES, c = p % PGeo::PIECES;
+            const int row = __shfl_sync(0xFFFFFFFFu, ids, r);
+            cp_async16_zfill(dst + (c / 8) * PGeo::PART + r * PGeo::ROW + (c % 8) * 16, P + (int64_t)(row < 0 ? 0 : row) * PGeo::PIECES + c, row >= 0);
+        }
+        ptx::cp_async_commit();
+    }
+    __device__ __forceinline__ void start_ids(int64_t beg, int64_t e, int lane)
+    {
+        at = beg;
+        end = e;
+        load_ids(lane);
+        y = y_next;
+        id_first = id;
+        load_ids(lane);
+    }
+    __device__ __forceinline__ void start_copies(int lane) { issue(g & 1, id_first, lane); }
+};
+
+__device__ __forceinline__ void sum_parts(PartsFeed &feed, int64_t len, Sums<64, float> &acc, float *b_s, int lane)
+{
+    const int stages = (int)((len + kEntries - 1) / kEntries);
+    float bacc[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) bacc[i][e] = 0.f;
+    const uint32_t lane_at = ((lane & 7) + 8 * (lane >> 4)) * PGeo::ROW + 16 * ((lane >> 3) & 1);
+#pragma unroll 1
+    for (int s = 0; s < stages; ++s) {
+        const float y = feed.y;
+        if (s + 1 < stages) {
+            feed.y = feed.y_next;
+            feed.issue((feed.g + 1) & 1, feed.id, lane);
+            feed.load_ids(lane);
+            ptx::cp_async_wait<1>();
+        } else {
+            ptx::cp_async_wait<0>();
+        }
+        __syncwarp();
+        uint32_t yb0 = lane < 4 ? 0x3F803F80u : 0u, yb1 = yb0;      // (labels of 1; entries past the end are zeros)
+        if (feed.val) {
+            const int q = 2 * (lane & 3);
+            label_operand(__shfl_sync(0xFFFFFFFFu, y, q), __shfl_sync(0xFFFFFFFFu, y, q + 1), __shfl_sync(0xFFFFFFFFu, y, q + 8),
+                          __shfl_sync(0xFFFFFFFFu, y, q + 9), yb0, yb1, lane);
+        }
+        const uint32_t src = feed.ring + (feed.g & 1) * PGeo::STAGE + lane_at;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            uint32_t a[3][4];
+#pragma unroll
+            for (int p = 0; p < 3; ++p) ldmatrix_x4_trans(src + p * PGeo::PART + 32 * i, a[p]);
+            float tb[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int p = 2; p >= 0; --p) mma_bf16(tb, a[p], yb0, yb1);
+            // the parts' products from the smallest up, each stage's from zero: the accumulator of an mma truncates.  (The other
+            // operand is loaded again for every block: four blocks' fragments at once do not fit the registers.)
+            constexpr int pa[6] = {2, 0, 1, 1, 0, 0}, pb[6] = {0, 2, 1, 0, 1, 0};
+#pragma unroll
+            for (int j = 0; j <= i; ++j) {
+                uint32_t b[3][4];
+#pragma unroll
+                for (int p = 0; p < 3; ++p) ldmatrix_x4_trans(src + p * PGeo::PART + 32 * j, b[p]);
+                float t[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+#pragma unroll
+                for (int q = 0; q < 6; ++q) {
+                    mma_bf16(t[0], a[pa[q]], b[pb[q]][0], b[pb[q]][2]);
+                    mma_bf16(t[1], a[pa[q]], b[pb[q]][1], b[pb[q]][3]);
+                }
+#pragma unroll
+                for (int n = 0; n < 2; ++n)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) acc.c[i * (i + 1) + 2 * j + n][e] += t[n][e];
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) bacc[i][e] += tb[e];
+        }
+        __syncwarp();      // the slot may be overwritten
+        ++feed.g;
+    }
+    // columns 0, 1 are in the quad's first lane, 2 in its second
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float u = bacc[i][0] + bacc[i][1], v = bacc[i][2] + bacc[i][3];
+        const float u1 = __shfl_down_sync(0xFFFFFFFFu, u, 1), v1 = __shfl_down_sync(0xFFFFFFFFu, v, 1);
+        if ((lane & 3) == 0) {
+            b_s[16 * i + lane / 4] = u + u1;
+            b_s[16 * i + 8 + lane / 4] = v + v1;
+        }
+    }
+    __syncwarp();
+}
+
+__global__ void __launch_bounds__(PGeo::WARPS * 32, 1)
+k_rows_cg64(SideView sv, int64_t last, int64_t count, const int *dual_flag, int64_t primal_count, const uint4 *__restrict__ P,
+            const float *__restrict__ Bmat, RowOut out, WarpCg cg, DevStatus *st)
+{
+    using G = WGeo<64, float>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float4 *base = reinterpret_cast<float4 *>(smem_raw);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    unsigned char *mine = smem_raw + G::BASE + warp * PGeo::WARP;
+    float *vec = reinterpret_cast<float *>(mine + 2 * PGeo::STAGE), *b_s = vec + 64;
+    if (dual_flag && *dual_flag) count = primal_count;      // the rows behind them have been solved in the dual form
+    if ((int64_t)blockIdx.x >= count) return;
+    load_base<64, float>(Bmat, base);
+    __syncthreads();
+    const int64_t warps = (int64_t)gridDim.x * PGeo::WARPS;
+    unsigned rows = 0, products = 0;
+    int64_t item = (int64_t)warp * gridDim.x + blockIdx.x;
+    if (item >= count) return;
+    PartsFeed feed;
+    feed.P = P;
+    feed.idx = sv.idx;
+    feed.val = sv.val;
+    feed.ring = ptx::smem_u32(mine);
+    feed.g = 0;
+    int64_t u = sv.order[last - item];
+    int64_t len = sv.ptr[u + 1] - sv.ptr[u];
+    feed.start_ids(sv.ptr[u], sv.ptr[u + 1], lane);
+    feed.start_copies(lane);
+    // the row after this one is looked up while this one is summed: its id a row ahead, its range now
+    int64_t un = item + warps < count ? sv.order[last - item - warps] : -1;
+    while (true) {
+        const int64_t after = item + 2 * warps;
+        const int64_t bn = un < 0 ? 0 : sv.ptr[un], en = un < 0 ? 0 : sv.ptr[un + 1];
+        const int64_t ua = after < count ? sv.order[last - after] : -1;
+        const float *stored = reinterpret_cast<const float *>(out.table) + u * 64;
+        float x0 = cg.warm ? stored[lane] : 0.f, x1 = cg.warm ? stored[lane + 32] : 0.f;
+        float a0[64], a1[64];
+        {
+            Sums<64, float> acc;
+            acc.zero();
+            sum_parts(feed, len, acc, b_s, lane);
+            if (un >= 0) feed.start_ids(bn, en, lane);
+            add_base<64, float>(acc, base, lane);
+            // (through the slot that the next row's first stage will not take)
+            symmetric_rows(acc, reinterpret_cast<float *>(mine + ((feed.g + 1) & 1) * PGeo::STAGE), a0, a1, lane);
+        }
+        if (un >= 0) feed.start_copies(lane);      // they travel while this row is solved
+        int spent = 0;
+        const bool ok = conjugate_gradients(cg, a0, a1, vec, b_s[lane], b_s[lane + 32], x0, x1, spent, lane);
+        ++rows;
+        products += spent;
+        if (ok) {
+            float *row = reinterpret_cast<float *>(out.table) + u * 64;
+            row[lane] = x0;
+            row[lane + 32] = x1;
+            if (out.cap_slot) {
+                const int slot = out.cap_slot[u];
+                if (slot >= 0) {
+                    out.cap_out[(int64_t)slot * 64 + lane] = x0;
+                    out.cap_out[(int64_t)slot * 64 + 32 + lane] = x1;
+                }
+            }
+        } else if (lane == 0) {
+            cg.fallback_list[atomicAdd(&cg.counters[2], 1ull)] = (int32_t)u;
+        }
+        if (un < 0) break;
+        __syncwarp();
+        item += warps;
+        u = un;
+        un = ua;
+        len = en - bn;
+    }
+    if (lane == 0) {
+        atomicAdd(&cg.counters[0], (unsigned long long)rows);
+        atomicAdd(&cg.counters[1], (unsigned long long)products);
+    }
+}
+
+// Sums of long rows and of the chunks of split rows: a block of four warps per item.  The warps share the gathered stages and have
+// the matrix's 16 x 16 blocks among them, three (or two) each, so that every accumulator sees all of an item's entries; the large
+// products and the five small ones have accumulators of their own, and the large sums are truncated once per 16 entries.
+template <int W> struct Blocks64 {      // blocks (i, j) of warp W: (3, 0 .. 2); (2, 0 .. 2); (1, 0), (1, 1); (0, 0), (3, 3)
+    static constexpr int N = W < 2 ? 3 : 2;
+    __host__ __device__ static constexpr int i(int k) { return W < 3 ? 3 - W : 3 * k; }
+    __host__ __device__ static constexpr int j(int k) { return W < 3 ? k : 3 * k; }
+};
+
+struct Sums64 {
+    float big[3][2][4], small[3][2][4], b[4];
+};
+
+template <int W> __device__ __forceinline__ void products64(uint32_t src, uint32_t yb0, uint32_t yb1, Sums64 &acc)
+{
+    using K = Blocks64<W>;
+    uint32_t f[3][4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const bool used = W == 0 || (W == 1 && i < 3) || (W == 2 && i < 2) || (W == 3 && (i == 0 || i == 3));
+        if (used)
+#pragma unroll
+            for (int p = 0; p < 3; ++p) ldmatrix_x4_trans(src + p * PGeo::PART + 32 * i, f[p][i]);
+    }
+    constexpr int pa[5] = {2, 0, 1, 1, 0}, pb[5] = {0, 2, 1, 0, 1};
+#pragma unroll
+    for (int k = 0; k < K::N; ++k) {
+        const int i = K::i(k), j = K::j(k);
+#pragma unroll
+        for (int n = 0; n < 2; ++n) mma_bf16(acc.big[k][n], f[0][i], f[0][j][n], f[0][j][2 + n]);
+    }
+#pragma unroll
+    for (int q = 0; q < 5; ++q)
+#pragma unroll
+        for (int k = 0; k < K::N; ++k)
+#pragma unroll
+            for (int n = 0; n < 2; ++n) mma_bf16(acc.small[k][n], f[pa[q]][K::i(k)], f[pb[q]][K::j(k)][n], f[pb[q]][K::j(k)][2 + n]);
+    constexpr int ib = W == 3 ? 0 : 3 - W;      // the warp's features of the right-hand side
+#pragma unroll
+    for (int p = 2; p >= 0; --p) mma_bf16(acc.b, f[p][ib], yb0, yb1);
+}
+
+template <int W> __device__ __forceinline__ void write64(const Sums64 &acc, float *dst, int lane)
+{
+    using K = Blocks64<W>;
+#pragma unroll
+    for (int k = 0; k < K::N; ++k)
+#pragma unroll
+        for (int n = 0; n < 2; ++n) {
+            const float *x = acc.big[k][n], *y = acc.small[k][n];
+            *reinterpret_cast<float4 *>(dst + ((K::i(k) * (K::i(k) + 1) + 2 * K::j(k) + n) * 32 + lane) * 4) =
+                make_float4(x[0] + y[0], x[1] + y[1], x[2] + y[2], x[3] + y[3]);
+        }
+    const float u = acc.b[0] + acc.b[1], v = acc.b[2] + acc.b[3];
+    const float u1 = __shfl_down_sync(0xFFFFFFFFu, u, 1), v1 = __shfl_down_sync(0xFFFFFFFFu, v, 1);
+    constexpr int ib = W == 3 ? 0 : 3 - W;
+    if ((lane & 3) == 0) {
+        dst[PGeo::G::NB * 128 + 16 * ib + lane / 4] = u + u1;
+        dst[PGeo::G::NB * 128 + 16 * ib + 8 + lane / 4] = v + v1;
+    }
+}
+
+__global__ void __launch_bounds__(128, 4) k_sums64(SideView sv, int64_t n_chunks, int64_t last_long, const uint4 *__restrict__ P, float *__restrict__ sums)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ float y_s[PGeo::RING][kEntries];
+    constexpr int R = PGeo::RING;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    int64_t beg, end;
+    if ((int64_t)blockIdx.x < n_chunks) {
+        beg = sv.chunk_desc[4 * (int64_t)blockIdx.x + 1];
+        end = sv.chunk_desc[4 * (int64_t)blockIdx.x + 2];
+    } else {
+        const int64_t u = sv.order[last_long - ((int64_t)blockIdx.x - n_chunks)];
+        beg = sv.ptr[u];
+        end = sv.ptr[u + 1];
+    }
+    const int stages = (int)((end - beg + kEntries - 1) / kEntries);
+    // a thread brings three 16-byte pieces of a stage; their rows' ids are looked up two stages before
+    const int r0 = tid / PGeo::PIECES, c0 = tid % PGeo::PIECES, r1 = (tid + 128) / PGeo::PIECES, c1 = (tid + 128) % PGeo::PIECES;
+    const int r2 = (tid + 256) / PGeo::PIECES, c2 = (tid + 256) % PGeo::PIECES;
+    int id[3];
+    float y = 0.f;
+    auto load_ids = [&](int s) {
+        const int64_t at = beg + (int64_t)s * kEntries;
+        id[0] = at + r0 < end ? __ldg(sv.idx + at + r0) : -1;
+        id[1] = at + r1 < end ? __ldg(sv.idx + at + r1) : -1;
+        id[2] = at + r2 < end ? __ldg(sv.idx + at + r2) : -1;
+        if (tid < kEntries) y = at + tid < end ? (sv.val ? __ldg(sv.val + at + tid) : 1.f) : 0.f;
+    };
+    const uint32_t ring = ptx::smem_u32(smem_raw);
+    auto issue = [&](int s) {
+        const uint32_t dst = ring + (uint32_t)(s % R) * PGeo::STAGE;
+        cp_async16_zfill(dst + (c0 / 8) * PGeo::PART + r0 * PGeo::ROW + (c0 % 8) * 16, P + (int64_t)(id[0] < 0 ? 0 : id[0]) * PGeo::PIECES + c0, id[0] >= 0);
+        cp_async16_zfill(dst + (c1 / 8) * PGeo::PART + r1 * PGeo::ROW + (c1 % 8) * 16, P + (int64_t)(id[1] < 0 ? 0 : id[1]) * PGeo::PIECES + c1, id[1] >= 0);
+        cp_async16_zfill(dst + (c2 / 8) * PGeo::PART + r2 * PGeo::ROW + (c2 % 8) * 16, P + (int64_t)(id[2] < 0 ? 0 : id[2]) * PGeo::PIECES + c2, id[2] >= 0);
+        if (tid < kEntries) y_s[s % R][tid] = y;
+    };
+#pragma unroll
+    for (int s = 0; s < R - 1; ++s) {
+        if (s < stages) {
+            load_ids(s);
+            issue(s);
+        }
+        ptx::cp_async_commit();
+    }
+    if (R - 1 < stages) load_ids(R - 1);
+    Sums64 acc;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+#pragma unroll
+            for (int n = 0; n < 2; ++n) acc.big[k][n][e] = acc.small[k][n][e] = 0.f;
+        acc.b[e] = 0.f;
+    }
+    const uint32_t lane_at = ((lane & 7) + 8 * (lane >> 4)) * PGeo::ROW + 16 * ((lane >> 3) & 1);
+#pragma unroll 1
+    for (int s = 0; s < stages; ++s) {
+        ptx::cp_async_wait<R - 2>();
+        __syncthreads();      // the stage is here for all, and the slot of the one before it is free
+        if (s + R - 1 < stages) {
+            issue(s + R - 1);
+            if (s + R < stages) load_ids(s + R);
+        }
+        ptx::cp_async_commit();
+        uint32_t yb0, yb1;
+        const float *ys = y_s[s % R] + 2 * (lane & 3);
+        label_operand(ys[0], ys[1], ys[8], ys[9], yb0, yb1, lane);
+        const uint32_t src = ring + (uint32_t)(s % R) * PGeo::STAGE + lane_at;
+        if (warp == 0) products64<0>(src, yb0, yb1, acc);
+        else if (warp == 1) products64<1>(src, yb0, yb1, acc);
+        else if (warp == 2) products64<2>(src, yb0, yb1, acc);
+        else products64<3>(src, yb0, yb1, acc);
+    }
+    float *dst = sums + (int64_t)blockIdx.x * PGeo::SUMS;
+    if (warp == 0) write64<0>(acc, dst, lane);
+    else if (warp == 1) write64<1>(acc, dst, lane);
+    else if (warp == 2) write64<2>(acc, dst, lane);
+    else write64<3>(acc, dst, lane);
 }
 
 // rows without observations: A^-1 0 = 0
@@ -859,6 +1228,7 @@ struct WarpRows {
     const int64_t *offs;
     int64_t n_chunks, n_split_rows;
     const void *X;
+    void *parts;               // fp32 tables of 64 features: room for the table's bfloat16 parts
     const float *Bmat;
     float *partials;
     RowOut out;
@@ -869,69 +1239,120 @@ struct WarpRows {
     int64_t *launches;
 };
 
-template <int D, typename T, bool CG> cudaError_t rows_warp_dt(const WarpRows &a)
+template <typename K> cudaError_t more_smem(K *kernel, size_t bytes)
 {
-    using G = WGeo<D, T>;
-    using B = BGeo<D, T>;
-    static_assert(B::SUMS <= D * D + D, "a chunk's sums fit its place in the workspace");
-    static_assert(B::SMEM <= 232448 && (size_t)G::BASE + G::REGS_WARPS * G::WARP <= 232448, "shared memory");
-    const T *X = reinterpret_cast<const T *>(a.X);
-    const int64_t *offs = a.offs;
-    const int kLongClass = warp_long_class(offs);
-    const size_t smem_warp = (size_t)G::BASE + G::REGS_WARPS * G::WARP;
-    const size_t smem_split = (size_t)G::BASE + G::WORK + 4 * B::SUMS;
-    cudaError_t e;
-    // longest work first
-    if (a.n_chunks > 0) {
-        if ((e = cudaFuncSetAttribute(k_rows_block<D, T, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B::SMEM)) != cudaSuccess) return e;
-        k_rows_block<D, T, true, false><<<(unsigned)a.n_chunks, B::kBlockWarps * 32, B::SMEM, a.s>>>(a.sv, 0, X, a.Bmat, a.partials, a.out, a.cg, a.st);
-        k_split_solve_warp<D, T, CG><<<(unsigned)a.n_split_rows, 32, smem_split, a.s>>>(a.sv, offs[kNClasses - 1], a.partials, a.Bmat, a.out, a.cg, a.st);
-        *a.launches += 2;
-    }
-    const int64_t n_long = offs[kNClasses - 1] - offs[kLongClass];
-    if (n_long > 0) {
-        if ((e = cudaFuncSetAttribute(k_rows_block<D, T, false, CG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B::SMEM)) != cudaSuccess) return e;
-        k_rows_block<D, T, false, CG><<<(unsigned)n_long, B::kBlockWarps * 32, B::SMEM, a.s>>>(a.sv, offs[kNClasses - 1] - 1, X, a.Bmat, a.partials, a.out,
-                                                                                          a.cg, a.st);
-        ++*a.launches;
-    }
-    const int64_t n_warp = offs[kLongClass] - offs[1];
-    if (n_warp > 0) {
-        if ((e = cudaFuncSetAttribute(k_rows_warp<D, T, CG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_warp)) != cudaSuccess) return e;
-        const int64_t blocks = (n_warp + G::ROWS - 1) / G::ROWS;      // few rows: one per SM before two
-        k_rows_warp<D, T, CG><<<(unsigned)(blocks < 148 ? blocks : 148), G::REGS_WARPS * 32, smem_warp, a.s>>>(
-            a.sv, offs[kLongClass] - 1, n_warp, a.dual_flag, offs[kLongClass] - offs[2], nullptr, nullptr, X, a.Bmat, a.out, a.cg, a.st);
-        ++*a.launches;
-    }
-    if (CG && offs[kNClasses] > offs[1]) {
-        // the rows conjugate gradients did not finish (none, as a rule: its blocks then return at once)
-        if ((e = cudaFuncSetAttribute(k_rows_warp<D, T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_warp)) != cudaSuccess) return e;
-        k_rows_warp<D, T, false><<<148, G::REGS_WARPS * 32, smem_warp, a.s>>>(a.sv, 0, 0, nullptr, 0, a.cg.fallback_list, a.cg.counters + 2, X, a.Bmat,
-                                                                             a.out, a.cg, a.st);
-        ++*a.launches;
-    }
-    const int64_t n_zero = offs[1] - offs[0];
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
+template <int D, typename T> cudaError_t zero_rows(const WarpRows &a)
+{
+    const int64_t n_zero = a.offs[1] - a.offs[0];
     if (n_zero > 0) {
-        k_zero_rows_warp<T><<<(unsigned)((n_zero * D + 255) / 256), 256, 0, a.s>>>(a.sv.order + offs[0], n_zero, D, a.out);
+        k_zero_rows_warp<T><<<(unsigned)((n_zero * D + 255) / 256), 256, 0, a.s>>>(a.sv.order + a.offs[0], n_zero, D, a.out);
         ++*a.launches;
     }
     return cudaGetLastError();
 }
 
+// rows order[end - 1], order[end - 2] .. by a warp each, down to class `first`; `list` (with its device-side count) instead
+template <int D, typename T>
+cudaError_t whole_rows(const WarpRows &a, int64_t end, const int32_t *list, const unsigned long long *list_count)
+{
+    using G = WGeo<D, T>;
+    static_assert((size_t)G::BASE + G::REGS_WARPS * G::WARP <= 232448, "shared memory");
+    const size_t smem = (size_t)G::BASE + G::REGS_WARPS * G::WARP;
+    const int64_t n = list ? 0 : end - a.offs[1];
+    if (!list && n <= 0) return cudaSuccess;
+    const cudaError_t e = more_smem(k_rows_warp<D, T>, smem);
+    if (e != cudaSuccess) return e;
+    const int64_t blocks = list ? 148 : (n + G::ROWS - 1) / G::ROWS;      // few rows: one per SM before two
+    k_rows_warp<D, T><<<(unsigned)(blocks < 148 ? blocks : 148), G::REGS_WARPS * 32, smem, a.s>>>(
+        a.sv, end - 1, n, list ? nullptr : a.dual_flag, end - a.offs[2], list, list_count, reinterpret_cast<const T *>(a.X), a.Bmat, a.out, a.st);
+    ++*a.launches;
+    return cudaGetLastError();
+}
+
+template <int D, typename T, bool CG> cudaError_t solve_rows(const WarpRows &a, int64_t n_long)
+{
+    if (a.n_split_rows + n_long <= 0) return cudaSuccess;
+    const size_t smem = (size_t)WGeo<D, T>::BASE + WGeo<D, T>::WORK + 4 * BGeo<D, T>::SUMS;
+    k_solve_sums_warp<D, T, CG><<<(unsigned)(a.n_split_rows + n_long), 32, smem, a.s>>>(a.sv, a.offs[kNClasses - 1], a.n_split_rows, a.n_chunks,
+                                                                                      a.partials, a.Bmat, a.out, a.cg, a.st);
+    ++*a.launches;
+    return cudaGetLastError();
+}
+
+template <int D, typename T> cudaError_t rows_warp_dt(const WarpRows &a)
+{
+    using B = BGeo<D, T>;
+    static_assert(B::SUMS <= D * D + D, "a chunk's sums fit its place in the workspace");
+    static_assert(B::SMEM <= 232448, "shared memory");
+    const T *X = reinterpret_cast<const T *>(a.X);
+    const int64_t *offs = a.offs, end_long = offs[kNClasses - 1], begin_long = offs[warp_long_class(offs)];
+    cudaError_t e;
+    // longest work first
+    if (a.n_chunks > 0) {
+        if ((e = more_smem(k_rows_block<D, T, true>, B::SMEM)) != cudaSuccess) return e;
+        k_rows_block<D, T, true><<<(unsigned)a.n_chunks, B::kBlockWarps * 32, B::SMEM, a.s>>>(a.sv, 0, X, a.Bmat, a.partials, a.out, a.st);
+        ++*a.launches;
+        if ((e = solve_rows<D, T, false>(a, 0)) != cudaSuccess) return e;
+    }
+    if (end_long > begin_long) {
+        if ((e = more_smem(k_rows_block<D, T, false>, B::SMEM)) != cudaSuccess) return e;
+        k_rows_block<D, T, false><<<(unsigned)(end_long - begin_long), B::kBlockWarps * 32, B::SMEM, a.s>>>(a.sv, end_long - 1, X, a.Bmat, a.partials,
+                                                                                                         a.out, a.st);
+        ++*a.launches;
+    }
+    if ((e = whole_rows<D, T>(a, begin_long, nullptr, nullptr)) != cudaSuccess) return e;
+    return zero_rows<D, T>(a);
+}
+
+// fp32 tables of 64 features: long rows and chunks over the parts whatever the solver, the other rows too with conjugate gradients
+cudaError_t rows_parts64(const WarpRows &a, bool use_cg, int64_t n_table)
+{
+    const int64_t *offs = a.offs, end_long = offs[kNClasses - 1], begin_long = offs[parts64_long_class(offs)];
+    const int64_t n_long = end_long - begin_long, n = begin_long - offs[1];
+    const uint4 *P = static_cast<const uint4 *>(a.parts);
+    cudaError_t e;
+    if (a.n_chunks + n_long > 0 || (use_cg && n > 0)) {
+        k_parts64<<<(unsigned)((n_table * 16 + 255) / 256), 256, 0, a.s>>>(static_cast<const float *>(a.X), n_table, static_cast<uint32_t *>(a.parts));
+        ++*a.launches;
+    }
+    if (a.n_chunks + n_long > 0) {
+        const size_t smem = PGeo::RING * PGeo::STAGE;
+        k_sums64<<<(unsigned)(a.n_chunks + n_long), 128, smem, a.s>>>(a.sv, a.n_chunks, end_long - 1, P, a.partials);
+        ++*a.launches;
+        e = use_cg ? solve_rows<64, float, true>(a, n_long) : solve_rows<64, float, false>(a, n_long);
+        if (e != cudaSuccess) return e;
+    }
+    if (use_cg) {
+        if (n > 0) {
+            const size_t smem = PGeo::G::BASE + PGeo::WARPS * PGeo::WARP;
+            if ((e = more_smem(k_rows_cg64, smem)) != cudaSuccess) return e;
+            k_rows_cg64<<<(unsigned)(n < 148 ? n : 148), PGeo::WARPS * 32, smem, a.s>>>(a.sv, begin_long - 1, n, a.dual_flag, begin_long - offs[2], P, a.Bmat,
+                                                                                     a.out, a.cg, a.st);
+            ++*a.launches;
+            // the rows conjugate gradients did not finish (none, as a rule: its blocks then return at once)
+            if ((e = whole_rows<64, float>(a, begin_long, a.cg.fallback_list, a.cg.counters + 2)) != cudaSuccess) return e;
+        }
+    } else if ((e = whole_rows<64, float>(a, begin_long, nullptr, nullptr)) != cudaSuccess) {
+        return e;
+    }
+    return zero_rows<64, float>(a);
+}
+
 }  // namespace
 
-cudaError_t launch_rows_warp(const SideView &sv, const int64_t *offs, int64_t n_chunks, int64_t n_split_rows, const void *X, int bf16, int d,
-                             const float *Bmat, float *partials, RowOut out, DevStatus *st, const CgOptions &cg, const int *dual_flag,
-                             cudaStream_t s, int64_t *launches)
+cudaError_t launch_rows_warp(const SideView &sv, const int64_t *offs, int64_t n_chunks, int64_t n_split_rows, const void *X, int64_t n_table,
+                             void *parts, int bf16, int d, const float *Bmat, float *partials, RowOut out, DevStatus *st, const CgOptions &cg,
+                             const int *dual_flag, cudaStream_t s, int64_t *launches)
 {
-    const bool use_cg = cg.enabled && d == 64 && !bf16;
-    const WarpRows a{sv, offs, n_chunks, n_split_rows, X, Bmat, partials, out, st,
-                     WarpCg{cg.max_iter, cg.warm_start ? 1 : 0, cg.tol * cg.tol, use_cg ? cg.counters : nullptr, cg.fallback_list},
-                     dual_flag, s, launches};
+    const WarpRows a{sv, offs, n_chunks, n_split_rows, X, parts, Bmat, partials, out, st,
+                     WarpCg{cg.max_iter, cg.warm_start ? 1 : 0, cg.tol * cg.tol, cg.counters, cg.fallback_list}, dual_flag, s, launches};
     switch (d) {
-    case 16: return bf16 ? rows_warp_dt<16, __nv_bfloat16, false>(a) : rows_warp_dt<16, float, false>(a);
-    case 32: return bf16 ? rows_warp_dt<32, __nv_bfloat16, false>(a) : rows_warp_dt<32, float, false>(a);
-    case 64: return bf16 ? rows_warp_dt<64, __nv_bfloat16, false>(a) : use_cg ? rows_warp_dt<64, float, true>(a) : rows_warp_dt<64, float, false>(a);
+    case 16: return bf16 ? rows_warp_dt<16, __nv_bfloat16>(a) : rows_warp_dt<16, float>(a);
+    case 32: return bf16 ? rows_warp_dt<32, __nv_bfloat16>(a) : rows_warp_dt<32, float>(a);
+    case 64: return bf16 ? rows_warp_dt<64, __nv_bfloat16>(a) : rows_parts64(a, cg.enabled, n_table);
     default: return cudaErrorInvalidValue;
     }
 }
