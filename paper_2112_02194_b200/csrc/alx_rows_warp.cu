@@ -894,11 +894,13 @@ struct PartsFeed {
     __device__ __forceinline__ void issue(int slot, int ids, int lane)
     {
         const uint32_t dst = ring + (uint32_t)slot * PGeo::STAGE;
-#pragma unroll
-        for (int k = 0; k < kEntries * PGeo::PIECES / 32; ++k) {
-            const int p = lane + 32 * k, r = p / PGeo::PIECES, c = p % PGeo::PIECES;
+#pragma unroll 1
+        for (int k = 0; k < kEntries; k += 4) {      // eight lanes per part of a row (unrolled in full it does not fit the registers)
+            const int r = k + (lane >> 3), c = lane & 7;
             const int row = __shfl_sync(0xFFFFFFFFu, ids, r);
-            cp_async16_zfill(dst + (c / 8) * PGeo::PART + r * PGeo::ROW + (c % 8) * 16, P + (int64_t)(row < 0 ? 0 : row) * PGeo::PIECES + c, row >= 0);
+            const uint4 *src = P + (int64_t)(row < 0 ? 0 : row) * PGeo::PIECES + c;
+#pragma unroll
+            for (int p = 0; p < 3; ++p) cp_async16_zfill(dst + p * PGeo::PART + r * PGeo::ROW + c * 16, src + 8 * p, row >= 0);
         }
         ptx::cp_async_commit();
     }
@@ -1004,7 +1006,7 @@ k_rows_cg64(SideView sv, int64_t last, int64_t count, const int *dual_flag, int6
     __syncthreads();
     const int64_t warps = (int64_t)gridDim.x * PGeo::WARPS;
     unsigned rows = 0, products = 0;
-    int64_t item = (int64_t)warp * gridDim.x + blockIdx.x;
+    const int64_t item = (int64_t)warp * gridDim.x + blockIdx.x;
     if (item >= count) return;
     PartsFeed feed;
     feed.P = P;
@@ -1012,35 +1014,36 @@ k_rows_cg64(SideView sv, int64_t last, int64_t count, const int *dual_flag, int6
     feed.val = sv.val;
     feed.ring = ptx::smem_u32(mine);
     feed.g = 0;
-    int64_t u = sv.order[last - item];
-    int64_t len = sv.ptr[u + 1] - sv.ptr[u];
+    // the walk: rows are looked up two ahead (id), one ahead (range); 32-bit ids and lengths, for the registers
+    const int32_t *walk = sv.order + (last - item);
+    int left = (int)((count - item - 1) / warps);      // rows after the current one
+    int u = *walk, un = left > 0 ? *(walk - warps) : -1;
+    int len = (int)(sv.ptr[u + 1] - sv.ptr[u]);
     feed.start_ids(sv.ptr[u], sv.ptr[u + 1], lane);
     feed.start_copies(lane);
-    // the row after this one is looked up while this one is summed: its id a row ahead, its range now
-    int64_t un = item + warps < count ? sv.order[last - item - warps] : -1;
     while (true) {
-        const int64_t after = item + 2 * warps;
-        const int64_t bn = un < 0 ? 0 : sv.ptr[un], en = un < 0 ? 0 : sv.ptr[un + 1];
-        const int64_t ua = after < count ? sv.order[last - after] : -1;
-        const float *stored = reinterpret_cast<const float *>(out.table) + u * 64;
-        float x0 = cg.warm ? stored[lane] : 0.f, x1 = cg.warm ? stored[lane + 32] : 0.f;
         float a0[64], a1[64];
+        const int ua = left > 1 ? *(walk - 2 * warps) : -1;
         {
+            const int64_t bn = left > 0 ? sv.ptr[un] : 0;
+            const int len_next = left > 0 ? (int)(sv.ptr[un + 1] - bn) : 0;
             Sums<64, float> acc;
             acc.zero();
             sum_parts(feed, len, acc, b_s, lane);
-            if (un >= 0) feed.start_ids(bn, en, lane);
+            len = len_next;
+            if (left > 0) feed.start_ids(bn, bn + len, lane);
             add_base<64, float>(acc, base, lane);
             // (through the slot that the next row's first stage will not take)
             symmetric_rows(acc, reinterpret_cast<float *>(mine + ((feed.g + 1) & 1) * PGeo::STAGE), a0, a1, lane);
         }
-        if (un >= 0) feed.start_copies(lane);      // they travel while this row is solved
+        if (left > 0) feed.start_copies(lane);      // they travel while this row is solved
+        float *row = reinterpret_cast<float *>(out.table) + (int64_t)u * 64;
+        float x0 = cg.warm ? row[lane] : 0.f, x1 = cg.warm ? row[lane + 32] : 0.f;
         int spent = 0;
         const bool ok = conjugate_gradients(cg, a0, a1, vec, b_s[lane], b_s[lane + 32], x0, x1, spent, lane);
         ++rows;
         products += spent;
         if (ok) {
-            float *row = reinterpret_cast<float *>(out.table) + u * 64;
             row[lane] = x0;
             row[lane + 32] = x1;
             if (out.cap_slot) {
@@ -1051,14 +1054,14 @@ k_rows_cg64(SideView sv, int64_t last, int64_t count, const int *dual_flag, int6
                 }
             }
         } else if (lane == 0) {
-            cg.fallback_list[atomicAdd(&cg.counters[2], 1ull)] = (int32_t)u;
+            cg.fallback_list[atomicAdd(&cg.counters[2], 1ull)] = u;
         }
-        if (un < 0) break;
+        if (left == 0) break;
         __syncwarp();
-        item += warps;
+        --left;
+        walk -= warps;
         u = un;
         un = ua;
-        len = en - bn;
     }
     if (lane == 0) {
         atomicAdd(&cg.counters[0], (unsigned long long)rows);
