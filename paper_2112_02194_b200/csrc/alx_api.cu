@@ -60,9 +60,14 @@ struct alx_ctx {
     void *dual_ws = nullptr;      // tensor path: B^-1 operand tiles and the flag of the dual form
     int64_t dual_candidates = 0;  // rows of classes 1 and 2 of the last half-epoch (solved in the dual form if the flag is set)
     int64_t dual_candidates32 = 0; // of them, the rows of 17 .. 32 observations (which the whole-rows kernel may have taken instead)
+    // The launches of a whole epoch on this matrix, for small matrices: captured behind the second alx_epoch, replayed from the third on
+    cudaGraphExec_t epoch_graph = nullptr;
+    int epochs_run = 0;            // alx_epoch calls since the matrix was set
+    int64_t epoch_launches = 0;    // kernels in the graph
+    bool capturing = false;
     int last_side = 0;             // side of the last half-epoch: its flag and policy record stay on the device until alx_get_stats asks
     double *loss_partials_buf = nullptr;
-    double *loss_result = nullptr;
+    unsigned *loss_counter = nullptr;              // zero between calls
     DevStatus *status = nullptr;
     unsigned long long *cg_counters = nullptr;   // tensor path, last half-epoch: rows solved by conjugate gradients, products, fall-backs; dual-form rows polished, their products
     int32_t *cg_fallback_list = nullptr;         // tensor path with conjugate gradients: the rows left to the Cholesky solve
@@ -283,16 +288,10 @@ struct Download {
     }
 };
 
-// wait for the stream, read and clear the device status word
-alx_status check_device_status(alx_ctx *c)
+// the status word that a copy or a kernel has put into the box and the stream has been waited for: report and clear it
+alx_status report_status(alx_ctx *c)
 {
     DevStatus h;
-    {
-        alx_status st = ensure_box(c);
-        if (st != ALX_OK) return st;
-    }
-    ALX_CUDA(c, cudaMemcpyAsync(c->box, c->status, sizeof h, cudaMemcpyDeviceToHost, c->stream));
-    ALX_CUDA(c, cudaStreamSynchronize(c->stream));
     memcpy(&h, c->box, sizeof h);
     c->stats.not_spd += (int64_t)h.not_spd;
     if (h.flags == 0) return ALX_OK;
@@ -306,6 +305,16 @@ alx_status check_device_status(alx_ctx *c)
                     h.first_bad % 1000000, (h.flags & kFlagNotSpd) ? "; rows also met non-positive pivots" : "");
     if (h.flags & kFlagNotSpd) return fail(c, ALX_ERR_NOT_SPD, "%llu rows met a non-positive pivot (first: row %lld); they were set to zero", h.not_spd, h.first_bad);
     return fail(c, ALX_ERR_CUDA, "device status flags 0x%x", h.flags);
+}
+
+// wait for the stream, read and clear the device status word
+alx_status check_device_status(alx_ctx *c)
+{
+    alx_status st = ensure_box(c);
+    if (st != ALX_OK) return st;
+    ALX_CUDA(c, cudaMemcpyAsync(c->box, c->status, sizeof(DevStatus), cudaMemcpyDeviceToHost, c->stream));
+    ALX_CUDA(c, cudaStreamSynchronize(c->stream));
+    return report_status(c);
 }
 
 SideView side_view(const alx_ctx *c, int side)
@@ -367,8 +376,16 @@ alx_status build_buckets(alx_ctx *c, int side, int64_t *scratch_a, int64_t *scra
     return ALX_OK;
 }
 
+void drop_epoch_graph(alx_ctx *c)
+{
+    if (c->epoch_graph) cudaGraphExecDestroy(c->epoch_graph);
+    c->epoch_graph = nullptr;
+    c->epochs_run = 0;
+}
+
 void release_matrix(alx_ctx *c)
 {
+    drop_epoch_graph(c);
     for (int s = 0; s < 2; ++s) {
         dev_free(c, c->ptr[s]); c->ptr[s] = nullptr;
         dev_free(c, c->idx[s]); c->idx[s] = nullptr;
@@ -460,67 +477,64 @@ alx_status gramian_of(alx_ctx *c, int table_side, bool solve)
     return ALX_OK;
 }
 
+// what the statistics say of a half-epoch
+void note_half_epoch(alx_ctx *c, int side)
+{
+    c->last_side = side;
+    c->dual_candidates = dual_rows_of(c, side);
+    c->dual_candidates32 = dual_form(c) && c->dual_candidates > 0 ? c->class_offs[side][3] - c->class_offs[side][2] : 0;
+    c->main_timed = tensor_path(c) || cg64(c);
+    c->stats.kernel_path[side] = warp_path(c) || tensor_path(c) || team_path(c) ? 1 : 0;
+}
+
 alx_status half_epoch_impl(alx_ctx *c, int side, const int32_t *cap_slot, float *cap_out)
 {
     if (c->nnz < 0) return fail(c, ALX_ERR_BAD_STATE, "alx_half_epoch before alx_set_csr");
     const int fixed = 1 - side;
     if (!c->have_table[fixed]) return fail(c, ALX_ERR_BAD_STATE, "the fixed table has not been set");
     NvtxRange range(side == ALX_ROWS ? "alx half-epoch: rows" : "alx half-epoch: columns");
-    ALX_CUDA(c, cudaEventRecord(c->ev[0], c->stream));
+    ALX_CUDA(c, record_event(c->ev[0], c->stream, c->capturing));
     alx_status st;
     {
         NvtxRange r("alx Gramian + base matrix");
         st = gramian_of(c, fixed, dual_rows_of(c, side) > 0);
     }
     if (st != ALX_OK) return st;
-    ALX_CUDA(c, cudaEventRecord(c->ev[1], c->stream));
+    ALX_CUDA(c, record_event(c->ev[1], c->stream, c->capturing));
     NvtxRange rows_range("alx rows: gather, sums, solve, store");
     RowOut out{c->table[side], cap_slot, cap_out};
-    c->dual_candidates = c->dual_candidates32 = 0;
-    c->last_side = side;
+    note_half_epoch(c, side);
+    const int64_t n_dual = c->dual_candidates;
     if (warp_path(c)) {
         if (cg64(c)) ALX_CUDA(c, cudaMemsetAsync(c->cg_counters, 0, 5 * sizeof(unsigned long long), c->stream));
-        const int64_t n_dual = dual_rows_of(c, side);
         if (n_dual > 0)
             ALX_CUDA(c, dual64(c) ? launch_rows_dual64(side_view(c, side), c->class_offs[side][1], n_dual, c->table[fixed], c->dual_ws, out,
                                                        c->stream, &c->launches)
                                   : launch_rows_dual_warp(side_view(c, side), c->class_offs[side][1], n_dual, c->table[fixed], c->bf16,
                                                           c->opt.d, c->dual_ws, out, c->status, c->stream, &c->launches));
-        ALX_CUDA(c, cudaEventRecord(c->ev[3], c->stream));
+        if (cg64(c)) ALX_CUDA(c, record_event(c->ev[3], c->stream, c->capturing));
         ALX_CUDA(c, launch_rows_warp(side_view(c, side), c->class_offs[side], c->n_chunks[side], c->n_split_rows[side], c->table[fixed],
                                      c->n[fixed], c->parts, c->bf16, c->opt.d, c->Bmat, c->split_partials, out, c->status, cg_options(c, side),
                                      n_dual > 0 ? dual_flag_of(c) : nullptr, c->stream, &c->launches));
-        ALX_CUDA(c, cudaEventRecord(c->ev[4], c->stream));
-        c->stats.kernel_path[side] = 1;
-        c->main_timed = true;
-        c->dual_candidates = n_dual;
+        if (cg64(c)) ALX_CUDA(c, record_event(c->ev[4], c->stream, c->capturing));
     } else if (tensor_path(c)) {
-        const int64_t n_dual = dual_rows_of(c, side);
         ALX_CUDA(c, cudaMemsetAsync(c->cg_counters, 0, 5 * sizeof(unsigned long long), c->stream));
         ALX_CUDA(c, launch_rows_umma(side_view(c, side), c->class_offs[side], c->n_chunks[side], c->n_split_rows[side],
                                      c->table[fixed], c->Bmat, c->split_partials, out, c->status, c->stream,
-                                     &c->launches, c->ev[3], c->ev[4], n_dual > 0 ? c->dual_ws : nullptr, c->n[fixed],
+                                     &c->launches, c->ev[3], c->ev[4], c->capturing, n_dual > 0 ? c->dual_ws : nullptr, c->n[fixed],
                                      cg_options(c, side), c->order16[side], c->n4[side], c->n8[side]));
-        c->stats.kernel_path[side] = 1;
-        c->main_timed = true;
-        c->dual_candidates = n_dual;
-        c->dual_candidates32 = n_dual > 0 ? c->class_offs[side][3] - c->class_offs[side][2] : 0;
     } else if (team_path(c)) {
-        const int64_t n_dual = dual_rows_of(c, side);
         if (n_dual > 0)
             ALX_CUDA(c, launch_rows_dual_warp(side_view(c, side), c->class_offs[side][1], n_dual, c->table[fixed], 0, c->opt.d, c->dual_ws, out,
                                               c->status, c->stream, &c->launches));
         ALX_CUDA(c, launch_rows_team(side_view(c, side), c->class_offs[side], c->n_chunks[side], c->n_split_rows[side],
                                      static_cast<const float *>(c->table[fixed]), c->Bmat, c->split_partials, out, c->status,
                                      n_dual > 0 ? dual_flag_of(c) : nullptr, c->stream, &c->launches));
-        c->stats.kernel_path[side] = 1;
-        c->dual_candidates = n_dual;
     } else {
         ALX_CUDA(c, launch_rows_simple(side_view(c, side), c->class_offs[side], c->n_chunks[side], c->n_split_rows[side], c->table[fixed],
                                        c->bf16, c->opt.d, c->Bmat, c->split_partials, out, c->status, c->stream, &c->launches));
-        c->stats.kernel_path[side] = 0;
     }
-    ALX_CUDA(c, cudaEventRecord(c->ev[2], c->stream));
+    ALX_CUDA(c, record_event(c->ev[2], c->stream, c->capturing));
     c->have_table[side] = true;
     c->have_gram[side] = false;
     return ALX_OK;
@@ -604,8 +618,8 @@ alx_status create_impl(const alx_options *opt, const alx_ctx *parent, alx_ctx **
         int64_t n_part = gramian_partials(nmax);
         if (gramian_umma_partials() > n_part) n_part = gramian_umma_partials();
         ALX_ALLOC(c, c->gram_partials, n_part * d * d);
-        ALX_ALLOC(c, c->loss_result, 4);
-        ALX_CUDA(c, cudaMemsetAsync(c->loss_result, 0, 4 * sizeof(double), c->stream));
+        ALX_ALLOC(c, c->loss_counter, 1);
+        ALX_CUDA(c, cudaMemsetAsync(c->loss_counter, 0, sizeof(unsigned), c->stream));
         ALX_ALLOC(c, c->status, 1);
         ALX_CUDA(c, cudaMemsetAsync(c->status, 0, sizeof(DevStatus), c->stream));
         ALX_ALLOC(c, c->cg_counters, 5);
@@ -635,6 +649,7 @@ alx_status alx_destroy(alx_ctx *c)
     DeviceGuard guard(c->device);
     cudaStreamSynchronize(c->stream);
     if (c->fold) alx_destroy(c->fold);
+    drop_epoch_graph(c);
     if (c->box) cudaFreeHost(c->box);
     for (auto &e : c->ev) if (e) cudaEventDestroy(e);
     if (c->copy_stream) { cudaStreamSynchronize(c->copy_stream); cudaStreamDestroy(c->copy_stream); }
@@ -881,13 +896,6 @@ alx_status alx_half_epoch(alx_ctx *c, alx_side side)
     return half_epoch_impl(c, side, nullptr, nullptr);
 }
 
-alx_status alx_epoch(alx_ctx *c)
-{
-    alx_status st = alx_half_epoch(c, ALX_ROWS);
-    if (st != ALX_OK) return st;
-    return alx_half_epoch(c, ALX_COLS);
-}
-
 namespace {
 alx_status ensure_copy_stream(alx_ctx *c)
 {
@@ -895,7 +903,61 @@ alx_status ensure_copy_stream(alx_ctx *c)
     if (!c->copy_ev) ALX_CUDA(c, cudaEventCreateWithFlags(&c->copy_ev, cudaEventDisableTiming));
     return ALX_OK;
 }
+
+// Matrices of at most this many entries replay their epochs as a graph: a half-epoch is five to ten launches and three events,
+// 20 us of host time, which the GPU outruns up to some million entries; beyond, it makes no difference
+constexpr int64_t kGraphEntries = 1ll << 24;
+
+// Captures the launches of one epoch (on the library's second stream, whatever stream the context works on).  The state the
+// launches depend on -- tables and matrix in place, both tables set -- is that of every later epoch on this matrix.  Where
+// capturing fails, epochs go on as single launches.
+void capture_epoch(alx_ctx *c)
+{
+    if (ensure_copy_stream(c) != ALX_OK) return;
+    cudaStream_t user = c->stream;
+    const int64_t launches = c->launches;
+    if (cudaStreamBeginCapture(c->copy_stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) { cudaGetLastError(); return; }
+    c->stream = c->copy_stream;
+    c->capturing = true;
+    alx_status st = half_epoch_impl(c, ALX_ROWS, nullptr, nullptr);
+    if (st == ALX_OK) st = half_epoch_impl(c, ALX_COLS, nullptr, nullptr);
+    c->capturing = false;
+    c->stream = user;
+    c->epoch_launches = c->launches - launches;
+    c->launches = launches;
+    cudaGraph_t graph = nullptr;
+    if (cudaStreamEndCapture(c->copy_stream, &graph) != cudaSuccess || !graph) { cudaGetLastError(); return; }
+    if (st == ALX_OK && cudaGraphInstantiate(&c->epoch_graph, graph, 0) != cudaSuccess) {
+        cudaGetLastError();
+        c->epoch_graph = nullptr;
+    }
+    cudaGraphDestroy(graph);
+}
 }  // namespace
+
+alx_status alx_epoch(alx_ctx *c)
+{
+    if (!c) return ALX_ERR_INVALID_ARG;
+    DeviceGuard guard(c->device);
+    if (c->epoch_graph && c->have_table[0] && c->have_table[1]) {
+        NvtxRange range("alx epoch (graph)");
+        ALX_CUDA(c, cudaGraphLaunch(c->epoch_graph, c->stream));
+        c->launches += c->epoch_launches;
+        // (the host-side state of a half-epoch is what the capture of the columns' half left)
+        c->have_gram[ALX_ROWS] = true;
+        c->have_gram[ALX_COLS] = false;
+        note_half_epoch(c, ALX_COLS);
+        return ALX_OK;
+    }
+    alx_status st = half_epoch_impl(c, ALX_ROWS, nullptr, nullptr);
+    if (st == ALX_OK) st = half_epoch_impl(c, ALX_COLS, nullptr, nullptr);
+    if (st != ALX_OK) return st;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (++c->epochs_run == 2 && c->nnz <= kGraphEntries && cudaStreamIsCapturing(c->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone)
+        capture_epoch(c);
+    return ALX_OK;
+}
+
 
 alx_status alx_load_host(alx_ctx *c, const int64_t *rowptr, const int32_t *colidx, const float *values, int64_t nnz,
                          const void *W, const void *H)
@@ -1009,15 +1071,15 @@ alx_status alx_loss(alx_ctx *c, double *total, double *components)
             alx_status st = gramian_of(c, s, false);
             if (st != ALX_OK) return st;
         }
-    ALX_CUDA(c, launch_loss(c->ptr[0], c->idx[0], c->val[0], c->n[0], c->nnz, c->table[0], c->table[1], c->bf16, c->opt.d, c->G64[0],
-                            c->G64[1], (double)c->opt.alpha0, (double)c->opt.lambda, c->loss_partials_buf, c->loss_result, c->stream,
-                            &c->launches));
-    double h[3];
-    Download down(c);
-    alx_status st = down.add(h, c->loss_result, sizeof h);
-    if (st == ALX_OK) st = check_device_status(c);
+    alx_status st = ensure_box(c);
     if (st != ALX_OK) return st;
-    down.take();
+    double *h = reinterpret_cast<double *>(c->box + 64);
+    ALX_CUDA(c, launch_loss(c->ptr[0], c->idx[0], c->val[0], c->n[0], c->nnz, c->table[0], c->table[1], c->bf16, c->opt.d, c->G64[0],
+                            c->G64[1], (double)c->opt.alpha0, (double)c->opt.lambda, c->loss_partials_buf, c->loss_counter, c->status,
+                            reinterpret_cast<DevStatus *>(c->box), h, c->stream, &c->launches));
+    ALX_CUDA(c, cudaStreamSynchronize(c->stream));
+    st = report_status(c);
+    if (st != ALX_OK) return st;
     *total = h[0] + h[1] + h[2];
     if (components) { components[0] = h[0]; components[1] = h[1]; components[2] = h[2]; }
     return ALX_OK;

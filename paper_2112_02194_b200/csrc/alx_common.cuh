@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 namespace alx {
 
 constexpr int kNClasses = 12;
@@ -79,6 +81,28 @@ struct RowOut {
     const int32_t *cap_slot; // nullptr, or per-row capture slot (-1 = none)
     float *cap_out;          // [slots x d] fp32 solutions before rounding
 };
+
+// ---- small host pieces of the launchers -----------------------------------------------------------
+// Lets a kernel use more than the default dynamic shared memory, once per device (the call costs a microsecond of host time,
+// which a half-epoch of a small matrix pays several times over).  One static object per kernel.
+struct SmemOnce {
+    std::atomic<unsigned long long> done{0};      // a bit per device
+    template <typename K> cudaError_t operator()(K *kernel, size_t bytes)
+    {
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        if (dev < 64 && (done.load(std::memory_order_relaxed) >> dev & 1)) return cudaSuccess;
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        if (e == cudaSuccess && dev < 64) done.fetch_or(1ull << dev, std::memory_order_relaxed);
+        return e;
+    }
+};
+// Records a timing event, as a node of its own where the stream is being captured into a graph.
+inline cudaError_t record_event(cudaEvent_t ev, cudaStream_t s, bool capturing)
+{
+    return cudaEventRecordWithFlags(ev, s, capturing ? cudaEventRecordExternal : cudaEventRecordDefault);
+}
 
 // ---- host entry points (one per .cu) ----------------------------------------------------------
 struct ScanScratch;
@@ -180,10 +204,16 @@ struct CgOptions {
     float switch_products;         // mean products per row beyond which the side's next half-epochs take Cholesky
 };
 
-// The degree class from which on a row gets a block of warps instead of one: more than 1024 entries (a warp takes about 50 us
-// for as many) where there are so many rows that every warp has several anyway, else more than 256, so that a few longer
-// rows do not outlast the others.
-inline int warp_long_class(const int64_t *class_offs_host) { return class_offs_host[8] - class_offs_host[1] >= 148 * 20 * 8 ? 8 : 6; }
+// The degree class from which on a row gets a block of warps instead of one.  Where there are so many rows that every warp has
+// several anyway: more than 1024 entries (a warp takes about 50 us for as many).  Else the longest rows must not outlast the
+// others: the lowest class from 65 entries up whose rows, with all longer ones, are at most one wave of blocks (148), at most 257.
+inline int warp_long_class(const int64_t *class_offs_host)
+{
+    if (class_offs_host[8] - class_offs_host[1] >= 148 * 20 * 8) return 8;
+    int c = 4;
+    while (c < 6 && class_offs_host[kNClasses - 1] - class_offs_host[c] > 148) ++c;
+    return c;
+}
 // ... and for fp32 tables of 64 features, where a long row's sums take a place in the workspace: more than 512 entries (256 where rows
 // are few), as long as those rows are at most kLongRowBudget
 inline int parts64_long_class(const int64_t *class_offs_host)
@@ -234,7 +264,7 @@ cudaError_t launch_recall(const int32_t *ids, int64_t m, int k_stride, int k, co
 cudaError_t launch_rows_umma(const SideView &sv, const int64_t *class_offs_host, int64_t n_chunks,
                              int64_t n_split_rows, const void *X, const float *Bmat, float *split_partials,
                              RowOut out, DevStatus *st, cudaStream_t s, int64_t *launches, cudaEvent_t main_begin,
-                             cudaEvent_t main_end, const void *dual_ws, int64_t n_table, const CgOptions &cg, const int32_t *order16 = nullptr, int64_t n4 = 0, int64_t n8 = 0);
+                             cudaEvent_t main_end, bool capturing, const void *dual_ws, int64_t n_table, const CgOptions &cg, const int32_t *order16 = nullptr, int64_t n4 = 0, int64_t n8 = 0);
 
 // alx_dual.cu: rows with at most 32 observations in the dual form (d = 128, bf16 tables)
 size_t dual_workspace_bytes();
@@ -267,9 +297,11 @@ cudaError_t launch_rows_dual(const SideView &sv, int64_t first16, int64_t count1
 
 // alx_loss.cu
 int64_t loss_partials(int64_t nnz);
-// result: [0] observed, [1] all-pairs, [2] regulariser, and [3] a counter that is zero between calls
+// host: page-locked, device-accessible: the status word goes to its start, [0] observed, [1] all-pairs, [2] regulariser to
+// host_result; counter: a device word that is zero between calls
 cudaError_t launch_loss(const int64_t *rowptr, const int32_t *colidx, const float *values, int64_t n_rows,
                             int64_t nnz, const void *W, const void *H, int bf16, int d, const double *GW, const double *GH,
-                            double alpha0, double lambda, double *partials, double *result, cudaStream_t s, int64_t *launches);
+                            double alpha0, double lambda, double *partials, unsigned *counter, const DevStatus *st, DevStatus *host_status,
+                            double *host_result, cudaStream_t s, int64_t *launches);
 
 }  // namespace alx

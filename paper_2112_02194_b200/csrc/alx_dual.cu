@@ -631,7 +631,8 @@ template <int KP> cudaError_t launch_dual_instance(DualParams p, int sms, cudaSt
     if (p.count <= 0) return cudaSuccess;
     p.n_tiles = (p.count + 128 / KP - 1) / (128 / KP);
     const size_t smem = sizeof(DualSmem) + 1024;
-    cudaError_t e = cudaFuncSetAttribute(k_dual<KP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static SmemOnce allow;
+    cudaError_t e = allow(k_dual<KP>, smem);
     if (e != cudaSuccess) return e;
     const int grid = (int)(p.n_tiles < sms ? p.n_tiles : (sms > 0 ? sms : 1));
     k_dual<KP><<<grid, kBlockThreads, smem, s>>>(p);

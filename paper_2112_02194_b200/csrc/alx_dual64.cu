@@ -206,7 +206,8 @@ cudaError_t launch_rows_dual64(const SideView &sv, int64_t first, int64_t count,
 {
     if (count <= 0) return cudaSuccess;
     const size_t smem = sizeof(float) * D * D + kWarps * sizeof(WarpScratch);
-    cudaError_t e = cudaFuncSetAttribute(k_dual64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static SmemOnce allow;
+    cudaError_t e = allow(k_dual64, smem);
     if (e != cudaSuccess) return e;
     int64_t blocks = (count + kWarps - 1) / kWarps;
     if (blocks > 148 * 6) blocks = 148 * 6;

@@ -252,7 +252,8 @@ cudaError_t launch_dt(const SideView &sv, int64_t first, int64_t count, const vo
 {
     using G = DGeo<D, T>;
     static_assert(G::SMEM <= 232448, "shared memory");
-    const cudaError_t e = cudaFuncSetAttribute(k_dual_warp<D, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM);
+    static SmemOnce allow;
+    const cudaError_t e = allow(k_dual_warp<D, T>, G::SMEM);
     if (e != cudaSuccess) return e;
     k_dual_warp<D, T><<<(unsigned)(count < 148 ? count : 148), G::WARPS * 32, G::SMEM, s>>>(
         sv, first, count, static_cast<const T *>(X), static_cast<const uint4 *>(ws), dual_warp_flag_ptr(ws, D), out, st);

@@ -201,7 +201,8 @@ cudaError_t gramian_tiles_dt(const void *X, int64_t n, float *partials, double *
 {
     using G = GramGeo<D, T>;
     static_assert(G::ELEMS <= D * D && G::SMEM <= 232448, "sizes");
-    const cudaError_t e = cudaFuncSetAttribute(k_gramian_tiles<D, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM);
+    static SmemOnce allow;
+    const cudaError_t e = allow(k_gramian_tiles<D, T>, G::SMEM);
     if (e != cudaSuccess) return e;
     const int64_t blocks = gramian_partials(n), per = (n + blocks - 1) / blocks;
     k_gramian_tiles<D, T><<<(unsigned)blocks, G::THREADS, G::SMEM, s>>>(static_cast<const T *>(X), n, per, partials);

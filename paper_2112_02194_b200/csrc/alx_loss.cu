@@ -14,7 +14,14 @@ constexpr int64_t kMostBlocks = 148 * kBlocksPerSm;
 // Entries a warp takes at a time; the warps then go on together to the next stretch of the matrix, so that at any time they
 // read neighbouring rows of W, and of H where the matrix is local (one long range per warp spread them over the whole table:
 // 70 ms instead of 35 ms for 1e9 entries within 1 % of the diagonal)
-constexpr int kSpan = 512;
+constexpr int kMostSpan = 512;
+
+// entries per span: as many as give every SM something to do, a multiple of 32
+int span_of(int64_t nnz)
+{
+    const int64_t s = nnz / (kMostBlocks * kWarps) / 32 * 32;
+    return s < 32 ? 32 : s < kMostSpan ? (int)s : kMostSpan;
+}
 
 // largest u in [0, n) with ptr[u] <= e, by the whole warp: 32 probes a round
 __device__ __forceinline__ int64_t warp_row_of(const int64_t *__restrict__ ptr, int64_t n, int64_t e, int lane)
@@ -86,10 +93,10 @@ __device__ __forceinline__ double block_sum(double v, double *buf)
 // block to finish adds the blocks' sums in order and the two Gramian terms.
 template <int D, typename T>
 __global__ void __launch_bounds__(kWarps * 32, kBlocksPerSm) k_loss(const int64_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
-                                                      const float *__restrict__ values, int64_t n_rows, int64_t nnz,
+                                                      const float *__restrict__ values, int64_t n_rows, int64_t nnz, int span,
                                                       const T *__restrict__ W, const T *__restrict__ H, const double *__restrict__ GW,
                                                       const double *__restrict__ GH, double alpha0, double lambda, double *partials,
-                                                      double *result)
+                                                      unsigned *counter, const DevStatus *st, DevStatus *host_status, double *host_result)
 {
     constexpr int EL = 16 / (int)sizeof(T), LANES = D / EL, U = LANES < 4 ? LANES : 4;
     __shared__ double buf[kWarps];
@@ -97,8 +104,8 @@ __global__ void __launch_bounds__(kWarps * 32, kBlocksPerSm) k_loss(const int64_
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int part = lane % LANES, first = lane - part;      // first lane of the group
     double acc = 0.0;
-    for (int64_t e0 = ((int64_t)blockIdx.x * kWarps + warp) * kSpan; e0 < nnz; e0 += (int64_t)gridDim.x * kWarps * kSpan) {
-        const int64_t e1 = e0 + kSpan < nnz ? e0 + kSpan : nnz;
+    for (int64_t e0 = ((int64_t)blockIdx.x * kWarps + warp) * span; e0 < nnz; e0 += (int64_t)gridDim.x * kWarps * span) {
+        const int64_t e1 = e0 + span < nnz ? e0 + span : nnz;
         int64_t u = warp_row_of(rowptr, n_rows, e0, lane);
         int w_row = -1;
         float w[EL];
@@ -159,7 +166,6 @@ __global__ void __launch_bounds__(kWarps * 32, kBlocksPerSm) k_loss(const int64_
         }
     }
     const double mine = block_sum(acc, buf);
-    unsigned *counter = reinterpret_cast<unsigned *>(result + 3);
     if (threadIdx.x == 0) {
         partials[blockIdx.x] = mine;
         __threadfence();
@@ -180,9 +186,11 @@ __global__ void __launch_bounds__(kWarps * 32, kBlocksPerSm) k_loss(const int64_
     f = block_sum(f, buf);
     t = block_sum(t, buf);
     if (threadIdx.x == 0) {
-        result[0] = nnz > 0 ? s : 0.0;
-        result[1] = alpha0 * f;
-        result[2] = lambda * t;
+        // straight to the host, with the status word: one wait and no copies
+        host_result[0] = nnz > 0 ? s : 0.0;
+        host_result[1] = alpha0 * f;
+        host_result[2] = lambda * t;
+        *host_status = *st;
         *counter = 0;
     }
 }
@@ -191,24 +199,22 @@ __global__ void __launch_bounds__(kWarps * 32, kBlocksPerSm) k_loss(const int64_
 
 int64_t loss_partials(int64_t nnz)
 {
-    const int64_t b = (nnz + kSpan * kWarps - 1) / (kSpan * kWarps);
+    const int64_t per = (int64_t)span_of(nnz) * kWarps, b = (nnz + per - 1) / per;
     return b < kMostBlocks ? (b > 0 ? b : 1) : kMostBlocks;
 }
 
 cudaError_t launch_loss(const int64_t *rowptr, const int32_t *colidx, const float *values, int64_t n_rows, int64_t nnz, const void *W,
                         const void *H, int bf16, int d, const double *GW, const double *GH, double alpha0, double lambda, double *partials,
-                        double *result, cudaStream_t s, int64_t *launches)
+                        unsigned *counter, const DevStatus *st, DevStatus *host_status, double *host_result, cudaStream_t s, int64_t *launches)
 {
     const unsigned grid = (unsigned)loss_partials(nnz);
-#define ALX_CASE(DD)                                                                                                              \
-    case DD:                                                                                                                      \
-        if (bf16)                                                                                                                 \
-            k_loss<DD, __nv_bfloat16><<<grid, kWarps * 32, 0, s>>>(rowptr, colidx, values, n_rows, nnz,                 \
-                                                                   (const __nv_bfloat16 *)W, (const __nv_bfloat16 *)H, GW, GH,    \
-                                                                   alpha0, lambda, partials, result);                             \
-        else                                                                                                                      \
-            k_loss<DD, float><<<grid, kWarps * 32, 0, s>>>(rowptr, colidx, values, n_rows, nnz, (const float *)W,       \
-                                                           (const float *)H, GW, GH, alpha0, lambda, partials, result);           \
+#define ALX_LOSS(DD, T)                                                                                                             \
+    k_loss<DD, T><<<grid, kWarps * 32, 0, s>>>(rowptr, colidx, values, n_rows, nnz, span_of(nnz), (const T *)W, (const T *)H, GW, GH,     \
+                                               alpha0, lambda, partials, counter, st, host_status, host_result)
+#define ALX_CASE(DD)                        \
+    case DD:                                \
+        if (bf16) ALX_LOSS(DD, __nv_bfloat16); \
+        else ALX_LOSS(DD, float);           \
         break;
     switch (d) {
         ALX_CASE(16)
@@ -218,6 +224,7 @@ cudaError_t launch_loss(const int64_t *rowptr, const int32_t *colidx, const floa
     default: return cudaErrorInvalidValue;
     }
 #undef ALX_CASE
+#undef ALX_LOSS
     ++*launches;
     return cudaGetLastError();
 }

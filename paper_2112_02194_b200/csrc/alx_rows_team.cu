@@ -524,9 +524,10 @@ cudaError_t launch_rows_team(const SideView &sv, const int64_t *offs, int64_t n_
 {
     const size_t smem = sizeof(TeamSmem);
     cudaError_t e;
-    if ((e = cudaFuncSetAttribute(k_rows_team, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_sums_team, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_solve_sums_team, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+    static SmemOnce allow_rows, allow_sums, allow_solve;
+    if ((e = allow_rows(k_rows_team, smem)) != cudaSuccess) return e;
+    if ((e = allow_sums(k_sums_team, smem)) != cudaSuccess) return e;
+    if ((e = allow_solve(k_solve_sums_team, smem)) != cudaSuccess) return e;
     if (n_chunks > 0) {
         const int slices = team_slices(n_chunks);
         k_sums_team<<<(unsigned)(n_chunks * slices), kTeam, smem, s>>>(sv, 0, 1, slices, X, sums);

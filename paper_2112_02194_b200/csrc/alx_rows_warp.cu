@@ -589,6 +589,24 @@ __device__ __forceinline__ void store_row(const float *x, bool ok, int64_t u, co
     }
 }
 
+// rows without observations: A^-1 0 = 0 (grid-wide)
+struct ZeroRows {
+    const int32_t *rows;
+    int64_t count;
+};
+template <int D, typename T> __device__ __forceinline__ void store_zeros(const ZeroRows &zero, const RowOut &out)
+{
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < zero.count * D; t += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t u = zero.rows[t / D];
+        const int c = (int)(t % D);
+        store_elem(reinterpret_cast<T *>(out.table) + u * D + c, 0.f);
+        if (out.cap_slot) {
+            const int slot = out.cap_slot[u];
+            if (slot >= 0) out.cap_out[(int64_t)slot * D + c] = 0.f;
+        }
+    }
+}
+
 // the base matrix in the order of the mma fragments (block-wide)
 template <int D, typename T> __device__ __forceinline__ void load_base(const float *__restrict__ Bmat, float4 *base)
 {
@@ -608,9 +626,10 @@ template <int D, typename T> __device__ __forceinline__ void load_base(const flo
 template <int D, typename T>
 __global__ void __launch_bounds__(WGeo<D, T>::REGS_WARPS * 32, 1)
 k_rows_warp(SideView sv, int64_t last, int64_t count, const int *dual_flag, int64_t primal_count, const int32_t *list,
-            const unsigned long long *list_count, const T *__restrict__ X, const float *__restrict__ Bmat, RowOut out, DevStatus *st)
+            const unsigned long long *list_count, const T *__restrict__ X, const float *__restrict__ Bmat, RowOut out, ZeroRows zero, DevStatus *st)
 {
     using G = WGeo<D, T>;
+    store_zeros<D, T>(zero, out);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float4 *base = reinterpret_cast<float4 *>(smem_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -992,9 +1011,10 @@ __device__ __forceinline__ void sum_parts(PartsFeed &feed, int64_t len, Sums<64,
 
 __global__ void __launch_bounds__(PGeo::WARPS * 32, 1)
 k_rows_cg64(SideView sv, int64_t last, int64_t count, const int *dual_flag, int64_t primal_count, const uint4 *__restrict__ P,
-            const float *__restrict__ Bmat, RowOut out, WarpCg cg, DevStatus *st)
+            const float *__restrict__ Bmat, RowOut out, ZeroRows zero, WarpCg cg, DevStatus *st)
 {
     using G = WGeo<64, float>;
+    store_zeros<64, float>(zero, out);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float4 *base = reinterpret_cast<float4 *>(smem_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1211,20 +1231,7 @@ __global__ void __launch_bounds__(128, 4) k_sums64(SideView sv, int64_t n_chunks
     else write64<3>(acc, dst, lane);
 }
 
-// rows without observations: A^-1 0 = 0
-template <typename T>
-__global__ void k_zero_rows_warp(const int32_t *__restrict__ rows, int64_t count, int d, RowOut out)
-{
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= count * d) return;
-    const int64_t u = rows[t / d];
-    const int c = (int)(t % d);
-    store_elem(reinterpret_cast<T *>(out.table) + u * d + c, 0.f);
-    if (out.cap_slot) {
-        const int slot = out.cap_slot[u];
-        if (slot >= 0) out.cap_out[(int64_t)slot * d + c] = 0.f;
-    }
-}
+template <int D, typename T> __global__ void __launch_bounds__(256) k_zero_rows_warp(ZeroRows zero, RowOut out) { store_zeros<D, T>(zero, out); }
 
 struct WarpRows {
     SideView sv;
@@ -1242,19 +1249,16 @@ struct WarpRows {
     int64_t *launches;
 };
 
-template <typename K> cudaError_t more_smem(K *kernel, size_t bytes)
+// The rows without observations: with the launch of the others (`blocks` of `threads`) where that has a thread for every 32 values,
+// else by a launch of their own, now.
+template <int D, typename T> ZeroRows zero_rows(const WarpRows &a, int64_t blocks, int64_t threads)
 {
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
-template <int D, typename T> cudaError_t zero_rows(const WarpRows &a)
-{
-    const int64_t n_zero = a.offs[1] - a.offs[0];
-    if (n_zero > 0) {
-        k_zero_rows_warp<T><<<(unsigned)((n_zero * D + 255) / 256), 256, 0, a.s>>>(a.sv.order + a.offs[0], n_zero, D, a.out);
-        ++*a.launches;
-    }
-    return cudaGetLastError();
+    const ZeroRows z{a.sv.order + a.offs[0], a.offs[1] - a.offs[0]};
+    if (z.count * D <= blocks * threads * 32) return z;
+    const int64_t grid = (z.count * D + 255) / 256;
+    k_zero_rows_warp<D, T><<<(unsigned)(grid < (1 << 20) ? grid : 1 << 20), 256, 0, a.s>>>(z, a.out);
+    ++*a.launches;
+    return ZeroRows{nullptr, 0};
 }
 
 // rows order[end - 1], order[end - 2] .. by a warp each, down to class `first`; `list` (with its device-side count) instead
@@ -1265,12 +1269,19 @@ cudaError_t whole_rows(const WarpRows &a, int64_t end, const int32_t *list, cons
     static_assert((size_t)G::BASE + G::REGS_WARPS * G::WARP <= 232448, "shared memory");
     const size_t smem = (size_t)G::BASE + G::REGS_WARPS * G::WARP;
     const int64_t n = list ? 0 : end - a.offs[1];
-    if (!list && n <= 0) return cudaSuccess;
-    const cudaError_t e = more_smem(k_rows_warp<D, T>, smem);
+    if (!list && n <= 0) {
+        zero_rows<D, T>(a, 0, 0);
+        return cudaGetLastError();
+    }
+    static SmemOnce allow;
+    const cudaError_t e = allow(k_rows_warp<D, T>, smem);
     if (e != cudaSuccess) return e;
-    const int64_t blocks = list ? 148 : (n + G::ROWS - 1) / G::ROWS;      // few rows: one per SM before two
-    k_rows_warp<D, T><<<(unsigned)(blocks < 148 ? blocks : 148), G::REGS_WARPS * 32, smem, a.s>>>(
-        a.sv, end - 1, n, list ? nullptr : a.dual_flag, end - a.offs[2], list, list_count, reinterpret_cast<const T *>(a.X), a.Bmat, a.out, a.st);
+    int64_t blocks = list ? 148 : (n + G::ROWS - 1) / G::ROWS;      // few rows: one per SM before two
+    if (blocks > 148) blocks = 148;
+    const ZeroRows zero = list ? ZeroRows{nullptr, 0} : zero_rows<D, T>(a, blocks, G::REGS_WARPS * 32);
+    k_rows_warp<D, T><<<(unsigned)blocks, G::REGS_WARPS * 32, smem, a.s>>>(
+        a.sv, end - 1, n, list ? nullptr : a.dual_flag, end - a.offs[2], list, list_count, reinterpret_cast<const T *>(a.X), a.Bmat, a.out, zero,
+        a.st);
     ++*a.launches;
     return cudaGetLastError();
 }
@@ -1295,19 +1306,20 @@ template <int D, typename T> cudaError_t rows_warp_dt(const WarpRows &a)
     cudaError_t e;
     // longest work first
     if (a.n_chunks > 0) {
-        if ((e = more_smem(k_rows_block<D, T, true>, B::SMEM)) != cudaSuccess) return e;
+        static SmemOnce allow;
+        if ((e = allow(k_rows_block<D, T, true>, B::SMEM)) != cudaSuccess) return e;
         k_rows_block<D, T, true><<<(unsigned)a.n_chunks, B::kBlockWarps * 32, B::SMEM, a.s>>>(a.sv, 0, X, a.Bmat, a.partials, a.out, a.st);
         ++*a.launches;
         if ((e = solve_rows<D, T, false>(a, 0)) != cudaSuccess) return e;
     }
     if (end_long > begin_long) {
-        if ((e = more_smem(k_rows_block<D, T, false>, B::SMEM)) != cudaSuccess) return e;
+        static SmemOnce allow;
+        if ((e = allow(k_rows_block<D, T, false>, B::SMEM)) != cudaSuccess) return e;
         k_rows_block<D, T, false><<<(unsigned)(end_long - begin_long), B::kBlockWarps * 32, B::SMEM, a.s>>>(a.sv, end_long - 1, X, a.Bmat, a.partials,
                                                                                                          a.out, a.st);
         ++*a.launches;
     }
-    if ((e = whole_rows<D, T>(a, begin_long, nullptr, nullptr)) != cudaSuccess) return e;
-    return zero_rows<D, T>(a);
+    return whole_rows<D, T>(a, begin_long, nullptr, nullptr);
 }
 
 // fp32 tables of 64 features: long rows and chunks over the parts whatever the solver, the other rows too with conjugate gradients
@@ -1331,17 +1343,19 @@ cudaError_t rows_parts64(const WarpRows &a, bool use_cg, int64_t n_table)
     if (use_cg) {
         if (n > 0) {
             const size_t smem = PGeo::G::BASE + PGeo::WARPS * PGeo::WARP;
-            if ((e = more_smem(k_rows_cg64, smem)) != cudaSuccess) return e;
-            k_rows_cg64<<<(unsigned)(n < 148 ? n : 148), PGeo::WARPS * 32, smem, a.s>>>(a.sv, begin_long - 1, n, a.dual_flag, begin_long - offs[2], P, a.Bmat,
-                                                                                     a.out, a.cg, a.st);
+            static SmemOnce allow;
+            if ((e = allow(k_rows_cg64, smem)) != cudaSuccess) return e;
+            const int64_t blocks = n < 148 ? n : 148;
+            k_rows_cg64<<<(unsigned)blocks, PGeo::WARPS * 32, smem, a.s>>>(a.sv, begin_long - 1, n, a.dual_flag, begin_long - offs[2], P, a.Bmat, a.out,
+                                                                          zero_rows<64, float>(a, blocks, PGeo::WARPS * 32), a.cg, a.st);
             ++*a.launches;
             // the rows conjugate gradients did not finish (none, as a rule: its blocks then return at once)
             if ((e = whole_rows<64, float>(a, begin_long, a.cg.fallback_list, a.cg.counters + 2)) != cudaSuccess) return e;
         }
-    } else if ((e = whole_rows<64, float>(a, begin_long, nullptr, nullptr)) != cudaSuccess) {
-        return e;
+        else zero_rows<64, float>(a, 0, 0);
+        return cudaGetLastError();
     }
-    return zero_rows<64, float>(a);
+    return whole_rows<64, float>(a, begin_long, nullptr, nullptr);
 }
 
 }  // namespace

@@ -381,7 +381,8 @@ template <int D, typename T, int QT> cudaError_t launch_fma(const FmaArgs &a)
 {
     using G = FmaGeo<D, T, QT>;
     static_assert(G::ITEMS <= kTopkTile, "a tile's items fit a candidate buffer");
-    const cudaError_t e = cudaFuncSetAttribute(k_topk_fma<D, T, QT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM);
+    static SmemOnce allow;
+    const cudaError_t e = allow(k_topk_fma<D, T, QT>, G::SMEM);
     if (e != cudaSuccess) return e;
     dim3 grid((unsigned)((a.m + QT - 1) / QT), (unsigned)a.slabs);
     k_topk_fma<D, T, QT><<<grid, kFmaThreads, G::SMEM, a.s>>>(static_cast<const T *>(a.H), a.i_begin, a.i_end, a.Q, a.m, a.k, a.cap,

@@ -310,7 +310,8 @@ cudaError_t launch_topk_umma(const TopkUmma &u, int64_t i_begin, int64_t i_end, 
                              DevStatus *st, cudaStream_t s)
 {
     const size_t smem = sizeof(TopkSmem) + 1024;
-    const cudaError_t e = cudaFuncSetAttribute(k_topk_umma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static SmemOnce allow;
+    const cudaError_t e = allow(k_topk_umma, smem);
     if (e != cudaSuccess) return e;
     dim3 grid((unsigned)(u.m_pad / kTopkQueries), (unsigned)slabs);
     k_topk_umma<<<grid, kThreads, smem, s>>>(u.items, u.queries, i_begin, i_end, m, u.m_pad, k, cap, ex_ptr, ex_idx, slab, lists,

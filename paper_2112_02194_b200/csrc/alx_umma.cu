@@ -1664,7 +1664,8 @@ cudaError_t table_tensor_map(const void *X, int64_t n, CUtensorMap *tm, int box_
 template <int MODE> cudaError_t launch_mode(const Params &p, int grid, cudaStream_t s)
 {
     const size_t smem = smem_bytes<MODE>();
-    cudaError_t e = cudaFuncSetAttribute(k_umma<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static SmemOnce allow;
+    cudaError_t e = allow(k_umma<MODE>, smem);
     if (e != cudaSuccess) return e;
     CUtensorMap tm;
     e = table_tensor_map(p.X, p.n_table, &tm, MODE == kModeGramian ? Ring<MODE>::kRows : 1);
@@ -1702,7 +1703,7 @@ cudaError_t launch_gramian_umma(const void *X, int64_t n, float *partials, cudaS
 
 cudaError_t launch_rows_umma(const SideView &sv, const int64_t *offs, int64_t n_chunks, int64_t n_split_rows,
                              const void *X, const float *Bmat, float *split_partials, RowOut out, DevStatus *st,
-                             cudaStream_t s, int64_t *launches, cudaEvent_t main_begin, cudaEvent_t main_end,
+                             cudaStream_t s, int64_t *launches, cudaEvent_t main_begin, cudaEvent_t main_end, bool capturing,
                              const void *dual_ws, int64_t n_table, const CgOptions &cg, const int32_t *order16, int64_t n4, int64_t n8)
 {
     const int sms = sm_count();
@@ -1731,7 +1732,8 @@ cudaError_t launch_rows_umma(const SideView &sv, const int64_t *offs, int64_t n_
         p.n_split_rows = n_split_rows;
         p.n_items = n_split_rows + n_long;
         const size_t smem = smem_bytes<kModeRows>();
-        e = cudaFuncSetAttribute(k_solve_sums, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        static SmemOnce allow;
+        e = allow(k_solve_sums, smem);
         if (e != cudaSuccess) return e;
         k_solve_sums<<<(int)(p.n_items < sms ? p.n_items : sms), 4 * 128, smem, s>>>(p);
         ++*launches;
@@ -1765,7 +1767,7 @@ cudaError_t launch_rows_umma(const SideView &sv, const int64_t *offs, int64_t n_
         p.fallback_list = cg.fallback_list;
         p.fallback_count = cg.counters + 2;
         const int grid = (int)(n_whole < sms ? n_whole : sms);
-        if (main_begin) cudaEventRecord(main_begin, s);
+        if (main_begin) record_event(main_begin, s, capturing);
         if (cg.enabled && p.dual_flag) {
             // The dual form beyond its condition limit (flag 2): its solutions, already in the table, are the start
             // vectors of a conjugate-gradient pass over the same rows, which works on the d x d system itself and stops
@@ -1803,7 +1805,7 @@ cudaError_t launch_rows_umma(const SideView &sv, const int64_t *offs, int64_t n_
             ++*launches;
         }
         if (e != cudaSuccess) return e;
-        if (main_end) cudaEventRecord(main_end, s);
+        if (main_end) record_event(main_end, s, capturing);
     }
     const int64_t n_zero = offs[1] - offs[0];
     if (n_zero > 0) {
