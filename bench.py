@@ -391,20 +391,21 @@ def run_ours(args, w):
     alu_cg_half = statistics.mean([alu_half - rows_side[sd] * chol_row - 2.0 * ent_side[sd] * d + alu_side[sd] for sd in (0, 1)])
     t_alu_cg = alu_cg_half / (fp32_peak * 1e12)
     t_roof_cg = max(t_bytes, t_tensor + t_alu_cg)
-    fold = st.kernel_path[0] == 1 and e == 4       # fp32 tables with d = 64 on the tensor cores: split operands
+    fold = st.kernel_path[0] == 1 and e == 4 and d == 64       # fp32 tables with d = 64: table of bfloat16 parts
     if st.kernel_path[0] != 1:
         kernel_txt = "k_rows_simple: whole rows on the FP32 ALUs (gather, outer products, Cholesky in shared memory, store)"
     elif fold:
-        kernel_txt = ("k_umma<4>: whole rows of 17..512 entries (item gather by TMA from the bfloat16 parts of the fp32 "
-                      "table, tcgen05 outer products into tensor memory, fold to the 64 x 64 matrix, conjugate gradients "
-                      "on the matrix in registers, Cholesky in shared memory for rows that do not converge, store)")
+        kernel_txt = ("k_rows_cg64: whole rows of 17..512 entries, a warp each (gather from the bfloat16 parts of the fp32 table, "
+                      "mma outer products and conjugate gradients with the matrix in registers, store)")
+    elif not (d == 128 and e == 2):
+        kernel_txt = "k_rows_warp / k_rows_team: whole rows, one or four warps each (gather, mma outer products, Cholesky, store)"
     else:
         kernel_txt = ("k_umma<3> + k_umma<0>: whole rows (item gather by TMA, tcgen05 outer products into tensor memory, "
                       "conjugate gradients on the matrix in tensor memory, Cholesky in tensor memory for rows that do not "
                       "converge or sides the policy moved, store)")
     short_txt = ("rows with at most 16 entries, solved by k_dual64 outside the dominant kernel" if fold else
                  "rows with at most 32 entries, solved by k_dual outside the dominant kernel")
-    long_txt = ("whole rows of more than 512 entries: sums by the chunks kernel, solve by k_solve_sums_fold, outside the "
+    long_txt = ("whole rows of more than 512 entries: sums by k_sums64, solve by k_solve_sums_warp, outside the "
                 "dominant kernel" if fold else
                 "whole rows of more than 1024 entries: sums by the chunks kernel, solve by k_solve_sums, outside the "
                 "dominant kernel")
