@@ -65,6 +65,8 @@ struct alx_ctx {
     int epochs_run = 0;            // alx_epoch calls since the matrix was set
     int64_t epoch_launches = 0;    // kernels in the graph
     bool capturing = false;
+    bool by_stamps = false;        // the last half-epoch's times are in `stamps`, not in the events
+    unsigned long long *stamps = nullptr;          // device, [kStampSlots]
     int last_side = 0;             // side of the last half-epoch: its flag and policy record stay on the device until alx_get_stats asks
     double *loss_partials_buf = nullptr;
     unsigned *loss_counter = nullptr;              // zero between calls
@@ -454,7 +456,7 @@ int64_t dual_rows_of(const alx_ctx *c, int side)
 }
 
 // the Gramian and the base matrix of a table; `solve`: also what the rows' dual form needs of the base matrix
-alx_status gramian_of(alx_ctx *c, int table_side, bool solve)
+alx_status gramian_of(alx_ctx *c, int table_side, bool solve, unsigned long long *stamps = nullptr)
 {
     if (tensor_path(c)) {
         ALX_CUDA(c, launch_gramian_umma(c->table[table_side], c->n[table_side], c->gram_partials, c->stream, &c->launches));
@@ -466,7 +468,7 @@ alx_status gramian_of(alx_ctx *c, int table_side, bool solve)
         return ALX_OK;
     }
     ALX_CUDA(c, launch_gramian(c->table[table_side], c->bf16, c->n[table_side], c->opt.d, c->gram_partials,
-                               c->G64[table_side], c->Bmat, c->opt.alpha0, c->opt.lambda, c->stream, &c->launches));
+                               c->G64[table_side], c->Bmat, c->opt.alpha0, c->opt.lambda, stamps, c->stream, &c->launches));
     if (solve && dual64(c)) ALX_CUDA(c, launch_dual64_prepare(c->Bmat, c->dual_ws, dual_cond_limit(c), c->stream, &c->launches));
     if (solve && dual_warp(c)) {
         const float most = c->bf16 ? kDualWarpLimitBf16 : kDualWarpLimitF32;
@@ -493,14 +495,16 @@ alx_status half_epoch_impl(alx_ctx *c, int side, const int32_t *cap_slot, float 
     const int fixed = 1 - side;
     if (!c->have_table[fixed]) return fail(c, ALX_ERR_BAD_STATE, "the fixed table has not been set");
     NvtxRange range(side == ALX_ROWS ? "alx half-epoch: rows" : "alx half-epoch: columns");
-    ALX_CUDA(c, record_event(c->ev[0], c->stream, c->capturing));
+    // (the launches of the d <= 64 kernels without conjugate gradients are the ones short enough to mind events in a graph)
+    unsigned long long *stamps = c->capturing && warp_path(c) && !cg64(c) ? c->stamps : nullptr;
+    if (!stamps) ALX_CUDA(c, record_event(c->ev[0], c->stream, c->capturing));
     alx_status st;
     {
         NvtxRange r("alx Gramian + base matrix");
-        st = gramian_of(c, fixed, dual_rows_of(c, side) > 0);
+        st = gramian_of(c, fixed, dual_rows_of(c, side) > 0, stamps);
     }
     if (st != ALX_OK) return st;
-    ALX_CUDA(c, record_event(c->ev[1], c->stream, c->capturing));
+    if (!stamps) ALX_CUDA(c, record_event(c->ev[1], c->stream, c->capturing));
     NvtxRange rows_range("alx rows: gather, sums, solve, store");
     RowOut out{c->table[side], cap_slot, cap_out};
     note_half_epoch(c, side);
@@ -515,7 +519,7 @@ alx_status half_epoch_impl(alx_ctx *c, int side, const int32_t *cap_slot, float 
         if (cg64(c)) ALX_CUDA(c, record_event(c->ev[3], c->stream, c->capturing));
         ALX_CUDA(c, launch_rows_warp(side_view(c, side), c->class_offs[side], c->n_chunks[side], c->n_split_rows[side], c->table[fixed],
                                      c->n[fixed], c->parts, c->bf16, c->opt.d, c->Bmat, c->split_partials, out, c->status, cg_options(c, side),
-                                     n_dual > 0 ? dual_flag_of(c) : nullptr, c->stream, &c->launches));
+                                     n_dual > 0 ? dual_flag_of(c) : nullptr, stamps, c->stream, &c->launches));
         if (cg64(c)) ALX_CUDA(c, record_event(c->ev[4], c->stream, c->capturing));
     } else if (tensor_path(c)) {
         ALX_CUDA(c, cudaMemsetAsync(c->cg_counters, 0, 5 * sizeof(unsigned long long), c->stream));
@@ -534,7 +538,8 @@ alx_status half_epoch_impl(alx_ctx *c, int side, const int32_t *cap_slot, float 
         ALX_CUDA(c, launch_rows_simple(side_view(c, side), c->class_offs[side], c->n_chunks[side], c->n_split_rows[side], c->table[fixed],
                                        c->bf16, c->opt.d, c->Bmat, c->split_partials, out, c->status, c->stream, &c->launches));
     }
-    ALX_CUDA(c, record_event(c->ev[2], c->stream, c->capturing));
+    if (!stamps) ALX_CUDA(c, record_event(c->ev[2], c->stream, c->capturing));
+    c->by_stamps = false;
     c->have_table[side] = true;
     c->have_gram[side] = false;
     return ALX_OK;
@@ -618,6 +623,8 @@ alx_status create_impl(const alx_options *opt, const alx_ctx *parent, alx_ctx **
         int64_t n_part = gramian_partials(nmax);
         if (gramian_umma_partials() > n_part) n_part = gramian_umma_partials();
         ALX_ALLOC(c, c->gram_partials, n_part * d * d);
+        ALX_ALLOC(c, c->stamps, kStampSlots);
+        ALX_CUDA(c, cudaMemsetAsync(c->stamps, 0, kStampSlots * sizeof(unsigned long long), c->stream));
         ALX_ALLOC(c, c->loss_counter, 1);
         ALX_CUDA(c, cudaMemsetAsync(c->loss_counter, 0, sizeof(unsigned), c->stream));
         ALX_ALLOC(c, c->status, 1);
@@ -947,6 +954,7 @@ alx_status alx_epoch(alx_ctx *c)
         c->have_gram[ALX_ROWS] = true;
         c->have_gram[ALX_COLS] = false;
         note_half_epoch(c, ALX_COLS);
+        c->by_stamps = warp_path(c) && !cg64(c);
         return ALX_OK;
     }
     alx_status st = half_epoch_impl(c, ALX_ROWS, nullptr, nullptr);
@@ -1338,9 +1346,17 @@ alx_status alx_get_stats(alx_ctx *c, alx_stats *out)
     DeviceGuard guard(c->device);
     ALX_CUDA(c, cudaStreamSynchronize(c->stream));
     float ms = 0.f;
-    if (cudaEventElapsedTime(&ms, c->ev[0], c->ev[1]) == cudaSuccess) c->stats.ms_gramian = ms; else cudaGetLastError();
-    if (cudaEventElapsedTime(&ms, c->ev[1], c->ev[2]) == cudaSuccess) c->stats.ms_rows = ms; else cudaGetLastError();
-    if (cudaEventElapsedTime(&ms, c->ev[0], c->ev[2]) == cudaSuccess) c->stats.ms_half_epoch = ms; else cudaGetLastError();
+    if (c->by_stamps) {
+        unsigned long long t[kStampSlots];
+        ALX_CUDA(c, cudaMemcpy(t, c->stamps, sizeof t, cudaMemcpyDeviceToHost));
+        c->stats.ms_gramian = 1e-6 * (double)(t[kStampGramian] - t[kStampBegin]);
+        c->stats.ms_rows = t[kStampEnd] > t[kStampGramian] ? 1e-6 * (double)(t[kStampEnd] - t[kStampGramian]) : 0.0;
+        c->stats.ms_half_epoch = c->stats.ms_gramian + c->stats.ms_rows;
+    } else {
+        if (cudaEventElapsedTime(&ms, c->ev[0], c->ev[1]) == cudaSuccess) c->stats.ms_gramian = ms; else cudaGetLastError();
+        if (cudaEventElapsedTime(&ms, c->ev[1], c->ev[2]) == cudaSuccess) c->stats.ms_rows = ms; else cudaGetLastError();
+        if (cudaEventElapsedTime(&ms, c->ev[0], c->ev[2]) == cudaSuccess) c->stats.ms_half_epoch = ms; else cudaGetLastError();
+    }
     c->stats.ms_main_kernel = 0.0;
     if (c->main_timed) {
         if (cudaEventElapsedTime(&ms, c->ev[3], c->ev[4]) == cudaSuccess) c->stats.ms_main_kernel = ms; else cudaGetLastError();

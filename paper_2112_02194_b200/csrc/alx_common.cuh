@@ -82,6 +82,19 @@ struct RowOut {
     float *cap_out;          // [slots x d] fp32 solutions before rounding
 };
 
+// ---- device-side time stamps ------------------------------------------------------------------
+// A timing event that is a node of a graph costs the GPU 4 to 5 us, more than a kernel of a small matrix: there the kernels note
+// the time themselves (nanoseconds of the global timer, which only grows: a slot needs no reset).  Null: not wanted.
+enum StampSlot { kStampBegin = 0, kStampGramian = 1, kStampEnd = 2, kStampSlots = 3 };
+__device__ __forceinline__ void stamp(unsigned long long *slot)
+{
+    if (slot && threadIdx.x == 0) {
+        unsigned long long t;
+        asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+        atomicMax(slot, t);
+    }
+}
+
 // ---- small host pieces of the launchers -----------------------------------------------------------
 // Lets a kernel use more than the default dynamic shared memory, once per device (the call costs a microsecond of host time,
 // which a half-epoch of a small matrix pays several times over).  One static object per kernel.
@@ -147,7 +160,7 @@ cudaError_t launch_convert(const void *src, int src_bf16, void *dst, int dst_bf1
 // alx_gramian.cu
 int64_t gramian_partials(int64_t n);
 cudaError_t launch_gramian(const void *X, int bf16, int64_t n, int d, float *partials, double *G64, float *Bmat,
-                           float alpha0, float lambda, cudaStream_t s, int64_t *launches);
+                           float alpha0, float lambda, unsigned long long *stamps, cudaStream_t s, int64_t *launches);
 
 cudaError_t launch_gramian_reduce(const float *partials, int64_t n_partials, int d, double *G64, float *Bmat,
                                   float alpha0, float lambda, cudaStream_t s, int64_t *launches);
@@ -227,7 +240,7 @@ inline int parts64_long_class(const int64_t *class_offs_host)
 // flag, set when the rows of class 1 have been solved in the dual form
 cudaError_t launch_rows_warp(const SideView &sv, const int64_t *class_offs_host, int64_t n_chunks, int64_t n_split_rows, const void *X,
                              int64_t n_table, void *parts, int bf16, int d, const float *Bmat, float *split_partials, RowOut out, DevStatus *st,
-                             const CgOptions &cg, const int *dual_flag, cudaStream_t s, int64_t *launches);
+                             const CgOptions &cg, const int *dual_flag, unsigned long long *stamps, cudaStream_t s, int64_t *launches);
 
 // alx_rows_team.cu: fp32 tables of 128 features, four warps per row (kernels != 1); `sums`: team_sums_floats() floats
 int64_t team_sums_floats(const int64_t *class_offs_host, int64_t n_chunks);

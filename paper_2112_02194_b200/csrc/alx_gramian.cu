@@ -64,8 +64,9 @@ template <int D> __device__ __forceinline__ void load_tile(const __nv_bfloat16 *
 
 template <int D, typename T>
 __global__ void __launch_bounds__(GramGeo<D, T>::THREADS, 1) k_gramian_tiles(const T *__restrict__ X, int64_t n, int64_t rows_per_block,
-                                                                            float *__restrict__ partials)
+                                                                            float *__restrict__ partials, unsigned long long *begin)
 {
+    if (blockIdx.x == 0) stamp(begin);
     using G = GramGeo<D, T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float *red = reinterpret_cast<float *>(smem_raw + 2 * G::STAGE);
@@ -177,7 +178,8 @@ __device__ __forceinline__ void reduce_partials(const float *__restrict__ partia
 
 template <int D, typename T>
 __global__ void __launch_bounds__(256) k_gramian_reduce_tiles(const float *__restrict__ partials, int64_t n_partials, double *__restrict__ G64,
-                                                              float *__restrict__ Bmat, float alpha0, float lambda)
+                                                              float *__restrict__ Bmat, float alpha0, float lambda,
+                                                              unsigned long long *done)
 {
     using G = GramGeo<D, T>;
     reduce_partials<true>(partials, n_partials, G::ELEMS, D, G64, Bmat, alpha0, lambda, [](int e, int &i, int &l) {
@@ -187,6 +189,7 @@ __global__ void __launch_bounds__(256) k_gramian_reduce_tiles(const float *__res
         i = G::feature(I, ab / G::TILE);
         l = G::feature(tile - I * (I + 1) / 2, ab % G::TILE);
     });
+    stamp(done);
 }
 
 // full d x d partials (the tensor-core Gramian)
@@ -197,7 +200,8 @@ __global__ void __launch_bounds__(256) k_gramian_reduce(const float *__restrict_
 }
 
 template <int D, typename T>
-cudaError_t gramian_tiles_dt(const void *X, int64_t n, float *partials, double *G64, float *Bmat, float alpha0, float lambda, cudaStream_t s)
+cudaError_t gramian_tiles_dt(const void *X, int64_t n, float *partials, double *G64, float *Bmat, float alpha0, float lambda,
+                             unsigned long long *stamps, cudaStream_t s)
 {
     using G = GramGeo<D, T>;
     static_assert(G::ELEMS <= D * D && G::SMEM <= 232448, "sizes");
@@ -205,26 +209,28 @@ cudaError_t gramian_tiles_dt(const void *X, int64_t n, float *partials, double *
     const cudaError_t e = allow(k_gramian_tiles<D, T>, G::SMEM);
     if (e != cudaSuccess) return e;
     const int64_t blocks = gramian_partials(n), per = (n + blocks - 1) / blocks;
-    k_gramian_tiles<D, T><<<(unsigned)blocks, G::THREADS, G::SMEM, s>>>(static_cast<const T *>(X), n, per, partials);
-    k_gramian_reduce_tiles<D, T><<<(G::ELEMS + 31) / 32, 256, 0, s>>>(partials, blocks, G64, Bmat, alpha0, lambda);
+    k_gramian_tiles<D, T><<<(unsigned)blocks, G::THREADS, G::SMEM, s>>>(static_cast<const T *>(X), n, per, partials, stamps ? stamps + kStampBegin : nullptr);
+    k_gramian_reduce_tiles<D, T><<<(G::ELEMS + 31) / 32, 256, 0, s>>>(partials, blocks, G64, Bmat, alpha0, lambda,
+                                                                             stamps ? stamps + kStampGramian : nullptr);
     return cudaGetLastError();
 }
 
 template <int D>
-cudaError_t gramian_tiles_d(const void *X, int bf16, int64_t n, float *partials, double *G64, float *Bmat, float alpha0, float lambda, cudaStream_t s)
+cudaError_t gramian_tiles_d(const void *X, int bf16, int64_t n, float *partials, double *G64, float *Bmat, float alpha0, float lambda,
+                            unsigned long long *stamps, cudaStream_t s)
 {
-    return bf16 ? gramian_tiles_dt<D, __nv_bfloat16>(X, n, partials, G64, Bmat, alpha0, lambda, s)
-                : gramian_tiles_dt<D, float>(X, n, partials, G64, Bmat, alpha0, lambda, s);
+    return bf16 ? gramian_tiles_dt<D, __nv_bfloat16>(X, n, partials, G64, Bmat, alpha0, lambda, stamps, s)
+                : gramian_tiles_dt<D, float>(X, n, partials, G64, Bmat, alpha0, lambda, stamps, s);
 }
 
 cudaError_t gramian_tiles(const void *X, int bf16, int64_t n, int d, float *partials, double *G64, float *Bmat, float alpha0, float lambda,
-                          cudaStream_t s)
+                          unsigned long long *stamps, cudaStream_t s)
 {
     switch (d) {
-    case 16: return gramian_tiles_d<16>(X, bf16, n, partials, G64, Bmat, alpha0, lambda, s);
-    case 32: return gramian_tiles_d<32>(X, bf16, n, partials, G64, Bmat, alpha0, lambda, s);
-    case 64: return gramian_tiles_d<64>(X, bf16, n, partials, G64, Bmat, alpha0, lambda, s);
-    case 128: return gramian_tiles_d<128>(X, bf16, n, partials, G64, Bmat, alpha0, lambda, s);
+    case 16: return gramian_tiles_d<16>(X, bf16, n, partials, G64, Bmat, alpha0, lambda, stamps, s);
+    case 32: return gramian_tiles_d<32>(X, bf16, n, partials, G64, Bmat, alpha0, lambda, stamps, s);
+    case 64: return gramian_tiles_d<64>(X, bf16, n, partials, G64, Bmat, alpha0, lambda, stamps, s);
+    case 128: return gramian_tiles_d<128>(X, bf16, n, partials, G64, Bmat, alpha0, lambda, stamps, s);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -247,10 +253,10 @@ cudaError_t launch_gramian_reduce(const float *partials, int64_t n_partials, int
 }
 
 cudaError_t launch_gramian(const void *X, int bf16, int64_t n, int d, float *partials, double *G64, float *Bmat,
-                           float alpha0, float lambda, cudaStream_t s, int64_t *launches)
+                           float alpha0, float lambda, unsigned long long *stamps, cudaStream_t s, int64_t *launches)
 {
     *launches += 2;
-    return gramian_tiles(X, bf16, n, d, partials, G64, Bmat, alpha0, lambda, s);
+    return gramian_tiles(X, bf16, n, d, partials, G64, Bmat, alpha0, lambda, stamps, s);
 }
 
 }  // namespace alx
@@ -384,7 +390,7 @@ alx_status alx_gramian_noalloc(const void *table, alx_dtype dtype, int64_t n, in
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     float *pieces = scratch, *base_out = scratch + kNoAllocPieceFloats;
     // every piece the reduction reads is written in full by the launch before it: nothing has to start at zero
-    const cudaError_t e = gramian_tiles(table, dtype == ALX_BF16, n, d, pieces, gramian, base_out, 0.f, 0.f, s);
+    const cudaError_t e = gramian_tiles(table, dtype == ALX_BF16, n, d, pieces, gramian, base_out, 0.f, 0.f, nullptr, s);
     if (e != cudaSuccess)
         return noalloc_fail(ALX_ERR_CUDA, std::string("alx_gramian_noalloc: launch failed: ") + cudaGetErrorString(e));
     g_noalloc_error.clear();

@@ -607,6 +607,14 @@ template <int D, typename T> __device__ __forceinline__ void store_zeros(const Z
     }
 }
 
+// The launch before this one may still run (programmatic dependent launch: it solves other rows).  The last thing a block does
+// is wait for it, so that whatever follows this grid follows both; then the time is noted.
+__device__ __forceinline__ void finish_after_previous(unsigned long long *done)
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    stamp(done);
+}
+
 // the base matrix in the order of the mma fragments (block-wide)
 template <int D, typename T> __device__ __forceinline__ void load_base(const float *__restrict__ Bmat, float4 *base)
 {
@@ -626,7 +634,7 @@ template <int D, typename T> __device__ __forceinline__ void load_base(const flo
 template <int D, typename T>
 __global__ void __launch_bounds__(WGeo<D, T>::REGS_WARPS * 32, 1)
 k_rows_warp(SideView sv, int64_t last, int64_t count, const int *dual_flag, int64_t primal_count, const int32_t *list,
-            const unsigned long long *list_count, const T *__restrict__ X, const float *__restrict__ Bmat, RowOut out, ZeroRows zero, DevStatus *st)
+            const unsigned long long *list_count, const T *__restrict__ X, const float *__restrict__ Bmat, RowOut out, ZeroRows zero, unsigned long long *done, DevStatus *st)
 {
     using G = WGeo<D, T>;
     store_zeros<D, T>(zero, out);
@@ -637,13 +645,16 @@ k_rows_warp(SideView sv, int64_t last, int64_t count, const int *dual_flag, int6
     unsigned char *work = mine + 2 * G::STAGE;
     if (dual_flag && *dual_flag) count = primal_count;
     if (list_count) count = (int64_t)*list_count;
-    if ((int64_t)blockIdx.x * G::ROWS >= count) return;
+    if ((int64_t)blockIdx.x * G::ROWS >= count) {
+        finish_after_previous(done);
+        return;
+    }
     load_base<D, T>(Bmat, base);
     __syncthreads();
     const int64_t warps = (int64_t)gridDim.x * G::REGS_WARPS;
     auto row_at = [&](int64_t k) -> int64_t { return list ? list[k] : sv.order[last - k]; };
     int64_t item = ((int64_t)warp * gridDim.x + blockIdx.x) * G::ROWS;
-    if (item >= count) return;
+    if (item >= count) return;      // (never a block's first warp)
     Feed<D, T> feed;
     feed.X = X;
     feed.idx = sv.idx;
@@ -695,6 +706,7 @@ k_rows_warp(SideView sv, int64_t last, int64_t count, const int *dual_flag, int6
         beg = bn;
         end = en;
     }
+    if (warp == 0) finish_after_previous(done);
 }
 
 // ---- long rows and chunks of split rows: a block of warps, each a slice of the entries; the slices' sums are added in warp
@@ -768,6 +780,7 @@ k_rows_block(SideView sv, int64_t last, const T *__restrict__ X, const float *__
     using G = WGeo<D, T>;
     using B = BGeo<D, T>;
     constexpr int kBlockWarps = B::kBlockWarps;
+    asm volatile("griddepcontrol.launch_dependents;");      // the rows of a warp each may start beside these
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float4 *base = reinterpret_cast<float4 *>(smem_raw);
     float *work = reinterpret_cast<float *>(smem_raw + G::BASE);
@@ -1245,6 +1258,7 @@ struct WarpRows {
     DevStatus *st;
     WarpCg cg;
     const int *dual_flag;      // set on the device when the rows of class 1 have been solved in the dual form
+    unsigned long long *stamps;      // time stamps of the half-epoch, or null
     cudaStream_t s;
     int64_t *launches;
 };
@@ -1263,7 +1277,7 @@ template <int D, typename T> ZeroRows zero_rows(const WarpRows &a, int64_t block
 
 // rows order[end - 1], order[end - 2] .. by a warp each, down to class `first`; `list` (with its device-side count) instead
 template <int D, typename T>
-cudaError_t whole_rows(const WarpRows &a, int64_t end, const int32_t *list, const unsigned long long *list_count)
+cudaError_t whole_rows(const WarpRows &a, int64_t end, const int32_t *list, const unsigned long long *list_count, bool after_block_rows)
 {
     using G = WGeo<D, T>;
     static_assert((size_t)G::BASE + G::REGS_WARPS * G::WARP <= 232448, "shared memory");
@@ -1279,9 +1293,21 @@ cudaError_t whole_rows(const WarpRows &a, int64_t end, const int32_t *list, cons
     int64_t blocks = list ? 148 : (n + G::ROWS - 1) / G::ROWS;      // few rows: one per SM before two
     if (blocks > 148) blocks = 148;
     const ZeroRows zero = list ? ZeroRows{nullptr, 0} : zero_rows<D, T>(a, blocks, G::REGS_WARPS * 32);
-    k_rows_warp<D, T><<<(unsigned)blocks, G::REGS_WARPS * 32, smem, a.s>>>(
-        a.sv, end - 1, n, list ? nullptr : a.dual_flag, end - a.offs[2], list, list_count, reinterpret_cast<const T *>(a.X), a.Bmat, a.out, zero,
-        a.st);
+    cudaLaunchAttribute beside[1];
+    beside[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    beside[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(G::REGS_WARPS * 32);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = a.s;
+    cfg.attrs = beside;
+    // beside k_rows_block, where that is the launch before this one (a launch of the rows without observations may be between)
+    cfg.numAttrs = after_block_rows && zero.rows ? 1 : 0;
+    const cudaError_t el = cudaLaunchKernelEx(&cfg, k_rows_warp<D, T>, a.sv, end - 1, n, list ? (const int *)nullptr : a.dual_flag, end - a.offs[2], list,
+                                              list_count, reinterpret_cast<const T *>(a.X), a.Bmat, a.out, zero,
+                                              a.stamps ? a.stamps + kStampEnd : (unsigned long long *)nullptr, a.st);
+    if (el != cudaSuccess) return el;
     ++*a.launches;
     return cudaGetLastError();
 }
@@ -1319,7 +1345,7 @@ template <int D, typename T> cudaError_t rows_warp_dt(const WarpRows &a)
                                                                                                          a.out, a.st);
         ++*a.launches;
     }
-    return whole_rows<D, T>(a, begin_long, nullptr, nullptr);
+    return whole_rows<D, T>(a, begin_long, nullptr, nullptr, end_long > begin_long);
 }
 
 // fp32 tables of 64 features: long rows and chunks over the parts whatever the solver, the other rows too with conjugate gradients
@@ -1350,22 +1376,22 @@ cudaError_t rows_parts64(const WarpRows &a, bool use_cg, int64_t n_table)
                                                                           zero_rows<64, float>(a, blocks, PGeo::WARPS * 32), a.cg, a.st);
             ++*a.launches;
             // the rows conjugate gradients did not finish (none, as a rule: its blocks then return at once)
-            if ((e = whole_rows<64, float>(a, begin_long, a.cg.fallback_list, a.cg.counters + 2)) != cudaSuccess) return e;
+            if ((e = whole_rows<64, float>(a, begin_long, a.cg.fallback_list, a.cg.counters + 2, false)) != cudaSuccess) return e;
         }
         else zero_rows<64, float>(a, 0, 0);
         return cudaGetLastError();
     }
-    return whole_rows<64, float>(a, begin_long, nullptr, nullptr);
+    return whole_rows<64, float>(a, begin_long, nullptr, nullptr, false);
 }
 
 }  // namespace
 
 cudaError_t launch_rows_warp(const SideView &sv, const int64_t *offs, int64_t n_chunks, int64_t n_split_rows, const void *X, int64_t n_table,
                              void *parts, int bf16, int d, const float *Bmat, float *partials, RowOut out, DevStatus *st, const CgOptions &cg,
-                             const int *dual_flag, cudaStream_t s, int64_t *launches)
+                             const int *dual_flag, unsigned long long *stamps, cudaStream_t s, int64_t *launches)
 {
     const WarpRows a{sv, offs, n_chunks, n_split_rows, X, parts, Bmat, partials, out, st,
-                     WarpCg{cg.max_iter, cg.warm_start ? 1 : 0, cg.tol * cg.tol, cg.counters, cg.fallback_list}, dual_flag, s, launches};
+                     WarpCg{cg.max_iter, cg.warm_start ? 1 : 0, cg.tol * cg.tol, cg.counters, cg.fallback_list}, dual_flag, stamps, s, launches};
     switch (d) {
     case 16: return bf16 ? rows_warp_dt<16, __nv_bfloat16>(a) : rows_warp_dt<16, float>(a);
     case 32: return bf16 ? rows_warp_dt<32, __nv_bfloat16>(a) : rows_warp_dt<32, float>(a);
