@@ -26,6 +26,7 @@ constexpr int kFmaQueries = 16;
 template <int D, typename T, int QT> struct FmaGeo {
     static constexpr int TQ = 4, QG = QT / TQ, IG = kFmaThreads / QG;
     static constexpr int TI = QT >= 64 ? 8 : QT / 4;
+    static constexpr int WQ = QG < 4 ? QG : 4, WI = 32 / WQ;     // a warp's lanes: WI item groups x WQ query groups
     static constexpr int ITEMS = IG * TI;                        // items per tile
     static constexpr int FC = D * (int)sizeof(T) < 128 ? D : 128 / (int)sizeof(T);      // features per pipeline step: whole lines
     static constexpr int NC = D / FC;
@@ -58,7 +59,7 @@ k_topk_fma(const T *__restrict__ H, int64_t i_begin, int64_t i_end, const float 
     __shared__ float thr_s[QT];
     __shared__ int cnt_s[QT], checked_s[QT];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int ig = tid % G::IG, qg = tid / G::IG;
+    const int ig = warp % (G::IG / G::WI) * G::WI + lane % G::WI, qg = warp / (G::IG / G::WI) * G::WQ + lane / G::WI;
     const int64_t q0 = (int64_t)blockIdx.x * QT;
     const int64_t i0 = i_begin + (int64_t)blockIdx.y * slab;
     const int64_t i1 = i0 + slab < i_end ? i0 + slab : i_end;
@@ -185,36 +186,48 @@ k_topk_fma(const T *__restrict__ H, int64_t i_begin, int64_t i_end, const float 
 }
 
 // ---- merge -------------------------------------------------------------------------------------------------------------
-constexpr int kMergeThreads = 256;
+constexpr int kMergeThreads = 512;
 constexpr int kMergeExcluded = 1024;      // exclusion lists up to this length are searched in shared memory
 constexpr int kMergeKeys = 4096;
 constexpr int kMergePer = kMergeKeys / kMergeThreads;
+constexpr int kMergeBins = 2048;
+constexpr int kMergeLists = kTopkMostSlabs * kTopkListsPerSlab;      // no phase has more lists per query
 
 // A block per query, after each phase: the phase's candidates and the k best of the phases before (carry), without the
-// excluded ids and those below the threshold the phase started from, are cut to the k best -- bisection over the keys' bits as
-// in warp_keep_best, here with block-wide counts.  `last`: they are ranked by counting and written out; otherwise they are
+// excluded ids and those below the threshold the phase started from, are cut to the k best -- a histogram of the scores finds
+// the bin of the k-th, then bisection as in warp_keep_best (here with block-wide counts) has the few steps within it left.  `last`: they are ranked by counting and written out; otherwise they are
 // carried on and the k-th score becomes the next phase's threshold.  Lists in groups, so that any number of candidates fits.
 // (The lists of query q: entry p of list l at ((l * query blocks + q / qb) * cap + p) * qb + q % qb, qb queries interleaved.)
-__global__ void __launch_bounds__(kMergeThreads) k_topk_merge(const uint64_t *__restrict__ lists, const int32_t *__restrict__ list_cnt,
+// Bound: latency.  The counts of all lists are one load, scanned; then every candidate of the group has a thread's register,
+// whose loads are all in flight together (a warp per list, list after list, took 23 us for 3 queries and now 7 to 11,
+// 71 us for 2048 and now 52 to 71: there it is bound by the 32-byte sectors of the interleaved lists).
+__global__ void __launch_bounds__(kMergeThreads, 3) k_topk_merge(const uint64_t *__restrict__ lists, const int32_t *__restrict__ list_cnt,
                                                               unsigned *gtau, uint64_t *carry, int first, int last, int64_t m, int k,
                                                               int cap, int n_lists, int qb, const int64_t *__restrict__ ex_ptr,
                                                               const int32_t *__restrict__ ex_idx, int32_t *__restrict__ ids_out,
                                                               float *__restrict__ scores_out)
 {
-    __shared__ uint64_t keys[kMergeKeys];
-    __shared__ int n_s, cnt_s[2][kMergeThreads / 32];
+    __shared__ uint64_t best[kMergeThreads];          // the k best so far, in any order (0: none)
+    __shared__ int start_s[kMergeLists + 1];          // candidates of the lists before
+    __shared__ uint16_t list_s[kMergeKeys];           // the list that a candidate of the group is on
+    __shared__ int n_s, cnt_s[2][kMergeThreads / 32], max_s[2][kMergeThreads / 32];
     __shared__ int32_t ex_s[kMergeExcluded];
+    __shared__ int hist[kMergeBins], bin_s, bin_above;
+    __shared__ uint32_t bin_lo, bin_hi;
+    __shared__ uint32_t ex_bits[kMergeThreads];       // a bit per excluded id (by its low bits): most candidates need no search
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t q = blockIdx.x;
     const uint64_t thr = (uint64_t)gtau[q] << 32;
     const int64_t q_blocks = (m + qb - 1) / qb;
-    auto block_sum = [&](int c, int half) {
+    int flip = 0;
+    auto block_sum = [&](int c) {
+        flip ^= 1;
         c = __reduce_add_sync(0xFFFFFFFFu, c);
-        if (lane == 0) cnt_s[half][warp] = c;
+        if (lane == 0) cnt_s[flip][warp] = c;
         __syncthreads();
         c = 0;
 #pragma unroll
-        for (int w = 0; w < kMergeThreads / 32; ++w) c += cnt_s[half][w];
+        for (int w = 0; w < kMergeThreads / 32; ++w) c += cnt_s[flip][w];
         return c;
     };
     const int64_t ex0 = ex_ptr ? ex_ptr[q] : 0;
@@ -222,8 +235,10 @@ __global__ void __launch_bounds__(kMergeThreads) k_topk_merge(const uint64_t *__
     const bool ex_here = ex_n <= kMergeExcluded;
     if (ex_here)
         for (int p = tid; p < (int)ex_n; p += kMergeThreads) ex_s[p] = ex_idx[ex0 + p];
+    ex_bits[tid] = 0;
     auto left_out = [&](int32_t id) {
         if (!ex_here) return excluded(ex_ptr, ex_idx, q, id);
+        if (!(ex_bits[(uint32_t)id / 32 % kMergeThreads] >> ((uint32_t)id % 32) & 1u)) return false;
         int lo = 0, hi = (int)ex_n;
         while (lo < hi) {
             const int mid = (lo + hi) >> 1;
@@ -231,127 +246,193 @@ __global__ void __launch_bounds__(kMergeThreads) k_topk_merge(const uint64_t *__
         }
         return lo < (int)ex_n && ex_s[lo] == id;
     };
-    if (tid == 0) n_s = 0;
-    int c = 0, longest = 1;
-    for (int l = tid; l < n_lists; l += kMergeThreads) {
-        const int cl = list_cnt[(int64_t)l * m + q];
-        c += cl;
-        longest = max(longest, cl);
-    }
-    const int total = block_sum(c, 0);
-    longest = __reduce_max_sync(0xFFFFFFFFu, longest);
-    if (lane == 0) cnt_s[1][warp] = longest;
-    if (!first)
-        for (int p = tid; p < k; p += kMergeThreads) {
-            const uint64_t key = carry[q * k + p];
-            if (key) keys[atomicAdd(&n_s, 1)] = key;
-        }
-    __syncthreads();
+    if (tid < k) best[tid] = first ? 0 : carry[q * k + tid];
+    // where every list's candidates begin: thread t has lists kScan t .. kScan t + kScan - 1
+    constexpr int kScan = kMergeLists / kMergeThreads;
+    int cl[kScan], mine = 0, longest = 1;
 #pragma unroll
-    for (int w = 0; w < kMergeThreads / 32; ++w) longest = max(longest, cnt_s[1][w]);
+    for (int j = 0; j < kScan; ++j) {
+        const int l = tid * kScan + j;
+        cl[j] = l < n_lists ? list_cnt[(int64_t)l * m + q] : 0;
+        mine += cl[j];
+        longest = max(longest, cl[j]);
+    }
+    int upto = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xFFFFFFFFu, upto, o);
+        if (lane >= o) upto += v;
+    }
+    longest = __reduce_max_sync(0xFFFFFFFFu, longest);
+    if (lane == 31) { cnt_s[0][warp] = upto; max_s[0][warp] = longest; }
+    __syncthreads();
+    int at = upto - mine;
+#pragma unroll
+    for (int w = 0; w < kMergeThreads / 32; ++w) {
+        if (w < warp) at += cnt_s[0][w];
+        longest = max(longest, max_s[0][w]);
+    }
+#pragma unroll
+    for (int j = 0; j < kScan; ++j) {
+        start_s[tid * kScan + j] = at;
+        at += cl[j];
+    }
+    if (tid == kMergeThreads - 1) start_s[kMergeLists] = at;
+    if (ex_here)
+        for (int p = tid; p < (int)ex_n; p += kMergeThreads) atomicOr(&ex_bits[(uint32_t)ex_s[p] / 32 % kMergeThreads], 1u << ((uint32_t)ex_s[p] % 32));
+    __syncthreads();
+    const int total = start_s[kMergeLists];
     const int group = total <= kMergeKeys - k ? n_lists : (kMergeKeys - k) / longest;
-    int flip = 0;
+    int n_best = first ? 0 : k;
     for (int s0 = 0; s0 < n_lists; s0 += group) {
         const int s1 = s0 + group < n_lists ? s0 + group : n_lists;
-        for (int s = s0 + warp; s < s1; s += kMergeThreads / 32) {
-            const int cnt = list_cnt[(int64_t)s * m + q];
-            const uint64_t *src = lists + ((int64_t)s * q_blocks + q / qb) * cap * qb + q % qb;
-            for (int p0 = 0; p0 < cnt; p0 += 128) {      // four loads in flight
-                uint64_t key[4];
+        const int base = start_s[s0], n_new = start_s[s1] - base, n_in = n_new + n_best;
+        for (int l = s0 + tid / 8; l < s1; l += kMergeThreads / 8)      // eight threads per list: few long lists or many short ones
+            for (int p = start_s[l] - base + tid % 8, e = start_s[l + 1] - base; p < e; p += 8) list_s[p] = (uint16_t)l;
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int p = p0 + 32 * j + lane;
-                    key[j] = p < cnt ? src[(int64_t)p * qb] : 0;
-                }
+        for (int b = 0; b < kMergeBins / kMergeThreads; ++b) hist[tid + kMergeThreads * b] = 0;
+        if (tid == 0) { bin_lo = 0xFFFFFFFFu; bin_hi = 0; }
+        __syncthreads();
+        uint64_t e[kMergePer];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    if (p0 + 32 * j >= cnt) break;
-                    const bool in = key[j] != 0 && key[j] >= thr && !left_out(key_id(key[j]));
-                    const unsigned who = __ballot_sync(0xFFFFFFFFu, in);
-                    int at = 0;
-                    if (lane == 0 && who) at = atomicAdd(&n_s, __popc(who));
-                    at = __shfl_sync(0xFFFFFFFFu, at, 0);
-                    if (in) keys[at + __popc(who & ((1u << lane) - 1u))] = key[j];
-                }
+        for (int j = 0; j < kMergePer; ++j) {
+            const int p = tid + kMergeThreads * j;
+            e[j] = 0;
+            if (p < n_new) {
+                const int l = list_s[p];
+                e[j] = lists[(((int64_t)l * q_blocks + q / qb) * cap + (p + base - start_s[l])) * qb + q % qb];
+            } else if (p < n_in) {
+                e[j] = best[p - n_new];
             }
         }
-        __syncthreads();
-        const int n = n_s;
-        __syncthreads();      // (the next group's appends change n_s)
-        if (n > k) {
-            uint64_t e[kMergePer];
-            uint32_t lo = 0xFFFFFFFFu, hi = 0;
+        int have = 0;
+        uint32_t lo = 0xFFFFFFFFu, hi = 0;
 #pragma unroll
-            for (int j = 0; j < kMergePer; ++j) {
-                const int p = tid + kMergeThreads * j;
-                e[j] = p < n ? keys[p] : 0;
-                if (p < n) {
-                    lo = min(lo, (uint32_t)(e[j] >> 32));
-                    hi = max(hi, (uint32_t)(e[j] >> 32));
-                }
+        for (int j = 0; j < kMergePer; ++j) {
+            if (kMergeThreads * j >= n_in) break;
+            if (tid + kMergeThreads * j < n_new && e[j] != 0 && (e[j] < thr || (ex_n && left_out(key_id(e[j]))))) e[j] = 0;
+            if (e[j]) {
+                ++have;
+                lo = min(lo, (uint32_t)(e[j] >> 32));
+                hi = max(hi, (uint32_t)(e[j] >> 32));
             }
-            lo = __reduce_min_sync(0xFFFFFFFFu, lo);
-            hi = __reduce_max_sync(0xFFFFFFFFu, hi);
-            if (lane == 0) { cnt_s[0][warp] = (int)lo; cnt_s[1][warp] = (int)hi; }
-            __syncthreads();
+        }
+        lo = __reduce_min_sync(0xFFFFFFFFu, lo);
+        hi = __reduce_max_sync(0xFFFFFFFFu, hi);
+        if (lane == 0) { max_s[0][warp] = (int)lo; max_s[1][warp] = (int)hi; }
+        const int n = block_sum(have);
+        uint64_t bar = 1;      // keep keys >= bar
+        if (n > k) {
 #pragma unroll
             for (int w = 0; w < kMergeThreads / 32; ++w) {
-                lo = min(lo, (uint32_t)cnt_s[0][w]);
-                hi = max(hi, (uint32_t)cnt_s[1][w]);
+                lo = min(lo, (uint32_t)max_s[0][w]);
+                hi = max(hi, (uint32_t)max_s[1][w]);
+            }
+            // (a bin never falls as the score rises: every step of its formula is monotone.  One bin for all where the scores'
+            // range is zero, infinite or not a number.)
+            const float least = order_score(lo), range = order_score(hi) - least;
+            float per_score = (float)(kMergeBins - 1) / range;
+            if (!(range > 0.f && range < INFINITY && per_score < INFINITY)) per_score = 0.f;
+            auto bin_of = [&](uint64_t key) {
+                return per_score > 0.f ? min((int)((order_score((uint32_t)(key >> 32)) - least) * per_score), kMergeBins - 1) : 0;
+            };
+#pragma unroll
+            for (int j = 0; j < kMergePer; ++j)
+                if (e[j]) atomicAdd(&hist[bin_of(e[j])], 1);
+            __syncthreads();
+            constexpr int kBins = kMergeBins / kMergeThreads;
+            int c[kBins], from = 0;
+#pragma unroll
+            for (int b = 0; b < kBins; ++b) {
+                c[b] = hist[tid * kBins + b];
+                from += c[b];
+            }
+            int incl = from;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_down_sync(0xFFFFFFFFu, incl, o);
+                if (lane + o < 32) incl += v;
+            }
+            if (lane == 0) max_s[0][warp] = incl;
+            __syncthreads();
+            int above = incl - from;
+            for (int w = warp + 1; w < kMergeThreads / 32; ++w) above += max_s[0][w];
+#pragma unroll
+            for (int b = kBins - 1; b >= 0; --b) {
+                if (above < k && above + c[b] >= k) { bin_s = tid * kBins + b; bin_above = above + c[b]; }
+                above += c[b];
             }
             __syncthreads();
-            int at_lo = n;
+            const int bin = bin_s;
+            int at_lo = bin_above;
+            if (at_lo > k)
+#pragma unroll
+                for (int j = 0; j < kMergePer; ++j)
+                    if (e[j] && bin_of(e[j]) == bin) {
+                        atomicMin(&bin_lo, (uint32_t)(e[j] >> 32));
+                        atomicMax(&bin_hi, (uint32_t)(e[j] >> 32));
+                    }
+            if (at_lo == k) {
+                uint32_t kth = 0xFFFFFFFFu;
+#pragma unroll
+                for (int j = 0; j < kMergePer; ++j)
+                    if (e[j] && bin_of(e[j]) >= bin) kth = min(kth, (uint32_t)(e[j] >> 32));
+                kth = __reduce_min_sync(0xFFFFFFFFu, kth);
+                if (lane == 0) atomicMin(&bin_lo, kth);
+            }
+            __syncthreads();
+            lo = bin_lo;
+            hi = at_lo > k ? bin_hi : lo;
             for (int step = 0; at_lo > k && lo < hi; ++step) {
                 const uint32_t mid = bisect_at(lo, hi, step);
                 int cc = 0;
 #pragma unroll
                 for (int j = 0; j < kMergePer; ++j)
-                    if (kMergeThreads * j < n) cc += (uint32_t)(e[j] >> 32) >= mid;
-                cc = block_sum(cc, flip);
-                flip ^= 1;
+                    if (kMergeThreads * j < n_in) cc += (uint32_t)(e[j] >> 32) >= mid;
+                cc = block_sum(cc);
                 if (cc >= k) { lo = mid; at_lo = cc; } else hi = mid - 1;
             }
-            uint64_t bar = (uint64_t)lo << 32;
+            bar = (uint64_t)lo << 32;
             for (int bit = 31; bit >= 0 && at_lo > k; --bit) {      // scores equal to the k-th: the smaller ids
                 const uint64_t cand = bar | (1u << bit);
                 int cc = 0;
 #pragma unroll
                 for (int j = 0; j < kMergePer; ++j)
-                    if (kMergeThreads * j < n) cc += e[j] >= cand;
-                cc = block_sum(cc, flip);
-                flip ^= 1;
+                    if (kMergeThreads * j < n_in) cc += e[j] >= cand;
+                cc = block_sum(cc);
                 if (cc >= k) { bar = cand; at_lo = cc; }
             }
-            if (tid == 0) n_s = 0;
-            __syncthreads();
-#pragma unroll
-            for (int j = 0; j < kMergePer; ++j)
-                if (e[j] != 0 && e[j] >= bar) keys[atomicAdd(&n_s, 1)] = e[j];
-            __syncthreads();
         }
-    }
-    const int n = n_s;
-    if (!last) {
-        uint32_t least = 0xFFFFFFFFu;
-        for (int p = tid; p < k; p += kMergeThreads) {
-            const uint64_t key = p < n ? keys[p] : 0;
-            carry[q * k + p] = key;
-            least = min(least, (uint32_t)(key >> 32));
-        }
-        least = __reduce_min_sync(0xFFFFFFFFu, least);
-        if (lane == 0) cnt_s[flip][warp] = (int)least;
+        if (tid == 0) n_s = 0;
         __syncthreads();
-        if (tid == 0 && n == k) {
-            for (int w = 0; w < kMergeThreads / 32; ++w) least = min(least, (uint32_t)cnt_s[flip][w]);
-            gtau[q] = least;
+#pragma unroll
+        for (int j = 0; j < kMergePer; ++j)
+            if (e[j] != 0 && e[j] >= bar) best[atomicAdd(&n_s, 1)] = e[j];
+        __syncthreads();
+        n_best = n_s;
+    }
+    const int n = n_best;
+    if (!last) {
+        const uint64_t key = tid < n ? best[tid] : 0;
+        if (tid < k) carry[q * k + tid] = key;
+        if (n == k) {
+            const uint32_t least = __reduce_min_sync(0xFFFFFFFFu, tid < k ? (uint32_t)(key >> 32) : 0xFFFFFFFFu);
+            if (lane == 0) cnt_s[0][warp] = (int)least;
+            __syncthreads();
+            if (tid == 0) {
+                uint32_t all = least;
+                for (int w = 1; w < kMergeThreads / 32; ++w) all = min(all, (uint32_t)cnt_s[0][w]);
+                gtau[q] = all;
+            }
         }
         return;
     }
     if (tid < k) {
         if (tid < n) {
-            const uint64_t mine = keys[tid];
+            const uint64_t mine = best[tid];
             int rank = 0;
-            for (int p = 0; p < n; ++p) rank += keys[p] > mine;
+#pragma unroll 8
+            for (int p = 0; p < n; ++p) rank += best[p] > mine;
             ids_out[q * k + rank] = key_id(mine);
             if (scores_out) scores_out[q * k + rank] = order_score((uint32_t)(mine >> 32));
         } else {      // fewer than k candidates: the rest of the row says so
