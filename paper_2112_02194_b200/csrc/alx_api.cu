@@ -456,20 +456,21 @@ int64_t dual_rows_of(const alx_ctx *c, int side)
 }
 
 // the Gramian and the base matrix of a table; `solve`: also what the rows' dual form needs of the base matrix
-alx_status gramian_of(alx_ctx *c, int table_side, bool solve, unsigned long long *stamps = nullptr)
+alx_status gramian_of(alx_ctx *c, int table_side, bool solve, unsigned long long *stamps = nullptr, cudaStream_t aside = nullptr)
 {
+    const cudaStream_t s = aside ? aside : c->stream;
     if (tensor_path(c)) {
-        ALX_CUDA(c, launch_gramian_umma(c->table[table_side], c->n[table_side], c->gram_partials, c->stream, &c->launches));
+        ALX_CUDA(c, launch_gramian_umma(c->table[table_side], c->n[table_side], c->gram_partials, s, &c->launches));
         ALX_CUDA(c, launch_gramian_reduce(c->gram_partials, gramian_umma_partials(), c->opt.d, c->G64[table_side], c->Bmat,
-                                          c->opt.alpha0, c->opt.lambda, c->stream, &c->launches));
+                                          c->opt.alpha0, c->opt.lambda, s, &c->launches));
         if (solve && dual_form(c)) ALX_CUDA(c, launch_dual_prepare(c->Bmat, c->dual_ws, dual_cond_limit(c), c->opt.solver == ALX_SOLVER_AUTO, c->stream,
                                                          &c->launches));
         c->have_gram[table_side] = true;
         return ALX_OK;
     }
     ALX_CUDA(c, launch_gramian(c->table[table_side], c->bf16, c->n[table_side], c->opt.d, c->gram_partials,
-                               c->G64[table_side], c->Bmat, c->opt.alpha0, c->opt.lambda, stamps, c->stream, &c->launches));
-    if (solve && dual64(c)) ALX_CUDA(c, launch_dual64_prepare(c->Bmat, c->dual_ws, dual_cond_limit(c), c->stream, &c->launches));
+                               c->G64[table_side], c->Bmat, c->opt.alpha0, c->opt.lambda, stamps, s, &c->launches));
+    if (solve && dual64(c)) ALX_CUDA(c, launch_dual64_prepare(c->Bmat, c->dual_ws, dual_cond_limit(c), s, &c->launches));
     if (solve && dual_warp(c)) {
         const float most = c->bf16 ? kDualWarpLimitBf16 : kDualWarpLimitF32;
         ALX_CUDA(c, launch_dual_warp_prepare(c->Bmat, c->dual_ws, c->opt.d, dual_cond_limit(c) < most ? dual_cond_limit(c) : most, c->stream,
@@ -489,7 +490,8 @@ void note_half_epoch(alx_ctx *c, int side)
     c->stats.kernel_path[side] = warp_path(c) || tensor_path(c) || team_path(c) ? 1 : 0;
 }
 
-alx_status half_epoch_impl(alx_ctx *c, int side, const int32_t *cap_slot, float *cap_out)
+// gramian_aside: the Gramian was launched on the second stream, copy_ev follows it
+alx_status half_epoch_impl(alx_ctx *c, int side, const int32_t *cap_slot, float *cap_out, bool gramian_aside = false)
 {
     if (c->nnz < 0) return fail(c, ALX_ERR_BAD_STATE, "alx_half_epoch before alx_set_csr");
     const int fixed = 1 - side;
@@ -501,9 +503,9 @@ alx_status half_epoch_impl(alx_ctx *c, int side, const int32_t *cap_slot, float 
     alx_status st;
     {
         NvtxRange r("alx Gramian + base matrix");
-        st = gramian_of(c, fixed, dual_rows_of(c, side) > 0, stamps);
+        if (gramian_aside) ALX_CUDA(c, cudaStreamWaitEvent(c->stream, c->copy_ev, 0));
+        else if ((st = gramian_of(c, fixed, dual_rows_of(c, side) > 0, stamps)) != ALX_OK) return st;
     }
-    if (st != ALX_OK) return st;
     if (!stamps) ALX_CUDA(c, record_event(c->ev[1], c->stream, c->capturing));
     NvtxRange rows_range("alx rows: gather, sums, solve, store");
     RowOut out{c->table[side], cap_slot, cap_out};
@@ -1134,6 +1136,13 @@ alx_status fold_in_impl(alx_ctx *k, const int64_t *rowptr, const int32_t *colidx
     const int d = k->opt.d;
     alx_status st = ensure_box(k);
     if (st != ALX_OK) return st;
+    // The Gramian of the column table needs nothing of the new rows: it runs beside their upload, checks and classes, on the
+    // second stream (a request for a few rows waited 75 us for it after 60 us of those).  B^-1 too where the rows could have use for it.
+    if ((st = ensure_copy_stream(k)) != ALX_OK) return st;
+    ALX_CUDA(k, cudaEventRecord(k->copy_ev, k->stream));
+    ALX_CUDA(k, cudaStreamWaitEvent(k->copy_stream, k->copy_ev, 0));
+    if ((st = gramian_of(k, ALX_COLS, n >= kDualLeastRows, nullptr, k->copy_stream)) != ALX_OK) return st;
+    ALX_CUDA(k, cudaEventRecord(k->copy_ev, k->copy_stream));
     // what the last call left
     dev_free(k, k->chunk_desc[0]); k->chunk_desc[0] = nullptr;
     dev_free(k, k->split_first[0]); k->split_first[0] = nullptr;
@@ -1187,7 +1196,7 @@ alx_status fold_in_impl(alx_ctx *k, const int64_t *rowptr, const int32_t *colidx
         k->split_partials = static_cast<float *>(sums);
     }
     k->nnz = nnz;
-    if ((st = half_epoch_impl(k, ALX_ROWS, nullptr, nullptr)) != ALX_OK) return st;
+    if ((st = half_epoch_impl(k, ALX_ROWS, nullptr, nullptr, true)) != ALX_OK) return st;
     const size_t bytes = sizeof(float) * n * d;
     if (on_device) {
         ALX_CUDA(k, launch_convert(k->table[0], k->bf16, x_out, 0, n * d, k->stream, &k->launches));
@@ -1233,6 +1242,7 @@ alx_status alx_fold_in(alx_ctx *c, const int64_t *rowptr, const int32_t *colidx,
     c->launches += k->launches - before;
     if (st != ALX_OK) {
         cudaStreamSynchronize(k->stream);
+        if (k->copy_stream) cudaStreamSynchronize(k->copy_stream);
         c->err = "alx_fold_in: " + k->err;
     }
     give_back_large(k);
