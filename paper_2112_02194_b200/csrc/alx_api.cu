@@ -463,7 +463,7 @@ alx_status gramian_of(alx_ctx *c, int table_side, bool solve, unsigned long long
         ALX_CUDA(c, launch_gramian_umma(c->table[table_side], c->n[table_side], c->gram_partials, s, &c->launches));
         ALX_CUDA(c, launch_gramian_reduce(c->gram_partials, gramian_umma_partials(), c->opt.d, c->G64[table_side], c->Bmat,
                                           c->opt.alpha0, c->opt.lambda, s, &c->launches));
-        if (solve && dual_form(c)) ALX_CUDA(c, launch_dual_prepare(c->Bmat, c->dual_ws, dual_cond_limit(c), c->opt.solver == ALX_SOLVER_AUTO, c->stream,
+        if (solve && dual_form(c)) ALX_CUDA(c, launch_dual_prepare(c->Bmat, c->dual_ws, dual_cond_limit(c), c->opt.solver == ALX_SOLVER_AUTO, s,
                                                          &c->launches));
         c->have_gram[table_side] = true;
         return ALX_OK;
@@ -473,7 +473,7 @@ alx_status gramian_of(alx_ctx *c, int table_side, bool solve, unsigned long long
     if (solve && dual64(c)) ALX_CUDA(c, launch_dual64_prepare(c->Bmat, c->dual_ws, dual_cond_limit(c), s, &c->launches));
     if (solve && dual_warp(c)) {
         const float most = c->bf16 ? kDualWarpLimitBf16 : kDualWarpLimitF32;
-        ALX_CUDA(c, launch_dual_warp_prepare(c->Bmat, c->dual_ws, c->opt.d, dual_cond_limit(c) < most ? dual_cond_limit(c) : most, c->stream,
+        ALX_CUDA(c, launch_dual_warp_prepare(c->Bmat, c->dual_ws, c->opt.d, dual_cond_limit(c) < most ? dual_cond_limit(c) : most, s,
                                              &c->launches));
     }
     c->have_gram[table_side] = true;
