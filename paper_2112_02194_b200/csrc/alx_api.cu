@@ -329,6 +329,7 @@ SideView side_view(const alx_ctx *c, int side)
     v.chunk_desc = c->chunk_desc[side];
     v.split_first = c->split_first[side];
     v.n = c->n[side];
+    v.nnz = c->nnz;
     return v;
 }
 
@@ -1076,17 +1077,15 @@ alx_status alx_loss(alx_ctx *c, double *total, double *components)
     if (c->nnz < 0) return fail(c, ALX_ERR_BAD_STATE, "alx_loss before alx_set_csr");
     if (!c->have_table[0] || !c->have_table[1]) return fail(c, ALX_ERR_BAD_STATE, "both tables must be set");
     DeviceGuard guard(c->device);
-    for (int s = 0; s < 2; ++s)
-        if (!c->have_gram[s]) {
-            alx_status st = gramian_of(c, s, false);
-            if (st != ALX_OK) return st;
-        }
     alx_status st = ensure_box(c);
     if (st != ALX_OK) return st;
+    const bool beside_gramian = !tensor_path(c) && !(c->have_gram[0] && c->have_gram[1]);
+    for (int s = 0; s < 2; ++s)
+        if (!c->have_gram[s] && (st = gramian_of(c, s, false)) != ALX_OK) return st;
     double *h = reinterpret_cast<double *>(c->box + 64);
     ALX_CUDA(c, launch_loss(c->ptr[0], c->idx[0], c->val[0], c->n[0], c->nnz, c->table[0], c->table[1], c->bf16, c->opt.d, c->G64[0],
                             c->G64[1], (double)c->opt.alpha0, (double)c->opt.lambda, c->loss_partials_buf, c->loss_counter, c->status,
-                            reinterpret_cast<DevStatus *>(c->box), h, c->stream, &c->launches));
+                            reinterpret_cast<DevStatus *>(c->box), h, beside_gramian, c->stream, &c->launches));
     ALX_CUDA(c, cudaStreamSynchronize(c->stream));
     st = report_status(c);
     if (st != ALX_OK) return st;

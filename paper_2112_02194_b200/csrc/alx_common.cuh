@@ -73,7 +73,7 @@ struct SideView {
     const int32_t *order;  // [n] rows by (class, id)
     const int64_t *chunk_desc;   // [4 * n_chunks]
     const int64_t *split_first;  // [n_split_rows + 1]
-    int64_t n;
+    int64_t n, nnz;
 };
 
 struct RowOut {
@@ -93,6 +93,33 @@ __device__ __forceinline__ void stamp(unsigned long long *slot)
         asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
         atomicMax(slot, t);
     }
+}
+
+// ---- programmatic dependent launches ----------------------------------------------------------
+// In a chain of kernels of 2 to 10 us each, a kernel's launch and start cost about 1 us.  launch_early lets it start when every
+// block of the launch before it has called let_next_start (or ended); wait_for_previous then waits until that launch has ended and
+// its writes can be seen (it returns at once in a kernel that was launched plainly).
+// Blocks that are placed while others still hold shared memory crowd on the SMs that have room: with 10M entries of 32 features the
+// block rows took 150 us instead of 75.  So only where the entries are at most kEarlyEntries (some 20 us of work) does a kernel of
+// the rows or the loss start early (2000 x 1500, d = 16: 16 epochs 0.95 -> 0.84 ms).
+constexpr int64_t kEarlyEntries = 1 << 18;
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename... P, typename... A>
+inline cudaError_t launch_early(bool early_start, void (*kernel)(P...), int64_t blocks, int threads, size_t smem, cudaStream_t s, A... args)
+{
+    cudaLaunchAttribute early[1];
+    early[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    early[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = early;
+    cfg.numAttrs = early_start ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
 // ---- small host pieces of the launchers -----------------------------------------------------------
@@ -315,6 +342,6 @@ int64_t loss_partials(int64_t nnz);
 cudaError_t launch_loss(const int64_t *rowptr, const int32_t *colidx, const float *values, int64_t n_rows,
                             int64_t nnz, const void *W, const void *H, int bf16, int d, const double *GW, const double *GH,
                             double alpha0, double lambda, double *partials, unsigned *counter, const DevStatus *st, DevStatus *host_status,
-                            double *host_result, cudaStream_t s, int64_t *launches);
+                            double *host_result, bool beside_gramian, cudaStream_t s, int64_t *launches);
 
 }  // namespace alx

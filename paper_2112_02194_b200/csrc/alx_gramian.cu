@@ -67,6 +67,7 @@ __global__ void __launch_bounds__(GramGeo<D, T>::THREADS, 1) k_gramian_tiles(con
                                                                             float *__restrict__ partials, unsigned long long *begin)
 {
     if (blockIdx.x == 0) stamp(begin);
+    let_next_start();
     using G = GramGeo<D, T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float *red = reinterpret_cast<float *>(smem_raw + 2 * G::STAGE);
@@ -182,6 +183,8 @@ __global__ void __launch_bounds__(256) k_gramian_reduce_tiles(const float *__res
                                                               unsigned long long *done)
 {
     using G = GramGeo<D, T>;
+    let_next_start();
+    wait_for_previous();
     reduce_partials<true>(partials, n_partials, G::ELEMS, D, G64, Bmat, alpha0, lambda, [](int e, int &i, int &l) {
         const int tile = e % G::TILES, ab = e / G::TILES;
         int I = 0;
@@ -210,9 +213,8 @@ cudaError_t gramian_tiles_dt(const void *X, int64_t n, float *partials, double *
     if (e != cudaSuccess) return e;
     const int64_t blocks = gramian_partials(n), per = (n + blocks - 1) / blocks;
     k_gramian_tiles<D, T><<<(unsigned)blocks, G::THREADS, G::SMEM, s>>>(static_cast<const T *>(X), n, per, partials, stamps ? stamps + kStampBegin : nullptr);
-    k_gramian_reduce_tiles<D, T><<<(G::ELEMS + 31) / 32, 256, 0, s>>>(partials, blocks, G64, Bmat, alpha0, lambda,
-                                                                             stamps ? stamps + kStampGramian : nullptr);
-    return cudaGetLastError();
+    return launch_early(true, k_gramian_reduce_tiles<D, T>, (G::ELEMS + 31) / 32, 256, 0, s, partials, blocks, G64, Bmat, alpha0, lambda,
+                        stamps ? stamps + kStampGramian : nullptr);
 }
 
 template <int D>

@@ -174,6 +174,7 @@ __global__ void __launch_bounds__(kWarps * 32, kBlocksPerSm) k_loss(const int64_
     __syncthreads();
     if (!last_s) return;
     __threadfence();
+    wait_for_previous();      // the Gramians (the entries need none of them)
     double s = 0.0, f = 0.0, t = 0.0;
     for (unsigned p = threadIdx.x; p < gridDim.x; p += kWarps * 32) s += __ldcg(partials + p);
 #pragma unroll 8
@@ -205,16 +206,23 @@ int64_t loss_partials(int64_t nnz)
 
 cudaError_t launch_loss(const int64_t *rowptr, const int32_t *colidx, const float *values, int64_t n_rows, int64_t nnz, const void *W,
                         const void *H, int bf16, int d, const double *GW, const double *GH, double alpha0, double lambda, double *partials,
-                        unsigned *counter, const DevStatus *st, DevStatus *host_status, double *host_result, cudaStream_t s, int64_t *launches)
+                        unsigned *counter, const DevStatus *st, DevStatus *host_status, double *host_result, bool beside_gramian, cudaStream_t s, int64_t *launches)
 {
     const unsigned grid = (unsigned)loss_partials(nnz);
-#define ALX_LOSS(DD, T)                                                                                                             \
-    k_loss<DD, T><<<grid, kWarps * 32, 0, s>>>(rowptr, colidx, values, n_rows, nnz, span_of(nnz), (const T *)W, (const T *)H, GW, GH,     \
-                                               alpha0, lambda, partials, counter, st, host_status, host_result)
+    // beside_gramian: the launch before this one is the reduction of a Gramian, which starts when the tables are complete and which
+    // this kernel waits for at its end
+    const bool early = beside_gramian && nnz <= kEarlyEntries;
+#define ALX_LOSS(DD, T)                                                                                                              \
+    {                                                                                                                                \
+        const cudaError_t e = launch_early(early, k_loss<DD, T>, grid, kWarps * 32, 0, s, rowptr, colidx, values, n_rows, nnz,       \
+                                           span_of(nnz), (const T *)W, (const T *)H, GW, GH, alpha0, lambda, partials, counter, st,  \
+                                           host_status, host_result);                                                                \
+        if (e != cudaSuccess) return e;                                                                                              \
+    }
 #define ALX_CASE(DD)                        \
     case DD:                                \
-        if (bf16) ALX_LOSS(DD, __nv_bfloat16); \
-        else ALX_LOSS(DD, float);           \
+        if (bf16) ALX_LOSS(DD, __nv_bfloat16) \
+        else ALX_LOSS(DD, float)            \
         break;
     switch (d) {
         ALX_CASE(16)

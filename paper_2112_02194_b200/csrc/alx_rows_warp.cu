@@ -611,7 +611,7 @@ template <int D, typename T> __device__ __forceinline__ void store_zeros(const Z
 // is wait for it, so that whatever follows this grid follows both; then the time is noted.
 __device__ __forceinline__ void finish_after_previous(unsigned long long *done)
 {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    wait_for_previous();
     stamp(done);
 }
 
@@ -634,9 +634,10 @@ template <int D, typename T> __device__ __forceinline__ void load_base(const flo
 template <int D, typename T>
 __global__ void __launch_bounds__(WGeo<D, T>::REGS_WARPS * 32, 1)
 k_rows_warp(SideView sv, int64_t last, int64_t count, const int *dual_flag, int64_t primal_count, const int32_t *list,
-            const unsigned long long *list_count, const T *__restrict__ X, const float *__restrict__ Bmat, RowOut out, ZeroRows zero, unsigned long long *done, DevStatus *st)
+            const unsigned long long *list_count, const T *__restrict__ X, const float *__restrict__ Bmat, RowOut out, ZeroRows zero, int wait_first, unsigned long long *done, DevStatus *st)
 {
     using G = WGeo<D, T>;
+    if (wait_first) wait_for_previous();
     store_zeros<D, T>(zero, out);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float4 *base = reinterpret_cast<float4 *>(smem_raw);
@@ -780,7 +781,8 @@ k_rows_block(SideView sv, int64_t last, const T *__restrict__ X, const float *__
     using G = WGeo<D, T>;
     using B = BGeo<D, T>;
     constexpr int kBlockWarps = B::kBlockWarps;
-    asm volatile("griddepcontrol.launch_dependents;");      // the rows of a warp each may start beside these
+    wait_for_previous();
+    let_next_start();      // the rows of a warp each may start beside these
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float4 *base = reinterpret_cast<float4 *>(smem_raw);
     float *work = reinterpret_cast<float *>(smem_raw + G::BASE);
@@ -1259,6 +1261,7 @@ struct WarpRows {
     WarpCg cg;
     const int *dual_flag;      // set on the device when the rows of class 1 have been solved in the dual form
     unsigned long long *stamps;      // time stamps of the half-epoch, or null
+    bool early;                      // few entries: the kernels may start while the one before them ends
     cudaStream_t s;
     int64_t *launches;
 };
@@ -1293,20 +1296,12 @@ cudaError_t whole_rows(const WarpRows &a, int64_t end, const int32_t *list, cons
     int64_t blocks = list ? 148 : (n + G::ROWS - 1) / G::ROWS;      // few rows: one per SM before two
     if (blocks > 148) blocks = 148;
     const ZeroRows zero = list ? ZeroRows{nullptr, 0} : zero_rows<D, T>(a, blocks, G::REGS_WARPS * 32);
-    cudaLaunchAttribute beside[1];
-    beside[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    beside[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)blocks);
-    cfg.blockDim = dim3(G::REGS_WARPS * 32);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = a.s;
-    cfg.attrs = beside;
-    // beside k_rows_block, where that is the launch before this one (a launch of the rows without observations may be between)
-    cfg.numAttrs = after_block_rows && zero.rows ? 1 : 0;
-    const cudaError_t el = cudaLaunchKernelEx(&cfg, k_rows_warp<D, T>, a.sv, end - 1, n, list ? (const int *)nullptr : a.dual_flag, end - a.offs[2], list,
-                                              list_count, reinterpret_cast<const T *>(a.X), a.Bmat, a.out, zero,
-                                              a.stamps ? a.stamps + kStampEnd : (unsigned long long *)nullptr, a.st);
+    // where k_rows_block is the launch before this one (a launch of the rows without observations may be between) the two run
+    // side by side: everything this one reads was complete before k_rows_block let it start
+    const bool beside = after_block_rows && zero.rows;
+    const cudaError_t el = launch_early(beside || (!list && a.early), k_rows_warp<D, T>, blocks, G::REGS_WARPS * 32, smem, a.s, a.sv, end - 1, n, list ? nullptr : a.dual_flag,
+                                        end - a.offs[2], list, list_count, reinterpret_cast<const T *>(a.X), a.Bmat, a.out, zero, beside ? 0 : 1,
+                                        a.stamps ? a.stamps + kStampEnd : nullptr, a.st);
     if (el != cudaSuccess) return el;
     ++*a.launches;
     return cudaGetLastError();
@@ -1334,15 +1329,17 @@ template <int D, typename T> cudaError_t rows_warp_dt(const WarpRows &a)
     if (a.n_chunks > 0) {
         static SmemOnce allow;
         if ((e = allow(k_rows_block<D, T, true>, B::SMEM)) != cudaSuccess) return e;
-        k_rows_block<D, T, true><<<(unsigned)a.n_chunks, B::kBlockWarps * 32, B::SMEM, a.s>>>(a.sv, 0, X, a.Bmat, a.partials, a.out, a.st);
+        e = launch_early(a.early, k_rows_block<D, T, true>, a.n_chunks, B::kBlockWarps * 32, B::SMEM, a.s, a.sv, 0, X, a.Bmat, a.partials, a.out, a.st);
+        if (e != cudaSuccess) return e;
         ++*a.launches;
         if ((e = solve_rows<D, T, false>(a, 0)) != cudaSuccess) return e;
     }
     if (end_long > begin_long) {
         static SmemOnce allow;
         if ((e = allow(k_rows_block<D, T, false>, B::SMEM)) != cudaSuccess) return e;
-        k_rows_block<D, T, false><<<(unsigned)(end_long - begin_long), B::kBlockWarps * 32, B::SMEM, a.s>>>(a.sv, end_long - 1, X, a.Bmat, a.partials,
-                                                                                                         a.out, a.st);
+        e = launch_early(a.early, k_rows_block<D, T, false>, end_long - begin_long, B::kBlockWarps * 32, B::SMEM, a.s, a.sv, end_long - 1, X, a.Bmat,
+                         a.partials, a.out, a.st);
+        if (e != cudaSuccess) return e;
         ++*a.launches;
     }
     return whole_rows<D, T>(a, begin_long, nullptr, nullptr, end_long > begin_long);
@@ -1391,7 +1388,7 @@ cudaError_t launch_rows_warp(const SideView &sv, const int64_t *offs, int64_t n_
                              const int *dual_flag, unsigned long long *stamps, cudaStream_t s, int64_t *launches)
 {
     const WarpRows a{sv, offs, n_chunks, n_split_rows, X, parts, Bmat, partials, out, st,
-                     WarpCg{cg.max_iter, cg.warm_start ? 1 : 0, cg.tol * cg.tol, cg.counters, cg.fallback_list}, dual_flag, stamps, s, launches};
+                     WarpCg{cg.max_iter, cg.warm_start ? 1 : 0, cg.tol * cg.tol, cg.counters, cg.fallback_list}, dual_flag, stamps, sv.nnz <= kEarlyEntries, s, launches};
     switch (d) {
     case 16: return bf16 ? rows_warp_dt<16, __nv_bfloat16>(a) : rows_warp_dt<16, float>(a);
     case 32: return bf16 ? rows_warp_dt<32, __nv_bfloat16>(a) : rows_warp_dt<32, float>(a);
