@@ -84,16 +84,17 @@ typedef struct alx_options {
                                 kernels, rows with at most 32 observations solved in the dual (push-through) form
                                 of Eq. 4 while alpha0 G + lambda I is well conditioned (see dual_cond_limit; the rows of
                                 17 .. 32 observations go to the conjugate-gradient kernel instead where that is the cheaper
-                                solve); for d = 64 with fp32 tables the same tensor-core kernels over bfloat16 parts of
-                                the fixed table (x = x1 + x2 + x3, so to fp32 accuracy), rows with at most 16
-                                observations in the dual form; every other (d, storage) the FP32-ALU kernels.
+                                solve); every other (d, storage) kernels of one warp (d <= 64) or four (d = 128) per row,
+                                their sums warp-level tensor-core products, of bfloat16 parts for fp32 tables (x = x1 + x2 +
+                                x3, so to fp32 accuracy), rows with at most 16 observations in the dual form for d = 64
+                                and for fp32 tables of 128.
                                 1 = force the plain FP32-ALU kernels (reference path inside the library; every d, every
                                 storage); 2 = as 0 but every row in the primal form */
     int32_t solver;          /* how the d x d system of Eq. 4 is solved (Sec. 4.5 compares the choices):
-                                ALX_SOLVER_AUTO (0): conjugate gradients where the library has them (the whole-rows
-                                tensor-core kernel), started as cg_start says and stopped at |r| <= cg_tol |b|; a row that has not
+                                ALX_SOLVER_AUTO (0): conjugate gradients where the library has them (d = 128 with
+                                bfloat16 tables, d = 64 with fp32 tables), started as cg_start says and stopped at |r| <= cg_tol |b|; a row that has not
                                 converged after cg_max_iter steps, and every row elsewhere, is solved by Cholesky.  A side
-                                whose conjugate-gradient half-epoch spent more than cg_switch_products (28) products per row on average (where
+                                (d = 128) whose conjugate-gradient half-epoch spent more than cg_switch_products (28) products per row on average (where
                                 the in-place Cholesky is the faster solve on B200) takes Cholesky for its next half-epochs,
                                 with one conjugate-gradient half-epoch in every eight to look again; the choice is made
                                 on the device from the counts of the side's last run.
@@ -110,11 +111,12 @@ typedef struct alx_options {
                                 is under way; costs one product for r = b - A x0, and falls back to zero when |r| > |b|);
                                 ALX_CG_START_ZERO (1): x = 0, so that a row's work does not depend on the table's history */
     float dual_cond_limit;   /* 0 => ALX_DEFAULT_DUAL_COND_LIMIT.  Rows with at most 32 observations (d = 128, bfloat16 tables)
-                                or 16 (d = 64, fp32 tables) are solved in the dual form of Eq. 4 while
-                                ||B||_F ||B^-1||_F <= this limit, B = alpha0 G + lambda I (the form's rounding error grows
+                                or 16 (d = 64; d = 128 with fp32 tables) are solved in the dual form of Eq. 4 while
+                                ||B||_F ||B^-1||_F <= this limit (at most 1024 for d = 64 with bfloat16 tables and 512 for
+                                d = 128 with fp32 tables, whatever is given), B = alpha0 G + lambda I (the form's rounding error grows
                                 with the condition of B; the product is d for a multiple of the identity and about
                                 sqrt(d) cond_2(B) when one direction dominates).  Beyond the limit, with solver =
-                                ALX_SOLVER_AUTO and d = 128: the dual-form solutions become the start vectors of a
+                                ALX_SOLVER_AUTO and bfloat16 tables of 128: the dual-form solutions become the start vectors of a
                                 conjugate-gradient pass over those rows (alx_stats.dual_polished_rows); otherwise the
                                 rows take the d x d solve like every other row */
 } alx_options;
@@ -124,15 +126,17 @@ typedef struct alx_stats {
     int64_t rows_in_class[2][ALX_N_CLASSES]; /* [side][class] */
     int64_t n_chunks[2];                     /* chunk descriptors of the split class, per side */
     int64_t not_spd;                         /* rows whose factorisation met a non-positive pivot, so far */
-    double ms_gramian, ms_rows, ms_half_epoch; /* device time of the phases of the LAST half-epoch */
+    double ms_gramian, ms_rows, ms_half_epoch; /* device time of the phases of the LAST half-epoch (of a
+                                                replayed epoch of d <= 64 by the device's global timer) */
     int64_t kernel_launches;                 /* kernels this context has launched so far */
     int64_t workspace_bytes;                 /* device memory the context holds */
-    int32_t kernel_path[2];                  /* [side]: 0 = FP32-ALU kernels, 1 = tensor-core kernels */
-    double ms_main_kernel;                   /* tensor path: device time of the whole-rows kernel of the LAST half-epoch, else 0 */
+    int32_t kernel_path[2];                  /* [side]: 0 = FP32-ALU kernels (kernels = 1), 1 = the others */
+    double ms_main_kernel;                   /* with conjugate gradients: device time of the whole-rows kernels of the LAST half-epoch, else 0 */
     int64_t dual_rows;                       /* rows the LAST half-epoch solved in the dual form of Eq. 4 (0: none, or the
                                                 form stepped aside because alpha0 G + lambda I was ill conditioned) */
-    int64_t long_rows[2];                    /* [side], tensor-core kernels only: whole rows of more than 1024 entries
-                                                whose sums the chunks kernel forms (as it does for the split rows) */
+    int64_t long_rows[2];                    /* [side], kernels != 1: whole rows whose sums several warps form, or the
+                                                chunks kernel (as it does for the split rows); more than 1024 entries for d = 128
+                                                with bfloat16 tables, fewer elsewhere */
     int64_t long_entries[2];                 /* [side]: the entries those rows hold */
     int64_t cg_rows;                         /* LAST half-epoch: rows the conjugate-gradient solve took, */
     int64_t cg_products;                     /* the matrix-vector products it spent on them (steps + 1 per row), */
@@ -266,8 +270,8 @@ alx_status alx_get_stats(alx_ctx *ctx, alx_stats *out);
  * on new rows.  rowptr[n_new + 1] / colidx[nnz] / values[nnz] (or NULL: y = 1) give the new rows as CSR over the
  * context's columns, with the rules of alx_set_csr; x_out receives n_new x d floats, the solutions after the round
  * to the storage type (the values a trained table would hold).  The arrays are host or device memory as on_device
- * says, x_out included.  The context's own matrix and tables are not touched; the call allocates what the half-step
- * needs for n_new rows, runs the same kernels as alx_half_epoch and synchronises.  A row with no entry gets 0.
+ * says, x_out included.  The context's own matrix and tables are not touched; the call runs the
+ * same kernels as alx_half_epoch, in buffers that the context keeps for the next call (large ones are given back), and synchronises.  A row with no entry gets 0.
  * ALX_ERR_BAD_STATE before the column table holds anything, ALX_ERR_BAD_CSR as alx_set_csr.
  */
 alx_status alx_fold_in(alx_ctx *ctx, const int64_t *rowptr, const int32_t *colidx, const float *values, int64_t n_new,
@@ -282,8 +286,8 @@ alx_status alx_fold_in(alx_ctx *ctx, const int64_t *rowptr, const int32_t *colid
  * scores.  exclude_ptr[m + 1] / exclude_idx (may both be NULL) list, per query and ascending, ids that must not be
  * returned (the kept links of a fold-in row, for example; the paper does not say whether it leaves them out).  Where
  * fewer than k items qualify the row is filled with id -1 and score -inf.  1 <= k <= ALX_MAX_TOPK.
- * Scores are fp32: for d = 128 with bfloat16 tables products of bfloat16 parts summed in fp32 on the tensor cores
- * (the query as three parts, so to fp32 accuracy); otherwise fp32 FMAs.  Two items whose exact scores differ by less
+ * Scores are fp32: for d = 128 with bfloat16 tables and more than 16 queries products of bfloat16 parts summed in
+ * fp32 on the tensor cores (the query as three parts, so to fp32 accuracy); otherwise fp32 FMAs.  Two items whose exact scores differ by less
  * than that rounding may come out in either order.  All arrays host or device as on_device says; synchronises.
  */
 alx_status alx_topk(alx_ctx *ctx, alx_side items, const float *queries, int64_t m, int32_t k, const int64_t *exclude_ptr,

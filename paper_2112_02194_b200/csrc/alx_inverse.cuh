@@ -8,8 +8,8 @@ namespace alx {
 // Symmetric sweep (Gauss-Jordan on a positive definite matrix): pivot j turns a_ic into a_ic - a_ij a_jc / a_jj, the pivot's
 // row and column into a_ij / a_jj and the pivot into -1 / a_jj; after all D pivots the matrix is -B^-1.  A thread keeps a
 // 4 x 4 tile of the lower triangle in registers; a step hands on one column through shared memory (two buffers, one barrier).
-// Bound: 128 dependent steps of barrier, shared-memory read, 16 FMAs a thread and the reciprocal of the next pivot, about 300
-// cycles each.  d = 128: 475 -> 24 us, d = 64: 137 -> 11 us (the Cholesky it replaces gave a row to a thread, with a division,
+// Bound: D dependent steps of barrier, shared-memory read, 16 FMAs a thread and the reciprocal of the next pivot, all in fp64 on
+// one SM: about 1300 cycles each at d = 128, 680 at 64.  d = 128: 475 -> 92 us, d = 64: 137 -> 23 us (the Cholesky it replaces gave a row to a thread, with a division,
 // a square root and three barriers per column, and then two triangular products as chains of shared-memory reads).
 template <int D> struct SweepGeo {
     static constexpr int T = D / 4, TILES = T * (T + 1) / 2, THREADS = (TILES + 31) / 32 * 32;

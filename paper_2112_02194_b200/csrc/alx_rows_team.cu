@@ -8,7 +8,8 @@
 // the column steps need shuffles only; the block meets at a barrier before and after a panel.
 //
 // The FP32-ALU kernels (alx_rows.cu) gave such a row 256 threads that met at a barrier three times per 16 columns and did the
-// trailing update with FMAs from shared memory: 60k x 25k, 2e6 entries, one epoch 17.4 ms; here 8.7 ms.
+// trailing update with FMAs from shared memory: 60k x 25k, 2e6 entries, one epoch 17.4 ms; here 6.8 ms
+// with the dual form for the rows of at most 16 entries (this kernel 5.1, the sums of long rows 0.7).
 // Bound: the chain of 64 double column steps and the 128 steps of the back substitution (three teams per SM hide what they can).
 #include "alx_common.cuh"
 #include "alx_mma.cuh"

@@ -3,13 +3,13 @@
 // For each row u of the solved side (Alg. 1 lines 3-10, Eq. 4): gather, A = sum x (x) x and b = sum y x, add the base
 // matrix, Cholesky, solve, round, store.  The FP32-ALU kernels (alx_rows.cu) give a row a block of 256 threads that meets at a
 // barrier several times per 16 columns; at these d a row is a few thousand operations and the barriers were the run time
-// (d = 64, bfloat16: 25 ns of the chip per row of 20 entries).  Here
+// (d = 64, bfloat16: 25 ns of the chip per row of 20 entries, here 6).  Here
 //   - 16 entries at a time come through a two-stage cp.async ring of the warp's own; the next row's first entries are on their
 //     way while the warp solves this one;
 //   - the sums are mma.sync m16n8k16 products on the lower triangle's 16 x 8 blocks.  A gathered tile is both operands: one
 //     ldmatrix.trans per 16 features gives the A fragment, and its registers are the B fragments of the same features.
 //     bfloat16 tables: products exact, sums in fp32.  fp32 tables: x = x1 + x2 + x3 in bfloat16 parts, the six products down to
-//     2^-24 (the scheme of the d = 64 tcgen05 path).  The warp-level instruction because a row's matrix is a fraction of a
+//     2^-24.  The warp-level instruction because a row's matrix is a fraction of a
 //     tcgen05 tile: m16n8k16 runs at 1024 FMA per cycle and SM (measured, 550 TFLOP/s), which at these d leaves the sums
 //     behind the solve, and the result is where the solve wants it, in the warp's registers;
 //   - Cholesky with lane = row (d = 64: rows l and l + 32; d = 16: two matrices per warp), two columns per step, the finished
@@ -18,7 +18,9 @@
 // Long rows (warp_long_class), and the chunks of rows longer than `split`, are summed by a block of warps, each a slice of the
 // entries; the slices are added in a fixed order.
 //
-// Bound: issue slots of the solve (d = 64: about 3400 per row) and, for long rows, the mma rate.
+// fp32 tables of 64 features with conjugate gradients: k_rows_cg64, the same over a table of the bfloat16 parts.
+//
+// Bound: issue slots of the solve (d = 64: about 3000 per row) and, for long rows, the mma rate.
 #include "alx_common.cuh"
 #include "alx_mma.cuh"
 #include "alx_ptx.cuh"
