@@ -3,6 +3,7 @@
 // the all-pairs term uses sum_u sum_i <w_u, h_i>^2 = <W^T W, H^T H>_F, the Gramian identity the paper
 // states under Eq. 4 applied to the objective; the regulariser is the trace of the two Gramians.
 #include "alx_common.cuh"
+#include "alx_mma.cuh"
 
 namespace alx {
 
@@ -10,6 +11,10 @@ namespace {
 
 constexpr int kWarps = 8;
 constexpr int kBlocksPerSm = 3;
+// bfloat16 tables of 32 features and more: products by mma (fewer features would leave half of its K empty), two blocks per SM, as 16
+// loads of 16 bytes a lane are in flight
+template <int D, typename T> constexpr bool by_mma() { return sizeof(T) == 2 && D >= 32; }
+template <int D, typename T> constexpr int blocks_per_sm() { return by_mma<D, T>() ? 2 : kBlocksPerSm; }
 constexpr int64_t kMostBlocks = 148 * kBlocksPerSm;
 // Entries a warp takes at a time; the warps then go on together to the next stretch of the matrix, so that at any time they
 // read neighbouring rows of W, and of H where the matrix is local (one long range per warp spread them over the whole table:
@@ -86,13 +91,70 @@ __device__ __forceinline__ double block_sum(double v, double *buf)
     return r;
 }
 
+// The 16 entries from `half` on of the batch by mma.sync m16n8k16: A = their H rows (lane (g, q) = (lane / 4, lane % 4) has the 16-byte
+// pieces q + 4j of rows g and g + 8), B = the W rows of every second entry as columns (pieces alike, so that the features of A
+// and B go by the same permutation), C[e][e / 2] the dot products.  Entries whose row is not the one of the entry before them
+// and have an odd number need their own B: a second set of products, only where there is one.  The products start from zero
+// and are added by FADD, as the instruction truncates its accumulator.  Returns the dot product of entry half + g + 8 (q / 2)
+// to the lanes with q % 2 = g / 4.
+// 27 instructions an entry of 128 features became about 7: MMA_NOTE.
+template <int CH> struct HRows {
+    uint4 a[CH], b[CH];
+};
+template <int CH> __device__ __forceinline__ void load_h(HRows<CH> &h, const __nv_bfloat16 *__restrict__ H, int c, int half, int lane)
+{
+    const int64_t ca = __shfl_sync(0xFFFFFFFFu, c, half + (lane >> 2)), cb = __shfl_sync(0xFFFFFFFFu, c, half + (lane >> 2) + 8);
+#pragma unroll
+    for (int j = 0; j < CH; ++j) {
+        h.a[j] = __ldg(reinterpret_cast<const uint4 *>(H + ca * (32 * CH)) + (lane & 3) + 4 * j);
+        h.b[j] = __ldg(reinterpret_cast<const uint4 *>(H + cb * (32 * CH)) + (lane & 3) + 4 * j);
+    }
+}
+template <int CH> __device__ __forceinline__ void products(const HRows<CH> &h, const uint4 (&w)[CH], float (&d)[4])
+{
+#pragma unroll
+    for (int k = 0; k < 4; ++k) d[k] = 0.f;
+#pragma unroll
+    for (int j = 0; j < CH; ++j) {
+        const uint32_t lo[4] = {h.a[j].x, h.b[j].x, h.a[j].y, h.b[j].y}, hi[4] = {h.a[j].z, h.b[j].z, h.a[j].w, h.b[j].w};
+        float p[4] = {0.f, 0.f, 0.f, 0.f}, r[4] = {0.f, 0.f, 0.f, 0.f};
+        mma_bf16(p, lo, w[j].x, w[j].y);
+        mma_bf16(r, hi, w[j].z, w[j].w);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) d[k] += p[k] + r[k];
+    }
+}
+template <int CH>
+__device__ __forceinline__ float dots(const HRows<CH> &h, const __nv_bfloat16 *__restrict__ W, int row, int half, int &w_row, uint4 (&w)[CH], int lane)
+{
+    const int g = lane >> 2, q = lane & 3;
+    const int even = __shfl_sync(0xFFFFFFFFu, row, half + 2 * g), odd = __shfl_sync(0xFFFFFFFFu, row, half + 2 * g + 1);
+    if (__any_sync(0xFFFFFFFFu, even != w_row)) {
+        w_row = even;
+#pragma unroll
+        for (int j = 0; j < CH; ++j) w[j] = __ldg(reinterpret_cast<const uint4 *>(W + (int64_t)even * (32 * CH)) + q + 4 * j);
+    }
+    float d[4];
+    products(h, w, d);
+    const bool second = (g >> 1) & 1;      // (entry g: column g / 2, entry g + 8: column 4 + g / 2, columns 2q and 2q + 1 are here)
+    float v = q < 2 ? (second ? d[1] : d[0]) : (second ? d[3] : d[2]);
+    if (__any_sync(0xFFFFFFFFu, odd != even)) {
+        w_row = odd;
+#pragma unroll
+        for (int j = 0; j < CH; ++j) w[j] = __ldg(reinterpret_cast<const uint4 *>(W + (int64_t)odd * (32 * CH)) + q + 4 * j);
+        products(h, w, d);
+        if (g & 1) v = q < 2 ? (second ? d[1] : d[0]) : (second ? d[3] : d[2]);
+    }
+    return v;
+}
+
 // A warp takes spans of entries, 32 at a time: every lane looks up its entry's column, label and row (a window of the row offsets,
 // searched by shuffles).  A group of LANES lanes then works through LANES of the entries in turn, 16 bytes of a row a lane, so
 // that the W row stays in registers while the row goes on; four entries' loads are in flight and their sums share a
 // butterfly.  Bound: the latency of the H rows' gather (two rounds in flight, 24 warps per SM), and the 16 instructions an entry of 128 bfloat16 features takes.  The last
 // block to finish adds the blocks' sums in order and the two Gramian terms.
 template <int D, typename T>
-__global__ void __launch_bounds__(kWarps * 32, kBlocksPerSm) k_loss(const int64_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
+__global__ void __launch_bounds__(kWarps * 32, blocks_per_sm<D, T>()) k_loss(const int64_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
                                                       const float *__restrict__ values, int64_t n_rows, int64_t nnz, int span,
                                                       const T *__restrict__ W, const T *__restrict__ H, const double *__restrict__ GW,
                                                       const double *__restrict__ GH, double alpha0, double lambda, double *partials,
@@ -109,6 +171,7 @@ __global__ void __launch_bounds__(kWarps * 32, kBlocksPerSm) k_loss(const int64_
         int64_t u = warp_row_of(rowptr, n_rows, e0, lane);
         int w_row = -1;
         float w[EL];
+        [[maybe_unused]] uint4 wm[D / 32 > 0 ? D / 32 : 1];
         for (int64_t base = e0; base < e1; base += 32) {
             const int64_t e = base + lane;
             const int64_t last = e1 - 1 < base + 31 ? e1 - 1 : base + 31;
@@ -131,6 +194,19 @@ __global__ void __launch_bounds__(kWarps * 32, kBlocksPerSm) k_loss(const int64_
                 at += 32;
             }
             u = __shfl_sync(0xFFFFFFFFu, row, (int)(last - base));
+            if constexpr (by_mma<D, T>()) {
+                HRows<D / 32> h[2];
+                load_h(h[0], H, c, 0, lane);
+                load_h(h[1], H, c, 16, lane);
+#pragma unroll
+                for (int t = 0; t < 2; ++t) {
+                    const float v = dots(h[t], W, (int)row, 16 * t, w_row, wm, lane);
+                    const int k = 16 * t + (lane >> 2) + ((lane & 2) << 2);
+                    const double r = (double)__shfl_sync(0xFFFFFFFFu, y, k) - (double)v;
+                    if ((lane & 1) == lane >> 4 && base + k < e1) acc = fma(r, r, acc);
+                }
+                continue;
+            } else {
             float dot = 0.f;
             uint4 h[2][U];
             auto load = [&](int t0, uint4(&to)[U]) {
@@ -163,6 +239,7 @@ __global__ void __launch_bounds__(kWarps * 32, kBlocksPerSm) k_loss(const int64_
             }
             const double r = (double)y - (double)dot;
             if (e < e1) acc = fma(r, r, acc);
+            }
         }
     }
     const double mine = block_sum(acc, buf);
@@ -208,13 +285,13 @@ cudaError_t launch_loss(const int64_t *rowptr, const int32_t *colidx, const floa
                         const void *H, int bf16, int d, const double *GW, const double *GH, double alpha0, double lambda, double *partials,
                         unsigned *counter, const DevStatus *st, DevStatus *host_status, double *host_result, bool beside_gramian, cudaStream_t s, int64_t *launches)
 {
-    const unsigned grid = (unsigned)loss_partials(nnz);
+    const int64_t partial_sums = loss_partials(nnz);
     // beside_gramian: the launch before this one is the reduction of a Gramian, which starts when the tables are complete and which
     // this kernel waits for at its end
     const bool early = beside_gramian && nnz <= kEarlyEntries;
 #define ALX_LOSS(DD, T)                                                                                                              \
     {                                                                                                                                \
-        const cudaError_t e = launch_early(early, k_loss<DD, T>, grid, kWarps * 32, 0, s, rowptr, colidx, values, n_rows, nnz,       \
+        const cudaError_t e = launch_early(early, k_loss<DD, T>, partial_sums < 148 * blocks_per_sm<DD, T>() ? partial_sums : 148 * blocks_per_sm<DD, T>(), kWarps * 32, 0, s, rowptr, colidx, values, n_rows, nnz,       \
                                            span_of(nnz), (const T *)W, (const T *)H, GW, GH, alpha0, lambda, partials, counter, st,  \
                                            host_status, host_result);                                                                \
         if (e != cudaSuccess) return e;                                                                                              \
