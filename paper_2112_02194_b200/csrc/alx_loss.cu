@@ -11,10 +11,11 @@ namespace {
 
 constexpr int kWarps = 8;
 constexpr int kBlocksPerSm = 3;
-// bfloat16 tables of 32 features and more: products by mma (fewer features would leave half of its K empty), two blocks per SM, as 16
-// loads of 16 bytes a lane are in flight
-template <int D, typename T> constexpr bool by_mma() { return sizeof(T) == 2 && D >= 32; }
-template <int D, typename T> constexpr int blocks_per_sm() { return by_mma<D, T>() ? 2 : kBlocksPerSm; }
+// bfloat16 tables of 128 features: products by mma where rows hold 16 entries or more on average (shorter rows need the second set
+// of products and another load of W rows in most steps: 12 a row 488 us against 471 for 1.2e7 entries, 24 a row 412 against 460,
+// 120 a row 315 against 444; 64 features: 164 against 134 us at 20 a row).  Two blocks per SM: 16 loads of 16 bytes a lane are in flight
+constexpr int64_t kMmaLeastRow = 16;
+constexpr int64_t kMostBlocksMma = 148 * 2;
 constexpr int64_t kMostBlocks = 148 * kBlocksPerSm;
 // Entries a warp takes at a time; the warps then go on together to the next stretch of the matrix, so that at any time they
 // read neighbouring rows of W, and of H where the matrix is local (one long range per warp spread them over the whole table:
@@ -97,7 +98,7 @@ __device__ __forceinline__ double block_sum(double v, double *buf)
 // and have an odd number need their own B: a second set of products, only where there is one.  The products start from zero
 // and are added by FADD, as the instruction truncates its accumulator.  Returns the dot product of entry half + g + 8 (q / 2)
 // to the lanes with q % 2 = g / 4.
-// 27 instructions an entry of 128 features became about 7: MMA_NOTE.
+// 27 instructions an entry became about 7, and the gather through L2 is the bound: 1e9 entries 42 -> 31 ms.
 template <int CH> struct HRows {
     uint4 a[CH], b[CH];
 };
@@ -151,10 +152,10 @@ __device__ __forceinline__ float dots(const HRows<CH> &h, const __nv_bfloat16 *_
 // A warp takes spans of entries, 32 at a time: every lane looks up its entry's column, label and row (a window of the row offsets,
 // searched by shuffles).  A group of LANES lanes then works through LANES of the entries in turn, 16 bytes of a row a lane, so
 // that the W row stays in registers while the row goes on; four entries' loads are in flight and their sums share a
-// butterfly.  Bound: the latency of the H rows' gather (two rounds in flight, 24 warps per SM), and the 16 instructions an entry of 128 bfloat16 features takes.  The last
+// butterfly (with MMA: dots, above).  Bound without MMA: the latency of the H rows' gather (two rounds in flight, 24 warps per SM), and the 16 instructions an entry of 128 bfloat16 features takes.  The last
 // block to finish adds the blocks' sums in order and the two Gramian terms.
-template <int D, typename T>
-__global__ void __launch_bounds__(kWarps * 32, blocks_per_sm<D, T>()) k_loss(const int64_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
+template <int D, typename T, bool MMA>
+__global__ void __launch_bounds__(kWarps * 32, MMA ? 2 : kBlocksPerSm) k_loss(const int64_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
                                                       const float *__restrict__ values, int64_t n_rows, int64_t nnz, int span,
                                                       const T *__restrict__ W, const T *__restrict__ H, const double *__restrict__ GW,
                                                       const double *__restrict__ GH, double alpha0, double lambda, double *partials,
@@ -171,12 +172,28 @@ __global__ void __launch_bounds__(kWarps * 32, blocks_per_sm<D, T>()) k_loss(con
         int64_t u = warp_row_of(rowptr, n_rows, e0, lane);
         int w_row = -1;
         float w[EL];
-        [[maybe_unused]] uint4 wm[D / 32 > 0 ? D / 32 : 1];
+        [[maybe_unused]] uint4 wm[D >= 32 ? D / 32 : 1];
+        // MMA: columns two batches ahead, labels one; the first 16 H rows of a batch are fetched while the batch before it is multiplied
+        [[maybe_unused]] int32_t c0 = 0, c1 = 0;
+        [[maybe_unused]] float y0 = 1.f;
+        [[maybe_unused]] HRows<(D >= 32 ? D / 32 : 1)> h[2];
+        if constexpr (MMA) {
+            c0 = e0 + lane < e1 ? colidx[e0 + lane] : 0;
+            c1 = e0 + 32 + lane < e1 ? colidx[e0 + 32 + lane] : 0;
+            if (values && e0 + lane < e1) y0 = values[e0 + lane];
+            load_h(h[0], H, c0, 0, lane);
+        }
         for (int64_t base = e0; base < e1; base += 32) {
             const int64_t e = base + lane;
             const int64_t last = e1 - 1 < base + 31 ? e1 - 1 : base + 31;
-            const int32_t c = e < e1 ? colidx[e] : 0;
-            const float y = values && e < e1 ? values[e] : 1.f;
+            const int32_t c = MMA ? c0 : e < e1 ? colidx[e] : 0;
+            const float y = MMA ? y0 : values && e < e1 ? values[e] : 1.f;
+            if constexpr (MMA) {
+                load_h(h[1], H, c, 16, lane);
+                c0 = c1;
+                c1 = e + 64 < e1 ? colidx[e + 64] : 0;
+                y0 = values && e + 32 < e1 ? values[e + 32] : 1.f;
+            }
             // row of this lane's entry: count the offsets ptr[u + 1 ..] that are <= e
             int64_t row = u, at = u + 1;
             while (true) {
@@ -194,13 +211,11 @@ __global__ void __launch_bounds__(kWarps * 32, blocks_per_sm<D, T>()) k_loss(con
                 at += 32;
             }
             u = __shfl_sync(0xFFFFFFFFu, row, (int)(last - base));
-            if constexpr (by_mma<D, T>()) {
-                HRows<D / 32> h[2];
-                load_h(h[0], H, c, 0, lane);
-                load_h(h[1], H, c, 16, lane);
+            if constexpr (MMA) {
 #pragma unroll
                 for (int t = 0; t < 2; ++t) {
                     const float v = dots(h[t], W, (int)row, 16 * t, w_row, wm, lane);
+                    if (t == 0 && base + 32 < e1) load_h(h[0], H, c0, 0, lane);
                     const int k = 16 * t + (lane >> 2) + ((lane & 2) << 2);
                     const double r = (double)__shfl_sync(0xFFFFFFFFu, y, k) - (double)v;
                     if ((lane & 1) == lane >> 4 && base + k < e1) acc = fma(r, r, acc);
@@ -208,7 +223,7 @@ __global__ void __launch_bounds__(kWarps * 32, blocks_per_sm<D, T>()) k_loss(con
                 continue;
             } else {
             float dot = 0.f;
-            uint4 h[2][U];
+            uint4 hr[2][U];
             auto load = [&](int t0, uint4(&to)[U]) {
 #pragma unroll
                 for (int k = 0; k < U; ++k) {
@@ -216,10 +231,10 @@ __global__ void __launch_bounds__(kWarps * 32, blocks_per_sm<D, T>()) k_loss(con
                     to[k] = __ldg(reinterpret_cast<const uint4 *>(H + hc * D) + part);
                 }
             };
-            load(0, h[0]);
+            load(0, hr[0]);
 #pragma unroll
             for (int t0 = 0; t0 < LANES; t0 += U) {
-                if (t0 + U < LANES) load(t0 + U, h[(t0 / U + 1) & 1]);      // one round ahead
+                if (t0 + U < LANES) load(t0 + U, hr[(t0 / U + 1) & 1]);      // one round ahead
                 float s[U];
 #pragma unroll
                 for (int k = 0; k < U; ++k) {
@@ -229,7 +244,7 @@ __global__ void __launch_bounds__(kWarps * 32, blocks_per_sm<D, T>()) k_loss(con
                         unpack16(__ldg(reinterpret_cast<const uint4 *>(W + (int64_t)w_row * D) + part), w);
                     }
                     float hv[EL];
-                    unpack16(h[(t0 / U) & 1][k], hv);
+                    unpack16(hr[(t0 / U) & 1][k], hv);
                     s[k] = w[0] * hv[0];
 #pragma unroll
                     for (int j = 1; j < EL; ++j) s[k] = fmaf(w[j], hv[j], s[k]);
@@ -285,21 +300,23 @@ cudaError_t launch_loss(const int64_t *rowptr, const int32_t *colidx, const floa
                         const void *H, int bf16, int d, const double *GW, const double *GH, double alpha0, double lambda, double *partials,
                         unsigned *counter, const DevStatus *st, DevStatus *host_status, double *host_result, bool beside_gramian, cudaStream_t s, int64_t *launches)
 {
-    const int64_t partial_sums = loss_partials(nnz);
+    const int64_t sums = loss_partials(nnz);
     // beside_gramian: the launch before this one is the reduction of a Gramian, which starts when the tables are complete and which
     // this kernel waits for at its end
     const bool early = beside_gramian && nnz <= kEarlyEntries;
-#define ALX_LOSS(DD, T)                                                                                                              \
+#define ALX_LOSS(DD, T, MMA)                                                                                                         \
     {                                                                                                                                \
-        const cudaError_t e = launch_early(early, k_loss<DD, T>, partial_sums < 148 * blocks_per_sm<DD, T>() ? partial_sums : 148 * blocks_per_sm<DD, T>(), kWarps * 32, 0, s, rowptr, colidx, values, n_rows, nnz,       \
+        const int64_t blocks = MMA && sums > kMostBlocksMma ? kMostBlocksMma : sums;                                                 \
+        const cudaError_t e = launch_early(early, k_loss<DD, T, MMA>, blocks, kWarps * 32, 0, s, rowptr, colidx, values, n_rows, nnz, \
                                            span_of(nnz), (const T *)W, (const T *)H, GW, GH, alpha0, lambda, partials, counter, st,  \
                                            host_status, host_result);                                                                \
         if (e != cudaSuccess) return e;                                                                                              \
     }
-#define ALX_CASE(DD)                        \
-    case DD:                                \
-        if (bf16) ALX_LOSS(DD, __nv_bfloat16) \
-        else ALX_LOSS(DD, float)            \
+#define ALX_CASE(DD)                                                       \
+    case DD:                                                               \
+        if (!bf16) ALX_LOSS(DD, float, false)                              \
+        else if (DD == 128 && nnz >= kMmaLeastRow * n_rows) ALX_LOSS(DD, __nv_bfloat16, (DD == 128)) \
+        else ALX_LOSS(DD, __nv_bfloat16, false)                            \
         break;
     switch (d) {
         ALX_CASE(16)
